@@ -249,6 +249,23 @@ int sm_count() {
   return n[dev];
 }
 
+// cudaFuncAttributeMaxDynamicSharedMemorySize belongs to the (kernel, device) pair: set once per device (mu and done
+// belong to the kernel)
+template <typename Kern>
+cudaError_t set_max_smem(Kern kern, int bytes, std::mutex& mu, bool (&done)[kMaxDevices]) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!done[dev]) {
+    const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (r != cudaSuccess) return r;
+    done[dev] = true;
+  }
+  return cudaSuccess;
+}
+
 template <int MODE, int MTOK, bool GRP, bool FQ, bool A16, bool SPLIT, bool SDBG, bool SB = false>
 int launch_stream_s(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
   // cudaFuncAttributeMaxDynamicSharedMemorySize belongs to the (kernel, device) pair: set once per device
@@ -668,6 +685,16 @@ int rcp_ldp_export(const void* w_f16, const float* sig_beta, const float* sig_ga
   lp.N = N; lp.K = K; lp.G = group;
   lp.units = (long long)N * (K / group);
   const int block = 256;
+  if (group == rcp::kLdpGroup) {
+    static std::mutex mu;
+    static bool attr_set[kMaxDevices] = {};
+    RCP_CUDA(set_max_smem(rcp::ldp_export128_kernel, (int)rcp::kLdpSmem, mu, attr_set));
+    const long long tiles = (lp.units + 31) / 32;   // a warp per 32 units, two CTAs per SM
+    const int g128 = (int)std::min<long long>((tiles + rcp::kLdpWarps - 1) / rcp::kLdpWarps, 2 * sm_count());
+    rcp::ldp_export128_kernel<<<g128, rcp::kLdpWarps * 32, rcp::kLdpSmem, static_cast<cudaStream_t>(stream)>>>(lp);
+    RCP_CUDA(cudaGetLastError());
+    return RCP_OK;
+  }
   const long long want = (lp.units + (block / 32) - 1) / (block / 32);
   const int grid = (int)std::min<long long>(want, (long long)sm_count() * 16);
   rcp::ldp_export_kernel<<<grid, block, 0, static_cast<cudaStream_t>(stream)>>>(lp);

@@ -111,6 +111,44 @@ def test_export_directly_followed_by_the_linear_call_on_one_stream(N, K, G, M):
         assert np.all(np.isfinite(got)) and np.all(np.abs(got - ref["y"]) <= ref["tol"]), f"repetition {rep}"
 
 
+@pytest.mark.parametrize("N,K", [(1, 128), (1, 31 * 128), (1, 32 * 128), (3, 11 * 128), (257, 128), (40, 2048)])
+def test_ldp_export_groups_of_128_at_tile_edges_and_hard_thresholds(N, K):
+    """The form for units of 128 compares weights with the smallest fp16 number that reaches each threshold. Unit
+    counts around its tiles of 32; thresholds that are hit exactly, that nothing or everything reaches, ranges so wide
+    that the threshold lies among numbers far smaller than the range's rounding, subnormal ranges, signed zeros."""
+    G = 128
+    w, sb, sg, s1, s2 = _inputs(N, K, G, 5 * N + K)
+    wv = w.view(N * K // G, G)
+    for i in range(wv.shape[0]):
+        a = (sb, sg, s1, s2)
+        flat = [t.view(-1) for t in a]
+        kind = i % 8
+        if kind == 1:      # thresholds 1/4, 5/8, 7/8 of [0, 1] hit exactly
+            wv[i] = (torch.arange(G) % 17 / 16.0).to(torch.float16)
+            flat[0][i] = flat[1][i] = 1.0
+            flat[2][i] = flat[3][i] = 0.5
+        elif kind == 2:    # -60000 .. 60000 with a threshold near zero, met by subnormal weights of both signs
+            wv[i] = (torch.arange(G) - 64).to(torch.float16) * 2.0 ** -24
+            wv[i, 0], wv[i, 1] = -60000.0, 60000.0
+            flat[0][i] = flat[1][i] = 1.0
+            flat[2][i] = 0.999999 if i % 16 == 2 else 1.0
+        elif kind == 3:    # t_1 = 0: everything reaches it; t_3 = 1
+            flat[2][i], flat[3][i] = 0.0, 1.0
+        elif kind == 4:    # subnormal weights only
+            wv[i] = (torch.arange(G) * 7 % 53 - 20).to(torch.float16) * 2.0 ** -24
+        elif kind == 5:    # no range, negative
+            wv[i] = -0.25
+        elif kind == 6:    # zeros of both signs and a positive maximum
+            wv[i] = torch.where(torch.arange(G) % 2 == 0, 0.0, -0.0).to(torch.float16)
+            wv[i, 5] = 0.5
+    ref = oracle.ldp_export(f16_bits(w), sb.numpy(), sg.numpy(), s1.numpy(), s2.numpy(), G)
+    words, lut = rcp.rcp_ldp_export(w.to(DEV), sb.to(DEV), sg.to(DEV), s1.to(DEV), s2.to(DEV), G)
+    assert np.array_equal(words.cpu().numpy().view(np.uint32), oracle.pack_weights(ref["codes"]))
+    # levels bit for bit, except that a zero level may carry either sign (which zero is the minimum is not defined)
+    got = f16_bits(lut)
+    assert np.all((got == ref["lut"]) | (((got | ref["lut"]) & 0x7FFF) == 0))
+
+
 def test_ldp_export_argument_errors():
     L = rcp.lib()
     z = torch.zeros(4096, dtype=torch.int32, device=DEV)
