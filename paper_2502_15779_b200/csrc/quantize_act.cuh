@@ -5,8 +5,8 @@
 // CTAs (1, 2, 4 or 8) shares it, each CTA whole rotation blocks, every thread 8 consecutive
 // elements. The butterfly strides run in ascending order: 1,2,4 inside the thread's registers,
 // 8..128 by warp shuffles, 256 and up through the CTA's shared memory in radix-8 passes. (A rotation
-// block never spans CTAs: one block over a token of 4096 or 8192 elements takes the one-CTA kernel
-// further down, shorter tokens fit one CTA.) Each butterfly is one fp32 add and one fp32 subtract
+// block never spans CTAs: one block over a token of 2048, 4096 or 8192 elements takes a one-CTA kernel
+// further down, as do blocks of at most 512 in most cases.) Each butterfly is one fp32 add and one fp32 subtract
 // (lower index first), then one fp32 multiply by 1/sqrt(B): the rounding order is fixed, so the int4
 // decision is reproducible bit for bit. The token's absmax meets in distributed shared memory.
 #pragma once
@@ -312,34 +312,251 @@ __device__ __forceinline__ float rotate_token_words(const __half* x, int W, floa
   return __half2float(__float2half_rn(s32));
 }
 
-// One CTA of 512 threads per token, for a token of 4096 or 8192 elements under one rotation block:
-// faster than the cluster form above for these shapes (no cluster launch, no passes through
-// distributed shared memory).
-__global__ void __launch_bounds__(512) quantize_act_wide_kernel(const QuantParams p) {
-  extern __shared__ __align__(16) float sbuf[];   // rotate_scratch_bytes(K)
-  __shared__ float s_amax[16];
-  const int m = blockIdx.x, tid = threadIdx.x;
+// ---------------------------------------------------------------------------------------------
+// One CTA per token. The cluster kernel above shares a token out to get at its latency; with many tokens (the
+// activations of a prompt) most of its threads wait at barriers or for the cluster while little else is resident. Here
+// a persistent CTA takes token after token, one thread per word (16 consecutive elements) or two, the next token's
+// activations already on their way, several CTAs per SM, so that one computes while another waits. That is bound by
+// instruction issue (17 to 19 warp instructions per 32 elements against 2.5 bytes per element of traffic), so
+// adds, products and the rounding work on pairs (the two-wide fp32 instructions round each half like the scalar ones)
+// and the clamp of the rounding is left out where it cannot act. Same operations on the same operands in the same
+// order as above: bit-identical results. 2048 tokens, us before (cluster, or one CTA of 512 threads with four barriers)
+// and now, memory floor: K = 4096 27.1, 12.2, 3.3; K = 8192 33.8, 23.9, 6.5; K = 14336 in blocks of 128 78.4, 28.5, 11.4.
+// Fewer barriers also make it the faster form for one token (K = 4096: 2.8 -> 1.8 us).
+
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }   // a - b, rounded once
+
+// the sixteen values of a word, pair i holding elements 2 i and 2 i + 1: the four stages that pair them (strides below B)
+__device__ __forceinline__ void butterflies_word(float2 (&a)[8], int B) {
+  if (B > 1) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      const float u = a[i].x, w = a[i].y;
+      a[i] = make_float2(__fadd_rn(u, w), __fsub_rn(u, w));
+    }
+  }
+#pragma unroll
+  for (int h = 1; h < 8; h *= 2) {
+    if (2 * h < B) {
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        if ((i & h) == 0) {
+          const float2 u = a[i], w = a[i + h];
+          a[i] = add2(u, w);
+          a[i + h] = sub2(u, w);
+        }
+      }
+    }
+  }
+}
+__device__ __forceinline__ void word_from_halves(uint4 r0, uint4 r1, float2 (&v)[8]) {
+  const uint32_t w[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+#pragma unroll
+  for (int i = 0; i < 8; i++) v[i] = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
+}
+// Eight packed nibbles from the fp32 numbers 1.5 * 2^23 + q: the low four bits of the pattern are q's.
+__device__ __forceinline__ uint32_t pack_nibbles(const float2* b) {
+  uint32_t e[4], o[4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) { e[i] = __float_as_uint(b[i].x); o[i] = __float_as_uint(b[i].y); }
+  const uint32_t lo = __byte_perm(__byte_perm(e[0], e[1], 0x0040), __byte_perm(e[2], e[3], 0x0040), 0x5410);
+  const uint32_t hi = __byte_perm(__byte_perm(o[0], o[1], 0x0040), __byte_perm(o[2], o[3], 0x0040), 0x5410);
+  return (lo & 0x0F0F0F0Fu) | ((hi << 4) & 0xF0F0F0F0u);
+}
+// The word's sixteen int4 values for scale s > 0, packed. `clamped` false (the same for the whole warp): the caller
+// knows that |v / s| < 7.5. Then v * (1 / s), rounded to an integer in the same operation, differs by less than 1e-6
+// from the IEEE quotient, so the two round alike unless the remainder is within 4e-6 of a half; such a warp divides.
+// Every lane of the warp must call.
+__device__ __forceinline__ uint2 quantize_word(const float2 (&v)[8], float s, bool clamped) {
+  float2 b[8];
+  bool redo = clamped;
+  if (!clamped) {
+    const float rinv = __frcp_rn(s);
+    const float2 r2 = make_float2(rinv, rinv), magic = make_float2(12582912.f, 12582912.f);
+    const float2 minus = make_float2(-1.f, -1.f);
+    float worst = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      b[i] = __ffma2_rn(v[i], r2, magic);
+      const float2 rest = __ffma2_rn(v[i], r2, __ffma2_rn(b[i], minus, magic));   // (magic - b: minus the integer, exactly)
+      worst = fmaxf(worst, fmaxf(fabsf(rest.x), fabsf(rest.y)));
+    }
+    redo = __any_sync(0xffffffffu, worst > 0.499996f);
+  }
+  if (redo) {
+    float t[16];
+    int q[16];
+#pragma unroll
+    for (int i = 0; i < 8; i++) { t[2 * i] = v[i].x; t[2 * i + 1] = v[i].y; }
+    quantize_int4<16>(t, s, q);
+#pragma unroll
+    for (int i = 0; i < 8; i++) b[i] = make_float2(__int_as_float(q[2 * i] + 0x4B400000), __int_as_float(q[2 * i + 1] + 0x4B400000));
+  }
+  return make_uint2(pack_nibbles(b), pack_nibbles(b + 4));
+}
+// |v| <= amax and s = fp16(amax * clip / 7): with clip >= 0.94 and a normal s, |v / s| <= 7 / 0.94 * (1 + 2^-10) < 7.5.
+__device__ __forceinline__ bool needs_clamp(float clip_ratio, float s) { return !(clip_ratio >= 0.94f && s >= 6.103515625e-5f); }
+
+// Rotation blocks of at most 512 elements (or none): a block lies within a warp (strides 16, 32, .. are lane
+// exchanges), only the token's absmax crosses warps. R words per thread, blockDim.x * R >= K / 16, at most T_MAX threads. BLOCK: the
+// block size where it is known at compile time, 0: p.B.
+template <int R, int T_MAX, int BLOCK>
+__global__ void __launch_bounds__(T_MAX, 1024 / T_MAX) quantize_act_rows_kernel(const QuantParams p, int M) {
+  __shared__ unsigned s_max[2][32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
   asm volatile("griddepcontrol.launch_dependents;");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int W = p.K / 16;
-  float v[16];
-  const float s = rotate_token_words<512>(p.x + (size_t)m * p.K, W, p.inv_sqrt_b, p.clip_ratio, sbuf, s_amax, v);
-  if (tid == 0) p.scale[m] = __float2half_rn(s);
-  int q[16];
-  if (s != 0.f) {   // the same for the whole CTA; threads beyond the token hold zeros
-    quantize_int4<16>(v, s, q);
-  } else {
+  extern __shared__ __align__(16) uint4 s_next[];   // [R][2][T]: the next token's activations; a thread copies its own
+  const int W = p.K / 16, T = blockDim.x, B = BLOCK ? BLOCK : p.B;
+  auto fetch = [&](int m) {
+    const __half* const src = p.x + (size_t)m * p.K;
 #pragma unroll
-    for (int e = 0; e < 16; e++) q[e] = 0;
-  }
-  if (tid < W) {
-    uint32_t lo32 = 0, hi32 = 0;
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-      lo32 |= (uint32_t)(q[e] & 0xF) << (4 * e);
-      hi32 |= (uint32_t)(q[8 + e] & 0xF) << (4 * e);
+    for (int r = 0; r < R; r++) {
+      const int w = r * T + tid;
+      if (w < W) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_next + 2 * r * T + tid);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + 16 * w) : "memory");
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * T), "l"(src + 16 * w + 8) : "memory");
+      }
     }
-    *reinterpret_cast<uint2*>(p.xq + (size_t)m * (p.K / 2) + (size_t)tid * 8) = make_uint2(lo32, hi32);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int i = 0; i < 2 * R; i++) s_next[i * T + tid] = make_uint4(0, 0, 0, 0);   // (threads beyond the token keep zeros)
+  int par = 0;
+  fetch(blockIdx.x);
+  for (int m = blockIdx.x; m < M; m += gridDim.x, par ^= 1) {
+    float2 v[R][8];
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll
+    for (int r = 0; r < R; r++) word_from_halves(s_next[2 * r * T + tid], s_next[(2 * r + 1) * T + tid], v[r]);
+    if (m + (int)gridDim.x < M) fetch(m + gridDim.x);   // (the values above have been read)
+    float amax = 0.f;
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      butterflies_word(v[r], B);
+#pragma unroll
+      for (int d = 1; d < 32; d *= 2) {   // stride 16 d
+        if (16 * d < B) {
+          // lower lane: mine + other; upper lane: other - mine (one rounding either way)
+          const float sign = (lane & d) ? -1.f : 1.f;
+          const float2 s2 = make_float2(sign, sign);
+#pragma unroll
+          for (int i = 0; i < 8; i++) {
+            const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, v[r][i].x, d), __shfl_xor_sync(0xffffffffu, v[r][i].y, d));
+            v[r][i] = __ffma2_rn(v[r][i], s2, other);
+          }
+        }
+      }
+      if (B > 1) {
+        const float2 f2 = make_float2(p.inv_sqrt_b, p.inv_sqrt_b);
+#pragma unroll
+        for (int i = 0; i < 8; i++) v[r][i] = __fmul2_rn(v[r][i], f2);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; i++) amax = fmaxf(amax, fmaxf(fabsf(v[r][i].x), fabsf(v[r][i].y)));
+    }
+    // non-negative floats order like their patterns
+    unsigned am = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
+    if (lane == 0) s_max[par][warp] = am;
+    __syncthreads();   // (the other half of s_max is free: everybody has read it before coming here)
+    am = __reduce_max_sync(0xffffffffu, lane < nwarp ? s_max[par][lane] : 0u);
+    const __half s16 = __float2half_rn(__fdiv_rn(__fmul_rn(__uint_as_float(am), p.clip_ratio), 7.0f));
+    const float s = __half2float(s16);
+    if (tid == 0) p.scale[m] = s16;
+    const bool clamped = needs_clamp(p.clip_ratio, s);
+    uint2* const dst = reinterpret_cast<uint2*>(p.xq + (size_t)m * (p.K / 2));
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const int w = r * T + tid;
+      const uint2 packed = s != 0.f ? quantize_word(v[r], s, clamped) : make_uint2(0, 0);   // (s: the same for the CTA)
+      if (w < W) dst[w] = packed;
+    }
+  }
+}
+
+// One rotation block over the whole token, NT = K / 16 threads (K = 2048, 4096 or 8192). Strides 1..8 inside the word;
+// 16..128 after a transposition inside the warp, 256 by one lane exchange; 512 and up after a transposition across the
+// R = NT / 32 warps, every thread taking 16 / R columns of R values; then back to words, the absmax meeting at the same
+// barrier. The buffer of the cross-warp passes is used in turn with a second one: two barriers per token.
+template <int NT>
+__host__ __device__ constexpr size_t full_rows_smem() { return (size_t)(NT * 17 + 2 * 16 * (NT + 4)) * 4; }
+
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) quantize_act_full_rows_kernel(const QuantParams p, int M) {
+  extern __shared__ __align__(16) float sbuf[];   // full_rows_smem<NT>()
+  constexpr int R = NT / 32, kPitch = 17, QP = NT + 4;
+  __shared__ unsigned s_max[2][R];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  float* const wbuf = sbuf + warp * (32 * kPitch);
+  const int e1 = lane & 15, hi = lane & 16;
+  uint4 raw[2];
+  auto fetch = [&](int m) {
+    const uint4* const src = reinterpret_cast<const uint4*>(p.x + (size_t)m * (NT * 16)) + 2 * tid;
+    raw[0] = __ldg(src);
+    raw[1] = __ldg(src + 1);
+  };
+  int par = 0;
+  fetch(blockIdx.x);
+  for (int m = blockIdx.x; m < M; m += gridDim.x, par ^= 1) {
+    float* const qbuf = sbuf + NT * 17 + par * (16 * QP);
+    float2 v[8];
+    word_from_halves(raw[0], raw[1], v);
+    if (m + (int)gridDim.x < M) fetch(m + gridDim.x);
+    butterflies_word(v, 16);   // strides 1..8
+#pragma unroll
+    for (int i = 0; i < 8; i++) { wbuf[lane * kPitch + 2 * i] = v[i].x; wbuf[lane * kPitch + 2 * i + 1] = v[i].y; }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; i++)   // element e1 of the words hi + 2 i, hi + 2 i + 1
+      v[i] = make_float2(wbuf[(hi | (2 * i)) * kPitch + e1], wbuf[(hi | (2 * i + 1)) * kPitch + e1]);
+    __syncwarp();
+    butterflies_word(v, 16);   // strides 16..128
+    {
+      const float sign = hi ? -1.f : 1.f;
+      const float2 s2 = make_float2(sign, sign);
+#pragma unroll
+      for (int i = 0; i < 8; i++) {   // stride 256
+        const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, v[i].x, 16), __shfl_xor_sync(0xffffffffu, v[i].y, 16));
+        v[i] = __ffma2_rn(v[i], s2, other);
+      }
+    }
+    {
+      float4* const dst = reinterpret_cast<float4*>(qbuf + e1 * QP + warp * 32 + hi);
+#pragma unroll
+      for (int j = 0; j < 4; j++) dst[j] = make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
+    }
+    __syncthreads();
+    float amax = 0.f;
+    // element c R + warp: its R words 32 apart (values 2 i and 2 i + 1 of the thread are words 2 i and 2 i + 1 of R)
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      const float* const col = qbuf + ((2 * i / R) * R + warp) * QP + lane;
+      v[i] = make_float2(col[(2 * i % R) * 32], col[((2 * i + 1) % R) * 32]);
+    }
+    butterflies_word(v, R);   // strides 512 ..
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      v[i] = __fmul2_rn(v[i], make_float2(p.inv_sqrt_b, p.inv_sqrt_b));
+      amax = fmaxf(amax, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
+      float* const col = qbuf + ((2 * i / R) * R + warp) * QP + lane;
+      col[(2 * i % R) * 32] = v[i].x;
+      col[((2 * i + 1) % R) * 32] = v[i].y;
+    }
+    unsigned am = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
+    if (lane == 0) s_max[par][warp] = am;
+    __syncthreads();
+    am = __reduce_max_sync(0xffffffffu, s_max[par][lane % R]);
+    const __half s16 = __float2half_rn(__fdiv_rn(__fmul_rn(__uint_as_float(am), p.clip_ratio), 7.0f));
+    const float s = __half2float(s16);
+    if (tid == 0) p.scale[m] = s16;
+#pragma unroll
+    for (int i = 0; i < 8; i++) v[i] = make_float2(qbuf[2 * i * QP + tid], qbuf[(2 * i + 1) * QP + tid]);
+    const uint2 packed = s != 0.f ? quantize_word(v, s, needs_clamp(p.clip_ratio, s)) : make_uint2(0, 0);
+    reinterpret_cast<uint2*>(p.xq + (size_t)m * (NT * 8))[tid] = packed;
   }
 }
 

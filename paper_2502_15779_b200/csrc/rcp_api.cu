@@ -525,6 +525,58 @@ int static_scratch_address(void** out) {
   return RCP_OK;
 }
 
+// Whether one CTA takes a whole token (quantize_act_rows_kernel, quantize_act_full_rows_kernel) or a cluster shares it.
+// Measured on B200, cluster -> one CTA, us a call. One block over the token: one CTA at any count (K = 4096: 2.8 -> 1.8
+// for one token, 27 -> 12 for 2048). Blocks inside a warp: one CTA up to K = 8192 (2560: 1.95 -> 1.61 and 9.3 -> 6.7;
+// 8064: 2.8 -> 2.1 and 38 -> 19), above that once the tokens fill the GPU better than eight CTAs each would: 11008 and
+// 14336 even at 24 tokens (14336: 3.4 -> 3.6 at 16, 4.25 -> 3.5 at 32, 78 -> 28 at 2048), 28672 at 40 (5.2 -> 5.7
+// at 32, 8.0 -> 5.8 at 64, 178 -> 60 at 2048).
+bool rows_form(int M, int K, int B) {
+  if (B > 512) return B == K && (K == 2048 || K == 4096 || K == 8192);
+  return K <= 8192 || (K <= 16384 && M >= 24) || (K <= 32768 && M >= 40);
+}
+
+template <int NT>
+int launch_full_rows(const rcp::QuantParams& qp, int M, cudaStream_t st) {
+  static std::mutex mu;
+  static bool attr_set[kMaxDevices] = {};
+  auto kern = rcp::quantize_act_full_rows_kernel<NT>;
+  RCP_CUDA(set_max_smem(kern, (int)rcp::full_rows_smem<NT>(), mu, attr_set));
+  const int grid = std::min(M, sm_count() * (1024 / NT));
+  RCP_CUDA(launch_overlapped(kern, dim3(grid), dim3(NT), rcp::full_rows_smem<NT>(), st, qp, M));
+  return RCP_OK;
+}
+
+template <int R, int T_MAX, int BLOCK>
+int launch_block_rows(const rcp::QuantParams& qp, int M, cudaStream_t st) {
+  static std::mutex mu;
+  static bool attr_set[kMaxDevices] = {};
+  auto kern = rcp::quantize_act_rows_kernel<R, T_MAX, BLOCK>;
+  RCP_CUDA(set_max_smem(kern, R * T_MAX * 32, mu, attr_set));
+  const int T = ((qp.K / 16 + R - 1) / R + 31) / 32 * 32;
+  const int grid = std::min(M, sm_count() * std::max(1, 1024 / T));
+  RCP_CUDA(launch_overlapped(kern, dim3(grid), dim3(T), (size_t)R * T * 32, st, qp, M));
+  return RCP_OK;
+}
+
+int launch_quantize_rows(const rcp::QuantParams& qp, int M, cudaStream_t st) {
+  if (qp.B > 512) {
+    if (qp.K == 2048) return launch_full_rows<128>(qp, M, st);
+    if (qp.K == 4096) return launch_full_rows<256>(qp, M, st);
+    return launch_full_rows<512>(qp, M, st);
+  }
+  const int W = qp.K / 16;
+  if (qp.B == 128) {
+    if (W <= 512) return launch_block_rows<1, 512, 128>(qp, M, st);
+    // up to one token per SM a thread per word (14336, 96 tokens: 3.6 us against 4.9 with two words per thread), beyond
+    // that two smaller CTAs per SM (2048 tokens: 28.5 against 30.0)
+    if (W <= 1024 && M <= sm_count()) return launch_block_rows<1, 1024, 128>(qp, M, st);
+    if (W <= 896) return launch_block_rows<2, 448, 128>(qp, M, st);
+    return launch_block_rows<2, 1024, 128>(qp, M, st);
+  }
+  return W <= 512 ? launch_block_rows<1, 512, 0>(qp, M, st) : launch_block_rows<2, 1024, 0>(qp, M, st);
+}
+
 template <bool GRP, bool SDBG>
 int launch_w3(const rcp::W3Params& wp, size_t smem, cudaStream_t st) {
   static std::mutex mu;
@@ -722,14 +774,8 @@ int rcp_quantize_act(const void* x_f16, int M, int K, int had_block, float clip_
   while ((1 << qp.lgB) < B) qp.lgB++;
   qp.inv_sqrt_b = (float)(1.0 / std::sqrt((double)B));
   qp.clip_ratio = clip_ratio;
-  if (B == K && (K == 4096 || K == 8192)) {
-    // one rotation block over a long token: one CTA of 512 threads per token (measured faster than a cluster)
-    qp.unit = K; qp.nunits = 1; qp.lg_local = qp.lgB;
-    RCP_CUDA(launch_overlapped(rcp::quantize_act_wide_kernel, dim3((unsigned)M), dim3(512), rcp::rotate_scratch_bytes(K), st, qp));
-    return RCP_OK;
-  }
-  // whole rotation blocks per CTA (a block is at most 2048 elements here: longer single blocks went above,
-  // and B <= 8192 < K otherwise means at least two blocks)
+  if (rows_form(M, K, B)) return launch_quantize_rows(qp, M, st);
+  // whole rotation blocks per CTA
   int C = 1;
   while (C < 8 && K / (2 * C) >= 2048) C *= 2;
   qp.unit = std::max(B, 64);

@@ -67,6 +67,25 @@ def test_quantize_act_bit_exact(M, K, B, clip):
     assert np.array_equal(xq.cpu().numpy(), ref["xq"])
 
 
+@pytest.mark.parametrize("M,K,B,clip", [
+    (1, 64, 64, 1.0), (2, 576, 2, 0.94), (3, 576, 64, 1.0), (5, 2112, 32, 0.5), (1200, 2048, 2048, 1.0), (600, 4096, 4096, 0.93),
+    (300, 8192, 8192, 1.0), (600, 4096, 128, 1.0), (150, 8192, 512, 1.0), (24, 8320, 128, 1.0), (150, 8704, 128, 0.9),
+    (148, 14336, 128, 1.0), (300, 14336, 128, 1.0), (24, 9216, 512, 1.0), (40, 28672, 128, 1.0), (40, 32768, 1, 1.0)])
+def test_quantize_act_one_cta_per_token(M, K, B, clip):
+    """The kernels with a CTA per token, at the ends of their ranges: token counts around the CTAs of the grid, words
+    that fill no warp, one and two words per thread; all-zero tokens, scales among the fp16 subnormals (where the
+    clamp of the rounding acts) and quotients on and next to ties."""
+    x = synth.make_activations(M, K, 31 * M + K)
+    x[M // 2] = 0
+    if M > 2:
+        x[0] = x[0] * 1e-6                                     # a subnormal scale
+        x[1] = (torch.arange(K) % 15 - 7).to(torch.float16) * 0.5   # with no rotation: halves of the scale, ties
+    ref = oracle.quantize_act(f16_bits(x), B, clip)
+    xq, scale = rcp.rcp_quantize_act(x.to(DEV), B, clip)
+    assert np.array_equal(f16_bits(scale), ref["scale"])
+    assert np.array_equal(xq.cpu().numpy(), ref["xq"])
+
+
 def test_quantize_act_zero_token_and_errors():
     x = synth.make_activations(3, 512, seed=1)
     x[1] = 0
