@@ -303,12 +303,12 @@ int rcp_gemv_w2a4_grouped_variant(int variant, const uint32_t* words, const void
  * == 0) or rcp_gemv_w2a4_grouped (group > 0), same arguments, same results bit for bit in xq and
  * scale and within the GEMV's tolerance in y (Section 4.4 data path; Appendix A.7 counts the
  * separate activation quantizer as the overhead this removes).
- *   For one token of 4096 or 8192 elements under one rotation block (had_block == K) and group in
- *   {0, 128}, a single kernel does both: every CTA rotates and quantizes the token itself while its
- *   first weight requests are in flight (measured faster than two kernels for these shapes only).
- *   xq and scale_f16 are then optional outputs (NULL: not written). Every other case runs the two
- *   kernels one after the other and needs xq [M][K/2] and scale_f16 [M] as staging: RCP_ERR_NULL
- *   without them.
+ *   For one token under one rotation block of 2048, 4096 or 8192 elements (had_block == K), or in blocks
+ *   of at most 512 with K <= 16384, and group in {0, 128}, a single kernel does both: every CTA rotates
+ *   and quantizes the token itself while its first weight requests are in flight (measured faster than
+ *   two kernels for these shapes). Every other case runs the two kernels one after the other.
+ *   xq [M][K/2] and scale_f16 [M] are written either way. They may be NULL only for one token of 4096 or
+ *   8192 elements under one block; RCP_ERR_NULL otherwise.
  *   x_f16 obeys stream order; words and lut_f16 are layer constants (see rcp_gemv_w2a4).
  * Never synchronizes.
  */

@@ -334,9 +334,9 @@ def rcp_gemv_w2a4_static(words, lut, xq, scale, y=None):
 def rcp_linear_w2a4(x, had_block, clip_ratio, words, lut, group=0, y=None, xq=None, scale=None, workspace=None,
                     S_dbg=None):
     """x fp16 [M][K] -> y fp16 [M][N]: activation quantization and LUT GEMV in one call (one kernel for
-    one token of 4096 or 8192 under one rotation block). lut fp16 [N][4] with group=0, [N][K/group][4]
-    otherwise. xq / scale: optional outputs on the one-kernel path, required staging otherwise (pass them to
-    be safe). S_dbg int32 [M][N][4] ([M][N][K/group][4]): the integer sums, from the checked instantiation
+    most one-token shapes). lut fp16 [N][4] with group=0, [N][K/group][4]
+    otherwise. xq / scale: optional for one token of 4096 or 8192 under one rotation block, required otherwise (pass
+    them to be safe). S_dbg int32 [M][N][4] ([M][N][K/group][4]): the integer sums, from the checked instantiation
     of the kernel that runs anyway."""
     _dev(x, torch.float16, "x")
     _dev(words, torch.int32, "words")

@@ -113,8 +113,9 @@ struct GemvParams {
   const __half* x;
   uint8_t* xq_out;      // optional [M][K/2]: the int4 activations, written by CTA 0
   __half* scale_out;    // optional [M]
-  float inv_sqrt_b, clip_ratio;   // the rotation block is the whole token, K = 4096 or 8192
-  int off_qbuf;         // the quantizer's scratch (rotate_scratch_bytes(K)) in shared memory
+  float inv_sqrt_b, clip_ratio;
+  int had_block;        // rotation block (1: none)
+  int off_qbuf;         // the scratch of a rotation over the whole token (full_rotate_bytes(K)) in shared memory
   int stages;           // ring depth
   int ramp_clk;         // clocks between the first `stages` requests of a CTA
   int off_bar, off_T0c, off_scale, off_red, off_bs;   // shared-memory byte offsets from the aligned base
@@ -233,13 +234,12 @@ __global__ void wait_timeout_kernel(int32_t* status, uint32_t polls) {
 // MTOK  tokens, fixed at compile time for the dp4a modes (1 or 2); kModeMma: 0 = run-time, up to 8; 8 = exactly eight
 //       (one MMA column tile), 16 = run-time, 9 to 16 (two column tiles fed from the same masks)
 // GRP   one grid per group of 128 weights instead of one per row (kModeHybrid has no such form)
-// FQ    one token of 4096 or 8192 activations under one rotation block: the activations arrive as
-//       fp16 and every CTA rotates and quantizes them itself (Appendix A.2, Section 4.4), in the
-//       arithmetic order of the stand-alone quantizer: bit-identical int4 values. For these shapes
-//       (where the stand-alone kernel needs a cluster and passes through distributed shared memory)
-//       it costs less than a kernel of its own. A thread takes one word (16 consecutive activations):
-//       strides 1..8 in registers, 16..256 by lane exchanges, 512 and up through shared memory, one
-//       thread per (lane, element) column over the warps.
+// FQ    one token arriving as fp16: every CTA rotates and quantizes it itself (Appendix A.2, Section 4.4), in the
+//       arithmetic order of the stand-alone quantizer: bit-identical int4 values. The arithmetic is done 148 times over,
+//       but the launch in front, its end and the way of xq through memory are on the critical path of a decode step, and
+//       the weights are on their way meanwhile. FQ = 4, 8, 16: one rotation block over the token of 512 FQ elements, FQ
+//       elements per thread (rotate_full_token); FQ = -1, -2: blocks of at most 512 elements, up to -FQ
+//       words of 16 per thread (rotate_block_token). 0: xq and scale are inputs.
 // A16   weight-only form: the "tokens" are the four base-64 fixed-point digits of up to two (MTOK 16: four)
 //       fp16 tokens, one signed byte per element (p.xq is [4 tokens][K] bytes, p.unit their fp32 units, p.M
 //       the number of digit columns); the digits of a token are combined in fp32 when its rows are finished.
@@ -253,7 +253,7 @@ __global__ void wait_timeout_kernel(int32_t* status, uint32_t polls) {
 //       consumers like the producer does. The token count and K then no longer meet in shared memory: no K in
 //       parts, up to sixteen tokens for any K, and the expansion (2 us at eight tokens of 8192) leaves the
 //       critical path. The host keeps (warps sharing a group) x tokens at 32 or less per stage.
-template <int MODE, int MTOK, bool GRP, bool FQ = false, bool A16 = false, bool SPLIT = false, bool SDBG = false,
+template <int MODE, int MTOK, bool GRP, int FQ = 0, bool A16 = false, bool SPLIT = false, bool SDBG = false,
           bool SB = false>
 __global__ void __launch_bounds__(SB ? kGThreads + 32 * kExpWarps : kGThreads, 1)
 gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
@@ -265,16 +265,16 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   const int g = lane >> 2, t = lane & 3;
   const int M = (MTOK > 0 && MTOK != 16) ? MTOK : p.M;   // (kModeMma with MTOK 8: exactly eight tokens, known at compile time)
   constexpr bool kTwoTiles = (MODE == kModeMma && MTOK == 16);   // tokens 8..15 in a second set of accumulators
-  static_assert(!(kTwoTiles && (GRP || FQ)), "two column tiles: per-row grid, quantized activations only");
-  static_assert(!A16 || (MODE == kModeMma && !GRP && !FQ), "digit columns: tensor-core mode, per-row grid");
+  static_assert(!(kTwoTiles && (GRP || FQ != 0)), "two column tiles: per-row grid, quantized activations only");
+  static_assert(!A16 || (MODE == kModeMma && !GRP && FQ == 0), "digit columns: tensor-core mode, per-row grid");
   // Long K with several tokens: the expanded activations of the whole K do not fit in shared memory. The kernel
   // then goes through K in nsplit parts: activations of the part expanded, every phase run over the part's
   // chunks, the integer sums of this CTA's rows parked in shared memory until the last part finishes them. The
   // plan is the same for every part, so the same lane meets the same sums again: nothing crosses warps.
   // A form of its own, so that the kernels that never need it keep their code.
   constexpr bool kSplit = SPLIT;
-  static_assert(!SPLIT || (MODE == kModeMma && MTOK == 0 && !GRP && !FQ), "K in parts: eight-column tensor-core kernels, per-row grid");
-  static_assert(!SB || (MODE == kModeMma && !FQ && !A16 && !SPLIT), "streamed activations: tensor-core kernels");
+  static_assert(!SPLIT || (MODE == kModeMma && MTOK == 0 && !GRP && FQ == 0), "K in parts: eight-column tensor-core kernels, per-row grid");
+  static_assert(!SB || (MODE == kModeMma && FQ == 0 && !A16 && !SPLIT), "streamed activations: tensor-core kernels");
   constexpr int kThreads = SB ? kGThreads + 32 * kExpWarps : kGThreads;   // consumers, producer warp, and the expander warps (SB)
   const uint32_t stage_stride = SB ? (uint32_t)p.stage_stride : (uint32_t)kStageBytes;
   const int nsplit = kSplit ? p.nsplit : 1;
@@ -477,67 +477,98 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   const int nch = kSplit ? min(p.nchunk, p.nchunk_total - chunk0) : p.nchunk;
   if (kp > 0) asm volatile("bar.sync 1, %0;" ::"n"(kCWarps * 32) : "memory");        // every warp is done with the last part's activations
   // ------------------------------------------------------------------ fused quantizer (consumer warps)
-  if constexpr (FQ) {
-    static_assert(!FQ || (MODE == kModeDp4a && MTOK == 1), "the fused quantizer serves the one-token kernels");
-    constexpr int NT = kCWarps * 32;
-    const int W = p.K / 16;                                           // 256 or 512 words: one per thread
-    float* const qbuf = reinterpret_cast<float*>(gen + p.off_qbuf);   // rotate_scratch_bytes(K)
-    float* const s_amax = s_scale + 16;                               // [16 warps] behind the scales
-    float v[16];
-    const float sc = rotate_token_words<NT>(p.x, W, p.inv_sqrt_b, p.clip_ratio, qbuf, s_amax, v);
+  // Bytes of a word's position p, even positions times 4: where word w's four 32-bit operands go in the expanded
+  // activations of one token (position p at + {0, 8, 64, 72}).
+  auto act_slot = [&](int w) { return bs + (size_t)(((w >> 5) * 4 + ((w >> 1) & 3)) * 2) * 64 + ((w >> 3) & 3) * 16 + (w & 1) * 4; };
+  if constexpr (FQ != 0) {
+    static_assert(FQ == 0 || (MODE == kModeDp4a && MTOK == 1), "the fused quantizer serves the one-token kernels");
+    static_assert(kCWarps == 16, "512 threads share the rotation");
+    unsigned* const s_amax = reinterpret_cast<unsigned*>(s_scale + 16);   // [16 warps] behind the scales
+    const int W = p.K / 16;
+    constexpr int NR = FQ > 0 ? 1 : -FQ;           // words (or parts of one) per thread
+    constexpr int E = FQ > 0 ? FQ : 16;            // elements of each
+    constexpr int NP = E / 2;
+    float2 v[NR][NP];
+    float amax;
+    if constexpr (FQ > 0) amax = rotate_full_token<E>(p.x, p.inv_sqrt_b, reinterpret_cast<float*>(gen + p.off_qbuf), s_amax, v[0]);
+    else amax = rotate_block_token<NR>(p.x, W, p.had_block, p.inv_sqrt_b, s_amax, v);
+    const __half s16 = __float2half_rn(__fdiv_rn(__fmul_rn(amax, p.clip_ratio), 7.0f));
+    const float sc = __half2float(s16);
     if (tid == 0) {
       s_scale[0] = sc;
-      if (b == 0 && p.scale_out) p.scale_out[0] = __float2half_rn(sc);
+      if (b == 0 && p.scale_out) p.scale_out[0] = s16;
     }
-    int q[16];
-    int tsum = 0;
-    if (sc != 0.f) {   // the same for the whole CTA; threads beyond the token hold zeros
-      quantize_int4<16>(v, sc, q);
-    } else {
+    const bool clamped = needs_clamp(p.clip_ratio, sc);
+    int total = 0;
 #pragma unroll
-      for (int e = 0; e < 16; e++) q[e] = 0;
-    }
+    for (int r = 0; r < NR; r++) {
+      const int first = (r * 512 + tid) * E, w = first >> 4;   // this thread's elements: first .. first + E - 1
+      if (r * 512 + warp * 32 < p.nchunk * (kChunkWords * 16 / E)) {   // (whole warps; the last chunk is padded with zeros)
+        float2 f[NP];   // 1.5 * 2^23 + q: the low byte of the pattern is q's
+        if (sc != 0.f) {   // the same for the whole CTA; words beyond the token hold zeros
+          quantize_pairs<NP>(v[r], sc, clamped, f);
+        } else {
 #pragma unroll
-    for (int e = 0; e < 16; e++) tsum += q[e];
-    const int ch = tid >> 5, wi = tid & 31;
-    if (tid < p.nchunk * kChunkWords) {
-      uint32_t Q[4];
+          for (int i = 0; i < NP; i++) f[i] = make_float2(12582912.f, 12582912.f);
+        }
+        // position p of the E / 4 bytes of codes: elements p, 4 + p, ..
+        uint32_t Q[4];
 #pragma unroll
-      for (int pp = 0; pp < 4; pp++) {
-        const int m = (pp & 1) ? 1 : 4;   // even positions carry 4 q
-        Q[pp] = (uint32_t)((q[pp] * m) & 0xFF) | ((uint32_t)((q[4 + pp] * m) & 0xFF) << 8) |
-                ((uint32_t)((q[8 + pp] * m) & 0xFF) << 16) | ((uint32_t)((q[12 + pp] * m) & 0xFF) << 24);
+        for (int pp = 0; pp < 4; pp++) {
+          uint32_t d[E / 4];
+#pragma unroll
+          for (int j = 0; j < E / 4; j++) {
+            const float2 fp = f[2 * j + (pp >> 1)];
+            d[j] = __float_as_uint((pp & 1) ? fp.y : fp.x);
+          }
+          if constexpr (E == 16) Q[pp] = __byte_perm(__byte_perm(d[0], d[1], 0x0040), __byte_perm(d[2], d[3], 0x0040), 0x5410);
+          else if constexpr (E == 8) Q[pp] = __byte_perm(d[0], d[1], 0x0040) & 0xFFFFu;
+          else Q[pp] = d[0] & 0xFFu;
+        }
+        int tsum = 0;
+#pragma unroll
+        for (int pp = 0; pp < 4; pp++) tsum = __dp4a((int)Q[pp], 0x01010101, tsum);   // (absent bytes are zeros)
+        const uint32_t E0 = (Q[0] << 2) & 0xFCFCFCFCu, E2 = (Q[2] << 2) & 0xFCFCFCFCu;
+        uint8_t* const dst = act_slot(w) + ((first >> 2) & 3);
+        if (RCP_CK(dst >= bs && dst + 72 + E / 4 <= bs + p.bs_bytes, 2)) {
+          if constexpr (E == 16) {
+            *reinterpret_cast<uint32_t*>(dst) = E0;
+            *reinterpret_cast<uint32_t*>(dst + 8) = Q[1];
+            *reinterpret_cast<uint32_t*>(dst + 64) = E2;
+            *reinterpret_cast<uint32_t*>(dst + 72) = Q[3];
+          } else if constexpr (E == 8) {
+            *reinterpret_cast<uint16_t*>(dst) = (uint16_t)E0;
+            *reinterpret_cast<uint16_t*>(dst + 8) = (uint16_t)Q[1];
+            *reinterpret_cast<uint16_t*>(dst + 64) = (uint16_t)E2;
+            *reinterpret_cast<uint16_t*>(dst + 72) = (uint16_t)Q[3];
+          } else {
+            dst[0] = (uint8_t)E0;
+            dst[8] = (uint8_t)Q[1];
+            dst[64] = (uint8_t)E2;
+            dst[72] = (uint8_t)Q[3];
+          }
+        }
+        if (b == 0 && p.xq_out && w < W) {
+          uint8_t* const xo = p.xq_out + (first >> 1);
+          if constexpr (E == 16) *reinterpret_cast<uint2*>(xo) = make_uint2(pack_nibbles(f), pack_nibbles(f + 4));
+          else if constexpr (E == 8) *reinterpret_cast<uint32_t*>(xo) = pack_nibbles(f);
+          else *reinterpret_cast<uint16_t*>(xo) = (uint16_t)((Q[0] & 0xFu) | (Q[1] & 0xFu) << 4 | (Q[2] & 0xFu) << 8 | (Q[3] & 0xFu) << 12);
+        }
+        // sums of q: 128 / E lanes hold a group of 128
+        if constexpr (GRP) {
+#pragma unroll
+          for (int d = 1; d < 128 / E; d *= 2) tsum += __shfl_xor_sync(0xffffffffu, tsum, d);
+          if (lane % (128 / E) == 0) s_T0c[first >> 7] = tsum;
+        } else {
+          total += tsum;
+        }
       }
-      uint8_t* dst = bs + (size_t)((ch * 4 + ((wi >> 1) & 3)) * 2) * 64 + (wi >> 3) * 16 + (wi & 1) * 4;
-      if (RCP_CK(dst >= bs && dst + 64 + 12 <= bs + p.bs_bytes, 2)) {
-        *reinterpret_cast<uint32_t*>(dst) = Q[0];
-        *reinterpret_cast<uint32_t*>(dst + 8) = Q[1];
-        *reinterpret_cast<uint32_t*>(dst + 64) = Q[2];
-        *reinterpret_cast<uint32_t*>(dst + 64 + 8) = Q[3];
-      }
     }
-    if (b == 0 && p.xq_out && tid < W) {
-      uint32_t lo32 = 0, hi32 = 0;
-#pragma unroll
-      for (int e = 0; e < 8; e++) {
-        lo32 |= (uint32_t)(q[e] & 0xF) << (4 * e);
-        hi32 |= (uint32_t)(q[8 + e] & 0xF) << (4 * e);
-      }
-      *reinterpret_cast<uint2*>(p.xq_out + (size_t)tid * 8) = make_uint2(lo32, hi32);
-    }
-    // sums of q: a warp holds exactly one chunk (32 consecutive words), eight lanes one group of 128
-    tsum += __shfl_xor_sync(0xffffffffu, tsum, 1);
-    tsum += __shfl_xor_sync(0xffffffffu, tsum, 2);
-    tsum += __shfl_xor_sync(0xffffffffu, tsum, 4);
-    if constexpr (GRP) {
-      if ((lane & 7) == 0 && ch < p.nchunk) s_T0c[tid >> 3] = tsum;
-    } else {
-      tsum += __shfl_xor_sync(0xffffffffu, tsum, 8);
-      tsum += __shfl_xor_sync(0xffffffffu, tsum, 16);
-      if (lane == 0 && ch < p.nchunk) atomicAdd(&s_T0tot[0], tsum);
-    }
-    if constexpr (!GRP)
+    if constexpr (!GRP) {
+      total = __reduce_add_sync(0xffffffffu, total);
+      if (lane == 0) atomicAdd(&s_T0tot[0], total);
       for (int i = tid; i < 2 * 8 * 16 * M * 3; i += kCWarps * 32) s_red[i] = 0;
+    }
   } else if constexpr (SB && GRP) {
     // Streamed activations, group-wise grid: the sum of q of every (token, group of 128) is needed up front, as
     // 8 x the sum in fp32 (what the finish works with). A group is 64 bytes of packed activations.

@@ -192,127 +192,6 @@ __global__ void __launch_bounds__(1024) quantize_act_kernel(const QuantParams p)
 }
 
 // ---------------------------------------------------------------------------------------------
-// One token of W = K / 16 words (256 or 512) under a single rotation block, by NT = 512 threads of one
-// CTA: thread tid holds word tid (16 consecutive activations). Every butterfly stage runs in registers, the
-// data changing hands through shared memory in between, in ascending order of the strides (the order of
-// quantize_act_kernel: same operations on the same operands, bit-identical results):
-//   strides 1..8      inside the word;
-//   strides 16..128   after a transposition inside the warp (thread (h, e) of a warp, h = lane >> 4,
-//                     e = lane & 15, takes element e of the warp's words 16 h .. 16 h + 15);
-//   stride 256        one lane exchange (lane ^ 16);
-//   strides 512 ..    after a transposition across the warps (thread (warp = element, lane) takes the
-//                     R = W / 32 values of its column, 32 words apart);
-// then the scale by 1/sqrt(K) and the token's absmax. Leaves the rotated, scaled activations of the thread's
-// word in v and returns the quantization scale (as rounded to fp16). Uses named barrier 1 with NT threads;
-// qbuf: rotate_scratch_bytes(K) bytes, 16-byte aligned; s_amax: NT / 32 floats.
-__host__ __device__ constexpr size_t rotate_scratch_bytes(int K) { return (size_t)17 * (K / 16) * 4; }
-
-template <int NT>
-__device__ __forceinline__ float rotate_token_words(const __half* x, int W, float inv_sqrt_b, float clip_ratio,
-                                                    float* qbuf, float* s_amax, float (&v)[16]) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kPitch = 17;   // rows of the in-warp transposition: 16 floats and one of padding (no bank conflicts)
-  const int QP = W + 4;        // pitch of the cross-warp buffer [16 elements][W words]: the 16-byte stores of eight
-                               // lanes with different elements then fall into different banks
-  if (tid < W) {
-    const uint4* src = reinterpret_cast<const uint4*>(x + (size_t)tid * 16);
-    const uint4 r0 = __ldg(src), r1 = __ldg(src + 1);
-    const __half2* h0 = reinterpret_cast<const __half2*>(&r0);
-    const __half2* h1 = reinterpret_cast<const __half2*>(&r1);
-#pragma unroll
-    for (int e = 0; e < 4; e++) {
-      const float2 f0 = __half22float2(h0[e]), f1 = __half22float2(h1[e]);
-      v[2 * e] = f0.x; v[2 * e + 1] = f0.y; v[8 + 2 * e] = f1.x; v[8 + 2 * e + 1] = f1.y;
-    }
-  } else {
-#pragma unroll
-    for (int e = 0; e < 16; e++) v[e] = 0.f;
-  }
-  // sixteen values in registers: the four stages that pair them
-  auto butterflies16 = [](float (&a)[16]) {
-#pragma unroll
-    for (int h = 1; h < 16; h *= 2) {
-#pragma unroll
-      for (int e = 0; e < 16; e++) {
-        if ((e & h) == 0) {
-          const float u = a[e], w = a[e + h];
-          a[e] = __fadd_rn(u, w);
-          a[e + h] = __fsub_rn(u, w);
-        }
-      }
-    }
-  };
-  butterflies16(v);   // strides 1..8
-  const bool data_warp = warp * 32 < W;   // (W is a multiple of 256: a warp holds 32 words or none)
-  const int e1 = lane & 15, hi = lane & 16;
-  float u[16];
-#pragma unroll
-  for (int j = 0; j < 16; j++) u[j] = 0.f;
-  if (data_warp) {
-    float* const wbuf = qbuf + warp * (32 * kPitch);
-#pragma unroll
-    for (int e = 0; e < 16; e++) wbuf[lane * kPitch + e] = v[e];
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < 16; j++) u[j] = wbuf[(hi | j) * kPitch + e1];   // element e1 of the words hi + j
-    butterflies16(u);   // strides 16..128
-#pragma unroll
-    for (int j = 0; j < 16; j++) {   // stride 256
-      const float other = __shfl_xor_sync(0xffffffffu, u[j], 16);
-      u[j] = hi ? __fsub_rn(other, u[j]) : __fadd_rn(u[j], other);
-    }
-  }
-  asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");   // every warp is done with its transposition area
-  if (data_warp) {   // u[j]: element e1 of word warp * 32 + hi + j
-    float4* const dst = reinterpret_cast<float4*>(qbuf + e1 * QP + warp * 32 + hi);
-#pragma unroll
-    for (int j = 0; j < 4; j++) dst[j] = make_float4(u[4 * j], u[4 * j + 1], u[4 * j + 2], u[4 * j + 3]);
-  }
-  asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
-  {
-    const int R = W >> 5;   // 8 or 16 warps hold data
-    float* const colp = qbuf + warp * QP + lane;
-    float tv[16];
-#pragma unroll
-    for (int w = 0; w < 16; w++) tv[w] = (w < R) ? colp[w * 32] : 0.f;
-#pragma unroll
-    for (int h = 1; h < 16; h *= 2) {
-      if (h < R) {
-#pragma unroll
-        for (int w = 0; w < 16; w++) {
-          if ((w & h) == 0) {
-            const float a = tv[w], z = tv[w + h];
-            tv[w] = __fadd_rn(a, z);
-            tv[w + h] = __fsub_rn(a, z);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int w = 0; w < 16; w++) if (w < R) colp[w * 32] = tv[w];
-  }
-  asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
-  if (tid < W) {
-#pragma unroll
-    for (int e = 0; e < 16; e++) v[e] = qbuf[e * QP + tid];
-  }
-  float amax = 0.f;
-#pragma unroll
-  for (int e = 0; e < 16; e++) {
-    v[e] = __fmul_rn(v[e], inv_sqrt_b);
-    amax = fmaxf(amax, fabsf(v[e]));
-  }
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
-  if (lane == 0) s_amax[warp] = amax;
-  asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
-#pragma unroll
-  for (int w = 0; w < NT / 32; w++) amax = fmaxf(amax, s_amax[w]);
-  const float s32 = __fdiv_rn(__fmul_rn(amax, clip_ratio), 7.0f);
-  return __half2float(__float2half_rn(s32));
-}
-
-// ---------------------------------------------------------------------------------------------
 // One CTA per token. The cluster kernel above shares a token out to get at its latency; with many tokens (the
 // activations of a prompt) most of its threads wait at barriers or for the cluster while little else is resident. Here
 // a persistent CTA takes token after token, one thread per word (16 consecutive elements) or two, the next token's
@@ -364,12 +243,12 @@ __device__ __forceinline__ uint32_t pack_nibbles(const float2* b) {
   const uint32_t hi = __byte_perm(__byte_perm(o[0], o[1], 0x0040), __byte_perm(o[2], o[3], 0x0040), 0x5410);
   return (lo & 0x0F0F0F0Fu) | ((hi << 4) & 0xF0F0F0F0u);
 }
-// The word's sixteen int4 values for scale s > 0, packed. `clamped` false (the same for the whole warp): the caller
-// knows that |v / s| < 7.5. Then v * (1 / s), rounded to an integer in the same operation, differs by less than 1e-6
-// from the IEEE quotient, so the two round alike unless the remainder is within 4e-6 of a half; such a warp divides.
-// Every lane of the warp must call.
-__device__ __forceinline__ uint2 quantize_word(const float2 (&v)[8], float s, bool clamped) {
-  float2 b[8];
+// Rounds NP pairs of values over s > 0 to int4, as the fp32 numbers 1.5 * 2^23 + q. `clamped` false (the same for the
+// whole warp): the caller knows that |v / s| < 7.5. Then v * (1 / s), rounded to an integer in the same operation,
+// differs by less than 1e-6 from the IEEE quotient, so the two round alike unless the remainder is within 4e-6 of a
+// half; such a warp divides. Every lane of the warp must call.
+template <int NP>
+__device__ __forceinline__ void quantize_pairs(const float2 (&v)[NP], float s, bool clamped, float2 (&b)[NP]) {
   bool redo = clamped;
   if (!clamped) {
     const float rinv = __frcp_rn(s);
@@ -377,7 +256,7 @@ __device__ __forceinline__ uint2 quantize_word(const float2 (&v)[8], float s, bo
     const float2 minus = make_float2(-1.f, -1.f);
     float worst = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; i++) {
+    for (int i = 0; i < NP; i++) {
       b[i] = __ffma2_rn(v[i], r2, magic);
       const float2 rest = __ffma2_rn(v[i], r2, __ffma2_rn(b[i], minus, magic));   // (magic - b: minus the integer, exactly)
       worst = fmaxf(worst, fmaxf(fabsf(rest.x), fabsf(rest.y)));
@@ -385,18 +264,40 @@ __device__ __forceinline__ uint2 quantize_word(const float2 (&v)[8], float s, bo
     redo = __any_sync(0xffffffffu, worst > 0.499996f);
   }
   if (redo) {
-    float t[16];
-    int q[16];
+    float t[2 * NP];
+    int q[2 * NP];
 #pragma unroll
-    for (int i = 0; i < 8; i++) { t[2 * i] = v[i].x; t[2 * i + 1] = v[i].y; }
-    quantize_int4<16>(t, s, q);
+    for (int i = 0; i < NP; i++) { t[2 * i] = v[i].x; t[2 * i + 1] = v[i].y; }
+    quantize_int4<2 * NP>(t, s, q);
 #pragma unroll
-    for (int i = 0; i < 8; i++) b[i] = make_float2(__int_as_float(q[2 * i] + 0x4B400000), __int_as_float(q[2 * i + 1] + 0x4B400000));
+    for (int i = 0; i < NP; i++) b[i] = make_float2(__int_as_float(q[2 * i] + 0x4B400000), __int_as_float(q[2 * i + 1] + 0x4B400000));
   }
+}
+// The word's sixteen int4 values, packed.
+__device__ __forceinline__ uint2 quantize_word(const float2 (&v)[8], float s, bool clamped) {
+  float2 b[8];
+  quantize_pairs<8>(v, s, clamped, b);
   return make_uint2(pack_nibbles(b), pack_nibbles(b + 4));
 }
 // |v| <= amax and s = fp16(amax * clip / 7): with clip >= 0.94 and a normal s, |v / s| <= 7 / 0.94 * (1 + 2^-10) < 7.5.
 __device__ __forceinline__ bool needs_clamp(float clip_ratio, float s) { return !(clip_ratio >= 0.94f && s >= 6.103515625e-5f); }
+
+// Strides of 16 and up inside a warp whose lanes hold one word each, below B
+__device__ __forceinline__ void butterflies_lanes(float2 (&v)[8], int B, int lane) {
+#pragma unroll
+  for (int d = 1; d < 32; d *= 2) {   // stride 16 d
+    if (16 * d < B) {
+      // lower lane: mine + other; upper lane: other - mine (one rounding either way)
+      const float sign = (lane & d) ? -1.f : 1.f;
+      const float2 s2 = make_float2(sign, sign);
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, v[i].x, d), __shfl_xor_sync(0xffffffffu, v[i].y, d));
+        v[i] = __ffma2_rn(v[i], s2, other);
+      }
+    }
+  }
+}
 
 // Rotation blocks of at most 512 elements (or none): a block lies within a warp (strides 16, 32, .. are lane
 // exchanges), only the token's absmax crosses warps. R words per thread, blockDim.x * R >= K / 16, at most T_MAX threads. BLOCK: the
@@ -436,19 +337,7 @@ __global__ void __launch_bounds__(T_MAX, 1024 / T_MAX) quantize_act_rows_kernel(
 #pragma unroll
     for (int r = 0; r < R; r++) {
       butterflies_word(v[r], B);
-#pragma unroll
-      for (int d = 1; d < 32; d *= 2) {   // stride 16 d
-        if (16 * d < B) {
-          // lower lane: mine + other; upper lane: other - mine (one rounding either way)
-          const float sign = (lane & d) ? -1.f : 1.f;
-          const float2 s2 = make_float2(sign, sign);
-#pragma unroll
-          for (int i = 0; i < 8; i++) {
-            const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, v[r][i].x, d), __shfl_xor_sync(0xffffffffu, v[r][i].y, d));
-            v[r][i] = __ffma2_rn(v[r][i], s2, other);
-          }
-        }
-      }
+      butterflies_lanes(v[r], B, lane);
       if (B > 1) {
         const float2 f2 = make_float2(p.inv_sqrt_b, p.inv_sqrt_b);
 #pragma unroll
@@ -558,6 +447,160 @@ __global__ void __launch_bounds__(NT, 1024 / NT) quantize_act_full_rows_kernel(c
     const uint2 packed = s != 0.f ? quantize_word(v, s, needs_clamp(p.clip_ratio, s)) : make_uint2(0, 0);
     reinterpret_cast<uint2*>(p.xq + (size_t)m * (NT * 8))[tid] = packed;
   }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The rotation of one token by 512 threads inside another kernel (the GEMV's in-kernel quantizer), latency bound: as few
+// barriers as possible and all threads at work. Same operations in the same order as above: bit-identical results.
+
+// One rotation block over the whole token of K = 512 E elements (E = 4, 8 or 16): thread t holds the elements t E ..
+// t E + E - 1 on return, rotated and scaled, and the token's absmax is returned (the same bits in every thread). Strides
+// below E in registers; the next log2 E after a transposition inside the warp; up to 16 E by lane exchanges; the sixteen
+// warps' strides after a transposition across the warps: there a column of sixteen values, one per warp, is shared by
+// 16 / E lanes, E values each, and a last lane exchange or two. Two barriers (named barrier 1, 512 threads).
+// buf: full_rotate_bytes<E>() bytes, 16-byte aligned; s_amax: 16 words.
+//   Cross-warp buffer: element e of lane l of warp w at e kQP + 32 w + (w / E) kPL + l. The pads make every access below
+// free of bank conflicts.
+template <int E>
+struct FullRotate {
+  static constexpr int kP = E + 1;              // pitch of the in-warp transposition
+  static constexpr int kPL = 2 * E;             // the lanes that share a column are kPL apart
+  static constexpr int kQP = E == 16 ? 516 : E == 8 ? 548 : 552;
+  static constexpr size_t kBytes = (size_t)(512 * kP + E * kQP) * 4;
+};
+__host__ constexpr size_t full_rotate_bytes(int K) {
+  return K == 2048 ? FullRotate<4>::kBytes : K == 4096 ? FullRotate<8>::kBytes : FullRotate<16>::kBytes;
+}
+
+// the stages that pair 2 NP register values (strides 1 .. NP)
+template <int NP>
+__device__ __forceinline__ void butterflies_pairs(float2 (&a)[NP]) {
+#pragma unroll
+  for (int i = 0; i < NP; i++) {
+    const float u = a[i].x, w = a[i].y;
+    a[i] = make_float2(__fadd_rn(u, w), __fsub_rn(u, w));
+  }
+#pragma unroll
+  for (int h = 1; h < NP; h *= 2) {
+#pragma unroll
+    for (int i = 0; i < NP; i++) {
+      if ((i & h) == 0) {
+        const float2 u = a[i], w = a[i + h];
+        a[i] = add2(u, w);
+        a[i + h] = sub2(u, w);
+      }
+    }
+  }
+}
+template <int NP>
+__device__ __forceinline__ void butterfly_exchange(float2 (&a)[NP], int d, bool upper) {
+  const float sign = upper ? -1.f : 1.f;
+  const float2 s2 = make_float2(sign, sign);
+#pragma unroll
+  for (int i = 0; i < NP; i++) {
+    const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, a[i].x, d), __shfl_xor_sync(0xffffffffu, a[i].y, d));
+    a[i] = __ffma2_rn(a[i], s2, other);
+  }
+}
+
+template <int E>
+__device__ __forceinline__ float rotate_full_token(const __half* x, float inv_sqrt_b, float* buf, unsigned* s_amax,
+                                                   float2 (&v)[E / 2]) {
+  using F = FullRotate<E>;
+  constexpr int NP = E / 2;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* const wbuf = buf + warp * (32 * F::kP);
+  float* const qbuf = buf + 512 * F::kP;
+  {
+    uint32_t raw[NP];
+    if constexpr (E == 4) {
+      const uint2 r = __ldg(reinterpret_cast<const uint2*>(x) + tid);
+      raw[0] = r.x; raw[1] = r.y;
+    } else {
+#pragma unroll
+      for (int i = 0; i < E / 8; i++) {
+        const uint4 r = __ldg(reinterpret_cast<const uint4*>(x) + tid * (E / 8) + i);
+        raw[4 * i] = r.x; raw[4 * i + 1] = r.y; raw[4 * i + 2] = r.z; raw[4 * i + 3] = r.w;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NP; i++) v[i] = __half22float2(*reinterpret_cast<const __half2*>(&raw[i]));
+  }
+  butterflies_pairs<NP>(v);   // strides 1 .. E / 2
+#pragma unroll
+  for (int i = 0; i < NP; i++) { wbuf[lane * F::kP + 2 * i] = v[i].x; wbuf[lane * F::kP + 2 * i + 1] = v[i].y; }
+  __syncwarp();
+  const int e1 = lane % E, l1 = lane - e1;   // this lane: element e1 of the lanes l1 .. l1 + E - 1
+#pragma unroll
+  for (int i = 0; i < NP; i++) v[i] = make_float2(wbuf[(l1 + 2 * i) * F::kP + e1], wbuf[(l1 + 2 * i + 1) * F::kP + e1]);
+  butterflies_pairs<NP>(v);   // strides E .. E E / 2
+#pragma unroll
+  for (int d = E; d < 32; d *= 2) butterfly_exchange<NP>(v, d, (lane & d) != 0);   // .. 16 E
+  {
+    float4* const dst = reinterpret_cast<float4*>(qbuf + e1 * F::kQP + warp * 32 + (warp / E) * F::kPL + l1);
+#pragma unroll
+    for (int j = 0; j < E / 4; j++) dst[j] = make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
+  }
+  asm volatile("bar.sync 1, 512;" ::: "memory");
+  {
+    constexpr int kLC = 16 / E;              // warps that share an element's columns, and lanes that share a column
+    const int wq = lane / F::kPL;            // this lane: the values of the warps wq E .. wq E + E - 1
+    float* const col = qbuf + (warp / kLC) * F::kQP + wq * (E * 32 + F::kPL) + (warp % kLC) * F::kPL + lane % F::kPL;
+#pragma unroll
+    for (int i = 0; i < NP; i++) v[i] = make_float2(col[2 * i * 32], col[(2 * i + 1) * 32]);
+    butterflies_pairs<NP>(v);
+#pragma unroll
+    for (int d = F::kPL; d < 32; d *= 2) butterfly_exchange<NP>(v, d, (lane & d) != 0);
+    float amax = 0.f;
+#pragma unroll
+    for (int i = 0; i < NP; i++) {
+      v[i] = __fmul2_rn(v[i], make_float2(inv_sqrt_b, inv_sqrt_b));
+      amax = fmaxf(amax, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
+      col[2 * i * 32] = v[i].x;
+      col[(2 * i + 1) * 32] = v[i].y;
+    }
+    const unsigned am = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));   // non-negative: ordered like the patterns
+    if (lane == 0) s_amax[warp] = am;
+  }
+  asm volatile("bar.sync 1, 512;" ::: "memory");
+  const float* const mine = qbuf + warp * 32 + (warp / E) * F::kPL + lane;
+#pragma unroll
+  for (int i = 0; i < NP; i++) v[i] = make_float2(mine[2 * i * F::kQP], mine[(2 * i + 1) * F::kQP]);
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, s_amax[lane & 15]));
+}
+
+// Rotation blocks of B <= 512 elements (1: none): thread t takes the words t, t + 512, .. (NR at most) of the token's W;
+// words beyond it are zeros. Returns the token's absmax; one barrier.
+template <int NR>
+__device__ __forceinline__ float rotate_block_token(const __half* x, int W, int B, float inv_sqrt_b, unsigned* s_amax,
+                                                    float2 (&v)[NR][8]) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint4 raw[NR][2];
+#pragma unroll
+  for (int r = 0; r < NR; r++) {
+    const int w = r * 512 + tid;
+    raw[r][0] = raw[r][1] = make_uint4(0, 0, 0, 0);
+    if (w < W) { raw[r][0] = __ldg(reinterpret_cast<const uint4*>(x) + 2 * w); raw[r][1] = __ldg(reinterpret_cast<const uint4*>(x) + 2 * w + 1); }
+  }
+  float amax = 0.f;
+#pragma unroll
+  for (int r = 0; r < NR; r++) {
+    word_from_halves(raw[r][0], raw[r][1], v[r]);
+    if (r * 512 + warp * 32 < W) {   // (whole warps)
+      butterflies_word(v[r], B);
+      butterflies_lanes(v[r], B, lane);
+      if (B > 1) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) v[r][i] = __fmul2_rn(v[r][i], make_float2(inv_sqrt_b, inv_sqrt_b));
+      }
+#pragma unroll
+      for (int i = 0; i < 8; i++) amax = fmaxf(amax, fmaxf(fabsf(v[r][i].x), fabsf(v[r][i].y)));
+    }
+  }
+  const unsigned am = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
+  if (lane == 0) s_amax[warp] = am;
+  asm volatile("bar.sync 1, 512;" ::: "memory");
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, s_amax[lane & 15]));
 }
 
 }  // namespace rcp

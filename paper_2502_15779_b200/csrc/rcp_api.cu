@@ -266,7 +266,7 @@ cudaError_t set_max_smem(Kern kern, int bytes, std::mutex& mu, bool (&done)[kMax
   return cudaSuccess;
 }
 
-template <int MODE, int MTOK, bool GRP, bool FQ, bool A16, bool SPLIT, bool SDBG, bool SB = false>
+template <int MODE, int MTOK, bool GRP, int FQ, bool A16, bool SPLIT, bool SDBG, bool SB = false>
 int launch_stream_s(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
   // cudaFuncAttributeMaxDynamicSharedMemorySize belongs to the (kernel, device) pair: set once per device
   static std::mutex mu;
@@ -289,12 +289,12 @@ int launch_stream_s(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const 
 // streamed activations (tensor-core kernels of the per-row grid; MTOK 0: up to eight tokens, 16: nine to sixteen)
 template <int MTOK>
 int launch_stream_sb(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
-  if (gp.S_out) return launch_stream_s<rcp::kModeMma, MTOK, false, false, false, false, true, true>(maps, gp, pl, st);
-  return launch_stream_s<rcp::kModeMma, MTOK, false, false, false, false, false, true>(maps, gp, pl, st);
+  if (gp.S_out) return launch_stream_s<rcp::kModeMma, MTOK, false, 0, false, false, true, true>(maps, gp, pl, st);
+  return launch_stream_s<rcp::kModeMma, MTOK, false, 0, false, false, false, true>(maps, gp, pl, st);
 }
 
 // gp.S_out set: the checked instantiation of the same kernel, which also stores its integer sums.
-template <int MODE, int MTOK, bool GRP = false, bool FQ = false, bool A16 = false, bool SPLIT = false>
+template <int MODE, int MTOK, bool GRP = false, int FQ = 0, bool A16 = false, bool SPLIT = false>
 int launch_stream_t(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
   if (gp.S_out) return launch_stream_s<MODE, MTOK, GRP, FQ, A16, SPLIT, true>(maps, gp, pl, st);
   return launch_stream_s<MODE, MTOK, GRP, FQ, A16, SPLIT, false>(maps, gp, pl, st);
@@ -311,9 +311,6 @@ struct FusedAct {
   void* scale_out;       // optional
 };
 
-// Shapes the in-kernel quantizer takes: one token of 4096 or 8192 elements under one rotation block.
-// Measured on B200: there the fused kernel beats the two kernels by 0.7 to 1.9 us a call; for shorter
-// tokens, block-wise rotation or two tokens the stand-alone quantizer (several CTAs per token) wins.
 // Weight-only form, activations still in fp16: the GEMV kernel makes the digit planes itself.
 struct SplitAct {
   const void* x_f16;    // [tokens][K]
@@ -321,7 +318,24 @@ struct SplitAct {
   float* unit_out;      // [tokens][4], written by CTA 0
 };
 
-bool fused_ok(int M, int K, int B) { return M == 1 && B == K && (K == 4096 || K == 8192); }
+// Shapes the in-kernel quantizer takes: one token under one rotation block of 2048, 4096 or 8192 elements, or in blocks
+// of at most 512 with K up to 16384. Measured on B200, us a call in a chain of calls, cold weights, two kernels -> one:
+// 2048x2048 3.95 -> 2.74, 4096x4096 5.4 -> 3.9, 57344x8192 33.4 -> 31.6, 333x5184 4.6 -> 3.6, 4096x14336 9.6 -> 8.4.
+// At K = 28672 (four words per thread) the stand-alone quantizer's cluster of eight CTAs is faster than all CTAs doing
+// the whole token (8192x28672 21.6 -> 22.3), and two tokens are twice the serial work.
+bool full_block(int K, int B) { return B == K && (K == 2048 || K == 4096 || K == 8192); }
+bool fused_ok(int M, int K, int B) { return M == 1 && (full_block(K, B) || (B <= 512 && K <= 16384)); }
+
+template <bool GRP>
+int launch_fused(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
+  if (full_block(gp.K, gp.had_block)) {
+    if (gp.K == 2048) return launch_stream_t<rcp::kModeDp4a, 1, GRP, 4>(maps, gp, pl, st);
+    if (gp.K == 4096) return launch_stream_t<rcp::kModeDp4a, 1, GRP, 8>(maps, gp, pl, st);
+    return launch_stream_t<rcp::kModeDp4a, 1, GRP, 16>(maps, gp, pl, st);
+  }
+  if (gp.K <= 8192) return launch_stream_t<rcp::kModeDp4a, 1, GRP, -1>(maps, gp, pl, st);
+  return launch_stream_t<rcp::kModeDp4a, 1, GRP, -2>(maps, gp, pl, st);
+}
 
 int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16,
                   int M, int N, int K, void* y_f16, void* workspace, cudaStream_t st, bool grouped = false,
@@ -338,7 +352,7 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
   if (fa && (mode != rcp::kModeDp4a || !fused_ok(M, K, fa->B))) return RCP_ERR_VARIANT;
   EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return cuda_fail(cudaErrorNotSupported);
-  const StreamPlan pl = make_plan(M, N, K, sm_count(), grouped, fa ? rcp::rotate_scratch_bytes(K) : (sa ? (size_t)M * K : 0), nsplit,
+  const StreamPlan pl = make_plan(M, N, K, sm_count(), grouped, fa ? (full_block(K, fa->B) ? rcp::full_rotate_bytes(K) : 0) : (sa ? (size_t)M * K : 0), nsplit,
                                   stream_act);
   if (pl.stages < 2 || pl.smem > kSmemMax) return RCP_ERR_SHAPE;
   // Tensor maps of the phases in use (the others repeat the first). Encoding one costs the host about a
@@ -401,35 +415,35 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
   gp.stage_stride = pl.stage_stride;
   gp.off_qbuf = pl.off_qbuf;
   gp.x = nullptr; gp.xq_out = nullptr; gp.scale_out = nullptr; gp.unit_out = nullptr;
-  gp.inv_sqrt_b = 1.f; gp.clip_ratio = 1.f;
+  gp.inv_sqrt_b = 1.f; gp.clip_ratio = 1.f; gp.had_block = 1;
   if (fa) {
     gp.x = static_cast<const __half*>(fa->x_f16);
     gp.xq_out = fa->xq_out;
     gp.scale_out = static_cast<__half*>(fa->scale_out);
     gp.inv_sqrt_b = (float)(1.0 / std::sqrt((double)fa->B));
     gp.clip_ratio = fa->clip_ratio;
-    return grouped ? launch_stream_t<rcp::kModeDp4a, 1, true, true>(maps, gp, pl, st)
-                   : launch_stream_t<rcp::kModeDp4a, 1, false, true>(maps, gp, pl, st);
+    gp.had_block = fa->B;
+    return grouped ? launch_fused<true>(maps, gp, pl, st) : launch_fused<false>(maps, gp, pl, st);
   }
   if (sa) {
     gp.x = static_cast<const __half*>(sa->x_f16);
     gp.xq_out = reinterpret_cast<uint8_t*>(sa->digits_out);
     gp.unit_out = sa->unit_out;
-    return launch_stream_t<rcp::kModeMma, 0, false, false, true>(maps, gp, pl, st);
+    return launch_stream_t<rcp::kModeMma, 0, false, 0, true>(maps, gp, pl, st);
   }
   if (unit) {
-    if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, false, true, true>(maps, gp, pl, st);
-    return M > 8 ? launch_stream_t<rcp::kModeMma, 16, false, false, true>(maps, gp, pl, st)
-                 : launch_stream_t<rcp::kModeMma, 0, false, false, true>(maps, gp, pl, st);
+    if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, 0, true, true>(maps, gp, pl, st);
+    return M > 8 ? launch_stream_t<rcp::kModeMma, 16, false, 0, true>(maps, gp, pl, st)
+                 : launch_stream_t<rcp::kModeMma, 0, false, 0, true>(maps, gp, pl, st);
   }
   if (grouped) {
     if (mode == rcp::kModeDp4a)
       return M == 1 ? launch_stream_t<rcp::kModeDp4a, 1, true>(maps, gp, pl, st)
                     : launch_stream_t<rcp::kModeDp4a, 2, true>(maps, gp, pl, st);
     if (stream_act)
-      return gp.S_out ? launch_stream_s<rcp::kModeMma, 0, true, false, false, false, true, true>(maps, gp, pl, st)
-                      : launch_stream_s<rcp::kModeMma, 0, true, false, false, false, false, true>(maps, gp, pl, st);
-    if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, true, false, false, false, false>(maps, gp, pl, st);
+      return gp.S_out ? launch_stream_s<rcp::kModeMma, 0, true, 0, false, false, true, true>(maps, gp, pl, st)
+                      : launch_stream_s<rcp::kModeMma, 0, true, 0, false, false, false, true>(maps, gp, pl, st);
+    if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, true, 0, false, false, false>(maps, gp, pl, st);
     return launch_stream_t<rcp::kModeMma, 0, true>(maps, gp, pl, st);
   }
   if (mode == rcp::kModeHybrid)
@@ -442,8 +456,8 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
     if (M == 8 && !gp.S_out) return launch_stream_sb<8>(maps, gp, pl, st);
     return M > 8 ? launch_stream_sb<16>(maps, gp, pl, st) : launch_stream_sb<0>(maps, gp, pl, st);
   }
-  if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, false, false, true>(maps, gp, pl, st);
-  if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, false, false, false, false, false>(maps, gp, pl, st);   // token count known at compile time
+  if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, 0, false, true>(maps, gp, pl, st);
+  if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, false, 0, false, false, false>(maps, gp, pl, st);   // token count known at compile time
   return M > 8 ? launch_stream_t<rcp::kModeMma, 16>(maps, gp, pl, st) : launch_stream_t<rcp::kModeMma, 0>(maps, gp, pl, st);
 }
 
@@ -1057,6 +1071,7 @@ int rcp_linear_w2a4_checked(const void* x_f16, int M, int K, int had_block, floa
     return RCP_ERR_ALIGN;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (!workspace) return RCP_ERR_WORKSPACE;
+  if (!(M == 1 && B == K && (K == 4096 || K == 8192)) && (!xq || !scale_f16)) return RCP_ERR_NULL;
   if (fused_ok(M, K, B) && (group == 0 || group == 128)) {
     const FusedAct fa{x_f16, B, clip_ratio, xq, scale_f16};
     return launch_stream(rcp::kModeDp4a, words, lut_f16, nullptr, nullptr, M, N, K, y_f16, workspace, st, group == 128,

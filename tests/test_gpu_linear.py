@@ -70,6 +70,29 @@ def test_linear_matches_oracle(N, K, B, M, group):
     _check(N, K, B, M, group, 1.0, seed=N + K + M + group, kind="rotated_laplace" if K >= 512 else "uniform")
 
 
+@pytest.mark.parametrize("group", [0, 128])
+@pytest.mark.parametrize("N,K,B,clip", [(37, 128, 1, 1.0), (37, 640, 64, 0.9), (50, 2048, 2048, 0.9), (37, 8064, 128, 1.0),
+                                        (37, 8192, 512, 1.0), (37, 8320, 128, 0.94), (37, 16384, 256, 0.5), (2400, 2560, 2, 1.0),
+                                        (37, 4096, 4096, 0.93), (37, 8192, 8192, 1.0)])
+def test_linear_one_kernel_forms(N, K, B, clip, group):
+    """The in-kernel quantizer at the ends of its ranges: words that fill no warp and no chunk, one and two words per
+    thread, every thread layout of the single block; clip ratios on both sides of the clamp."""
+    _check(N, K, B, 1, group, clip, seed=7 * N + K + B)
+    assert rcp.rcp_linear_w2a4_launches(1, N, K, B, group) == 1
+    # a token of zeros and one whose scale is an fp16 subnormal
+    codes, lut = synth.make_layer(N, K, B, "uniform", 3, device=DEV)
+    words = rcp.rcp_pack_weights(codes)
+    for factor in (0.0, 2.0 ** -22):
+        x = synth.make_activations(1, K, 12, device=DEV) * factor
+        xq = torch.empty(1, K // 2, dtype=torch.uint8, device=DEV)
+        scale = torch.empty(1, dtype=torch.float16, device=DEV)
+        y = rcp.rcp_linear_w2a4(x, B, clip, words, lut, xq=xq, scale=scale)
+        qa = oracle.quantize_act(f16_bits(x), B, clip)
+        assert np.array_equal(xq.cpu().numpy(), qa["xq"]) and np.array_equal(f16_bits(scale), qa["scale"])
+        y2 = rcp.rcp_gemv_w2a4(words, lut, xq, scale)
+        assert torch.equal(y.view(torch.int16), y2.view(torch.int16))
+
+
 def test_linear_clip_ratio_zero_token_and_optional_outputs():
     _check(70, 2048, 2048, 2, 0, 0.9, seed=3)
     _check(70, 4096, 4096, 1, 0, 0.9, seed=5)
