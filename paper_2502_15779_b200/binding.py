@@ -1,11 +1,13 @@
 """Thin Python binding over the C ABI declared in include/rcp.h.
 
 Argument marshalling only: tensors are allocated by torch (device memory and streams), every
-computation runs in the library's CUDA kernels.  There is no fallback: if the shared library
-is missing or a call fails, an exception is raised.
+computation runs in the library's CUDA kernels.  The calls of a decode step are marshalled in native
+code (csrc/binding.cpp, the module _marshal), the offline ones here with ctypes.  There is no fallback:
+if the shared library or the module is missing or a call fails, an exception is raised.
 """
 import contextlib
 import ctypes as C
+import importlib.util
 import os
 
 import torch
@@ -19,6 +21,10 @@ VARIANTS = {"auto": GEMV_AUTO, "simple": GEMV_SIMPLE, "dp4a": GEMV_DP4A, "mma": 
             "mma_stream": GEMV_MMA_STREAM}
 
 _lib = None
+_m = None   # the native marshalling module, bound to _lib
+_MARSHAL_PATH = os.path.join(_HERE, "_marshal.so")
+_MARSHALLED = ("rcp_quantize_act", "rcp_gemv_w2a4_variant", "rcp_gemv_w2a4_grouped_variant", "rcp_gemv_w2a16_checked",
+               "rcp_gemv_w3a4", "rcp_linear_w2a4_checked", "rcp_linear_w2a4_host")
 
 
 class RcpError(RuntimeError):
@@ -82,6 +88,21 @@ def lib():
         L.rcp_linear_w2a4_checked.argtypes = [vp, i, i, i, C.c_float, vp, vp, i, i, vp, vp, vp, vp, vp, vp]
         _lib = L
     return _lib
+
+
+def _native():
+    """The marshalling module, loaded and bound to the library on first use."""
+    global _m
+    if _m is None:
+        L = lib()
+        if not os.path.exists(_MARSHAL_PATH):
+            raise RuntimeError(f"{_MARSHAL_PATH} not found: build it with `python -m paper_2502_15779_b200.build`")
+        spec = importlib.util.spec_from_file_location(__package__ + "._marshal", _MARSHAL_PATH)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        m.bind({name: C.cast(getattr(L, name), C.c_void_p).value for name in _MARSHALLED})
+        _m = m
+    return _m
 
 
 def _check(fn, status):
@@ -171,16 +192,16 @@ def rcp_nf3_export(w, sig_beta, sig_gamma, sig_s1, table, zero_index, group):
 
 def rcp_quantize_act(x: torch.Tensor, had_block: int, clip_ratio: float = 1.0, xq=None, scale=None):
     """x fp16 [M][K] -> (xq uint8 [M][K/2], scale fp16 [M])."""
-    _dev(x, torch.float16, "x")
-    M, K = x.shape
-    if xq is None:
-        xq = torch.empty((M, K // 2), dtype=torch.uint8, device=x.device)
-    if scale is None:
-        scale = torch.empty((M,), dtype=torch.float16, device=x.device)
-    with _on(x):
-        _check("rcp_quantize_act",
-               lib().rcp_quantize_act(_ptr(x), M, K, int(had_block), float(clip_ratio), _ptr(xq), _ptr(scale),
-                                      _stream(x)))
+    if xq is None or scale is None:
+        _dev(x, torch.float16, "x")
+        M, K = x.shape
+        if xq is None:
+            xq = torch.empty((M, K // 2), dtype=torch.uint8, device=x.device)
+        if scale is None:
+            scale = torch.empty((M,), dtype=torch.float16, device=x.device)
+    st = (_m or _native()).quantize_act(x, had_block, clip_ratio, xq, scale)
+    if st:
+        _check("rcp_quantize_act", st)
     return xq, scale
 
 
@@ -194,51 +215,42 @@ def make_workspace(M: int, N: int, K: int, device) -> torch.Tensor:
     return torch.zeros((n + 3) // 4, dtype=torch.int32, device=device)
 
 
+def _variant(variant):
+    return VARIANTS[variant] if isinstance(variant, str) else int(variant)
+
+
 def rcp_gemv_w2a4(words, lut, xq, scale, y=None, workspace=None, S_dbg=None, variant="auto"):
     """words int32 [N][K/16], lut fp16 [N][4], xq uint8 [M][K/2], scale fp16 [M] -> y fp16 [M][N]."""
+    if y is None or workspace is None:
+        y, workspace = _results(words, xq, y, workspace)
+    st = (_m or _native()).gemv_w2a4(_variant(variant), words, lut, 0, xq, scale, y, workspace, S_dbg)
+    if st:
+        _check("rcp_gemv_w2a4", st)
+    return y
+
+
+def _results(words, x, y, workspace):
+    """The buffers a caller did not pass: y fp16 [M][N] and the workspace."""
     _dev(words, torch.int32, "words")
-    _dev(lut, torch.float16, "lut")
-    _dev(xq, torch.uint8, "xq")
-    _dev(scale, torch.float16, "scale")
-    N, W = words.shape
-    K = W * 16
-    M = xq.shape[0]
-    if xq.shape != (M, K // 2) or lut.shape != (N, 4) or scale.shape != (M,):
-        raise ValueError("shape mismatch between words, lut, xq and scale")
+    N, K = words.shape[0], words.shape[1] * 16
+    M = x.shape[0]
     if y is None:
         y = torch.empty((M, N), dtype=torch.float16, device=words.device)
     if workspace is None and rcp_gemv_workspace_bytes(M, N, K) > 0:
         workspace = make_workspace(M, N, K, words.device)
-    v = VARIANTS[variant] if isinstance(variant, str) else int(variant)
-    with _on(words):
-        _check("rcp_gemv_w2a4",
-               lib().rcp_gemv_w2a4_variant(v, _ptr(words), _ptr(lut), _ptr(xq), _ptr(scale), M, N, K, _ptr(y),
-                                           _ptr(workspace), _ptr(S_dbg), _stream(words)))
-    return y
+    return y, workspace
 
 
 def rcp_gemv_w2a4_grouped(words, lut, xq, scale, group=128, y=None, workspace=None, S_dbg=None, variant="auto"):
     """Group-wise grid: words int32 [N][K/16], lut fp16 [N][K/group][4], xq uint8 [M][K/2], scale fp16 [M]
     -> y fp16 [M][N]. S_dbg: int32 [M][N][K/group][4]."""
-    _dev(words, torch.int32, "words")
-    _dev(lut, torch.float16, "lut")
-    _dev(xq, torch.uint8, "xq")
-    _dev(scale, torch.float16, "scale")
-    N, W = words.shape
-    K = W * 16
-    M = xq.shape[0]
-    group = int(group)
-    if group < 1 or K % group or xq.shape != (M, K // 2) or lut.shape != (N, K // group, 4) or scale.shape != (M,):
+    if int(group) < 1:
         raise ValueError("shape mismatch between words, lut, group, xq and scale")
-    if y is None:
-        y = torch.empty((M, N), dtype=torch.float16, device=words.device)
-    if workspace is None and rcp_gemv_workspace_bytes(M, N, K) > 0:
-        workspace = make_workspace(M, N, K, words.device)
-    v = VARIANTS[variant] if isinstance(variant, str) else int(variant)
-    with _on(words):
-        _check("rcp_gemv_w2a4_grouped",
-               lib().rcp_gemv_w2a4_grouped_variant(v, _ptr(words), _ptr(lut), group, _ptr(xq), _ptr(scale), M, N, K,
-                                                   _ptr(y), _ptr(workspace), _ptr(S_dbg), _stream(words)))
+    if y is None or workspace is None:
+        y, workspace = _results(words, xq, y, workspace)
+    st = (_m or _native()).gemv_w2a4(_variant(variant), words, lut, int(group), xq, scale, y, workspace, S_dbg)
+    if st:
+        _check("rcp_gemv_w2a4_grouped", st)
     return y
 
 
@@ -246,26 +258,15 @@ def rcp_gemv_w2a16(words, lut, x, y=None, digits=None, unit=None, workspace=None
     """Weight-only form: words int32 [N][K/16], lut fp16 [N][4], x fp16 [M][K] -> y fp16 [M][N].
     digits int8 [M][4][K] and unit fp32 [M][4] receive the fixed-point form of x the kernels used.
     S_dbg int32 [4 M][N][4]: the per-code sums of every digit plane (checked instantiation of the kernel)."""
-    _dev(words, torch.int32, "words")
-    _dev(lut, torch.float16, "lut")
-    _dev(x, torch.float16, "x")
-    N, W = words.shape
-    K = W * 16
-    M = x.shape[0]
-    if x.shape != (M, K) or lut.shape != (N, 4):
-        raise ValueError("shape mismatch between words, lut and x")
-    if y is None:
-        y = torch.empty((M, N), dtype=torch.float16, device=words.device)
+    if y is None or workspace is None:
+        y, workspace = _results(words, x, y, workspace)
     if digits is None:
-        digits = torch.empty((M, 4, K), dtype=torch.int8, device=words.device)
+        digits = torch.empty((x.shape[0], 4, x.shape[1]), dtype=torch.int8, device=words.device)
     if unit is None:
-        unit = torch.empty((M, 4), dtype=torch.float32, device=words.device)
-    if workspace is None:
-        workspace = make_workspace(M, N, K, words.device)
-    with _on(words):
-        _check("rcp_gemv_w2a16",
-               lib().rcp_gemv_w2a16_checked(_ptr(words), _ptr(lut), _ptr(x), M, N, K, _ptr(y), _ptr(digits), _ptr(unit),
-                                            _ptr(workspace), _ptr(S_dbg), _stream(words)))
+        unit = torch.empty((x.shape[0], 4), dtype=torch.float32, device=words.device)
+    st = (_m or _native()).gemv_w2a16(words, lut, x, y, digits, unit, workspace, S_dbg)
+    if st:
+        _check("rcp_gemv_w2a16", st)
     return y
 
 
@@ -284,24 +285,12 @@ def rcp_pack_weights3(codes: torch.Tensor):
 def rcp_gemv_w3a4(words2, words1, lut, xq, scale, group=0, y=None, S_dbg=None):
     """W3A4 GEMV: words2 int32 [N][K/16], words1 int32 [N][K/32], lut fp16 [N][8] (group=0) or [N][K/128][8]
     (group=128), xq uint8 [M][K/2], scale fp16 [M] -> y fp16 [M][N]."""
-    _dev(words2, torch.int32, "words2")
-    _dev(words1, torch.int32, "words1")
-    _dev(lut, torch.float16, "lut")
-    _dev(xq, torch.uint8, "xq")
-    _dev(scale, torch.float16, "scale")
-    N, W = words2.shape
-    K = W * 16
-    M = xq.shape[0]
-    group = int(group)
-    want = (N, 8) if group == 0 else (N, K // max(group, 1), 8)
-    if words1.shape != (N, K // 32) or xq.shape != (M, K // 2) or tuple(lut.shape) != want or scale.shape != (M,):
-        raise ValueError("shape mismatch between words2, words1, lut, group, xq and scale")
     if y is None:
-        y = torch.empty((M, N), dtype=torch.float16, device=words2.device)
-    with _on(words2):
-        _check("rcp_gemv_w3a4",
-               lib().rcp_gemv_w3a4(_ptr(words2), _ptr(words1), _ptr(lut), group, _ptr(xq), _ptr(scale), M, N, K, _ptr(y),
-                                   _ptr(S_dbg), _stream(words2)))
+        _dev(words2, torch.int32, "words2")
+        y = torch.empty((xq.shape[0], words2.shape[0]), dtype=torch.float16, device=words2.device)
+    st = (_m or _native()).gemv_w3a4(words2, words1, lut, int(group), xq, scale, y, S_dbg)
+    if st:
+        _check("rcp_gemv_w3a4", st)
     return y
 
 
@@ -338,24 +327,11 @@ def rcp_linear_w2a4(x, had_block, clip_ratio, words, lut, group=0, y=None, xq=No
     otherwise. xq / scale: optional for one token of 4096 or 8192 under one rotation block, required otherwise (pass
     them to be safe). S_dbg int32 [M][N][4] ([M][N][K/group][4]): the integer sums, from the checked instantiation
     of the kernel that runs anyway."""
-    _dev(x, torch.float16, "x")
-    _dev(words, torch.int32, "words")
-    _dev(lut, torch.float16, "lut")
-    M, K = x.shape
-    N, W = words.shape
-    group = int(group)
-    want = (N, 4) if group == 0 else (N, K // max(group, 1), 4)
-    if W * 16 != K or tuple(lut.shape) != want:
-        raise ValueError("shape mismatch between x, words, lut and group")
-    if y is None:
-        y = torch.empty((M, N), dtype=torch.float16, device=words.device)
-    if workspace is None:
-        workspace = make_workspace(M, N, K, words.device)
-    with _on(words):
-        _check("rcp_linear_w2a4",
-               lib().rcp_linear_w2a4_checked(_ptr(x), M, K, int(had_block), float(clip_ratio), _ptr(words), _ptr(lut),
-                                             group, N, _ptr(y), _ptr(xq), _ptr(scale), _ptr(workspace), _ptr(S_dbg),
-                                             _stream(words)))
+    if y is None or workspace is None:
+        y, workspace = _results(words, x, y, workspace)
+    st = (_m or _native()).linear_w2a4(x, had_block, clip_ratio, words, lut, group, y, xq, scale, workspace, S_dbg)
+    if st:
+        _check("rcp_linear_w2a4", st)
     return y
 
 
@@ -370,13 +346,8 @@ def rcp_linear_w2a4_launches(M: int, N: int, K: int, had_block: int, group: int 
 def rcp_linear_w2a4_host(x_host, had_block, clip_ratio, words, lut, y_host, x_dev, xq_dev, scale_dev, y_dev, workspace):
     """x_host fp16 [M][K] (host, ideally pinned) -> y_host fp16 [M][N] (host). Asynchronous on the
     current stream: synchronize before reading y_host."""
-    M, K = x_host.shape
-    N = words.shape[0]
-    if x_host.is_cuda or y_host.is_cuda or x_host.dtype != torch.float16 or y_host.dtype != torch.float16:
-        raise TypeError("x_host / y_host must be fp16 host tensors")
-    with _on(words):
-        _check("rcp_linear_w2a4_host",
-               lib().rcp_linear_w2a4_host(_ptr(x_host), M, K, int(had_block), float(clip_ratio), _ptr(words), _ptr(lut),
-                                          N, _ptr(y_host), _ptr(x_dev), _ptr(xq_dev), _ptr(scale_dev), _ptr(y_dev),
-                                          _ptr(workspace), _stream(words)))
+    st = (_m or _native()).linear_w2a4_host(x_host, had_block, clip_ratio, words, lut, y_host, x_dev, xq_dev, scale_dev,
+                                            y_dev, workspace)
+    if st:
+        _check("rcp_linear_w2a4_host", st)
     return y_host

@@ -1,17 +1,20 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds the CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the native argument
+marshalling of the Python binding with the host compiler."""
 import os
 import subprocess
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "librcp_w2a4.so")
 LIB_CHECKED = os.path.join(HERE, "librcp_w2a4_checked.so")   # the guarded build (-DRCP_CHECKED), for tests
 DRIVER = os.path.join(HERE, "e2e_driver")                     # host program: a decode step through the C ABI
+MARSHAL = os.path.join(HERE, "_marshal.so")                   # csrc/binding.cpp, a Python extension module
 SOURCES = ["rcp_api.cu"]
 
 
 def _newest_source_mtime() -> float:
-    paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")]
     paths.append(os.path.join(os.path.dirname(HERE), "include", "rcp.h"))
     return max(os.path.getmtime(p) for p in paths)
 
@@ -41,6 +44,20 @@ def build_checked(force: bool = False) -> str:
     return _compile(LIB_CHECKED, defines=("RCP_CHECKED",))
 
 
+def build_marshal(force: bool = False) -> str:
+    src = os.path.join(CSRC, "binding.cpp")
+    header = os.path.join(os.path.dirname(HERE), "include", "rcp.h")
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= max(os.path.getmtime(src), os.path.getmtime(header)):
+        return MARSHAL
+    import torch
+    from torch.utils import cpp_extension
+    flags = ["-I" + d for d in cpp_extension.include_paths()] + ["-I" + sysconfig.get_paths()["include"], "-I/usr/local/cuda/include"]
+    libs = ["-L" + d for d in cpp_extension.library_paths()] + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    abi = f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", abi] + flags + ["-o", MARSHAL, src] + libs)
+    return MARSHAL
+
+
 def build_driver(force: bool = False) -> str:
     """The end-to-end driver (e2e_driver.cu): a C++ host program linked against the library, run by bench.py."""
     build()
@@ -56,6 +73,7 @@ def build_driver(force: bool = False) -> str:
 if __name__ == "__main__":
     import sys
     print(build(force=True, verbose=True))
+    print(build_marshal(force=True))
     print(build_driver(force=True))
     if "--checked" in sys.argv[1:]:
         print(build_checked(force=True))
