@@ -286,7 +286,8 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   int* const s_T0c = reinterpret_cast<int*>(gen + p.off_T0c);           // [M][nchunk]: sum of q per chunk; GRP: [M][4 nchunk] per group
   float* const s_scale = reinterpret_cast<float*>(gen + p.off_scale);   // [16]
   int* const s_red = reinterpret_cast<int*>(gen + p.off_red);           // [2][8 groups][16 rows][M][3]
-  float* const s_redf = reinterpret_cast<float*>(gen + p.off_red);      // GRP: [2][16 warps][16 rows][M]
+  float* const s_redf = reinterpret_cast<float*>(gen + p.off_red);      // GRP: a slot per warp, [token pairs][32], see red_index
+  const int red_plane = ((M + 1) >> 1) * 32;
   // tensor-core GRP: the same area as floats [4 nchunk][Mp], 8 x the sum of q of a group, tokens padded to even
   float* const s_T0f = reinterpret_cast<float*>(gen + p.off_T0c);
   const int ng4 = 4 * p.nchunk;
@@ -464,7 +465,13 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
     }
   }
 
-  // The packed weights and the LUT are constants of the layer; everything else (xq, scale, y) may
+  // What needs nothing of the kernel before this one: clearing the sums, and x in fp16 on its way to L2 if it is not there
+  // (the L2 is where a kernel in front would write it, so this can fetch nothing stale).
+  if constexpr (!GRP)
+    for (int i = tid; i < 2 * 8 * 16 * M * 3; i += kCWarps * 32) s_red[i] = 0;
+  if constexpr (FQ != 0 || A16)
+    if (tid == 0 && p.x && b * 64 < (A16 ? p.M / 4 : 1) * p.K) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.x + b * 64));
+  // The packed weights and the LUT are constants of the layer; everything else (x, xq, scale, y) may
   // belong to the kernel before this one: wait for it.
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -567,7 +574,6 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
     if constexpr (!GRP) {
       total = __reduce_add_sync(0xffffffffu, total);
       if (lane == 0) atomicAdd(&s_T0tot[0], total);
-      for (int i = tid; i < 2 * 8 * 16 * M * 3; i += kCWarps * 32) s_red[i] = 0;
     }
   } else if constexpr (SB && GRP) {
     // Streamed activations, group-wise grid: the sum of q of every (token, group of 128) is needed up front, as
@@ -616,7 +622,6 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
       if (lane == 0) atomicAdd(&s_T0tot[col], tsum);
     }
     if (tid < M) s_scale[tid] = __half2float(p.scale[tid]);
-    for (int i = tid; i < 2 * 8 * 16 * M * 3; i += kCWarps * 32) s_red[i] = 0;
   } else
   // ------------------------------------------------------------------ activations (consumer warps)
   // One unit = (column, chunk, i, pr, t) = two words. The 16 units of a (column, chunk) are 16
@@ -631,7 +636,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
         // One token (the host asks for this form only then: with two, the stand-alone kernel in front was
         // measured faster), its values held in registers between the two passes (up to four vectors of eight
         // per thread: K <= 16384, which the host checks).
-        unsigned* const s_am = reinterpret_cast<unsigned*>(s_red);   // [16 warps]; s_red is cleared further down
+        unsigned* const s_am = reinterpret_cast<unsigned*>(s_scale + 16);   // [16 warps]
         const int nvec = p.K / 8;
         uint4 xr[4];
         unsigned amax = 0u;
@@ -669,9 +674,11 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
             }
           }
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(kCWarps * 32) : "memory");   // planes complete; s_red free to be cleared
+        asm volatile("bar.sync 1, %0;" ::"n"(kCWarps * 32) : "memory");   // planes complete
       }
     }
+    float my_scale = 0.f;   // asked for now, stored when the activations are done
+    if (tid < M && !(A16 && p.x)) my_scale = A16 ? __ldg(p.unit + tid) : __half2float(__ldg(p.scale + tid));
     const int W = p.K / 16;
     const int total = ncol * p.nchunk * 16;
     // the two words of unit u (zeros past the end of the row or of the units)
@@ -697,30 +704,38 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
       }
       return x;
     };
-    // tensor-core kernels of the per-row grid (several tokens, so several units per thread): the next unit's
-    // words are fetched while this one is expanded. Measured: the one- and two-token kernels lose 1 % with
-    // it, the group-wise kernels have no registers to spare for it.
-    constexpr bool kPrefetch = !GRP && !A16 && MODE == kModeMma;
-    uint4 x_next = make_uint4(0, 0, 0, 0);
-    if constexpr (kPrefetch) x_next = load_unit(warp * 32 + lane);
+    // The words of a thread's next units are on their way while one is expanded (a unit takes some 250 clocks, its words
+    // 700 to arrive from L2): four in flight, or two of twice the size for the digit columns. One at a time, 8192x8192 took
+    // 10.2 us at eight tokens and 8192x28672 18.6 at one, now 9.4 and 18.1.
+    constexpr int kAhead = A16 ? 2 : 4;
+    uint4 xq_ahead[kAhead][A16 ? 2 : 1];
+    auto fetch_unit = [&](int u, uint4 (&x)[A16 ? 2 : 1]) {
+      if constexpr (A16) { x[0] = load_unit_bytes(u, 0); x[1] = load_unit_bytes(u, 1); }
+      else x[0] = load_unit(u);
+    };
+#pragma unroll
+    for (int i = 0; i < kAhead; i++) fetch_unit(warp * 32 + lane + i * kCWarps * 32, xq_ahead[i]);
+#pragma unroll 1
     for (int u0 = warp * 32; u0 < total; u0 += kCWarps * 32) {
       const int u = u0 + lane;
       int tsum = 0;
       const int pair = u >> 4;
       const int col = (int)(((uint32_t)pair * (uint32_t)p.inv_nchunk) >> 20), ch = pair - col * p.nchunk;   // pair / nchunk
-      uint4 x = x_next;
-      if constexpr (kPrefetch) x_next = load_unit(u + kCWarps * 32);
+      uint4 xu[A16 ? 2 : 1];
+#pragma unroll
+      for (int w = 0; w < (A16 ? 2 : 1); w++) {
+        xu[w] = xq_ahead[0][w];
+#pragma unroll
+        for (int i = 0; i + 1 < kAhead; i++) xq_ahead[i][w] = xq_ahead[i + 1][w];
+      }
+      fetch_unit(u + kAhead * kCWarps * 32, xq_ahead[kAhead - 1]);
       if (u < total) {
         const int lo = u & 3, hi = (u >> 2) & 3;   // lo: 16-byte slot t of the column block; hi: 2 i + pr, or the group
-        if constexpr (!kPrefetch && !A16) {
-          const int wx = (chunk0 + ch) * kChunkWords + (kRelabel ? 8 * hi + 2 * lo : 8 * lo + 2 * hi);   // word index in the row
-          if (wx < W) x = __ldg(reinterpret_cast<const uint4*>(p.xq + (size_t)col * (p.K / 2)) + (wx >> 1));
-        }
         uint32_t q[4][2];
         if constexpr (A16) {
 #pragma unroll
           for (int w = 0; w < 2; w++) {
-            const uint4 d = load_unit_bytes(u, w);   // bytes 4b..4b+3 of d: the digits that meet byte b of the weight word
+            const uint4 d = xu[w];   // bytes 4b..4b+3 of d: the digits that meet byte b of the weight word
             tsum = __dp4a((int)d.x, 0x01010101, tsum); tsum = __dp4a((int)d.y, 0x01010101, tsum);
             tsum = __dp4a((int)d.z, 0x01010101, tsum); tsum = __dp4a((int)d.w, 0x01010101, tsum);
             // 4 x 4 byte transpose: position p gathers byte p of each of the four
@@ -734,7 +749,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
         } else
 #pragma unroll
         for (int w = 0; w < 2; w++) {
-          const uint32_t lo32 = w ? x.z : x.x, hi32 = w ? x.w : x.y;   // codes 0..7 and 8..15 of the word
+          const uint32_t lo32 = w ? xu[0].z : xu[0].x, hi32 = w ? xu[0].w : xu[0].y;   // codes 0..7 and 8..15 of the word
           // even and odd codes of each half as bytes, each nibble sign-extended to a byte
           uint32_t n4[4] = {lo32 & 0x0F0F0F0Fu, (lo32 >> 4) & 0x0F0F0F0Fu, hi32 & 0x0F0F0F0Fu, (hi32 >> 4) & 0x0F0F0F0Fu};
 #pragma unroll
@@ -769,9 +784,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
         if ((u & 12) == 0 && u < total) s_T0c[col * ng4 + ch * 4 + (u & 3)] = tsum;
       }
     }
-    if (tid < M && !(A16 && p.x)) s_scale[tid] = A16 ? p.unit[tid] : __half2float(p.scale[tid]);
-    if constexpr (!GRP)
-      for (int i = tid; i < 2 * 8 * 16 * M * 3; i += kCWarps * 32) s_red[i] = 0;
+    if (tid < M && !(A16 && p.x)) s_scale[tid] = my_scale;
   }
   asm volatile("bar.sync 1, %0;" ::"n"(kCWarps * 32) : "memory");   // consumer warps only
 
@@ -1081,6 +1094,9 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
       }
     }
   };
+  // Place of a (row, token) in a reduction slot: blocks of two tokens x 16 rows, the rows of neighbouring
+  // blocks rotated by eight so that the stores of a warp (rows g, tokens 2 t and 2 t + 1) meet no bank conflicts.
+  auto red_index = [](int tok, int row) { return ((tok >> 1) << 5) + ((((tok & 1) << 4) + row) ^ (((tok >> 1) & 3) << 3)); };
   // end of a row group: the fp32 sums of this warp's chunks, for the entries this lane emits
   auto emit_grp = [&](int row_first, bool active, int KS, int grp, int ks, int& nred) {
     if constexpr (GRP) {
@@ -1091,35 +1107,34 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
           yacc[e] += __shfl_xor_sync(0xffffffffu, yacc[e], 2);
         }
       }
-      if (KS > 1) {
-        // every warp of the group leaves its sums in its own slot; the first adds them up in order
-        float* const red = s_redf + (nred & 1) * (kCWarps * 16 * M);
-        nred++;
+      // The KS warps that shared the group (or the one that had it) leave their terms in a slot each, then every warp adds
+      // up, in the order of the warps, and finishes every KS-th pair of tokens: lane & 15 is the row, lane >> 4 the token.
+      // (4096x14336 at eight tokens 14.2 -> 13.0 us, at one 8.0 -> 7.7, against one warp finishing the whole group. For
+      // the per-row grid, with three integer sums a row and token, the same was slower than its atomics: 2048x2048 2.7 -> 3.0.)
+      float* const mine = s_redf + warp * red_plane;
+      // a shared reduction before this one: its slots must have been read by everybody
+      if (nred) asm volatile("bar.sync 2, %0;" ::"n"(kCWarps * 32) : "memory");
+      nred = KS > 1;
 #pragma unroll
-        for (int e = 0; e < NE; e++)
-          if (active && etok[e] < M &&
-              RCP_CK(((nred - 1) & 1) * (kCWarps * 16 * M) + (warp * 16 + g + 8 * err[e]) * M + etok[e] < p.red_bytes / 4, 10))
-            red[(warp * 16 + g + 8 * err[e]) * M + etok[e]] = yacc[e];
-        asm volatile("bar.sync 2, %0;" ::"n"(kCWarps * 32) : "memory");   // consumer warps only
-        if (active && ks == 0) {
-#pragma unroll
-          for (int e = 0; e < NE; e++) {
-            if (etok[e] < M) {
-              float a = 0.f;
-              for (int k = 0; k < KS; k++) a += red[((grp * KS + k) * 16 + g + 8 * err[e]) * M + etok[e]];
-              yacc[e] = a;
-            }
-          }
+      for (int e = 0; e < NE; e++)
+        if (active && etok[e] < M && RCP_CK((warp * red_plane + red_index(etok[e], grow + 8 * err[e])) * 4 < p.red_bytes, 10))
+          mine[red_index(etok[e], grow + 8 * err[e])] = yacc[e];
+      if (KS > 1) asm volatile("bar.sync 2, %0;" ::"n"(kCWarps * 32) : "memory");   // consumer warps only
+      else __syncwarp();
+      if (active) {
+        const int row = row_first + (lane & 15);
+#pragma unroll 1
+        for (int tp = ks; 2 * tp < M; tp += KS) {
+          const int tok = 2 * tp + (lane >> 4);
+          const float* d = s_redf + grp * KS * red_plane + red_index(tok, lane & 15);
+          float a = 0.f;
+#pragma unroll 4
+          for (int k = 0; k < KS; k++, d += red_plane) a += *d;
+          if (tok < M && row < p.N)
+            p.y[(size_t)tok * p.N + row] = __float2half_rn(s_scale[tok] * (kRelabel ? 0.125f * a : a));
         }
       }
-      if (active && ks == 0) {
-#pragma unroll
-        for (int e = 0; e < NE; e++) {
-          const int row = row_first + grow + 8 * err[e];
-          if (etok[e] < M && row < p.N)
-            p.y[(size_t)etok[e] * p.N + row] = __float2half_rn(s_scale[etok[e]] * (kRelabel ? 0.125f * yacc[e] : yacc[e]));
-        }
-      }
+      if (KS == 1) __syncwarp();   // the slot is written again
 #pragma unroll
       for (int e = 0; e < NE; e++) yacc[e] = 0.f;
     }
@@ -1239,7 +1254,8 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
 
   int slot = slot_keep;
   uint32_t phase = phase_keep;
-  int nred = nred_keep;   // phases with a shared-memory reduction so far (its two buffers alternate)
+  // shared-memory reductions so far (two buffers alternate); group-wise grid: whether the last end of a group was one
+  int nred = nred_keep;
   int gbase = 0;   // groups of this CTA before the current repetition, the same count in every part
   for (int pi = 0; pi < p.nphase; pi++) {
     const GemvPhase ph = p.phase[pi];

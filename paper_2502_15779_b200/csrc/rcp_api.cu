@@ -197,9 +197,9 @@ StreamPlan make_plan(int M, int N, int K, int sms, bool grouped, size_t qbuf, in
   pl.stage_stride = (int)(rcp::kStageBytes + bstage);
   const size_t bs_bytes = stream_act ? 0 : (size_t)pl.nchunk * rcp::kChunkWords * 16 * M;
   // sums of q per chunk (per group of 128: four per chunk); reduction buffers: integer sums of 8
-  // row groups x 3 planes, or (group-wise grid) one fp32 term per warp
+  // row groups x 3 planes, or (group-wise grid) fp32 terms of every warp, tokens in pairs x 16 rows
   const size_t t0c_bytes = grouped ? (size_t)(M + 1) * pl.nchunk * 16 : (((size_t)M * pl.nchunk * 4) + 15) / 16 * 16;
-  const size_t red_bytes = grouped ? (size_t)2 * rcp::kCWarps * 16 * M * 4 : (size_t)2 * 8 * 16 * M * 3 * 4;
+  const size_t red_bytes = grouped ? (size_t)rcp::kCWarps * ((M + 1) / 2) * 32 * 4 : (size_t)2 * 8 * 16 * M * 3 * 4;
   // K in parts: the integer sums of every group this CTA owns wait in shared memory between the parts
   int own_groups = 0;
   for (int i = 0; i < pl.nphase; i++) own_groups += pl.phase[i].reps * (pl.phase[i].q + (pl.phase[i].r ? 1 : 0));
