@@ -596,24 +596,14 @@ int launch_w3(const rcp::W3Params& wp, size_t smem, cudaStream_t st) {
   static std::mutex mu;
   static bool attr_set[kMaxDevices] = {};
   auto kern = rcp::gemv_w3a4_kernel<GRP, SDBG>;
-  int dev = 0;
-  RCP_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= kMaxDevices) return RCP_ERR_LIMIT;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    if (!attr_set[dev]) {
-      RCP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, rcp::kMaxK + 128));
-      attr_set[dev] = true;
-    }
-  }
+  RCP_CUDA(set_max_smem(kern, rcp::kMaxK + 128, mu, attr_set));
   // One wave of resident CTAs, rows dealt round-robin to their warps (measured: CTAs beyond the resident wave,
-  // and warps sharing a row along K, both cost more than the evener load returns).
-  int per_sm = 0;
-  RCP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, rcp::kW3Threads, smem));
+  // and warps sharing a row along K, both cost more than the evener load returns). CTAs per SM: four by registers, or
+  // what the expanded activations (and some 9 KB beside them, 1 KB of it the system's) leave of 228 KB.
+  const int per_sm = std::max<int>(1, std::min<size_t>(4, 228 * 1024 / (smem + 9472 + 1024)));
   const int warps_per_cta = rcp::kW3Threads / 32;
-  const int grid = std::min(sm_count() * std::max(per_sm, 1), (wp.N + warps_per_cta - 1) / warps_per_cta);
-  kern<<<grid, rcp::kW3Threads, smem, st>>>(wp);
-  RCP_CUDA(cudaGetLastError());
+  const int grid = std::min(sm_count() * per_sm, (wp.N + warps_per_cta - 1) / warps_per_cta);
+  RCP_CUDA(launch_overlapped(kern, dim3(grid), dim3(rcp::kW3Threads), smem, st, wp));
   return RCP_OK;
 }
 
