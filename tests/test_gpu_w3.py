@@ -204,3 +204,10 @@ def test_exported_3bit_layer_through_the_gemv(N, K, G, M):
     out = oracle.gemv_w3a4(r2, r1, ref["lut"], qa["xq"], qa["scale"], G)
     err = np.abs(y.float().cpu().numpy().astype(np.float64) - out["y"])
     assert np.all(err <= out["tol"]), f"max err/tol {np.max(err / out['tol'])}"
+
+
+def test_w3a4_more_rows_than_a_warp_finishes_at_once():
+    """So many rows that a warp's sums are finished in several batches of 32 (592 CTAs x 8 warps x 32 rows = 151552)."""
+    N = 592 * 8 * 32 + 4736 + 77
+    rows = np.unique(np.concatenate([np.arange(40), np.arange(151540, 151570), np.arange(N - 40, N)]))
+    _check(N, 64, 1, 0, seed=5, rows=rows)
