@@ -927,8 +927,10 @@ int rcp_gemv_w2a16_checked(const uint32_t* words, const void* lut_f16, const voi
     return launch_stream(rcp::kModeMma, words, lut_f16, nullptr, nullptr, cols, N, K, y_f16, workspace, st, false,
                          nullptr, nullptr, 1, &sa, S_dbg);
   }
-  RCP_CUDA(launch_overlapped(rcp::split_act16_kernel, dim3(M), dim3(rcp::kSplitThreads), 0, st,
-                             static_cast<const __half*>(x_f16), K, digits, unit));
+  // half of the threads have a vector of eight elements (a whole one each: 0.1 to 0.4 us a call slower)
+  const int parts = std::max(1, std::min(16, K / (4 * rcp::kSplitThreads)));
+  RCP_CUDA(launch_overlapped(rcp::split_act16_kernel, dim3(M * parts), dim3(rcp::kSplitThreads), 0, st,
+                             static_cast<const __half*>(x_f16), K, parts, digits, unit));
   for (int c0 = 0; c0 < cols; c0 += cp) {
     const int cc = std::min(cp, cols - c0);
     const int rc = launch_stream(rcp::kModeMma, words, lut_f16, reinterpret_cast<const uint8_t*>(digits) + (size_t)c0 * K,

@@ -126,3 +126,16 @@ def test_w2a16_argument_errors():
     assert L.rcp_gemv_w2a16(p, p, p, 17, 16, 64, p, p, p, p, None) == -2
     assert L.rcp_gemv_w2a16(p, p, p, 1, 16, 65600, p, p, p, p, None) == -2   # K above the library's limit
     assert L.rcp_gemv_w2a16(p, p, p + 2, 1, 16, 64, p, p, p, p, None) == -3
+
+
+@pytest.mark.parametrize("K", [2112, 4160, 16448, 40960, 65536])
+def test_w2a16_largest_magnitude_in_any_part_of_the_token(K):
+    """The digits of a token are shared out over several CTAs, each of which finds the largest magnitude itself: planted
+    at the ends of the token and around the seams of the parts (one token per place), in one launch of the kernel."""
+    parts = max(1, min(16, K // 2048))
+    seams = sorted({K // 8 * p // parts * 8 for p in range(1, parts)})
+    places = sorted({0, K - 1, *[s for s in seams[:3]], *[s - 1 for s in seams[-3:]]})
+    x = synth.make_activations(len(places), K, K, device=DEV)
+    for m, at in enumerate(places):
+        x[m, at] = -3000.0 - 500.0 * m
+    _check(33, K, len(places), seed=K, kind="uniform", x=x)
