@@ -27,6 +27,14 @@ __device__ __forceinline__ float ld_cluster_f32(const float* local, uint32_t ran
   return v;
 }
 
+// Sends `halves` fp16 numbers at x on their way to L2, one 128-byte line per thread of the first ones. For use before the
+// wait for the kernel in front: the L2 is where that kernel would write them, so this can fetch nothing stale. (Activations
+// that are not in L2 otherwise arrive behind the next GEMV's weights: 8192x28672 at one token 21.5 -> 20.7 us, 10007x4096 at
+// three 8.5 -> 8.4, 28672x4096 at sixteen 24.7 -> 24.3.)
+__device__ __forceinline__ void prefetch_token(const __half* x, int halves, int tid) {
+  if (tid * 64 < halves) asm volatile("prefetch.global.L2 [%0];" ::"l"(x + tid * 64));
+}
+
 struct QuantParams {
   const __half* x;
   uint8_t* xq;
@@ -50,6 +58,7 @@ __global__ void __launch_bounds__(1024) quantize_act_kernel(const QuantParams p)
   // Launched with programmatic stream serialization: let the next kernel get started, then wait
   // for the kernel before this one, whose output x may be and whose input xq and scale may be.
   asm volatile("griddepcontrol.launch_dependents;");
+  prefetch_token(p.x + (size_t)m * p.K + (size_t)p.K / C / 8 * rank * 8, p.K / C, tid);
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // this CTA's slice of the token
@@ -307,6 +316,7 @@ __global__ void __launch_bounds__(T_MAX, 1024 / T_MAX) quantize_act_rows_kernel(
   __shared__ unsigned s_max[2][32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
   asm volatile("griddepcontrol.launch_dependents;");
+  prefetch_token(p.x + (size_t)blockIdx.x * p.K, p.K, tid);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   extern __shared__ __align__(16) uint4 s_next[];   // [R][2][T]: the next token's activations; a thread copies its own
   const int W = p.K / 16, T = blockDim.x, B = BLOCK ? BLOCK : p.B;
@@ -379,6 +389,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) quantize_act_full_rows_kernel(c
   __shared__ unsigned s_max[2][R];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   asm volatile("griddepcontrol.launch_dependents;");
+  prefetch_token(p.x + (size_t)blockIdx.x * (NT * 16), NT * 16, tid);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   float* const wbuf = sbuf + warp * (32 * kPitch);
   const int e1 = lane & 15, hi = lane & 16;

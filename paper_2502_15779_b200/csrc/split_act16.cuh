@@ -61,6 +61,8 @@ __global__ void __launch_bounds__(kSplitThreads) split_act16_kernel(const __half
   const int nvec = K / 8;
   asm volatile("griddepcontrol.launch_dependents;");
   asm volatile("griddepcontrol.launch_dependents;");
+  // the token on its way to L2 (nothing stale: that is where the kernel in front would write it)
+  if (part == 0 && tid * 64 < K) asm volatile("prefetch.global.L2 [%0];" ::"l"(x + (size_t)m * K + tid * 64));
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // this part's vectors, and the first of them asked for at once
   const int v0 = (int)((long long)nvec * part / parts), v1 = (int)((long long)nvec * (part + 1) / parts);
