@@ -106,7 +106,7 @@ struct GemvParams {
   int nchunk_total;     // chunks per row over the whole K
   int nsplit;           // parts of K gone through one after the other (tensor-core kernels of the per-row grid; else 1)
   int off_part;         // nsplit > 1: partial sums of this CTA's rows between the parts
-  int inv_nchunk;       // ceil(2^20 / nchunk): x / nchunk == (x * inv_nchunk) >> 20 for x < 2^20 / nchunk
+  int act_parts, inv_act_parts;   // warps that share the expansion of a column: max(1, 16 / M), and ceil(256 / that)
   int nphase;
   GemvPhase phase[kMaxPhases];
   // fused activation quantizer (FQ): x fp16 [M][K] replaces xq and scale as input
@@ -208,6 +208,25 @@ __device__ __forceinline__ void dp4a_s8s8(int& d, uint32_t a, uint32_t b) {
   asm("dp4a.s32.s32 %0, %1, %2, %0;" : "+r"(d) : "r"(a), "r"(b));
 }
 
+// The sixteen int4 activations of a word of codes (lo32: codes 0..7, hi32: codes 8..15) as the four dot-product operands:
+// byte j of q[p] meets code 4 j + p, 16 q for even positions and 4 q for odd ones. (16 q is the nibble in the upper half of
+// a byte as it stands, 4 q that shifted by two with its sign brought in, so no nibble is sign-extended to a byte first.)
+// tsum += 16 x their sum.
+__device__ __forceinline__ uint32_t sign_bytes(uint32_t x) {   // 0xFF in every byte whose top bit is set, else 0
+  uint32_t d;
+  asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(d) : "r"(x));
+  return d;
+}
+__device__ __forceinline__ void expand_word(uint32_t lo32, uint32_t hi32, uint32_t (&q)[4], int& tsum) {
+  const uint32_t p01 = __byte_perm(lo32, hi32, 0x6420), p23 = __byte_perm(lo32, hi32, 0x7531);   // positions 0 | 1, 2 | 3
+  const uint32_t h1 = p01 & 0xF0F0F0F0u, h3 = p23 & 0xF0F0F0F0u;
+  q[0] = (p01 << 4) & 0xF0F0F0F0u;
+  q[2] = (p23 << 4) & 0xF0F0F0F0u;
+  q[1] = (h1 >> 2) | (sign_bytes(h1) & 0xC0C0C0C0u);
+  q[3] = (h3 >> 2) | (sign_bytes(h3) & 0xC0C0C0C0u);
+  tsum = __dp4a((int)q[0], 0x01010101, __dp4a((int)q[2], 0x01010101, __dp4a((int)q[1], 0x04040404, __dp4a((int)q[3], 0x04040404, tsum))));
+}
+
 // Self-test of the bounded wait and its report (a test aid, not part of the data path): one thread waits, with
 // the routine the GEMV kernels wait with and a limit of the caller's choice, on a barrier that nobody ever
 // arrives at. The wait gives up, the status word receives the consumer-side code, the kernel returns.
@@ -281,6 +300,9 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   const int ncol = M;
   const int stages = p.stages;
   const uint32_t full0 = base + p.off_bar, empty0 = full0 + 8 * kMaxStages;
+  // How far the activation operands are scaled: even positions carry 4 q << kQ, odd ones q << kQ (16 q and 4 q; the
+  // quantizer inside and the digit columns keep 4 q and q)
+  constexpr int kQ = (A16 || FQ != 0) ? 0 : 2;
   static_assert(!(GRP && MODE == kModeHybrid), "no group-wise hybrid mode");
   constexpr bool kRelabel = GRP && MODE == kModeMma;   // a quad shares a group: lane t takes words 8j+2t, 8j+2t+1
   int* const s_T0c = reinterpret_cast<int*>(gen + p.off_T0c);           // [M][nchunk]: sum of q per chunk; GRP: [M][4 nchunk] per group
@@ -433,17 +455,13 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
                   const int col = w >> 4, lo = w & 3, hi = (w >> 2) & 3;
                   const uint4 x = xa[r];
                   uint32_t q[4][2];
+                  int unused = 0;
 #pragma unroll
                   for (int ww = 0; ww < 2; ww++) {
-                    const uint32_t lo32 = ww ? x.z : x.x, hi32 = ww ? x.w : x.y;
-                    uint32_t n4[4] = {lo32 & 0x0F0F0F0Fu, (lo32 >> 4) & 0x0F0F0F0Fu, hi32 & 0x0F0F0F0Fu, (hi32 >> 4) & 0x0F0F0F0Fu};
+                    uint32_t e[4];
+                    expand_word(ww ? x.z : x.x, ww ? x.w : x.y, e, unused);
 #pragma unroll
-                    for (int h = 0; h < 4; h++) n4[h] |= (n4[h] & 0x08080808u) * 0x1Eu;   // sign-extend the nibbles
-                    const uint32_t e0 = __byte_perm(n4[0], n4[2], 0x6420), e2 = __byte_perm(n4[0], n4[2], 0x7531);
-                    q[0][ww] = (e0 << 2) & 0xFCFCFCFCu;
-                    q[1][ww] = __byte_perm(n4[1], n4[3], 0x6420);
-                    q[2][ww] = (e2 << 2) & 0xFCFCFCFCu;
-                    q[3][ww] = __byte_perm(n4[1], n4[3], 0x7531);
+                    for (int pp = 0; pp < 4; pp++) q[pp][ww] = e[pp];
                   }
                   uint8_t* dst = sb + ((size_t)(((j * 4 + hi) * 2) * ncol + col)) * 64 + lo * 16;
                   if (RCP_CK(dst >= gen && dst + (size_t)ncol * 64 + 16 <= gen + (size_t)(slot + 1) * stage_stride, 13)) {
@@ -598,7 +616,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
           tsum = __dp4a((int)o, 0x01010101, tsum);
         }
       }
-      s_T0f[gi * Mp + col] = (float)(8 * tsum);
+      s_T0f[gi * Mp + col] = (float)((8 << kQ) * tsum);
     }
     if (tid < M) s_scale[tid] = __half2float(p.scale[tid]);
   } else if constexpr (SB) {
@@ -681,109 +699,91 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
     float my_scale = 0.f;   // asked for now, stored when the activations are done
     if (tid < M && !(A16 && p.x)) my_scale = A16 ? __ldg(p.unit + tid) : __half2float(__ldg(p.scale + tid));
     const int W = p.K / 16;
-    const int total = ncol * p.nchunk * 16;
-    // the two words of unit u (zeros past the end of the row or of the units)
-    auto load_unit = [&](int u) {
-      const int pair = u >> 4;
-      const int col = (int)(((uint32_t)pair * (uint32_t)p.inv_nchunk) >> 20), ch = pair - col * p.nchunk;   // pair / nchunk
-      const int lo = u & 3, hi = (u >> 2) & 3;
-      const int wx = (chunk0 + ch) * kChunkWords + (kRelabel ? 8 * hi + 2 * lo : 8 * lo + 2 * hi);   // word index in the row
-      uint4 x = make_uint4(0, 0, 0, 0);
-      if (u < total && wx < W) x = __ldg(reinterpret_cast<const uint4*>(p.xq + (size_t)col * (p.K / 2)) + (wx >> 1));
-      return x;
-    };
-    // digit columns: the 16 bytes of word wx + w of unit u
-    auto load_unit_bytes = [&](int u, int w) {
-      const int pair = u >> 4;
-      const int col = (int)(((uint32_t)pair * (uint32_t)p.inv_nchunk) >> 20), ch = pair - col * p.nchunk;
-      const int lo = u & 3, hi = (u >> 2) & 3;
-      const int wx = (chunk0 + ch) * kChunkWords + 8 * lo + 2 * hi + w;
-      uint4 x = make_uint4(0, 0, 0, 0);
-      if (u < total && wx < W) {
-        if (p.x) x = *(reinterpret_cast<const uint4*>(stg + (size_t)col * p.K) + wx);   // planes made above
-        else x = __ldg(reinterpret_cast<const uint4*>(p.xq + (size_t)col * p.K) + wx);
-      }
-      return x;
-    };
-    // The words of a thread's next units are on their way while one is expanded (a unit takes some 250 clocks, its words
-    // 700 to arrive from L2): four in flight, or two of twice the size for the digit columns. One at a time, 8192x8192 took
-    // 10.2 us at eight tokens and 8192x28672 18.6 at one, now 9.4 and 18.1.
+    // A column is shared by act_parts warps (16 / columns, at least one); a warp takes every act_parts-th pair of chunks, a
+    // lane one unit of two words in each: lo and hi say which. So nothing is worked out per unit but a bound, and
+    // the sum of q of a warp's units meets once at its end.
+    // (With the units dealt to all threads in a row, a division, an address, four shuffles and an atomic a unit, and nibbles
+    // sign-extended one mask at a time: 4096x4096 at sixteen tokens 7.45 us, now 6.83; 8192x8192 at eight 9.7, now 8.8;
+    // weight-only 4096x14336 at two 15.0, now 13.2.)
+    const int col = (warp * p.inv_act_parts) >> 8, part = warp - col * p.act_parts;
+    const int lo = lane & 3, hi = (lane >> 2) & 3;   // lo: 16-byte slot t of the column block; hi: 2 i + pr, or the group
+    int ch = col < ncol ? 2 * part + (lane >> 4) : p.nchunk;   // chunk of this part of K
+    int wx = (chunk0 + ch) * kChunkWords + (kRelabel ? 8 * hi + 2 * lo : 8 * lo + 2 * hi);   // first of the unit's two words
+    const int ch_step = 2 * p.act_parts, wx_step = ch_step * kChunkWords;
+    const uint8_t* src = A16 ? (p.x ? stg + (size_t)col * p.K : p.xq + (size_t)col * p.K) + (size_t)wx * 16
+                             : p.xq + (size_t)col * (p.K / 2) + (size_t)wx * 8;
+    uint8_t* dst = bs + ((size_t)(((ch * 4 + hi) * 2) * ncol + col)) * 64 + lo * 16;
+    const size_t dst_step = (size_t)ch_step * 8 * ncol * 64;
+    // The words of a thread's next units are on their way while one is expanded (a unit takes some 200 clocks, its words
+    // 700 to arrive from L2): four in flight, or two of twice the size for the digit columns.
     constexpr int kAhead = A16 ? 2 : 4;
-    uint4 xq_ahead[kAhead][A16 ? 2 : 1];
-    auto fetch_unit = [&](int u, uint4 (&x)[A16 ? 2 : 1]) {
-      if constexpr (A16) { x[0] = load_unit_bytes(u, 0); x[1] = load_unit_bytes(u, 1); }
-      else x[0] = load_unit(u);
+    uint4 ahead[kAhead][A16 ? 2 : 1];
+    auto fetch_unit = [&](int i, uint4 (&x)[A16 ? 2 : 1]) {   // the unit i steps on (zeros past the end of the row)
+#pragma unroll
+      for (int w = 0; w < (A16 ? 2 : 1); w++) {
+        x[w] = make_uint4(0, 0, 0, 0);
+        if (ch + i * ch_step < p.nchunk && wx + i * wx_step < W) {
+          const uint4* const at = reinterpret_cast<const uint4*>(src + (size_t)i * wx_step * (A16 ? 16 : 8)) + w;
+          if (A16 && p.x) x[w] = *at;   // planes made above
+          else x[w] = __ldg(at);
+        }
+      }
     };
 #pragma unroll
-    for (int i = 0; i < kAhead; i++) fetch_unit(warp * 32 + lane + i * kCWarps * 32, xq_ahead[i]);
+    for (int i = 0; i < kAhead; i++) fetch_unit(i, ahead[i]);
+    int total = 0;   // sum of q (of 16 q where kQ is 2) of this lane's units
 #pragma unroll 1
-    for (int u0 = warp * 32; u0 < total; u0 += kCWarps * 32) {
-      const int u = u0 + lane;
-      int tsum = 0;
-      const int pair = u >> 4;
-      const int col = (int)(((uint32_t)pair * (uint32_t)p.inv_nchunk) >> 20), ch = pair - col * p.nchunk;   // pair / nchunk
+    for (int c = 2 * part; c < p.nchunk; c += ch_step) {   // (the same trips for all lanes)
       uint4 xu[A16 ? 2 : 1];
 #pragma unroll
       for (int w = 0; w < (A16 ? 2 : 1); w++) {
-        xu[w] = xq_ahead[0][w];
+        xu[w] = ahead[0][w];
 #pragma unroll
-        for (int i = 0; i + 1 < kAhead; i++) xq_ahead[i][w] = xq_ahead[i + 1][w];
+        for (int i = 0; i + 1 < kAhead; i++) ahead[i][w] = ahead[i + 1][w];
       }
-      fetch_unit(u + kAhead * kCWarps * 32, xq_ahead[kAhead - 1]);
-      if (u < total) {
-        const int lo = u & 3, hi = (u >> 2) & 3;   // lo: 16-byte slot t of the column block; hi: 2 i + pr, or the group
-        uint32_t q[4][2];
+      fetch_unit(kAhead, ahead[kAhead - 1]);
+      int tsum = 0;
+      uint32_t q[4][2];
+#pragma unroll
+      for (int w = 0; w < 2; w++) {
         if constexpr (A16) {
+          const uint4 d = xu[w];   // bytes 4b..4b+3 of d: the digits that meet byte b of the weight word
+          tsum = __dp4a((int)d.x, 0x01010101, tsum); tsum = __dp4a((int)d.y, 0x01010101, tsum);
+          tsum = __dp4a((int)d.z, 0x01010101, tsum); tsum = __dp4a((int)d.w, 0x01010101, tsum);
+          // 4 x 4 byte transpose: position p gathers byte p of each of the four
+          const uint32_t t01 = __byte_perm(d.x, d.y, 0x5140), t23 = __byte_perm(d.z, d.w, 0x5140);
+          const uint32_t s01 = __byte_perm(d.x, d.y, 0x7362), s23 = __byte_perm(d.z, d.w, 0x7362);
+          q[0][w] = (__byte_perm(t01, t23, 0x5410) << 2) & 0xFCFCFCFCu;   // even positions carry 4 q (|q| <= 32)
+          q[1][w] = __byte_perm(t01, t23, 0x7632);
+          q[2][w] = (__byte_perm(s01, s23, 0x5410) << 2) & 0xFCFCFCFCu;
+          q[3][w] = __byte_perm(s01, s23, 0x7632);
+        } else {
+          uint32_t e[4];
+          expand_word(w ? xu[0].z : xu[0].x, w ? xu[0].w : xu[0].y, e, tsum);
 #pragma unroll
-          for (int w = 0; w < 2; w++) {
-            const uint4 d = xu[w];   // bytes 4b..4b+3 of d: the digits that meet byte b of the weight word
-            tsum = __dp4a((int)d.x, 0x01010101, tsum); tsum = __dp4a((int)d.y, 0x01010101, tsum);
-            tsum = __dp4a((int)d.z, 0x01010101, tsum); tsum = __dp4a((int)d.w, 0x01010101, tsum);
-            // 4 x 4 byte transpose: position p gathers byte p of each of the four
-            const uint32_t t01 = __byte_perm(d.x, d.y, 0x5140), t23 = __byte_perm(d.z, d.w, 0x5140);
-            const uint32_t s01 = __byte_perm(d.x, d.y, 0x7362), s23 = __byte_perm(d.z, d.w, 0x7362);
-            q[0][w] = (__byte_perm(t01, t23, 0x5410) << 2) & 0xFCFCFCFCu;   // even positions carry 4 q (|q| <= 32)
-            q[1][w] = __byte_perm(t01, t23, 0x7632);
-            q[2][w] = (__byte_perm(s01, s23, 0x5410) << 2) & 0xFCFCFCFCu;
-            q[3][w] = __byte_perm(s01, s23, 0x7632);
-          }
-        } else
-#pragma unroll
-        for (int w = 0; w < 2; w++) {
-          const uint32_t lo32 = w ? xu[0].z : xu[0].x, hi32 = w ? xu[0].w : xu[0].y;   // codes 0..7 and 8..15 of the word
-          // even and odd codes of each half as bytes, each nibble sign-extended to a byte
-          uint32_t n4[4] = {lo32 & 0x0F0F0F0Fu, (lo32 >> 4) & 0x0F0F0F0Fu, hi32 & 0x0F0F0F0Fu, (hi32 >> 4) & 0x0F0F0F0Fu};
-#pragma unroll
-          for (int h = 0; h < 4; h++) {
-            n4[h] |= (n4[h] & 0x08080808u) * 0x1Eu;
-            tsum = __dp4a((int)n4[h], 0x01010101, tsum);
-          }
-          // position p of a byte of codes: codes p, 4+p, 8+p, 12+p; even positions carry 4 q
-          const uint32_t v0 = __byte_perm(n4[0], n4[2], 0x6420), v2 = __byte_perm(n4[0], n4[2], 0x7531);
-          q[0][w] = (v0 << 2) & 0xFCFCFCFCu;
-          q[1][w] = __byte_perm(n4[1], n4[3], 0x6420);
-          q[2][w] = (v2 << 2) & 0xFCFCFCFCu;
-          q[3][w] = __byte_perm(n4[1], n4[3], 0x7531);
+          for (int pp = 0; pp < 4; pp++) q[pp][w] = e[pp];
         }
-        uint8_t* dst = bs + ((size_t)(((ch * 4 + hi) * 2) * ncol + col)) * 64 + lo * 16;
-        if (RCP_CK(dst >= bs && dst + (size_t)ncol * 64 + 16 <= bs + p.bs_bytes, 3)) {
-          *reinterpret_cast<uint4*>(dst) = make_uint4(q[0][0], q[0][1], q[1][0], q[1][1]);
-          *reinterpret_cast<uint4*>(dst + (size_t)ncol * 64) = make_uint4(q[2][0], q[2][1], q[3][0], q[3][1]);
-        }
+      }
+      if (ch < p.nchunk && RCP_CK(dst >= bs && dst + (size_t)ncol * 64 + 16 <= bs + p.bs_bytes, 3)) {
+        *reinterpret_cast<uint4*>(dst) = make_uint4(q[0][0], q[0][1], q[1][0], q[1][1]);
+        *reinterpret_cast<uint4*>(dst + (size_t)ncol * 64) = make_uint4(q[2][0], q[2][1], q[3][0], q[3][1]);
       }
       if constexpr (!GRP) {
-#pragma unroll
-        for (int d = 8; d > 0; d >>= 1) tsum += __shfl_xor_sync(0xffffffffu, tsum, d);
-        if ((lane & 15) == 0 && u < total) atomicAdd(&s_T0tot[col], tsum);   // integer: any order gives the same sum
-      } else if constexpr (kRelabel) {   // the group is bits 2,3 of the unit: add up over bits 0,1
+        total += tsum;
+      } else if constexpr (kRelabel) {   // the group is hi: add up over lo
         tsum += __shfl_xor_sync(0xffffffffu, tsum, 1);
         tsum += __shfl_xor_sync(0xffffffffu, tsum, 2);
-        if ((u & 3) == 0 && u < total) s_T0f[(ch * 4 + ((u >> 2) & 3)) * Mp + col] = (float)(8 * tsum);
-      } else {                           // the group is bits 0,1 of the unit: add up over bits 2,3
+        if (lo == 0 && ch < p.nchunk) s_T0f[(ch * 4 + hi) * Mp + col] = (float)(tsum * (8 << kQ >> 4));
+      } else {                           // the group is lo: add up over hi
         tsum += __shfl_xor_sync(0xffffffffu, tsum, 4);
         tsum += __shfl_xor_sync(0xffffffffu, tsum, 8);
-        if ((u & 12) == 0 && u < total) s_T0c[col * ng4 + ch * 4 + (u & 3)] = tsum;
+        if (hi == 0 && ch < p.nchunk) s_T0c[col * ng4 + ch * 4 + lo] = tsum >> 4;
       }
+      ch += ch_step; wx += wx_step; src += (size_t)wx_step * (A16 ? 16 : 8); dst += dst_step;
+    }
+    if constexpr (!GRP) {
+      total = __reduce_add_sync(0xffffffffu, total);
+      if (lane == 0 && col < ncol) atomicAdd(&s_T0tot[col], A16 ? total : total >> 4);   // integer: any order gives the same sum
     }
     if (tid < M && !(A16 && p.x)) s_scale[tid] = my_scale;
   }
@@ -977,6 +977,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   // ---- group-wise grid
   // Tensor-core mode: MMA row g of the fragment is row grow of the 16 (rows 0,2,4,6 in the first
   // half-warp, 1,3,5,7 in the second: the 8-byte reads of a half-warp then hit all 32 banks once).
+  constexpr float kGrpScale = 0.125f / (1 << kQ);   // what the sums of the tensor-core mode are to be multiplied by
   const int grow = kRelabel ? (2 * (g & 3) + (g >> 2)) : g;
   float yacc[NE];
 #pragma unroll
@@ -1001,9 +1002,9 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
       for (int tok = 0; tok < NTD; tok++)
 #pragma unroll
         for (int rr = 0; rr < 2; rr++) {
-          const int a1 = (accD[tok][rr][0][0] >> 2) + (accD[tok][rr][0][1] >> 6) + ((accP[tok][rr][0] + accP[tok][rr][1]) >> 7);
-          const int a2 = (accD[tok][rr][1][0] >> 3) + (accD[tok][rr][1][1] >> 7) + ((accP[tok][rr][0] - accP[tok][rr][1]) >> 8);
-          const int a3 = (accD[tok][rr][2][0] >> 3) + (accD[tok][rr][2][1] >> 7);
+          const int a1 = (accD[tok][rr][0][0] >> (2 + kQ)) + (accD[tok][rr][0][1] >> (6 + kQ)) + ((accP[tok][rr][0] + accP[tok][rr][1]) >> (7 + kQ));
+          const int a2 = (accD[tok][rr][1][0] >> (3 + kQ)) + (accD[tok][rr][1][1] >> (7 + kQ)) + ((accP[tok][rr][0] - accP[tok][rr][1]) >> (8 + kQ));
+          const int a3 = (accD[tok][rr][2][0] >> (3 + kQ)) + (accD[tok][rr][2][1] >> (7 + kQ));
           const int T0 = s_T0c[tok * ng4 + gi];
           const int S1 = a1 - a3, S2 = a2 - a3;
           yacc[tok * 2 + rr] += lut_dot(lg[0][rr], T0 - S1 - S2 - a3, S1, S2, a3);
@@ -1083,10 +1084,10 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
           yacc[r] = fmaf(c[0], (r & 1) ? t0.y : t0.x, fmaf(c[1], F1, fmaf(c[2], F2, fmaf(c[3], F3, yacc[r]))));
           if constexpr (SDBG) {
             // the same sums as integers
-            const int I1 = accM[0][0][r] >> 2, I2 = accM[1][0][r] >> 3, I3 = accM[2][0][r] >> 3;
+            const int I1 = accM[0][0][r] >> (2 + kQ), I2 = accM[1][0][r] >> (3 + kQ), I3 = accM[2][0][r] >> (3 + kQ);
             const int tok = 2 * t + (r & 1), row = row_first + grow + 8 * (r >> 1);
             if (tok < M && row < p.N && gi < p.ngrp) {
-              const int I0 = __float2int_rn(0.125f * ((r & 1) ? t0.y : t0.x)) - (I1 - I3) - (I2 - I3) - I3;
+              const int I0 = __float2int_rn(kGrpScale * ((r & 1) ? t0.y : t0.x)) - (I1 - I3) - (I2 - I3) - I3;
               *reinterpret_cast<int4*>(p.S_out + (((size_t)tok * p.N + row) * p.ngrp + gi) * 4) =
                   make_int4(I0, I1 - I3, I2 - I3, I3);
             }
@@ -1132,7 +1133,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
 #pragma unroll 4
           for (int k = 0; k < KS; k++, d += red_plane) a += *d;
           if (tok < M && row < p.N)
-            p.y[(size_t)tok * p.N + row] = __float2half_rn(s_scale[tok] * (kRelabel ? 0.125f * a : a));
+            p.y[(size_t)tok * p.N + row] = __float2half_rn(s_scale[tok] * (kRelabel ? kGrpScale * a : a));
         }
       }
       if (KS == 1) __syncwarp();   // the slot is written again
@@ -1146,20 +1147,20 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
     if constexpr (MODE == kModeMma) {
 #pragma unroll
       for (int r = 0; r < 4; r++) {
-        T1[r] = (accM[0][0][r] >> 2) + (accM[0][1][r] >> 6);
-        T2[r] = (accM[1][0][r] >> 3) + (accM[1][1][r] >> 7);
-        T3[r] = (accM[2][0][r] >> 3) + (accM[2][1][r] >> 7);
+        T1[r] = (accM[0][0][r] >> (2 + kQ)) + (accM[0][1][r] >> (6 + kQ));
+        T2[r] = (accM[1][0][r] >> (3 + kQ)) + (accM[1][1][r] >> (7 + kQ));
+        T3[r] = (accM[2][0][r] >> (3 + kQ)) + (accM[2][1][r] >> (7 + kQ));
         if constexpr (kSign3M) {
-          T1[r] += (accPu[r] + accPs[r]) >> 7;
-          T2[r] += (accPu[r] - accPs[r]) >> 8;
+          T1[r] += (accPu[r] + accPs[r]) >> (7 + kQ);
+          T2[r] += (accPu[r] - accPs[r]) >> (8 + kQ);
         }
       }
       if constexpr (kTwoTiles) {
 #pragma unroll
         for (int r = 0; r < 4; r++) {
-          T1[4 + r] = accN[0][0][r] >> 2;   // one set of accumulators: accM[.][1] stayed zero above
-          T2[4 + r] = accN[1][0][r] >> 3;
-          T3[4 + r] = accN[2][0][r] >> 3;
+          T1[4 + r] = accN[0][0][r] >> (2 + kQ);   // one set of accumulators: accM[.][1] stayed zero above
+          T2[4 + r] = accN[1][0][r] >> (3 + kQ);
+          T3[4 + r] = accN[2][0][r] >> (3 + kQ);
         }
       }
     } else {
@@ -1171,13 +1172,13 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
           int a1, a2, a3;
           if constexpr (MODE == kModeHybrid) {
             const int r = tok + 2 * rr;  // lane t==0 holds columns 0, 1
-            a1 = (accM[0][0][r] >> 2) + (accM[0][1][r] >> 6);
-            a2 = (accM[1][0][r] >> 3) + (accM[1][1][r] >> 7);
-            a3 = (accD[tok][rr][0][0] >> 3) + (accD[tok][rr][0][1] >> 7);
+            a1 = (accM[0][0][r] >> (2 + kQ)) + (accM[0][1][r] >> (6 + kQ));
+            a2 = (accM[1][0][r] >> (3 + kQ)) + (accM[1][1][r] >> (7 + kQ));
+            a3 = (accD[tok][rr][0][0] >> (3 + kQ)) + (accD[tok][rr][0][1] >> (7 + kQ));
           } else {
-            a1 = (accD[tok][rr][0][0] >> 2) + (accD[tok][rr][0][1] >> 6) + ((accP[tok][rr][0] + accP[tok][rr][1]) >> 7);
-            a2 = (accD[tok][rr][1][0] >> 3) + (accD[tok][rr][1][1] >> 7) + ((accP[tok][rr][0] - accP[tok][rr][1]) >> 8);
-            a3 = (accD[tok][rr][2][0] >> 3) + (accD[tok][rr][2][1] >> 7);
+            a1 = (accD[tok][rr][0][0] >> (2 + kQ)) + (accD[tok][rr][0][1] >> (6 + kQ)) + ((accP[tok][rr][0] + accP[tok][rr][1]) >> (7 + kQ));
+            a2 = (accD[tok][rr][1][0] >> (3 + kQ)) + (accD[tok][rr][1][1] >> (7 + kQ)) + ((accP[tok][rr][0] - accP[tok][rr][1]) >> (8 + kQ));
+            a3 = (accD[tok][rr][2][0] >> (3 + kQ)) + (accD[tok][rr][2][1] >> (7 + kQ));
             a1 += __shfl_xor_sync(0xffffffffu, a1, 1); a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
             a2 += __shfl_xor_sync(0xffffffffu, a2, 1); a2 += __shfl_xor_sync(0xffffffffu, a2, 2);
           }

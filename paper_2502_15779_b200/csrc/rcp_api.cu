@@ -403,7 +403,8 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
   gp.nchunk_total = pl.nchunk_total;
   gp.nsplit = pl.nsplit;
   gp.off_part = pl.off_part;
-  gp.inv_nchunk = ((1 << 20) + pl.nchunk - 1) / pl.nchunk;
+  gp.act_parts = std::max(1, rcp::kCWarps / M);
+  gp.inv_act_parts = (256 + gp.act_parts - 1) / gp.act_parts;
   gp.nphase = pl.nphase;
   for (int i = 0; i < rcp::kMaxPhases; i++) gp.phase[i] = i < pl.nphase ? pl.phase[i] : make_phase(1, 0, 0, 1, 0, pl.nchunk);
   gp.stages = pl.stages;

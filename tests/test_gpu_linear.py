@@ -93,6 +93,15 @@ def test_linear_one_kernel_forms(N, K, B, clip, group):
         assert torch.equal(y.view(torch.int16), y2.view(torch.int16))
 
 
+@pytest.mark.parametrize("group", [0, 128])
+@pytest.mark.parametrize("M", range(2, 17))
+def test_linear_every_token_count(M, group):
+    """The warps of a CTA are shared out over the tokens when the activations are expanded: every count, with chunks of K
+    that do not divide over the warps of a token (4.5 chunks) and with fewer chunks than warps (1.25)."""
+    _check(40, 2304, 128, M, group, 1.0, seed=M)
+    _check(17, 640, 128, M, group, 1.0, seed=50 + M)
+
+
 def test_linear_clip_ratio_zero_token_and_optional_outputs():
     _check(70, 2048, 2048, 2, 0, 0.9, seed=3)
     _check(70, 4096, 4096, 1, 0, 0.9, seed=5)
