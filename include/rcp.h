@@ -206,9 +206,8 @@ size_t rcp_gemv_workspace_bytes(int M, int N, int K);
  *   out[4] 128-byte chunks per row, out[5] number of phases, then per phase five ints:
  *   groups per CTA at most, first group, groups in the phase, CTAs taking part, repetitions;
  *   and one last int: the parts of K one launch goes through one after the other (1 unless several tokens
- *   meet a K so long that their expanded activations do not fit in shared memory at once; rcp_gemv_w2a4 then
- *   runs the RCP_GEMV_MMA_STREAM form, one pass over K, where that form's ring fits, and the weight-only form
- *   goes through K in parts).
+ *   meet a K so long that their expanded activations do not fit in shared memory at once; for more than four
+ *   parts rcp_gemv_w2a4 runs the RCP_GEMV_MMA_STREAM form, one pass over K, where that form's ring fits).
  * (A group is 16 consecutive output rows; see the kernel's description.) Returns the number of
  * ints the full description has, or a negative status.
  */

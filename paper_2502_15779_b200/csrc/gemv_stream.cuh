@@ -292,7 +292,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   // plan is the same for every part, so the same lane meets the same sums again: nothing crosses warps.
   // A form of its own, so that the kernels that never need it keep their code.
   constexpr bool kSplit = SPLIT;
-  static_assert(!SPLIT || (MODE == kModeMma && MTOK == 0 && !GRP && FQ == 0), "K in parts: eight-column tensor-core kernels, per-row grid");
+  static_assert(!SPLIT || (MODE == kModeMma && (MTOK == 0 || MTOK == 8) && !GRP && FQ == 0), "K in parts: eight-column tensor-core kernels, per-row grid");
   static_assert(!SB || (MODE == kModeMma && FQ == 0 && !A16 && !SPLIT), "streamed activations: tensor-core kernels");
   constexpr int kThreads = SB ? kGThreads + 32 * kExpWarps : kGThreads;   // consumers, producer warp, and the expander warps (SB)
   const uint32_t stage_stride = SB ? (uint32_t)p.stage_stride : (uint32_t)kStageBytes;

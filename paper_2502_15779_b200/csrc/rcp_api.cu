@@ -457,6 +457,7 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
     if (M == 8 && !gp.S_out) return launch_stream_sb<8>(maps, gp, pl, st);
     return M > 8 ? launch_stream_sb<16>(maps, gp, pl, st) : launch_stream_sb<0>(maps, gp, pl, st);
   }
+  if (pl.nsplit > 1 && M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, false, 0, false, true, false>(maps, gp, pl, st);
   if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, 0, false, true>(maps, gp, pl, st);
   if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, false, 0, false, false, false>(maps, gp, pl, st);   // token count known at compile time
   return M > 8 ? launch_stream_t<rcp::kModeMma, 16>(maps, gp, pl, st) : launch_stream_t<rcp::kModeMma, 0>(maps, gp, pl, st);
@@ -468,10 +469,12 @@ int launch_stream_passes(int mode, int cap, const uint32_t* words, const void* l
                          bool grouped = false, int32_t* S_out = nullptr) {
   int nsplit = 1;
   const int mp = (grouped || cap < 8) ? tokens_per_pass(M, K, cap) : tokens_and_parts(M, N, K, cap, sm_count(), &nsplit);
-  // Where the launch would have to go through K in parts (several tokens, a long K), the form that streams the
-  // activations beside the weights is faster (measured: 8192 x 28672 at eight tokens 29.4 against 32.9 us); elsewhere
-  // expanding once up front wins, because the expansion competes with the mask arithmetic for the logic pipe.
-  if (mode == rcp::kModeMma && !grouped && nsplit > 1 && mp == std::min(M, 8)) {
+  // Where the launch would have to go through K in more than four parts (several tokens, a very long K), the form that
+  // streams the activations beside the weights is faster: it expands them once per phase, but chunk by chunk among the mask
+  // arithmetic, where parts pay a barrier, a fill of the ring's first stage and a set of parked sums each. Measured at eight
+  // tokens, parts against streamed: 8192x28672 (three) 30.3 and 32.2 us, 8192x40960 (four) 39.8 and 43.6, 8192x65536 (six)
+  // 67.2 and 58.3.
+  if (mode == rcp::kModeMma && !grouped && nsplit > 4 && mp == std::min(M, 8)) {
     const StreamPlan sp = make_plan(mp, N, K, sm_count(), false, 0, 1, true);
     if (sp.stages >= 3 && sp.smem <= kSmemMax) {
       for (int m0 = 0; m0 < M; m0 += mp) {

@@ -179,3 +179,10 @@ def test_linear_host_buffers(N, K, B, M, pinned):
         ref = oracle.gemv_w2a4(w_ref, f16_bits(lut), qa["xq"], qa["scale"])
         got = yh.float().numpy().astype(np.float64)
         assert np.all(np.isfinite(got)) and np.all(np.abs(got - ref["y"]) <= ref["tol"])
+
+
+@pytest.mark.parametrize("M,K", [(8, 16512), (8, 49152), (8, 53248), (5, 28672), (13, 28672)])
+def test_linear_long_k_in_parts_and_streamed(M, K):
+    """Several tokens over a K that goes in parts: two to four parts, and beyond four the form that streams the
+    activations; exactly eight tokens (counted at compile time), fewer, and a second launch for the rest."""
+    _check(50, K, 128, M, 0, 1.0, seed=M + K)
