@@ -33,6 +33,21 @@ __device__ __forceinline__ float lut_sum(uint2 lut4, int S0, int S1, int S2, int
   return acc;
 }
 
+// x / 7 correctly rounded, for finite x >= 0: the product with the rounded reciprocal and one correction by its exact
+// remainder (division by a constant after Markstein; compared with the division itself for all 2^31 values of x). The
+// quotient is on the critical path of every quantization, and the general division is four times as long.
+__device__ __forceinline__ float div_by_7(float x) {
+  constexpr float y = 1.0f / 7.0f;
+  const float q = __fmul_rn(x, y);
+  return __fmaf_rn(__fmaf_rn(-7.0f, q, x), y, q);
+}
+// 1 / s within one unit in the last place
+__device__ __forceinline__ float reciprocal_within_ulp(float s) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s));
+  return r;
+}
+
 // q[e] = clamp(round-half-even(v[e] / s), -8, 7) for NV values, the quotient being the IEEE fp32
 // division the definition asks for, without dividing in the common case. With rinv = 1 / s (correctly
 // rounded), t = v * rinv lies within 2^-23 |v / s| of the exact quotient and the IEEE quotient within half

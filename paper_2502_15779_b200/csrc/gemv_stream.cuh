@@ -518,7 +518,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
     float amax;
     if constexpr (FQ > 0) amax = rotate_full_token<E>(p.x, p.inv_sqrt_b, reinterpret_cast<float*>(gen + p.off_qbuf), s_amax, v[0]);
     else amax = rotate_block_token<NR>(p.x, W, p.had_block, p.inv_sqrt_b, s_amax, v);
-    const __half s16 = __float2half_rn(__fdiv_rn(__fmul_rn(amax, p.clip_ratio), 7.0f));
+    const __half s16 = __float2half_rn(div_by_7(__fmul_rn(amax, p.clip_ratio)));
     const float sc = __half2float(s16);
     if (tid == 0) {
       s_scale[0] = sc;

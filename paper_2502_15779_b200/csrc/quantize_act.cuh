@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(1024) quantize_act_kernel(const QuantParams p)
     amax = s_amax;
   }
 
-  const float s32 = __fdiv_rn(__fmul_rn(amax, p.clip_ratio), 7.0f);
+  const float s32 = div_by_7(__fmul_rn(amax, p.clip_ratio));
   const __half s16 = __float2half_rn(s32);
   const float s = __half2float(s16);
   if (rank == 0 && tid == 0) p.scale[m] = s16;
@@ -254,13 +254,13 @@ __device__ __forceinline__ uint32_t pack_nibbles(const float2* b) {
 }
 // Rounds NP pairs of values over s > 0 to int4, as the fp32 numbers 1.5 * 2^23 + q. `clamped` false (the same for the
 // whole warp): the caller knows that |v / s| < 7.5. Then v * (1 / s), rounded to an integer in the same operation,
-// differs by less than 1e-6 from the IEEE quotient, so the two round alike unless the remainder is within 4e-6 of a
-// half; such a warp divides. Every lane of the warp must call.
+// differs by less than 1.2e-6 from the IEEE quotient (the reciprocal is within 2^-23 of its own size, the quotient within
+// 2^-22), so the two round alike unless the remainder is within 4e-6 of a half; such a warp divides. Every lane of the warp must call.
 template <int NP>
 __device__ __forceinline__ void quantize_pairs(const float2 (&v)[NP], float s, bool clamped, float2 (&b)[NP]) {
   bool redo = clamped;
   if (!clamped) {
-    const float rinv = __frcp_rn(s);
+    const float rinv = reciprocal_within_ulp(s);
     const float2 r2 = make_float2(rinv, rinv), magic = make_float2(12582912.f, 12582912.f);
     const float2 minus = make_float2(-1.f, -1.f);
     float worst = 0.f;
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(T_MAX, 1024 / T_MAX) quantize_act_rows_kernel(
     if (lane == 0) s_max[par][warp] = am;
     __syncthreads();   // (the other half of s_max is free: everybody has read it before coming here)
     am = __reduce_max_sync(0xffffffffu, lane < nwarp ? s_max[par][lane] : 0u);
-    const __half s16 = __float2half_rn(__fdiv_rn(__fmul_rn(__uint_as_float(am), p.clip_ratio), 7.0f));
+    const __half s16 = __float2half_rn(div_by_7(__fmul_rn(__uint_as_float(am), p.clip_ratio)));
     const float s = __half2float(s16);
     if (tid == 0) p.scale[m] = s16;
     const bool clamped = needs_clamp(p.clip_ratio, s);
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) quantize_act_full_rows_kernel(c
     if (lane == 0) s_max[par][warp] = am;
     __syncthreads();
     am = __reduce_max_sync(0xffffffffu, s_max[par][lane % R]);
-    const __half s16 = __float2half_rn(__fdiv_rn(__fmul_rn(__uint_as_float(am), p.clip_ratio), 7.0f));
+    const __half s16 = __float2half_rn(div_by_7(__fmul_rn(__uint_as_float(am), p.clip_ratio)));
     const float s = __half2float(s16);
     if (tid == 0) p.scale[m] = s16;
 #pragma unroll

@@ -352,8 +352,27 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
   if (fa && (mode != rcp::kModeDp4a || !fused_ok(M, K, fa->B))) return RCP_ERR_VARIANT;
   EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return cuda_fail(cudaErrorNotSupported);
-  const StreamPlan pl = make_plan(M, N, K, sm_count(), grouped, fa ? (full_block(K, fa->B) ? rcp::full_rotate_bytes(K) : 0) : (sa ? (size_t)M * K : 0), nsplit,
-                                  stream_act);
+  // The plan depends on sizes and form alone; working it out costs the host a quarter of a microsecond, so the last few
+  // are remembered per thread.
+  struct PlanKey { size_t qbuf; int M, N, K, sms, nsplit, grouped, stream_act, unused; };   // (no padding: compared as bytes)
+  struct PlanSlot { PlanKey key; StreamPlan plan; };
+  constexpr int kPlanSlots = 16;
+  thread_local PlanSlot plan_cache[kPlanSlots] = {};   // (M is 0 in an unused slot)
+  thread_local int plan_next = 0;
+  PlanKey pk = {};
+  pk.M = M; pk.N = N; pk.K = K; pk.sms = sm_count(); pk.nsplit = nsplit; pk.grouped = grouped; pk.stream_act = stream_act;
+  pk.qbuf = fa ? (full_block(K, fa->B) ? rcp::full_rotate_bytes(K) : 0) : (sa ? (size_t)M * K : 0);
+  const StreamPlan* found = nullptr;
+  for (int i = 0; i < kPlanSlots && !found; i++)
+    if (std::memcmp(&plan_cache[i].key, &pk, sizeof(PlanKey)) == 0) found = &plan_cache[i].plan;
+  if (!found) {
+    PlanSlot& slot = plan_cache[plan_next];
+    plan_next = (plan_next + 1) % kPlanSlots;
+    slot.plan = make_plan(M, N, K, pk.sms, grouped, pk.qbuf, nsplit, stream_act);
+    slot.key = pk;
+    found = &slot.plan;
+  }
+  const StreamPlan& pl = *found;
   if (pl.stages < 2 || pl.smem > kSmemMax) return RCP_ERR_SHAPE;
   // Tensor maps of the phases in use (the others repeat the first). Encoding one costs the host about a
   // microsecond, so the maps of the last few (weights, shape, boxes) combinations are remembered per thread.
