@@ -9,6 +9,14 @@ namespace rcp {
 constexpr int kMaxTokens = 16;   // skinny regime of the GEMV
 constexpr int kMaxK = 65536;
 
+// dot products of four bytes: unsigned or signed bytes of a, signed bytes of b
+__device__ __forceinline__ void dp4a_u8s8(int& d, uint32_t a, uint32_t b) {
+  asm("dp4a.u32.s32 %0, %1, %2, %0;" : "+r"(d) : "r"(a), "r"(b));
+}
+__device__ __forceinline__ void dp4a_s8s8(int& d, uint32_t a, uint32_t b) {
+  asm("dp4a.s32.s32 %0, %1, %2, %0;" : "+r"(d) : "r"(a), "r"(b));
+}
+
 __device__ __forceinline__ int sext4(uint32_t nib) { return (int)((nib ^ 8u) & 0xFu) - 8; }
 
 // y = s * (L0*S0 + L1*S1 + L2*S2 + L3*S3), fp32 arithmetic, integers converted exactly (|S| < 2^24).

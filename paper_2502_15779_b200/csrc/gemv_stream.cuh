@@ -201,12 +201,6 @@ __device__ __forceinline__ uint32_t and3(uint32_t a, uint32_t b, uint32_t c) {
   asm("lop3.b32 %0, %1, %2, %3, 0x80;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
   return d;
 }
-__device__ __forceinline__ void dp4a_u8s8(int& d, uint32_t a, uint32_t b) {
-  asm("dp4a.u32.s32 %0, %1, %2, %0;" : "+r"(d) : "r"(a), "r"(b));
-}
-__device__ __forceinline__ void dp4a_s8s8(int& d, uint32_t a, uint32_t b) {
-  asm("dp4a.s32.s32 %0, %1, %2, %0;" : "+r"(d) : "r"(a), "r"(b));
-}
 
 // The sixteen int4 activations of a word of codes (lo32: codes 0..7, hi32: codes 8..15) as the four dot-product operands:
 // byte j of q[p] meets code 4 j + p, 16 q for even positions and 4 q for odd ones. (16 q is the nibble in the upper half of

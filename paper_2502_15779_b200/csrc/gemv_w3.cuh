@@ -205,22 +205,36 @@ __device__ __forceinline__ uint32_t w3_and_mask(uint32_t a, uint32_t b) {
   asm("lop3.b32 %0, %1, %2, %3, 0x80;" : "=r"(d) : "r"(a), "r"(b), "n"(MASK));
   return d;
 }
-// In-byte position PP of a word: the seven products of code bits, one logic operation each (the mask keeps the
-// even bit of the position, so stray odd bits of hb and zz drop out), and their seven dot products.
+// In-byte position PP of a word: the seven products of code bits and their dot products. w: the word (b0 in the even, b1 in
+// the odd bits), s = 2 w (b0 in the odd bits), ws = w & s (b0 b1 there), Z: b2 in the odd bits. All but b0 are taken at the
+// odd bit of the position, where a plane word's second half stands as it is and its first half after one addition, so no
+// right shift is needed (additions run on either of two pipes, shifts and logic on one, which bounds this kernel); the
+// other bits drop out under the mask. Position 3 sits in bits 6 and 7: one mask keeps both, and read as unsigned and as
+// signed bytes it weighs 64 b0 + 128 b1 and 64 b0 - 128 b1, which gives b0 and b1 (accP).
 template <int PP>
-__device__ __forceinline__ void w3_position(uint32_t w, uint32_t hb, uint32_t whb, uint32_t zz, uint32_t q,
-                                            int (&acc)[7][2]) {
-  constexpr uint32_t m = 0x01010101u << (2 * PP);
-  uint32_t P[7];
-  P[0] = w & m;                          // b0
-  P[1] = hb & m;                         // b1
-  P[2] = whb & m;                        // b0 b1
-  P[3] = zz & m;                         // b2
-  P[4] = w3_and_mask<m>(w, zz);          // b0 b2
-  P[5] = w3_and_mask<m>(hb, zz);         // b1 b2
-  P[6] = w3_and_mask<m>(whb, zz);        // b0 b1 b2
+__device__ __forceinline__ void w3_position(uint32_t w, uint32_t s, uint32_t ws, uint32_t Z, uint32_t q, int (&acc)[7][2],
+                                            int (&accP)[2]) {
+  constexpr uint32_t m0 = 0x01010101u << (2 * PP), m1 = m0 << 1;
+  if constexpr (PP < 3) {
+    dp4a_u8s8(acc[0][PP >> 1], w & m0, q);                        // b0
+    dp4a_u8s8(acc[1][PP >> 1], w & m1, q);                        // b1, times 2 like all that follow
+  } else {
+    const uint32_t both = w & 0xC0C0C0C0u;
+    dp4a_u8s8(accP[0], both, q);
+    dp4a_s8s8(accP[1], both, q);
+  }
+  dp4a_u8s8(acc[2][PP >> 1], ws & m1, q);                         // b0 b1
+  dp4a_u8s8(acc[3][PP >> 1], Z & m1, q);                          // b2
+  dp4a_u8s8(acc[4][PP >> 1], w3_and_mask<m1>(s, Z), q);           // b0 b2
+  dp4a_u8s8(acc[5][PP >> 1], w3_and_mask<m1>(w, Z), q);           // b1 b2
+  dp4a_u8s8(acc[6][PP >> 1], w3_and_mask<m1>(ws, Z), q);          // b0 b1 b2
+}
+// the subset sums t[0..6] (b0, b1, b0 b1, b2, b0 b2, b1 b2, b0 b1 b2) from the accumulators
+__device__ __forceinline__ void w3_subset_sums(const int (&acc)[7][2], const int (&accP)[2], int (&t)[7]) {
+  t[0] = (acc[0][0] >> 2) + (acc[0][1] >> 6) + ((accP[0] + accP[1]) >> 7);
+  t[1] = (acc[1][0] >> 3) + (acc[1][1] >> 7) + ((accP[0] - accP[1]) >> 8);
 #pragma unroll
-  for (int f = 0; f < 7; f++) acc[f][PP >> 1] = __dp4a((int)P[f], (int)q, acc[f][PP >> 1]);
+  for (int f = 2; f < 7; f++) t[f] = (acc[f][0] >> 3) + (acc[f][1] >> 7);
 }
 
 // One token per launch. Shared memory: the token's activations expanded to one byte per code, 16 bytes per
@@ -311,9 +325,14 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
   const float s = __half2float(p.scale[0]);
   const int ngrp = p.K / 128;
   // The arithmetic of a lane step into the fourteen accumulators (weights beyond K are zeros: no guard needed).
-  int acc[7][2];
+  int acc[7][2], accP[2];
+  auto clear = [&]() {
 #pragma unroll
-  for (int f = 0; f < 7; f++) { acc[f][0] = 0; acc[f][1] = 0; }
+    for (int f = 0; f < 7; f++) { acc[f][0] = 0; acc[f][1] = 0; }
+    accP[0] = 0;
+    accP[1] = 0;
+  };
+  clear();
   const uint4* const act_lane = s_act + lane;
   auto lane_step = [&](const Step& c, int it) {
     const uint4* const act = act_lane + it * 256;
@@ -322,27 +341,25 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
       const uint32_t ww[4] = {c.a[h].x, c.a[h].y, c.a[h].z, c.a[h].w};
 #pragma unroll
       for (int i = 0; i < 4; i++) {
-        const uint32_t w = ww[i], hb = w >> 1, whb = w & hb;
-        const uint32_t zsel = (i < 2) ? c.z[h].x : c.z[h].y;
-        const uint32_t zz = (i & 1) ? (zsel >> 1) : zsel;   // top bits lined up with the b0 bits (odd bits: the other half's)
+        const uint32_t w = ww[i], s = w + w, ws = w & s;
+        const uint32_t z = (i < 2) ? c.z[h].x : c.z[h].y;
+        const uint32_t Z = (i & 1) ? z : z + z;   // the plane word's first half is in its even bits, the second in the odd ones
         const uint4 q = act[(h * 4 + i) * 32];
-        w3_position<0>(w, hb, whb, zz, q.x, acc);
-        w3_position<1>(w, hb, whb, zz, q.y, acc);
-        w3_position<2>(w, hb, whb, zz, q.z, acc);
-        w3_position<3>(w, hb, whb, zz, q.w, acc);
+        w3_position<0>(w, s, ws, Z, q.x, acc, accP);
+        w3_position<1>(w, s, ws, Z, q.y, acc, accP);
+        w3_position<2>(w, s, ws, Z, q.z, acc, accP);
+        w3_position<3>(w, s, ws, Z, q.w, acc, accP);
       }
     }
   };
   // Group-wise grid: this lane's 128 codes of step `it` are group lane + 32 it of the row; its term of y.
   auto finish_group = [&](int row, int it) -> float {
     const int gi = lane + 32 * it;
-    int t[8], S[8];
+    int sums[7], t[8], S[8];
+    w3_subset_sums(acc, accP, sums);
+    clear();
 #pragma unroll
-    for (int f = 0; f < 7; f++) {
-      t[f + 1] = (acc[f][0] >> 2) + (acc[f][1] >> 6);
-      acc[f][0] = 0;
-      acc[f][1] = 0;
-    }
+    for (int f = 0; f < 7; f++) t[f + 1] = sums[f];
     if (gi >= ngrp) return 0.f;
     t[0] = s_t0g[GRP ? gi : 0];
     w3_percode(t, S);
@@ -389,12 +406,10 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
       }
     } else if (last) {
       int t[7];
+      w3_subset_sums(acc, accP, t);
+      clear();
 #pragma unroll
-      for (int f = 0; f < 7; f++) {
-        t[f] = __reduce_add_sync(0xffffffffu, (acc[f][0] >> 2) + (acc[f][1] >> 6));   // one instruction per sum
-        acc[f][0] = 0;
-        acc[f][1] = 0;
-      }
+      for (int f = 0; f < 7; f++) t[f] = __reduce_add_sync(0xffffffffu, t[f]);   // one instruction per sum
       if (lane == 0) {
         s_sum[warp][cnt][0] = make_int4(t[0], t[1], t[2], t[3]);
         s_sum[warp][cnt][1] = make_int4(t[4], t[5], t[6], 0);
