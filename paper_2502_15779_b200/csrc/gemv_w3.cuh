@@ -239,18 +239,21 @@ __device__ __forceinline__ void w3_subset_sums(const int (&acc)[7][2], const int
 
 // One token per launch. Shared memory: the token's activations expanded to one byte per code, 16 bytes per
 // word of 16 codes: { position 0 (times 4), position 1, position 2 (times 4), position 3 }, byte j of a position =
-// activation of code 16 w + 4 j + p. A lane step covers 64 units of 64 codes; lane l takes units 2l and 2l + 1 of
-// it (128 consecutive codes, one group of the group-wise grid), i.e. eight words c = 0..7. Word c of lane l in
+// activation of code 16 w + 4 j + p. A lane step covers 64 units of 64 codes; lane l takes units 2l and 2l + 1 of it (128
+// consecutive codes, one group of the group-wise grid; HALF: units l and l + 32), i.e. eight words c = 0..7. Word c of lane l in
 // step `it` sits at 16-byte slot (it * 8 + c) * 32 + l: the lanes of a warp read consecutive slots (no bank
 // conflicts) at offsets from one address that are known at compile time. K is padded to whole lane steps with
 // zeros (weights beyond K are loaded as zeros as well, so the padding contributes nothing).
 // Four CTAs per SM (64 registers, no spills): 32 warps hide the weight loads better than the 24 that the
 // compiler's own choice of 80 registers leaves (57344x8192: 74.5 against 76.8 us).
+//   HALF: where the last step of a row is at most half full (K = 14336 is three and a half steps), every lane has a unit of
+// each half, and the empty half is left out by the whole warp: 4096x14336 15.1 -> 13.9 us. A form of its own, because the
+// branch costs spills at 64 registers (57344x8192 would take 74.7 us instead of 69.1).
 //   A warp's (row, lane step) pairs are one sequence, worked on from two buffers in turn, the weights of the next pair on
 // their way. A finished row leaves its seven sums in shared memory; the eight-level dot products are done for up to 32 rows
 // at once, one per lane. (One lane finishing one row at a time was a tenth of the instructions at K = 4096 and, with them,
 // its latency once a row: 28672x4096 23.1 -> 20.9 us, 57344x8192 74.2 -> 70.6.)
-template <bool GRP, bool SDBG>
+template <bool GRP, bool SDBG, bool HALF>
 __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params p) {
   extern __shared__ uint4 s_act[];           // [lane steps][8][32]
   constexpr int kWarps = kW3Threads / 32;
@@ -262,15 +265,18 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
   const int nunit = p.K / 64;
   const int nit = (nunit + 63) / 64;         // lane steps per row
   const int warps = gridDim.x * kWarps;
+  static_assert(!(GRP && HALF), "the group-wise grid wants both units of a group in one lane");
+  const int unit0 = HALF ? lane : 2 * lane;   // a lane's units in a step: unit0 and unit0 + unit_h
+  constexpr int unit_h = HALF ? 32 : 1;
   struct Step { uint4 a[2]; uint2 z[2]; };   // the weights of a lane step: two units, each one uint4 of words2, one uint2 of words1
   auto fetch = [&](int row, int it, Step& d) {
-    const int u = 2 * lane + 64 * it;
+    const int u = unit0 + 64 * it;
     const size_t e = (size_t)row * nunit + u;
 #pragma unroll
     for (int h = 0; h < 2; h++) {
-      const bool ok = row < p.N && u + h < nunit;
-      d.a[h] = ok ? __ldg(reinterpret_cast<const uint4*>(p.words2) + e + h) : make_uint4(0, 0, 0, 0);
-      d.z[h] = ok ? __ldg(reinterpret_cast<const uint2*>(p.words1) + e + h) : make_uint2(0, 0);
+      const bool ok = row < p.N && u + h * unit_h < nunit;
+      d.a[h] = ok ? __ldg(reinterpret_cast<const uint4*>(p.words2) + e + h * unit_h) : make_uint4(0, 0, 0, 0);
+      d.z[h] = ok ? __ldg(reinterpret_cast<const uint2*>(p.words1) + e + h * unit_h) : make_uint2(0, 0);
     }
   };
   // Rows are dealt round-robin to all warps of the grid (one resident wave of CTAs). Launched with programmatic stream
@@ -278,8 +284,8 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
   // first weights are sent on their way to L2, which is where such a kernel would put them (4096x14336: 15.7 -> 15.4 us).
   const int gw = blockIdx.x * kWarps + warp;
   Step A, B;
-  if (gw < p.N && 2 * lane < nunit) {
-    const size_t e = (size_t)gw * nunit + 2 * lane;
+  if (gw < p.N && unit0 < nunit) {
+    const size_t e = (size_t)gw * nunit + unit0;
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p.words2 + 4 * e));
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p.words1 + 2 * e));
   }
@@ -300,8 +306,9 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
     pos.z = (__byte_perm(e0, e1, 0x7531) << 2) & 0xFCFCFCFCu;   // codes 2,6,10,14, times 4
     pos.w = __byte_perm(o0, o1, 0x7531);                        // codes 3,7,11,15
     int wsum = __dp4a((int)e0, 0x01010101, __dp4a((int)o0, 0x01010101, __dp4a((int)e1, 0x01010101, __dp4a((int)o1, 0x01010101, 0))));
-    // word w = 8 (32 it + l) + c
-    s_act[((w >> 8) * 8 + (w & 7)) * 32 + ((w >> 3) & 31)] = pos;
+    // word c = 4 h + i of lane l in step w >> 8: word i of its unit h
+    if constexpr (HALF) s_act[((w >> 7) * 4 + (w & 3)) * 32 + ((w >> 2) & 31)] = pos;
+    else s_act[((w >> 8) * 8 + (w & 7)) * 32 + ((w >> 3) & 31)] = pos;
     if constexpr (GRP) {
       // eight consecutive words are one group; they belong to eight consecutive lanes
       wsum += __shfl_xor_sync(0xffffffffu, wsum, 1);
@@ -338,6 +345,7 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
     const uint4* const act = act_lane + it * 256;
 #pragma unroll
     for (int h = 0; h < 2; h++) {
+      if (HALF && h == 1 && 64 * it + 32 >= nunit) break;
       const uint32_t ww[4] = {c.a[h].x, c.a[h].y, c.a[h].z, c.a[h].w};
 #pragma unroll
       for (int i = 0; i < 4; i++) {

@@ -211,3 +211,10 @@ def test_w3a4_more_rows_than_a_warp_finishes_at_once():
     N = 592 * 8 * 32 + 4736 + 77
     rows = np.unique(np.concatenate([np.arange(40), np.arange(151540, 151570), np.arange(N - 40, N)]))
     _check(N, 64, 1, 0, seed=5, rows=rows)
+
+
+@pytest.mark.parametrize("K", [64, 2048, 2112, 4096, 6144, 6208, 14336, 18432, 22528])
+def test_w3a4_last_lane_step_half_full_or_more(K):
+    """Rows whose last lane step (4096 codes) holds 64, exactly half, just over half and all of its codes, on both sides of
+    the length up to which the empty half is left out."""
+    _check(70, K, 2, 0, seed=K)
