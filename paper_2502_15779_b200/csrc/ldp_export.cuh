@@ -104,8 +104,9 @@ __global__ void __launch_bounds__(256) ldp_export_kernel(const LdpParams p) {
 // definition itself (c_i reaches t_i, its predecessor does not); where that first guess is off by more than one
 // value, a bisection over the fp16 numbers finds it.
 //   A warp takes 32 units = 4096 consecutive weights (units are consecutive in memory whatever K is) and keeps them
-// in registers, 16 vectors of 8 weights per lane, so they are read once, the next tile being copied to shared memory meanwhile. Per-unit minima and maxima meet in a
-// transposing reduction (15 exchanges for 16 values instead of 4 per value), which leaves lane l with unit
+// in registers, 16 vectors of 8 weights per lane, so they are read once, the next tile being copied to shared memory
+// meanwhile. Per-unit minima and maxima meet in a transposing reduction (15 exchanges for 16 values instead of 4 per
+// value), which leaves lane l with unit
 // 2 (l & 15) + (l >> 4): the per-unit arithmetic runs once per unit, one unit per lane. About 8 instructions per
 // weight against 40. 28672 x 4096 weights: 56 us, 456 with the kernel above (memory floor 44).
 constexpr int kLdpGroup = 128;
