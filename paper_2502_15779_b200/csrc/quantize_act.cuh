@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(1024) quantize_act_kernel(const QuantParams p)
 // adds, products and the rounding work on pairs (the two-wide fp32 instructions round each half like the scalar ones)
 // and the clamp of the rounding is left out where it cannot act. Same operations on the same operands in the same
 // order as above: bit-identical results. 2048 tokens, us before (cluster, or one CTA of 512 threads with four barriers)
-// and now, memory floor: K = 4096 27.1, 12.2, 3.3; K = 8192 33.8, 23.9, 6.5; K = 14336 in blocks of 128 78.4, 28.5, 11.4.
+// and now, memory floor: K = 4096 27.1, 10.6, 3.3; K = 8192 33.8, 21.5, 6.5; K = 14336 in blocks of 128 78.4, 25.5, 11.4.
 // Fewer barriers also make it the faster form for one token (K = 4096: 2.8 -> 1.8 us).
 
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -273,13 +273,13 @@ __device__ __forceinline__ void quantize_pairs(const float2 (&v)[NP], float s, b
     redo = __any_sync(0xffffffffu, worst > 0.499996f);
   }
   if (redo) {
-    float t[2 * NP];
-    int q[2 * NP];
 #pragma unroll
-    for (int i = 0; i < NP; i++) { t[2 * i] = v[i].x; t[2 * i + 1] = v[i].y; }
-    quantize_int4<2 * NP>(t, s, q);
-#pragma unroll
-    for (int i = 0; i < NP; i++) b[i] = make_float2(__int_as_float(q[2 * i] + 0x4B400000), __int_as_float(q[2 * i + 1] + 0x4B400000));
+    for (int i = 0; i < NP; i++) {   // (pair by pair: rare, and fewer registers: 2048 tokens of 8064 in blocks of 64 16.4 -> 14.6 us)
+      const float t[2] = {v[i].x, v[i].y};
+      int q[2];
+      quantize_int4<2>(t, s, q);
+      b[i] = make_float2(__int_as_float(q[0] + 0x4B400000), __int_as_float(q[1] + 0x4B400000));
+    }
   }
 }
 // The word's sixteen int4 values, packed.
@@ -378,21 +378,25 @@ __global__ void __launch_bounds__(T_MAX, 1024 / T_MAX) quantize_act_rows_kernel(
 // One rotation block over the whole token, NT = K / 16 threads (K = 2048, 4096 or 8192). Strides 1..8 inside the word;
 // 16..128 after a transposition inside the warp, 256 by one lane exchange; 512 and up after a transposition across the
 // R = NT / 32 warps, every thread taking 16 / R columns of R values; then back to words, the absmax meeting at the same
-// barrier. The buffer of the cross-warp passes is used in turn with a second one: two barriers per token.
+// barrier: two barriers per token. One buffer serves all of it, element e of word t at e QP + t: outside the cross-warp
+// pass, which lies between the barriers, a warp touches only the columns of its own words.
+// Storing a word by element and reading sixteen words of one element with four 16-byte loads (no bank conflicts either
+// way) replaces a transposition through a buffer of its own: 2048 tokens of 4096 11.5 -> 10.6 us, of 8192 23.1 -> 21.5.
+constexpr int kFullRowsThreads = 1024;   // per SM; with 1280 or 1536 the registers spill (4096: 11.8 and 14.5 us)
 template <int NT>
-__host__ __device__ constexpr size_t full_rows_smem() { return (size_t)(NT * 17 + 2 * 16 * (NT + 4)) * 4; }
+__host__ __device__ constexpr size_t full_rows_smem() { return (size_t)16 * (NT + 4) * 4; }
 
 template <int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) quantize_act_full_rows_kernel(const QuantParams p, int M) {
-  extern __shared__ __align__(16) float sbuf[];   // full_rows_smem<NT>()
-  constexpr int R = NT / 32, kPitch = 17, QP = NT + 4;
+__global__ void __launch_bounds__(NT, kFullRowsThreads / NT) quantize_act_full_rows_kernel(const QuantParams p, int M) {
+  extern __shared__ __align__(16) float qbuf[];   // full_rows_smem<NT>()
+  constexpr int R = NT / 32, QP = NT + 4;
   __shared__ unsigned s_max[2][R];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   asm volatile("griddepcontrol.launch_dependents;");
   prefetch_token(p.x + (size_t)blockIdx.x * (NT * 16), NT * 16, tid);
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  float* const wbuf = sbuf + warp * (32 * kPitch);
   const int e1 = lane & 15, hi = lane & 16;
+  float4* const own = reinterpret_cast<float4*>(qbuf + e1 * QP + warp * 32 + hi);   // element e1 of the words hi .. hi + 15
   uint4 raw[2];
   auto fetch = [&](int m) {
     const uint4* const src = reinterpret_cast<const uint4*>(p.x + (size_t)m * (NT * 16)) + 2 * tid;
@@ -402,18 +406,19 @@ __global__ void __launch_bounds__(NT, 1024 / NT) quantize_act_full_rows_kernel(c
   int par = 0;
   fetch(blockIdx.x);
   for (int m = blockIdx.x; m < M; m += gridDim.x, par ^= 1) {
-    float* const qbuf = sbuf + NT * 17 + par * (16 * QP);
     float2 v[8];
     word_from_halves(raw[0], raw[1], v);
     if (m + (int)gridDim.x < M) fetch(m + gridDim.x);
     butterflies_word(v, 16);   // strides 1..8
 #pragma unroll
-    for (int i = 0; i < 8; i++) { wbuf[lane * kPitch + 2 * i] = v[i].x; wbuf[lane * kPitch + 2 * i + 1] = v[i].y; }
+    for (int i = 0; i < 8; i++) { qbuf[2 * i * QP + tid] = v[i].x; qbuf[(2 * i + 1) * QP + tid] = v[i].y; }
     __syncwarp();
 #pragma unroll
-    for (int i = 0; i < 8; i++)   // element e1 of the words hi + 2 i, hi + 2 i + 1
-      v[i] = make_float2(wbuf[(hi | (2 * i)) * kPitch + e1], wbuf[(hi | (2 * i + 1)) * kPitch + e1]);
-    __syncwarp();
+    for (int j = 0; j < 4; j++) {
+      const float4 f = own[j];
+      v[2 * j] = make_float2(f.x, f.y);
+      v[2 * j + 1] = make_float2(f.z, f.w);
+    }
     butterflies_word(v, 16);   // strides 16..128
     {
       const float sign = hi ? -1.f : 1.f;
@@ -424,11 +429,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) quantize_act_full_rows_kernel(c
         v[i] = __ffma2_rn(v[i], s2, other);
       }
     }
-    {
-      float4* const dst = reinterpret_cast<float4*>(qbuf + e1 * QP + warp * 32 + hi);
 #pragma unroll
-      for (int j = 0; j < 4; j++) dst[j] = make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
-    }
+    for (int j = 0; j < 4; j++) own[j] = make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
     __syncthreads();
     float amax = 0.f;
     // element c R + warp: its R words 32 apart (values 2 i and 2 i + 1 of the thread are words 2 i and 2 i + 1 of R)
@@ -470,14 +472,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) quantize_act_full_rows_kernel(c
 // warps' strides after a transposition across the warps: there a column of sixteen values, one per warp, is shared by
 // 16 / E lanes, E values each, and a last lane exchange or two. Two barriers (named barrier 1, 512 threads).
 // buf: full_rotate_bytes<E>() bytes, 16-byte aligned; s_amax: 16 words.
-//   Cross-warp buffer: element e of lane l of warp w at e kQP + 32 w + (w / E) kPL + l. The pads make every access below
-// free of bank conflicts.
+//   One buffer for both transpositions (57344x8192 30.8 -> 30.3 us a call, a ring stage more fitting beside it; with one
+// for each before): element e of lane l of warp w at e kQP + 32 w + (w / E) kPL + l. The pads make
+// every access below free of bank conflicts.
 template <int E>
 struct FullRotate {
-  static constexpr int kP = E + 1;              // pitch of the in-warp transposition
   static constexpr int kPL = 2 * E;             // the lanes that share a column are kPL apart
   static constexpr int kQP = E == 16 ? 516 : E == 8 ? 548 : 552;
-  static constexpr size_t kBytes = (size_t)(512 * kP + E * kQP) * 4;
+  static constexpr size_t kBytes = (size_t)E * kQP * 4;
 };
 __host__ constexpr size_t full_rotate_bytes(int K) {
   return K == 2048 ? FullRotate<4>::kBytes : K == 4096 ? FullRotate<8>::kBytes : FullRotate<16>::kBytes;
@@ -520,8 +522,9 @@ __device__ __forceinline__ float rotate_full_token(const __half* x, float inv_sq
   using F = FullRotate<E>;
   constexpr int NP = E / 2;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float* const wbuf = buf + warp * (32 * F::kP);
-  float* const qbuf = buf + 512 * F::kP;
+  float* const mine = buf + warp * 32 + (warp / E) * F::kPL + lane;
+  const int e1 = lane % E, l1 = lane - e1;   // after the transposition this lane has element e1 of the lanes l1 .. l1 + E - 1
+  float4* const own = reinterpret_cast<float4*>(buf + e1 * F::kQP + warp * 32 + (warp / E) * F::kPL + l1);
   {
     uint32_t raw[NP];
     if constexpr (E == 4) {
@@ -539,24 +542,24 @@ __device__ __forceinline__ float rotate_full_token(const __half* x, float inv_sq
   }
   butterflies_pairs<NP>(v);   // strides 1 .. E / 2
 #pragma unroll
-  for (int i = 0; i < NP; i++) { wbuf[lane * F::kP + 2 * i] = v[i].x; wbuf[lane * F::kP + 2 * i + 1] = v[i].y; }
+  for (int i = 0; i < NP; i++) { mine[2 * i * F::kQP] = v[i].x; mine[(2 * i + 1) * F::kQP] = v[i].y; }
   __syncwarp();
-  const int e1 = lane % E, l1 = lane - e1;   // this lane: element e1 of the lanes l1 .. l1 + E - 1
 #pragma unroll
-  for (int i = 0; i < NP; i++) v[i] = make_float2(wbuf[(l1 + 2 * i) * F::kP + e1], wbuf[(l1 + 2 * i + 1) * F::kP + e1]);
+  for (int j = 0; j < E / 4; j++) {
+    const float4 f = own[j];
+    v[2 * j] = make_float2(f.x, f.y);
+    v[2 * j + 1] = make_float2(f.z, f.w);
+  }
   butterflies_pairs<NP>(v);   // strides E .. E E / 2
 #pragma unroll
   for (int d = E; d < 32; d *= 2) butterfly_exchange<NP>(v, d, (lane & d) != 0);   // .. 16 E
-  {
-    float4* const dst = reinterpret_cast<float4*>(qbuf + e1 * F::kQP + warp * 32 + (warp / E) * F::kPL + l1);
 #pragma unroll
-    for (int j = 0; j < E / 4; j++) dst[j] = make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
-  }
+  for (int j = 0; j < E / 4; j++) own[j] = make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
   asm volatile("bar.sync 1, 512;" ::: "memory");
   {
     constexpr int kLC = 16 / E;              // warps that share an element's columns, and lanes that share a column
     const int wq = lane / F::kPL;            // this lane: the values of the warps wq E .. wq E + E - 1
-    float* const col = qbuf + (warp / kLC) * F::kQP + wq * (E * 32 + F::kPL) + (warp % kLC) * F::kPL + lane % F::kPL;
+    float* const col = buf + (warp / kLC) * F::kQP + wq * (E * 32 + F::kPL) + (warp % kLC) * F::kPL + lane % F::kPL;
 #pragma unroll
     for (int i = 0; i < NP; i++) v[i] = make_float2(col[2 * i * 32], col[(2 * i + 1) * 32]);
     butterflies_pairs<NP>(v);
@@ -574,7 +577,6 @@ __device__ __forceinline__ float rotate_full_token(const __half* x, float inv_sq
     if (lane == 0) s_amax[warp] = am;
   }
   asm volatile("bar.sync 1, 512;" ::: "memory");
-  const float* const mine = qbuf + warp * 32 + (warp / E) * F::kPL + lane;
 #pragma unroll
   for (int i = 0; i < NP; i++) v[i] = make_float2(mine[2 * i * F::kQP], mine[(2 * i + 1) * F::kQP]);
   return __uint_as_float(__reduce_max_sync(0xffffffffu, s_amax[lane & 15]));

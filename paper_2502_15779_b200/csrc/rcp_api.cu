@@ -579,7 +579,7 @@ int launch_full_rows(const rcp::QuantParams& qp, int M, cudaStream_t st) {
   static bool attr_set[kMaxDevices] = {};
   auto kern = rcp::quantize_act_full_rows_kernel<NT>;
   RCP_CUDA(set_max_smem(kern, (int)rcp::full_rows_smem<NT>(), mu, attr_set));
-  const int grid = std::min(M, sm_count() * (1024 / NT));
+  const int grid = std::min(M, sm_count() * (rcp::kFullRowsThreads / NT));
   RCP_CUDA(launch_overlapped(kern, dim3(grid), dim3(NT), rcp::full_rows_smem<NT>(), st, qp, M));
   return RCP_OK;
 }
