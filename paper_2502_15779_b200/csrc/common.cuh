@@ -49,6 +49,13 @@ __device__ __forceinline__ float div_by_7(float x) {
   const float q = __fmul_rn(x, y);
   return __fmaf_rn(__fmaf_rn(-7.0f, q, x), y, q);
 }
+// What keeps x = amax * clip_ratio finite, where the correction would turn infinity into NaN. The largest rotated magnitude
+// is below 6e6 and the smallest above 6e-10 (a multiple of 2^-24 over the root of 8192 at most), so beyond
+// kClipRatioCap every scale but zero is infinity in fp16 whatever the ratio is, and the host passes no larger one; the
+// warps' maxima are cut off at kAmaxCap, which only an infinite activation reaches. (Cut off where each warp leaves its
+// maximum: one minimum more behind the barrier cost 2.5 % at 2048 tokens of 4096, here it is free.)
+constexpr float kClipRatioCap = 1e18f, kAmaxCap = 1e20f;
+
 // 1 / s within one unit in the last place
 __device__ __forceinline__ float reciprocal_within_ulp(float s) {
   float r;

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(1024) quantize_act_kernel(const QuantParams p)
   for (int e = 0; e < 8; e++) amax = fmaxf(amax, fabsf(v[e]));
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
-  if (lane == 0) s_red[tid >> 5] = amax;
+  if (lane == 0) s_red[tid >> 5] = fminf(amax, kAmaxCap);
   __syncthreads();
   if (tid < 32) {
     float a = (tid < (int)((blockDim.x + 31) >> 5)) ? s_red[tid] : 0.f;
@@ -252,10 +252,18 @@ __device__ __forceinline__ uint32_t pack_nibbles(const float2* b) {
   const uint32_t hi = __byte_perm(__byte_perm(o[0], o[1], 0x0040), __byte_perm(o[2], o[3], 0x0040), 0x5410);
   return (lo & 0x0F0F0F0Fu) | ((hi << 4) & 0xF0F0F0F0u);
 }
+// the largest magnitude of the three, NaN where any of them is one
+__device__ __forceinline__ float max3_magnitude_or_nan(float a, float b, float c) {
+  float d;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
 // Rounds NP pairs of values over s > 0 to int4, as the fp32 numbers 1.5 * 2^23 + q. `clamped` false (the same for the
 // whole warp): the caller knows that |v / s| < 7.5. Then v * (1 / s), rounded to an integer in the same operation,
 // differs by less than 1.2e-6 from the IEEE quotient (the reciprocal is within 2^-23 of its own size, the quotient within
-// 2^-22), so the two round alike unless the remainder is within 4e-6 of a half; such a warp divides. Every lane of the warp must call.
+// 2^-22), so the two round alike unless the remainder is within 4e-6 of a half; such a warp
+// divides (and one that has met a NaN, or an infinity: s is infinite then, and the product a NaN). Every lane of the warp
+// must call.
 template <int NP>
 __device__ __forceinline__ void quantize_pairs(const float2 (&v)[NP], float s, bool clamped, float2 (&b)[NP]) {
   bool redo = clamped;
@@ -268,9 +276,9 @@ __device__ __forceinline__ void quantize_pairs(const float2 (&v)[NP], float s, b
     for (int i = 0; i < NP; i++) {
       b[i] = __ffma2_rn(v[i], r2, magic);
       const float2 rest = __ffma2_rn(v[i], r2, __ffma2_rn(b[i], minus, magic));   // (magic - b: minus the integer, exactly)
-      worst = fmaxf(worst, fmaxf(fabsf(rest.x), fabsf(rest.y)));
+      worst = max3_magnitude_or_nan(worst, rest.x, rest.y);
     }
-    redo = __any_sync(0xffffffffu, worst > 0.499996f);
+    redo = __any_sync(0xffffffffu, !(worst <= 0.499996f));
   }
   if (redo) {
 #pragma unroll
@@ -358,7 +366,7 @@ __global__ void __launch_bounds__(T_MAX, 1024 / T_MAX) quantize_act_rows_kernel(
     }
     // non-negative floats order like their patterns
     unsigned am = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
-    if (lane == 0) s_max[par][warp] = am;
+    if (lane == 0) s_max[par][warp] = min(am, __float_as_uint(kAmaxCap));
     __syncthreads();   // (the other half of s_max is free: everybody has read it before coming here)
     am = __reduce_max_sync(0xffffffffu, lane < nwarp ? s_max[par][lane] : 0u);
     const __half s16 = __float2half_rn(div_by_7(__fmul_rn(__uint_as_float(am), p.clip_ratio)));
@@ -449,7 +457,7 @@ __global__ void __launch_bounds__(NT, kFullRowsThreads / NT) quantize_act_full_r
       col[((2 * i + 1) % R) * 32] = v[i].y;
     }
     unsigned am = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
-    if (lane == 0) s_max[par][warp] = am;
+    if (lane == 0) s_max[par][warp] = min(am, __float_as_uint(kAmaxCap));
     __syncthreads();
     am = __reduce_max_sync(0xffffffffu, s_max[par][lane % R]);
     const __half s16 = __float2half_rn(div_by_7(__fmul_rn(__uint_as_float(am), p.clip_ratio)));
@@ -574,7 +582,7 @@ __device__ __forceinline__ float rotate_full_token(const __half* x, float inv_sq
       col[(2 * i + 1) * 32] = v[i].y;
     }
     const unsigned am = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));   // non-negative: ordered like the patterns
-    if (lane == 0) s_amax[warp] = am;
+    if (lane == 0) s_amax[warp] = min(am, __float_as_uint(kAmaxCap));
   }
   asm volatile("bar.sync 1, 512;" ::: "memory");
 #pragma unroll
@@ -611,7 +619,7 @@ __device__ __forceinline__ float rotate_block_token(const __half* x, int W, int 
     }
   }
   const unsigned am = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
-  if (lane == 0) s_amax[warp] = am;
+  if (lane == 0) s_amax[warp] = min(am, __float_as_uint(kAmaxCap));
   asm volatile("bar.sync 1, 512;" ::: "memory");
   return __uint_as_float(__reduce_max_sync(0xffffffffu, s_amax[lane & 15]));
 }

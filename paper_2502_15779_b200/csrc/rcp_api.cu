@@ -441,7 +441,7 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
     gp.xq_out = fa->xq_out;
     gp.scale_out = static_cast<__half*>(fa->scale_out);
     gp.inv_sqrt_b = (float)(1.0 / std::sqrt((double)fa->B));
-    gp.clip_ratio = fa->clip_ratio;
+    gp.clip_ratio = std::min(fa->clip_ratio, rcp::kClipRatioCap);
     gp.had_block = fa->B;
     return grouped ? launch_fused<true>(maps, gp, pl, st) : launch_fused<false>(maps, gp, pl, st);
   }
@@ -804,7 +804,7 @@ int rcp_quantize_act(const void* x_f16, int M, int K, int had_block, float clip_
   qp.lgB = 0;
   while ((1 << qp.lgB) < B) qp.lgB++;
   qp.inv_sqrt_b = (float)(1.0 / std::sqrt((double)B));
-  qp.clip_ratio = clip_ratio;
+  qp.clip_ratio = std::min(clip_ratio, rcp::kClipRatioCap);
   if (rows_form(M, K, B)) return launch_quantize_rows(qp, M, st);
   // whole rotation blocks per CTA
   int C = 1;

@@ -62,6 +62,23 @@ CASES = [
 ]
 
 
+@pytest.mark.parametrize("K,B", [(2048, 2048), (4096, 4096), (8192, 8192), (640, 128), (4096, 1), (16384, 512)])
+def test_scale_beyond_fp32(K, B):
+    """amax * clip_ratio overflows (both are finite): infinite scale and zero codes from the quantizer inside the GEMV too."""
+    N = 40
+    x = synth.make_activations(1, K, K)
+    x = x * (1000 / x.abs().max())
+    words = torch.zeros(N, K // 16, dtype=torch.int32, device=DEV)
+    lut = torch.ones(N, 4, dtype=torch.float16, device=DEV)
+    xq = torch.full((1, K // 2), 0xAB, dtype=torch.uint8, device=DEV)
+    scale = torch.zeros(1, dtype=torch.float16, device=DEV)
+    assert rcp.rcp_linear_w2a4_launches(1, N, K, B) == 1
+    rcp.rcp_linear_w2a4(x.to(DEV), B, 3e38, words, lut, xq=xq, scale=scale)
+    ref = oracle.quantize_act(f16_bits(x), B, 3e38)
+    assert ref["scale"][0] == 0x7C00 and f16_bits(scale)[0] == 0x7C00
+    assert not xq.cpu().numpy().any() and not ref["xq"].any()
+
+
 @pytest.mark.parametrize("group", [0, 128])
 @pytest.mark.parametrize("N,K,B,M", CASES)
 def test_linear_matches_oracle(N, K, B, M, group):

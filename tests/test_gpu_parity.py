@@ -86,6 +86,21 @@ def test_quantize_act_one_cta_per_token(M, K, B, clip):
     assert np.array_equal(xq.cpu().numpy(), ref["xq"])
 
 
+@pytest.mark.parametrize("M,K,B", [(1, 64, 64), (3, 1024, 1024), (2, 2048, 2048), (40, 4096, 4096), (3, 8192, 8192), (5, 4096, 128),
+                                   (24, 14336, 128), (3, 14336, 2048), (1, 28672, 128), (40, 32768, 1)])
+@pytest.mark.parametrize("clip", [1e35, 1e36, 3e38])
+def test_quantize_act_scale_beyond_fp32(M, K, B, clip):
+    """clip_ratio need only be finite: the product with the token's maximum overflows here in some tokens (every form of
+    the quantizer). The scale is infinity then and the codes are zero, as in every token whose scale overflows fp16."""
+    x = synth.make_activations(M, K, M + K)
+    x[0] = x[0] * (1000 / x[0].abs().max())
+    ref = oracle.quantize_act(f16_bits(x), B, clip)
+    assert ref["scale"][0] == 0x7C00
+    xq, scale = rcp.rcp_quantize_act(x.to(DEV), B, clip)
+    assert np.array_equal(f16_bits(scale), ref["scale"])
+    assert np.array_equal(xq.cpu().numpy(), ref["xq"])
+
+
 def test_quantize_act_zero_token_and_errors():
     x = synth.make_activations(3, 512, seed=1)
     x[1] = 0
