@@ -149,6 +149,60 @@ def test_ldp_export_groups_of_128_at_tile_edges_and_hard_thresholds(N, K):
     assert np.all((got == ref["lut"]) | (((got | ref["lut"]) & 0x7FFF) == 0))
 
 
+def _edge_units(wv, sig, kinds):
+    """Every second unit of wv [units][128] becomes one of the edge cases."""
+    sb, sg, s1, s2 = sig
+    i = torch.arange(128)
+    for u in range(0, wv.shape[0], 2):
+        kind = kinds[(u // 2) % len(kinds)]
+        if kind == "exact":        # thresholds 1/4, 5/8, 7/8 of [0, 1] hit exactly
+            wv[u] = (i % 17 / 16.0).to(torch.float16)
+            sb[u] = sg[u] = 1.0
+            s1[u] = s2[u] = 0.5
+        elif kind == "wide":       # a threshold among numbers far smaller than the rounding of the range
+            wv[u] = (i - 64).to(torch.float16) * 2.0 ** -24
+            wv[u, 0], wv[u, 1] = -60000.0, 60000.0
+            sb[u] = sg[u] = 1.0
+            s1[u] = 0.999999
+        elif kind == "ends":       # t_1 = 0, t_3 = 1
+            s1[u], s2[u] = 0.0, 1.0
+        elif kind == "subnormal":
+            wv[u] = (i * 7 % 53 - 20).to(torch.float16) * 2.0 ** -24
+        elif kind == "flat":
+            wv[u] = -0.25
+        elif kind == "zeros":      # zeros of both signs, one of them the minimum
+            wv[u] = torch.where(i % 2 == 0, 0.0, -0.0).to(torch.float16)
+            wv[u, 5] = 0.5
+        elif kind == "minus":      # zeros of both signs, one of them the maximum
+            wv[u] = torch.where(i % 2 == 0, 0.0, -0.0).to(torch.float16)
+            wv[u, 7] = -0.5
+
+
+def _export_whole_and_in_pieces(w, sig, N, K):
+    """The export of all rows in one call (tiles of units) and in calls of fewer than 4096 units (a warp per unit)."""
+    args = [w.to(DEV)] + [t.view(N, K // 128).to(DEV) for t in sig]
+    rows = 4095 // (K // 128)
+    parts = [rcp.rcp_ldp_export(*[t[r:r + rows] for t in args], 128) for r in range(0, N, rows)]
+    return rcp.rcp_ldp_export(*args, 128), (torch.cat([p[0] for p in parts]), torch.cat([p[1] for p in parts]))
+
+
+@pytest.mark.parametrize("N,K", [(4096, 128), (4097, 128), (4127, 128), (1366, 384), (75776 + 33, 128), (300, 14336)])
+def test_ldp_export_tiles_of_units_and_single_units_agree(N, K):
+    """Both forms for groups of 128, bit for bit, signs of zero levels included; the first rows against the oracle too."""
+    w, sb, sg, s1, s2 = _inputs(N, K, 128, N + K)
+    sig = [t.reshape(-1) for t in (sb, sg, s1, s2)]
+    _edge_units(w.view(-1, 128)[:400], sig, ["exact", "wide", "ends", "subnormal", "flat", "zeros", "minus"])
+    whole, pieces = _export_whole_and_in_pieces(w, sig, N, K)
+    assert torch.equal(whole[0], pieces[0])
+    assert torch.equal(whole[1].view(torch.int16), pieces[1].view(torch.int16))
+    n = 400 // (K // 128)
+    ref = oracle.ldp_export(f16_bits(w[:n]), *[t.view(N, K // 128)[:n].numpy() for t in sig], 128)
+    assert np.array_equal(whole[0][:n].cpu().numpy().view(np.uint32), oracle.pack_weights(ref["codes"]))
+    # a zero level may carry either sign against the oracle (which zero is the minimum is not defined)
+    got = f16_bits(whole[1][:n])
+    assert np.all((got == ref["lut"]) | (((got | ref["lut"]) & 0x7FFF) == 0))
+
+
 def test_ldp_export_argument_errors():
     L = rcp.lib()
     z = torch.zeros(4096, dtype=torch.int32, device=DEV)
