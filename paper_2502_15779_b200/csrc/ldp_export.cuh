@@ -197,6 +197,8 @@ __global__ void __launch_bounds__(kLdpWarps * 32, 2) ldp_export128_kernel(const 
     halve(std::integral_constant<int, 4>());
     halve(std::integral_constant<int, 2>());
     halve(std::integral_constant<int, 1>());
+    // (as from infinities of either sign: a unit of nothing but NaN has an empty range)
+    mm[0] = __hmin2(mm[0], __half2half2(__ushort_as_half((unsigned short)0x7C00)));
     const float wmin = __low2float(mm[0]), wmax = -__high2float(mm[0]);
     const float lo = __fmul_rn(sb, wmin);
     const float hi = __fmul_rn(sg, wmax);

@@ -203,6 +203,21 @@ def test_ldp_export_tiles_of_units_and_single_units_agree(N, K):
     assert np.all((got == ref["lut"]) | (((got | ref["lut"]) & 0x7FFF) == 0))
 
 
+def test_ldp_export_units_of_nan_have_an_empty_range():
+    """Nothing but NaN in a unit: no minimum and no maximum, so lo = +inf, no range, codes 0, four equal levels. A NaN among
+    numbers is ignored by the range and gets code 0. Alike in both forms."""
+    N, K = 4200, 128
+    w, sb, sg, s1, s2 = _inputs(N, K, 128, 3)
+    w[5] = w[4199] = float("nan")
+    w[7, ::2] = float("nan")
+    whole, pieces = _export_whole_and_in_pieces(w, [t.reshape(-1) for t in (sb, sg, s1, s2)], N, K)
+    assert torch.equal(whole[0], pieces[0])
+    assert torch.equal(whole[1].view(torch.int16), pieces[1].view(torch.int16))
+    for row in (5, 4199):
+        assert not whole[0][row].any() and torch.all(whole[1][row] == float("inf"))
+    assert torch.isfinite(whole[1][7]).all()
+
+
 def test_ldp_export_argument_errors():
     L = rcp.lib()
     z = torch.zeros(4096, dtype=torch.int32, device=DEV)
