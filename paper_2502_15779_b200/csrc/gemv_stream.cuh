@@ -1103,34 +1103,50 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
           yacc[e] += __shfl_xor_sync(0xffffffffu, yacc[e], 2);
         }
       }
-      // The KS warps that shared the group (or the one that had it) leave their terms in a slot each, then every warp adds
-      // up, in the order of the warps, and finishes every KS-th pair of tokens: lane & 15 is the row, lane >> 4 the token.
-      // (4096x14336 at eight tokens 14.2 -> 13.0 us, at one 8.0 -> 7.7, against one warp finishing the whole group. For
-      // the per-row grid, with three integer sums a row and token, the same was slower than its atomics: 2048x2048 2.7 -> 3.0.)
-      float* const mine = s_redf + warp * red_plane;
-      // a shared reduction before this one: its slots must have been read by everybody
-      if (nred) asm volatile("bar.sync 2, %0;" ::"n"(kCWarps * 32) : "memory");
-      nred = KS > 1;
+      // A group that one warp had: finished from the registers. (Through a slot like the shared ones, tensor-core kernels:
+      // 57344x8192 55.2 -> 57.6 us at eight tokens, 56.3 -> 60.5 at three. On the CUDA cores, where a quad holds two
+      // entries, the slot is as fast or faster: the linear call at 57344x8192 38.6 -> 38.1.)
+      constexpr bool kDirect = MODE == kModeMma;
+      if (kDirect && KS == 1) {
+        if (active) {
 #pragma unroll
-      for (int e = 0; e < NE; e++)
-        if (active && etok[e] < M && RCP_CK((warp * red_plane + red_index(etok[e], grow + 8 * err[e])) * 4 < p.red_bytes, 10))
-          mine[red_index(etok[e], grow + 8 * err[e])] = yacc[e];
-      if (KS > 1) asm volatile("bar.sync 2, %0;" ::"n"(kCWarps * 32) : "memory");   // consumer warps only
-      else __syncwarp();
-      if (active) {
-        const int row = row_first + (lane & 15);
-#pragma unroll 1
-        for (int tp = ks; 2 * tp < M; tp += KS) {
-          const int tok = 2 * tp + (lane >> 4);
-          const float* d = s_redf + grp * KS * red_plane + red_index(tok, lane & 15);
-          float a = 0.f;
-#pragma unroll 4
-          for (int k = 0; k < KS; k++, d += red_plane) a += *d;
-          if (tok < M && row < p.N)
-            p.y[(size_t)tok * p.N + row] = __float2half_rn(s_scale[tok] * (kRelabel ? kGrpScale * a : a));
+          for (int e = 0; e < NE; e++) {
+            const int row = row_first + grow + 8 * err[e];
+            if (etok[e] < M && row < p.N)
+              p.y[(size_t)etok[e] * p.N + row] = __float2half_rn(s_scale[etok[e]] * (kRelabel ? kGrpScale * yacc[e] : yacc[e]));
+          }
         }
+      } else {
+        // The KS warps that shared the group (or the one that had it) leave their terms in a slot each, then every warp adds
+        // up, in the order of the warps, and finishes every KS-th pair of tokens: lane & 15 is the row, lane >> 4 the token.
+        // (4096x14336 at eight tokens 14.2 -> 13.0 us, at one 8.0 -> 7.7, against one warp finishing the whole group. For
+        // the per-row grid, with three integer sums a row and token, the same was slower than its atomics: 2048x2048 2.7 -> 3.0.)
+        float* const mine = s_redf + warp * red_plane;
+        // a shared reduction before this one: its slots must have been read by everybody
+        if (nred) asm volatile("bar.sync 2, %0;" ::"n"(kCWarps * 32) : "memory");
+        const bool shared = kDirect || KS > 1;
+        nred = shared;
+#pragma unroll
+        for (int e = 0; e < NE; e++)
+          if (active && etok[e] < M && RCP_CK((warp * red_plane + red_index(etok[e], grow + 8 * err[e])) * 4 < p.red_bytes, 10))
+            mine[red_index(etok[e], grow + 8 * err[e])] = yacc[e];
+        if (shared) asm volatile("bar.sync 2, %0;" ::"n"(kCWarps * 32) : "memory");   // consumer warps only
+        else __syncwarp();
+        if (active) {
+          const int row = row_first + (lane & 15);
+#pragma unroll 1
+          for (int tp = ks; 2 * tp < M; tp += KS) {
+            const int tok = 2 * tp + (lane >> 4);
+            const float* d = s_redf + grp * KS * red_plane + red_index(tok, lane & 15);
+            float a = 0.f;
+#pragma unroll 4
+            for (int k = 0; k < KS; k++, d += red_plane) a += *d;
+            if (tok < M && row < p.N)
+              p.y[(size_t)tok * p.N + row] = __float2half_rn(s_scale[tok] * (kRelabel ? kGrpScale * a : a));
+          }
+        }
+        if (!shared) __syncwarp();   // the slot is written again
       }
-      if (KS == 1) __syncwarp();   // the slot is written again
 #pragma unroll
       for (int e = 0; e < NE; e++) yacc[e] = 0.f;
     }
@@ -1250,7 +1266,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
 
   int slot = slot_keep;
   uint32_t phase = phase_keep;
-  // shared-memory reductions so far (two buffers alternate); group-wise grid: whether the last end of a group was one
+  // shared-memory reductions so far (two buffers alternate); group-wise grid: whether the slots hold one's terms
   int nred = nred_keep;
   int gbase = 0;   // groups of this CTA before the current repetition, the same count in every part
   for (int pi = 0; pi < p.nphase; pi++) {

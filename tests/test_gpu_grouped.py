@@ -73,6 +73,14 @@ def test_grouped_gemv_small_and_ragged(N, K, B, M, variant):
     _check(N, K, 128, B, M, "rotated_laplace" if K >= 512 else "uniform", variant, seed=N + K + M)
 
 
+@pytest.mark.parametrize("M,variant", [(1, "dp4a"), (2, "dp4a"), (3, "mma_only"), (7, "mma_only"), (8, "mma_only")])
+@pytest.mark.parametrize("N", [148 * 256, 148 * 256 + 148 * 128 + 17, 148 * 16 * 9 - 5])
+def test_grouped_gemv_rows_of_one_warp_beside_rows_of_several(N, M, variant):
+    """Rounds and nine groups per CTA, where one warp owns a group and finishes it from its registers, alone and after a phase
+    whose groups are shared by two and by all warps (finished from the slots in shared memory)."""
+    _check(N, 256, 128, 128, M, "uniform", variant, seed=N + M)
+
+
 @pytest.mark.parametrize("N,K,G,M", [(50, 256, 16, 2), (33, 512, 64, 1), (20, 1024, 256, 3), (9, 2048, 2048, 1)])
 def test_grouped_gemv_other_group_sizes_take_the_plain_kernel(N, K, G, M):
     _check(N, K, G, 64, M, "uniform", "auto", seed=N + G)
