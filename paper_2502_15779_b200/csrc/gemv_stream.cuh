@@ -121,6 +121,7 @@ struct GemvParams {
   int off_bar, off_T0c, off_scale, off_red, off_bs;   // shared-memory byte offsets from the aligned base
   int bs_bytes, red_bytes, part_bytes;                // sizes of the areas at off_bs, off_red, off_part (guarded build)
   int stage_stride;     // bytes from one ring stage to the next: kStageBytes, plus the stage's activation area (SB)
+  int late_start;       // tensor-core kernels: the next kernel may start when this one ends, not at once (see the end)
 };
 
 // ----------------------------------------------------------------------------- PTX wrappers
@@ -319,8 +320,8 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
 
   const int b = blockIdx.x;
   // Launched with programmatic stream serialization; when the next kernel may start is explained at the end.
-  constexpr bool kLateStart = MODE == kModeMma;
-  if constexpr (!kLateStart) asm volatile("griddepcontrol.launch_dependents;");
+  const bool late_start = MODE == kModeMma && p.late_start;
+  if (!late_start) asm volatile("griddepcontrol.launch_dependents;");
   int* const s_T0tot = reinterpret_cast<int*>(s_scale + 32);   // [16]: sum of q per token, behind scales and maxima
   // The producer warp sets up the ring's barriers and only announces that (bar.arrive): its first
   // requests go out without waiting for anybody. The consumer warps wait for the announcement.
@@ -1368,11 +1369,13 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   }   // parts of K
   // When the next kernel may start. The one-token kernels let it start at once: it is a GEMV as a rule (the quantizer is
   // inside), cannot fit beside this CTA, and takes over SM by SM (2048x2048 in a chain 2.76 us, 2.97 with the trigger here).
-  // Behind a kernel for more tokens comes a quantizer, and behind that a GEMV whose CTAs take every SM that the quantizer
-  // leaves and fill the memory system with weights while its few CTAs still fetch their tokens: started from here, a chain
-  // of quantizer and GEMV takes 9.6 us instead of 11.2 at 4096x4096 and sixteen tokens, 12.3 instead of 13.3 at
-  // 8192x8192 and eight, 8.6 instead of 9.7 at 4100x8192 and three (GEMVs without quantizers lose 0.1 to 0.4 us by it).
-  if constexpr (kLateStart) asm volatile("griddepcontrol.launch_dependents;");
+  // So do the kernels for more tokens when they are called on activations quantized before, one set of which serves
+  // several GEMVs (4096x4096 at three tokens 4.2 us a call, 4.6 with the trigger here; 10240x8192 at nine 17.9 and 19.2).
+  // Inside a call that has a quantizer of its own (late_start) the next kernel is the next call's quantizer, and behind
+  // that comes a GEMV whose CTAs take every SM that the quantizer leaves and fill the memory system with weights while
+  // its few CTAs still fetch their tokens: started from here, a chain of such calls takes 6.0 us instead of 7.1 at 4096x4096 and
+  // eight tokens, 8.6 instead of 9.9 at sixteen, 13.5 instead of 14.0 at 10240x8192 and eight.
+  if (late_start) asm volatile("griddepcontrol.launch_dependents;");
 }
 
 }  // namespace rcp

@@ -340,7 +340,7 @@ int launch_fused(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const Str
 int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16,
                   int M, int N, int K, void* y_f16, void* workspace, cudaStream_t st, bool grouped = false,
                   const FusedAct* fa = nullptr, const float* unit = nullptr, int nsplit = 1,
-                  const SplitAct* sa = nullptr, int32_t* S_out = nullptr, bool stream_act = false) {
+                  const SplitAct* sa = nullptr, int32_t* S_out = nullptr, bool stream_act = false, bool late_start = false) {
   if (stream_act && (mode != rcp::kModeMma || fa || unit || sa || nsplit > 1 || M > (grouped ? 8 : rcp::kMaxTokens))) return RCP_ERR_VARIANT;
   if (nsplit > 1 && (mode != rcp::kModeMma || grouped || fa || M > 8)) return RCP_ERR_VARIANT;
   if (sa && (mode != rcp::kModeMma || grouped || fa || unit || nsplit > 1 || M != 4 || K > 16384)) return RCP_ERR_VARIANT;
@@ -424,6 +424,7 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
   gp.off_part = pl.off_part;
   gp.act_parts = std::max(1, rcp::kCWarps / M);
   gp.inv_act_parts = (256 + gp.act_parts - 1) / gp.act_parts;
+  gp.late_start = late_start;
   gp.nphase = pl.nphase;
   for (int i = 0; i < rcp::kMaxPhases; i++) gp.phase[i] = i < pl.nphase ? pl.phase[i] : make_phase(1, 0, 0, 1, 0, pl.nchunk);
   gp.stages = pl.stages;
@@ -485,7 +486,7 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
 // All M tokens: as many launches as it takes for the expanded activations to fit (`cap` tokens at most each).
 int launch_stream_passes(int mode, int cap, const uint32_t* words, const void* lut_f16, const uint8_t* xq,
                          const void* scale_f16, int M, int N, int K, void* y_f16, void* workspace, cudaStream_t st,
-                         bool grouped = false, int32_t* S_out = nullptr) {
+                         bool grouped = false, int32_t* S_out = nullptr, bool late_start = false) {
   int nsplit = 1;
   const int mp = (grouped || cap < 8) ? tokens_per_pass(M, K, cap) : tokens_and_parts(M, N, K, cap, sm_count(), &nsplit);
   // Where the launch would have to go through K in more than four parts (several tokens, a very long K), the form that
@@ -501,7 +502,7 @@ int launch_stream_passes(int mode, int cap, const uint32_t* words, const void* l
         const int rc = launch_stream(mode, words, lut_f16, xq + (size_t)m0 * (K / 2),
                                      static_cast<const __half*>(scale_f16) + m0, mm, N, K,
                                      static_cast<__half*>(y_f16) + (size_t)m0 * N, workspace, st, false, nullptr, nullptr, 1,
-                                     nullptr, S_out ? S_out + (size_t)m0 * N * 4 : nullptr, true);
+                                     nullptr, S_out ? S_out + (size_t)m0 * N * 4 : nullptr, true, late_start);
         if (rc != RCP_OK) return rc;
       }
       return RCP_OK;
@@ -519,7 +520,7 @@ int launch_stream_passes(int mode, int cap, const uint32_t* words, const void* l
         const int rc = launch_stream(mode, words, lut_f16, xq + (size_t)m0 * (K / 2),
                                      static_cast<const __half*>(scale_f16) + m0, mm, N, K,
                                      static_cast<__half*>(y_f16) + (size_t)m0 * N, workspace, st, true, nullptr, nullptr, 1,
-                                     nullptr, S_out ? S_out + (size_t)m0 * N * 4 * (K / 128) : nullptr, true);
+                                     nullptr, S_out ? S_out + (size_t)m0 * N * 4 * (K / 128) : nullptr, true, late_start);
         if (rc != RCP_OK) return rc;
       }
       return RCP_OK;
@@ -533,7 +534,7 @@ int launch_stream_passes(int mode, int cap, const uint32_t* words, const void* l
                                  static_cast<const __half*>(scale_f16) + m0, mm, N, K,
                                  static_cast<__half*>(y_f16) + (size_t)m0 * N, workspace, st, grouped, nullptr, nullptr,
                                  md == rcp::kModeMma ? nsplit : 1, nullptr,
-                                 S_out ? S_out + (size_t)m0 * N * 4 * (grouped ? K / 128 : 1) : nullptr);
+                                 S_out ? S_out + (size_t)m0 * N * 4 * (grouped ? K / 128 : 1) : nullptr, false, late_start);
     if (rc != RCP_OK) return rc;
   }
   return RCP_OK;
@@ -874,9 +875,9 @@ size_t rcp_gemv_workspace_bytes(int M, int N, int K) {
   return 16;   // a status word for the kernels' bounded waits; no sums pass through global memory
 }
 
-int rcp_gemv_w2a4_variant(int variant, const uint32_t* words, const void* lut_f16, const uint8_t* xq,
-                          const void* scale_f16, int M, int N, int K, void* y_f16, void* workspace,
-                          int32_t* S_dbg, void* stream) {
+// late_start: the call quantizes its activations itself (see the end of gemv_stream_kernel)
+static int gemv_w2a4(int variant, const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16, int M,
+                     int N, int K, void* y_f16, void* workspace, int32_t* S_dbg, void* stream, bool late_start) {
   if (!words || !lut_f16 || !xq || !scale_f16 || !y_f16) return RCP_ERR_NULL;
   if (M < 1 || M > rcp::kMaxTokens || N < 1 || !k_ok(K)) return RCP_ERR_SHAPE;
   if (!aligned16(words) || !aligned16(xq) || !aligned16(S_dbg) ||
@@ -904,10 +905,10 @@ int rcp_gemv_w2a4_variant(int variant, const uint32_t* words, const void* lut_f1
     case RCP_GEMV_MMA:
       // tensor-core path; for one or two tokens the b0*b1 plane goes to dp4a (FMA pipe) instead
       return launch_stream_passes(M <= 2 ? rcp::kModeHybrid : rcp::kModeMma, 16, words, lut_f16, xq, scale_f16, M, N, K,
-                                  y_f16, workspace, st, false, S_dbg);
+                                  y_f16, workspace, st, false, S_dbg, late_start);
     case RCP_GEMV_MMA_ONLY:
       return launch_stream_passes(rcp::kModeMma, 16, words, lut_f16, xq, scale_f16, M, N, K, y_f16, workspace, st, false,
-                                  S_dbg);
+                                  S_dbg, late_start);
     case RCP_GEMV_DP4A:
       // CUDA-core path: two tokens per launch
       return launch_stream_passes(rcp::kModeDp4a, 2, words, lut_f16, xq, scale_f16, M, N, K, y_f16, workspace, st, false,
@@ -917,13 +918,19 @@ int rcp_gemv_w2a4_variant(int variant, const uint32_t* words, const void* lut_f1
       const StreamPlan pl = make_plan(M, N, K, sm_count(), false, 0, 1, true);
       if (pl.stages < 2 || pl.smem > kSmemMax) return RCP_ERR_VARIANT;
       return launch_stream(rcp::kModeMma, words, lut_f16, xq, scale_f16, M, N, K, y_f16, workspace, st, false, nullptr,
-                           nullptr, 1, nullptr, S_dbg, true);
+                           nullptr, 1, nullptr, S_dbg, true, late_start);
     }
     default:
       return RCP_ERR_VARIANT;
   }
   RCP_CUDA(cudaGetLastError());
   return RCP_OK;
+}
+
+int rcp_gemv_w2a4_variant(int variant, const uint32_t* words, const void* lut_f16, const uint8_t* xq,
+                          const void* scale_f16, int M, int N, int K, void* y_f16, void* workspace,
+                          int32_t* S_dbg, void* stream) {
+  return gemv_w2a4(variant, words, lut_f16, xq, scale_f16, M, N, K, y_f16, workspace, S_dbg, stream, false);
 }
 
 int rcp_gemv_w2a4(const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16,
@@ -965,7 +972,7 @@ int rcp_gemv_w2a16_checked(const uint32_t* words, const void* lut_f16, const voi
     const int cc = std::min(cp, cols - c0);
     const int rc = launch_stream(rcp::kModeMma, words, lut_f16, reinterpret_cast<const uint8_t*>(digits) + (size_t)c0 * K,
                                  nullptr, cc, N, K, static_cast<__half*>(y_f16) + (size_t)(c0 / 4) * N, workspace, st,
-                                 false, nullptr, unit + c0, nsplit, nullptr, S_dbg ? S_dbg + (size_t)c0 * N * 4 : nullptr);
+                                 false, nullptr, unit + c0, nsplit, nullptr, S_dbg ? S_dbg + (size_t)c0 * N * 4 : nullptr, false, true);
     if (rc != RCP_OK) return rc;
   }
   return RCP_OK;
@@ -976,9 +983,9 @@ int rcp_gemv_w2a16(const uint32_t* words, const void* lut_f16, const void* x_f16
   return rcp_gemv_w2a16_checked(words, lut_f16, x_f16, M, N, K, y_f16, digits, unit, workspace, nullptr, stream);
 }
 
-int rcp_gemv_w2a4_grouped_variant(int variant, const uint32_t* words, const void* lut_f16, int group,
-                                  const uint8_t* xq, const void* scale_f16, int M, int N, int K, void* y_f16,
-                                  void* workspace, int32_t* S_dbg, void* stream) {
+static int gemv_w2a4_grouped(int variant, const uint32_t* words, const void* lut_f16, int group, const uint8_t* xq,
+                             const void* scale_f16, int M, int N, int K, void* y_f16, void* workspace, int32_t* S_dbg,
+                             void* stream, bool late_start) {
   if (!words || !lut_f16 || !xq || !scale_f16 || !y_f16) return RCP_ERR_NULL;
   if (M < 1 || M > rcp::kMaxTokens || N < 1 || !k_ok(K)) return RCP_ERR_SHAPE;
   if (group < 16 || group % 16 || K % group) return RCP_ERR_SHAPE;
@@ -1004,7 +1011,7 @@ int rcp_gemv_w2a4_grouped_variant(int variant, const uint32_t* words, const void
     case RCP_GEMV_MMA_ONLY:
       if (group != 128) return RCP_ERR_VARIANT;
       return launch_stream_passes(rcp::kModeMma, 8, words, lut_f16, xq, scale_f16, M, N, K, y_f16, workspace, st, true,
-                                  S_dbg);
+                                  S_dbg, late_start);
     case RCP_GEMV_DP4A:
       if (group != 128) return RCP_ERR_VARIANT;
       return launch_stream_passes(rcp::kModeDp4a, 2, words, lut_f16, xq, scale_f16, M, N, K, y_f16, workspace, st, true,
@@ -1014,6 +1021,12 @@ int rcp_gemv_w2a4_grouped_variant(int variant, const uint32_t* words, const void
   }
   RCP_CUDA(cudaGetLastError());
   return RCP_OK;
+}
+
+int rcp_gemv_w2a4_grouped_variant(int variant, const uint32_t* words, const void* lut_f16, int group,
+                                  const uint8_t* xq, const void* scale_f16, int M, int N, int K, void* y_f16,
+                                  void* workspace, int32_t* S_dbg, void* stream) {
+  return gemv_w2a4_grouped(variant, words, lut_f16, group, xq, scale_f16, M, N, K, y_f16, workspace, S_dbg, stream, false);
 }
 
 int rcp_gemv_w2a4_grouped(const uint32_t* words, const void* lut_f16, int group, const uint8_t* xq,
@@ -1105,10 +1118,10 @@ int rcp_linear_w2a4_checked(const void* x_f16, int M, int K, int had_block, floa
   if (rc != RCP_OK) return rc;
   // with S_dbg: the streaming kernel AUTO would pick, in its checked instantiation
   if (group == 0)
-    return rcp_gemv_w2a4_variant(S_dbg ? (M == 1 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY) : RCP_GEMV_AUTO, words, lut_f16, xq,
-                                 scale_f16, M, N, K, y_f16, workspace, S_dbg, stream);
-  return rcp_gemv_w2a4_grouped_variant(S_dbg && group == 128 ? (M <= 2 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY) : RCP_GEMV_AUTO,
-                                       words, lut_f16, group, xq, scale_f16, M, N, K, y_f16, workspace, S_dbg, stream);
+    return gemv_w2a4(S_dbg ? (M == 1 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY) : RCP_GEMV_AUTO, words, lut_f16, xq, scale_f16, M,
+                     N, K, y_f16, workspace, S_dbg, stream, true);
+  return gemv_w2a4_grouped(S_dbg && group == 128 ? (M <= 2 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY) : RCP_GEMV_AUTO, words,
+                           lut_f16, group, xq, scale_f16, M, N, K, y_f16, workspace, S_dbg, stream, true);
 }
 
 int rcp_linear_w2a4(const void* x_f16, int M, int K, int had_block, float clip_ratio, const uint32_t* words,
@@ -1146,7 +1159,7 @@ int rcp_linear_w2a4_host(const void* x_host_f16, int M, int K, int had_block, fl
   if (x_mapped) {
     rc = rcp_quantize_act(x_mapped, M, K, had_block, clip_ratio, xq_dev, scale_dev, stream);
     if (rc == RCP_OK)
-      rc = rcp_gemv_w2a4(words, lut_f16, xq_dev, scale_dev, M, N, K, y_out, workspace, nullptr, stream);
+      rc = gemv_w2a4(RCP_GEMV_AUTO, words, lut_f16, xq_dev, scale_dev, M, N, K, y_out, workspace, nullptr, stream, true);
   } else {
     RCP_CUDA(cudaMemcpyAsync(x_dev, x_host_f16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st));
     rc = rcp_linear_w2a4(x_dev, M, K, had_block, clip_ratio, words, lut_f16, 0, N, y_out, xq_dev, scale_dev, workspace,

@@ -84,3 +84,69 @@ def test_host_threads_with_their_own_streams():
     assert not errors, errors
     for p in probs:
         assert int(p["ws"].abs().max()) == 0
+
+
+@pytest.mark.parametrize("M", [1, 2, 3, 8, 9, 16])
+@pytest.mark.parametrize("group", [0, 128])
+def test_back_to_back_calls_that_share_their_buffers(M, group):
+    """Kernels of neighbouring calls overlap (each starts before the one in front of it has ended, at its start or at its
+    end, depending on the form). Calls of all forms in a row on one stream, quantized activations and results in the same
+    few buffers: every result is that of the call alone."""
+    K, B, Ns = 4096, 4096, (4096, 300, 10240)
+    layers = []
+    for i, N in enumerate(Ns):
+        codes, lut = (synth.make_layer_grouped(N, K, group, B, "uniform", 300 + i, device=DEV) if group
+                      else synth.make_layer(N, K, B, "uniform", 300 + i, device=DEV))
+        layers.append((rcp.rcp_pack_weights(codes), lut, rcp.make_workspace(M, N, K, DEV)))
+    xs = [synth.make_activations(M, K, 400 + i, device=DEV) for i in range(2)]
+    xq = torch.empty(M, K // 2, dtype=torch.uint8, device=DEV)
+    scale = torch.empty(M, dtype=torch.float16, device=DEV)
+    digits = torch.empty(M, 4, K, dtype=torch.int8, device=DEV)
+    unit = torch.empty(M, 4, dtype=torch.float32, device=DEV)
+    ys = [torch.empty(M, N, dtype=torch.float16, device=DEV) for N in Ns]
+
+    def gemv(layer, y):
+        words, lut, ws = layer
+        if group:
+            return rcp.rcp_gemv_w2a4_grouped(words, lut, xq, scale, group=group, y=y, workspace=ws)
+        return rcp.rcp_gemv_w2a4(words, lut, xq, scale, y=y, workspace=ws)
+
+    steps = []   # (call, its result's buffer)
+    for x in xs:
+        steps.append((lambda x=x: rcp.rcp_quantize_act(x, B, 1.0, xq=xq, scale=scale), None))
+        for layer, y in zip(layers, ys):
+            steps.append((lambda layer=layer, y=y: gemv(layer, y), y))
+        for (words, lut, ws), y in zip(layers, ys):
+            if not group:
+                steps.append((lambda x=x, words=words, lut=lut, ws=ws, y=y: rcp.rcp_gemv_w2a16(
+                    words, lut, x, y=y, digits=digits, unit=unit, workspace=ws), y))
+            steps.append((lambda x=x, words=words, lut=lut, ws=ws, y=y: rcp.rcp_linear_w2a4(
+                x, B, 1.0, words, lut, group=group, y=y, xq=xq, scale=scale, workspace=ws), y))
+        for layer, y in zip(layers, ys):
+            steps.append((lambda layer=layer, y=y: gemv(layer, y), y))
+
+    want = []
+    for call, y in steps:
+        call()
+        torch.cuda.synchronize()
+        if y is not None:
+            want.append(y.clone())
+    last = {y.data_ptr(): (i, y) for i, (_, y) in enumerate(s for s in steps if s[1] is not None)}
+    for _ in range(20):
+        for y in ys:
+            y.fill_(float("nan"))
+        for call, _ in steps:
+            call()
+        torch.cuda.synchronize()
+        for i, y in last.values():   # nothing stood between the calls: what is left is each buffer's last result
+            assert torch.equal(y.view(torch.int16), want[i].view(torch.int16))
+    own = []
+    for call, y in steps:            # and every result, copied out between the calls
+        call()
+        if y is not None:
+            own.append(y.clone())
+    torch.cuda.synchronize()
+    for o, w in zip(own, want):
+        assert torch.equal(o.view(torch.int16), w.view(torch.int16))
+    for _, _, ws in layers:
+        assert int(ws.abs().max()) == 0
