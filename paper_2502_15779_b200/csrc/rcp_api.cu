@@ -615,6 +615,57 @@ int launch_quantize_rows(const rcp::QuantParams& qp, int M, cudaStream_t st) {
   return W <= 512 ? launch_block_rows<1, 512, 0>(qp, M, st) : launch_block_rows<2, 1024, 0>(qp, M, st);
 }
 
+// Shared memory of which r CTAs fit on an SM (228 KB, 1 KB of it per CTA for the system) and r + 1 do not.
+constexpr size_t smem_for_residency(int r) { return 228 * 1024 / (r + 1) - 768; }
+
+// C CTAs per token as a cluster. The CTAs of a cluster are packed onto as few SMs as hold them, so a launch that would fill the
+// GPU with one or two CTAs per SM leaves half of it idle at four. From nine tokens on the launch therefore asks for as much
+// shared memory as makes it spread: as few CTAs per SM as still hold all of it at once. (us a call in a chain of them,
+// without and with: 28672 in blocks of 128 at 16, 24, 39 tokens 4.2, 4.9, 5.8 and 3.5, 4.2, 5.2; 14336 in blocks of 2048 at 64
+// and 100 7.2, 8.4 and 5.3, 7.2. More tokens than fit at three per SM are faster packed: 200 of those 12.1 and 12.9; eight
+// and fewer do not notice.)
+template <int C>
+int launch_quantize_cluster(const rcp::QuantParams& qp, int M, int T, size_t smem, cudaStream_t st) {
+  static std::mutex mu;
+  static bool attr_set[kMaxDevices] = {};
+  static int fit[kMaxDevices][4] = {};   // clusters resident at once with r CTAs per SM
+  auto kern = rcp::quantize_act_kernel<C>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)M * C);
+  cfg.blockDim = dim3(T);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  if (C > 1 && M > 8) {
+    RCP_CUDA(set_max_smem(kern, (int)smem_for_residency(1), mu, attr_set));
+    int dev = 0;
+    RCP_CUDA(cudaGetDevice(&dev));   // (below kMaxDevices: set_max_smem has looked)
+    for (int r = 1; r <= 3 && (r + 1) * T <= 2048; r++) {   // (by its threads an SM takes no more than that anyway)
+      std::lock_guard<std::mutex> lock(mu);
+      if (!fit[dev][r]) {
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cfg.dynamicSmemBytes = smem_for_residency(r);
+        RCP_CUDA(cudaOccupancyMaxActiveClusters(&fit[dev][r], kern, &cfg));
+      }
+      if (M <= fit[dev][r]) {
+        smem = std::max(smem, smem_for_residency(r));
+        break;
+      }
+    }
+  }
+  cfg.dynamicSmemBytes = smem;
+  cfg.attrs = C > 1 ? attr : attr + 1;
+  cfg.numAttrs = C > 1 ? 2 : 1;
+  RCP_CUDA(cudaLaunchKernelEx(&cfg, kern, qp));
+  return RCP_OK;
+}
+
 template <bool GRP, bool SDBG, bool HALF = false>
 int launch_w3(const rcp::W3Params& wp, size_t smem, cudaStream_t st) {
   static std::mutex mu;
@@ -823,27 +874,12 @@ int rcp_quantize_act(const void* x_f16, int M, int K, int had_block, float clip_
   if ((long long)per * qp.unit > 8192) return RCP_ERR_SHAPE;
   const int T = (per * qp.unit / 8 + 31) / 32 * 32;
   const size_t smem = B > 256 ? (size_t)T * 8 * sizeof(float) : 0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)M * C);
-  cfg.blockDim = dim3(T);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = C;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = C > 1 ? 2 : 1;
   switch (C) {
-    case 1: RCP_CUDA(cudaLaunchKernelEx(&cfg, rcp::quantize_act_kernel<1>, qp)); break;
-    case 2: RCP_CUDA(cudaLaunchKernelEx(&cfg, rcp::quantize_act_kernel<2>, qp)); break;
-    case 4: RCP_CUDA(cudaLaunchKernelEx(&cfg, rcp::quantize_act_kernel<4>, qp)); break;
-    default: RCP_CUDA(cudaLaunchKernelEx(&cfg, rcp::quantize_act_kernel<8>, qp)); break;
+    case 1: return launch_quantize_cluster<1>(qp, M, T, smem, st);
+    case 2: return launch_quantize_cluster<2>(qp, M, T, smem, st);
+    case 4: return launch_quantize_cluster<4>(qp, M, T, smem, st);
+    default: return launch_quantize_cluster<8>(qp, M, T, smem, st);
   }
-  return RCP_OK;
 }
 
 int rcp_gemv_plan(int M, int N, int K, int sms, int* out, int cap) {

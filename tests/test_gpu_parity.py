@@ -86,6 +86,20 @@ def test_quantize_act_one_cta_per_token(M, K, B, clip):
     assert np.array_equal(xq.cpu().numpy(), ref["xq"])
 
 
+@pytest.mark.parametrize("K,B", [(5120, 1024), (14336, 2048), (28672, 128), (28672, 4096)])
+def test_quantize_act_clusters_spread_over_the_gpu(K, B):
+    """Clusters of two, four and eight CTAs per token at token counts where the launch asks for one, two, three and as many
+    CTAs per SM as fit, one after the other in both directions."""
+    Ms = [8, 9, 16, 33, 39, 70, 150, 100, 39, 16, 9]
+    x = synth.make_activations(max(Ms), K, K + B)
+    ref = oracle.quantize_act(f16_bits(x), B, 1.0)
+    xd = x.to(DEV)
+    outs = [rcp.rcp_quantize_act(xd[:M], B, 1.0) for M in Ms]
+    for M, (xq, scale) in zip(Ms, outs):
+        assert np.array_equal(f16_bits(scale), ref["scale"][:M])
+        assert np.array_equal(xq.cpu().numpy(), ref["xq"][:M])
+
+
 @pytest.mark.parametrize("M,K,B", [(1, 64, 64), (3, 1024, 1024), (2, 2048, 2048), (40, 4096, 4096), (3, 8192, 8192), (5, 4096, 128),
                                    (24, 14336, 128), (3, 14336, 2048), (1, 28672, 128), (40, 32768, 1)])
 @pytest.mark.parametrize("clip", [1e35, 1e36, 3e38])
