@@ -51,8 +51,9 @@ bool bad_shapes(const char* what) {
   PyErr_Format(PyExc_ValueError, "shape mismatch between %s", what);
   return false;
 }
+// What int(o) and float(o) take: whole-numbered floats, numpy scalars, one-element tensors as well.
 bool integer(PyObject* o, int* out) {
-  PyObject* v = PyNumber_Index(o);
+  PyObject* v = PyNumber_Long(o);
   if (!v) return false;
   const long x = PyLong_AsLong(v);
   Py_DECREF(v);
@@ -61,8 +62,10 @@ bool integer(PyObject* o, int* out) {
   return true;
 }
 bool real(PyObject* o, float* out) {
-  const double x = PyFloat_AsDouble(o);
-  if (x == -1.0 && PyErr_Occurred()) return false;
+  PyObject* v = PyNumber_Float(o);
+  if (!v) return false;
+  const double x = PyFloat_AS_DOUBLE(v);
+  Py_DECREF(v);
   *out = (float)x;
   return true;
 }
