@@ -24,7 +24,7 @@ _lib = None
 _m = None   # the native marshalling module, bound to _lib
 _MARSHAL_PATH = os.path.join(_HERE, "_marshal.so")
 _MARSHALLED = ("rcp_quantize_act", "rcp_gemv_w2a4_variant", "rcp_gemv_w2a4_grouped_variant", "rcp_gemv_w2a16_checked",
-               "rcp_gemv_w3a4", "rcp_linear_w2a4_checked", "rcp_linear_w2a4_host")
+               "rcp_gemv_w3a4", "rcp_linear_w2a4_checked", "rcp_linear_w2a4_host", "rcp_gemv_workspace_bytes")
 
 
 class RcpError(RuntimeError):
@@ -136,11 +136,20 @@ def _dev(t, dtype, name):
     return t
 
 
+def _room(t, dtype, numel, name, like):
+    """A buffer passed by the caller for a result of numel elements."""
+    _dev(t, dtype, name)
+    if t.numel() < numel or t.device != like.device:
+        raise ValueError(f"{name}: expected at least {numel} elements on {like.device}")
+    return t
+
+
 def rcp_pack_weights(codes: torch.Tensor, out: torch.Tensor = None) -> torch.Tensor:
     """codes uint8 [N][K] in {0..3} -> words int32 [N][K/16] (bit pattern of the uint32 words)."""
     _dev(codes, torch.uint8, "codes")
     N, K = codes.shape
-    words = out if out is not None else torch.empty((N, K // 16), dtype=torch.int32, device=codes.device)
+    words = (_room(out, torch.int32, N * (K // 16), "out", codes) if out is not None
+             else torch.empty((N, K // 16), dtype=torch.int32, device=codes.device))
     with _on(codes):
         _check("rcp_pack_weights", lib().rcp_pack_weights(_ptr(codes), N, K, _ptr(words), _stream(codes)))
     return words
@@ -313,6 +322,7 @@ def rcp_gemv_w2a4_static(words, lut, xq, scale, y=None):
         raise ValueError("shape mismatch between words, lut, xq and scale")
     if y is None:
         y = torch.empty((M, N), dtype=torch.float16, device=words.device)
+    _room(y, torch.float16, M * N, "y", words)
     with _on(words):
         _check("rcp_gemv_w2a4_static",
                lib().rcp_gemv_w2a4_static(_ptr(words), _ptr(lut), _ptr(xq), _ptr(scale), M, N, K, _ptr(y),

@@ -22,30 +22,63 @@ struct Entry {
   decltype(&rcp_gemv_w3a4) gemv_w3a4 = nullptr;
   decltype(&rcp_linear_w2a4_checked) linear = nullptr;
   decltype(&rcp_linear_w2a4_host) linear_host = nullptr;
+  decltype(&rcp_gemv_workspace_bytes) workspace_bytes = nullptr;
 } g_fn;
 
 
-// A contiguous CUDA tensor of the given type, or a TypeError.
-const at::Tensor* dev(PyObject* o, at::ScalarType type, const char* name) {
+const char* type_name(at::ScalarType t) {
+  return t == at::kHalf ? "float16" : t == at::kInt ? "int32" : t == at::kFloat ? "float32" : t == at::kChar ? "int8" : "uint8";
+}
+bool on_other_device(const char* name) {
+  PyErr_Format(PyExc_ValueError, "%s: not on the device of the call's first tensor", name);
+  return false;
+}
+// A contiguous CUDA tensor of the given type (on the device of `like`), or a TypeError.
+const at::Tensor* dev(PyObject* o, at::ScalarType type, const char* name, const at::Tensor* like = nullptr) {
   if (THPVariable_Check(o)) {
     const at::Tensor& t = THPVariable_Unpack(o);
-    if (t.is_cuda() && t.scalar_type() == type && t.is_contiguous()) return &t;
+    if (t.is_cuda() && t.scalar_type() == type && t.is_contiguous()) {
+      if (like && t.device() != like->device()) { on_other_device(name); return nullptr; }
+      return &t;
+    }
   }
-  PyErr_Format(PyExc_TypeError, "%s: expected a contiguous CUDA tensor of dtype torch.%s", name,
-               type == at::kHalf ? "float16" : type == at::kInt ? "int32" : "uint8");
+  PyErr_Format(PyExc_TypeError, "%s: expected a contiguous CUDA tensor of dtype torch.%s", name, type_name(type));
   return nullptr;
 }
-// The data pointer of an optional tensor (None: null).
-bool ptr(PyObject* o, const char* name, void** out) {
+// The address of an optional buffer (None: null) that the library knows nothing else of: at least `need` elements of the given
+// type (kByte: or int8; kAny: bytes of any type), contiguous, on the device of `like` or in page-locked host memory, which
+// the device reaches as well.
+constexpr at::ScalarType kAny = at::ScalarType::Undefined;
+bool buffer(PyObject* o, const char* name, at::ScalarType type, const at::Tensor& like, int64_t need, void** out) {
   *out = nullptr;
   if (o == Py_None) return true;
   if (!THPVariable_Check(o)) {
     PyErr_Format(PyExc_TypeError, "%s: expected a tensor or None", name);
     return false;
   }
-  *out = THPVariable_Unpack(o).data_ptr();
+  const at::Tensor& t = THPVariable_Unpack(o);
+  const at::ScalarType have = t.scalar_type();
+  if (have == type && t.is_cuda() && t.numel() >= need && t.is_contiguous() && t.get_device() == like.get_device()) {   // as a rule
+    *out = t.data_ptr();
+    return true;
+  }
+  const bool fits = type == kAny || have == type || ((type == at::kByte || type == at::kChar) && (have == at::kByte || have == at::kChar));
+  if (!fits || !t.is_contiguous() || !(t.is_cuda() || t.is_pinned())) {
+    PyErr_Format(PyExc_TypeError, "%s: expected a contiguous CUDA tensor%s%s", name, type == kAny ? "" : " of dtype torch.",
+                 type == kAny ? "" : type_name(type));
+    return false;
+  }
+  if (t.is_cuda() && t.device() != like.device()) return on_other_device(name);
+  if ((type == kAny ? (int64_t)t.nbytes() : t.numel()) < need) {
+    PyErr_Format(PyExc_ValueError, "%s: %lld %s, %lld are needed", name, (long long)(type == kAny ? (int64_t)t.nbytes() : t.numel()),
+                 type == kAny ? "bytes" : "elements", (long long)need);
+    return false;
+  }
+  *out = t.data_ptr();
   return true;
 }
+// bytes of workspace the library wants (0 for shapes it refuses)
+int64_t workspace_bytes(int64_t M, int64_t N, int64_t K) { return (int64_t)g_fn.workspace_bytes((int)M, (int)N, (int)K); }
 bool has_shape(const at::Tensor& t, std::initializer_list<int64_t> want) { return t.sizes() == at::IntArrayRef(want); }
 bool bad_shapes(const char* what) {
   PyErr_Format(PyExc_ValueError, "shape mismatch between %s", what);
@@ -53,15 +86,24 @@ bool bad_shapes(const char* what) {
 }
 // What int(o) and float(o) take: whole-numbered floats, numpy scalars, one-element tensors as well.
 bool integer(PyObject* o, int* out) {
-  PyObject* v = PyNumber_Long(o);
-  if (!v) return false;
-  const long x = PyLong_AsLong(v);
-  Py_DECREF(v);
+  long x;
+  if (PyLong_CheckExact(o)) {
+    x = PyLong_AsLong(o);
+  } else {
+    PyObject* v = PyNumber_Long(o);
+    if (!v) return false;
+    x = PyLong_AsLong(v);
+    Py_DECREF(v);
+  }
   if (x == -1 && PyErr_Occurred()) return false;
   *out = (int)x;
   return true;
 }
 bool real(PyObject* o, float* out) {
+  if (PyFloat_CheckExact(o)) {
+    *out = (float)PyFloat_AS_DOUBLE(o);
+    return true;
+  }
   PyObject* v = PyNumber_Float(o);
   if (!v) return false;
   const double x = PyFloat_AS_DOUBLE(v);
@@ -120,7 +162,7 @@ PyObject* bind(PyObject*, PyObject* table) {
   if (!take("rcp_quantize_act", g_fn.quantize_act) || !take("rcp_gemv_w2a4_variant", g_fn.gemv) ||
       !take("rcp_gemv_w2a4_grouped_variant", g_fn.gemv_grouped) || !take("rcp_gemv_w2a16_checked", g_fn.gemv_w2a16) ||
       !take("rcp_gemv_w3a4", g_fn.gemv_w3a4) || !take("rcp_linear_w2a4_checked", g_fn.linear) ||
-      !take("rcp_linear_w2a4_host", g_fn.linear_host))
+      !take("rcp_linear_w2a4_host", g_fn.linear_host) || !take("rcp_gemv_workspace_bytes", g_fn.workspace_bytes))
     return nullptr;
   Py_RETURN_NONE;
 }
@@ -133,9 +175,11 @@ PyObject* quantize_act(PyObject*, PyObject* const* a, Py_ssize_t n) {
     void *xq, *scale;
     if (!count(n, 5)) return nullptr;
     const at::Tensor* x = dev(a[0], at::kHalf, "x");
-    if (!x || !integer(a[1], &B) || !real(a[2], &clip) || !ptr(a[3], "xq", &xq) || !ptr(a[4], "scale", &scale)) return nullptr;
+    if (!x || !integer(a[1], &B) || !real(a[2], &clip)) return nullptr;
     if (x->dim() != 2) { bad_shapes("x and [M][K]"); return nullptr; }
     const int M = (int)x->size(0), K = (int)x->size(1);
+    if (!buffer(a[3], "xq", at::kByte, *x, x->size(0) * (x->size(1) / 2), &xq) || !buffer(a[4], "scale", at::kHalf, *x, x->size(0), &scale))
+      return nullptr;
     const void* const xp = x->data_ptr();
     return on_device(*x, [&](void* st) { return g_fn.quantize_act(xp, M, K, B, clip, static_cast<uint8_t*>(xq), scale, st); });
   });
@@ -149,12 +193,12 @@ PyObject* gemv_w2a4(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!count(n, 9) || !integer(a[0], &variant) || !integer(a[3], &group)) return nullptr;
     const at::Tensor* words = dev(a[1], at::kInt, "words");
     if (!words) return nullptr;
-    const at::Tensor* lut = dev(a[2], at::kHalf, "lut");
+    const at::Tensor* lut = dev(a[2], at::kHalf, "lut", words);
     if (!lut) return nullptr;
-    const at::Tensor* xq = dev(a[4], at::kByte, "xq");
+    const at::Tensor* xq = dev(a[4], at::kByte, "xq", words);
     if (!xq) return nullptr;
-    const at::Tensor* scale = dev(a[5], at::kHalf, "scale");
-    if (!scale || !ptr(a[6], "y", &y) || !ptr(a[7], "workspace", &ws) || !ptr(a[8], "S_dbg", &S)) return nullptr;
+    const at::Tensor* scale = dev(a[5], at::kHalf, "scale", words);
+    if (!scale) return nullptr;
     const bool two = words->dim() == 2 && xq->dim() == 2;
     const int64_t N = two ? words->size(0) : 0, K = two ? 16 * words->size(1) : 0, M = two ? xq->size(0) : 0;
     const bool grid = group == 0 ? has_shape(*lut, {N, 4}) : group > 0 && K % group == 0 && has_shape(*lut, {N, K / group, 4});
@@ -162,6 +206,9 @@ PyObject* gemv_w2a4(PyObject*, PyObject* const* a, Py_ssize_t n) {
       bad_shapes(group == 0 ? "words, lut, xq and scale" : "words, lut, group, xq and scale");
       return nullptr;
     }
+    if (!buffer(a[6], "y", at::kHalf, *words, M * N, &y) || !buffer(a[7], "workspace", kAny, *words, workspace_bytes(M, N, K), &ws) ||
+        !buffer(a[8], "S_dbg", at::kInt, *words, M * N * (group ? K / group : 1) * 4, &S))
+      return nullptr;
     const uint32_t* const wp = static_cast<const uint32_t*>(words->data_ptr());
     const void *lp = lut->data_ptr(), *sp = scale->data_ptr();
     const uint8_t* const qp = static_cast<const uint8_t*>(xq->data_ptr());
@@ -179,15 +226,17 @@ PyObject* gemv_w2a16(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!count(n, 8)) return nullptr;
     const at::Tensor* words = dev(a[0], at::kInt, "words");
     if (!words) return nullptr;
-    const at::Tensor* lut = dev(a[1], at::kHalf, "lut");
+    const at::Tensor* lut = dev(a[1], at::kHalf, "lut", words);
     if (!lut) return nullptr;
-    const at::Tensor* x = dev(a[2], at::kHalf, "x");
-    if (!x || !ptr(a[3], "y", &y) || !ptr(a[4], "digits", &digits) || !ptr(a[5], "unit", &unit) || !ptr(a[6], "workspace", &ws) ||
-        !ptr(a[7], "S_dbg", &S))
-      return nullptr;
+    const at::Tensor* x = dev(a[2], at::kHalf, "x", words);
+    if (!x) return nullptr;
     const bool two = words->dim() == 2 && x->dim() == 2;
     const int64_t N = two ? words->size(0) : 0, K = two ? 16 * words->size(1) : 0, M = two ? x->size(0) : 0;
     if (!two || !has_shape(*x, {M, K}) || !has_shape(*lut, {N, 4})) { bad_shapes("words, lut and x"); return nullptr; }
+    if (!buffer(a[3], "y", at::kHalf, *words, M * N, &y) || !buffer(a[4], "digits", at::kChar, *words, M * 4 * K, &digits) ||
+        !buffer(a[5], "unit", at::kFloat, *words, M * 4, &unit) ||
+        !buffer(a[6], "workspace", kAny, *words, workspace_bytes(M, N, K), &ws) || !buffer(a[7], "S_dbg", at::kInt, *words, 4 * M * N * 4, &S))
+      return nullptr;
     const uint32_t* const wp = static_cast<const uint32_t*>(words->data_ptr());
     const void *lp = lut->data_ptr(), *xp = x->data_ptr();
     return on_device(*words, [&](void* st) {
@@ -205,14 +254,14 @@ PyObject* gemv_w3a4(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!count(n, 8) || !integer(a[3], &group)) return nullptr;
     const at::Tensor* words2 = dev(a[0], at::kInt, "words2");
     if (!words2) return nullptr;
-    const at::Tensor* words1 = dev(a[1], at::kInt, "words1");
+    const at::Tensor* words1 = dev(a[1], at::kInt, "words1", words2);
     if (!words1) return nullptr;
-    const at::Tensor* lut = dev(a[2], at::kHalf, "lut");
+    const at::Tensor* lut = dev(a[2], at::kHalf, "lut", words2);
     if (!lut) return nullptr;
-    const at::Tensor* xq = dev(a[4], at::kByte, "xq");
+    const at::Tensor* xq = dev(a[4], at::kByte, "xq", words2);
     if (!xq) return nullptr;
-    const at::Tensor* scale = dev(a[5], at::kHalf, "scale");
-    if (!scale || !ptr(a[6], "y", &y) || !ptr(a[7], "S_dbg", &S)) return nullptr;
+    const at::Tensor* scale = dev(a[5], at::kHalf, "scale", words2);
+    if (!scale) return nullptr;
     const bool two = words2->dim() == 2 && xq->dim() == 2;
     const int64_t N = two ? words2->size(0) : 0, K = two ? 16 * words2->size(1) : 0, M = two ? xq->size(0) : 0;
     const bool grid = group == 0 ? has_shape(*lut, {N, 8}) : has_shape(*lut, {N, K / std::max(group, 1), 8});
@@ -220,6 +269,9 @@ PyObject* gemv_w3a4(PyObject*, PyObject* const* a, Py_ssize_t n) {
       bad_shapes("words2, words1, lut, group, xq and scale");
       return nullptr;
     }
+    if (!buffer(a[6], "y", at::kHalf, *words2, M * N, &y) ||
+        !buffer(a[7], "S_dbg", at::kInt, *words2, M * N * (group ? K / std::max(group, 1) : 1) * 8, &S))
+      return nullptr;
     const uint32_t *w2 = static_cast<const uint32_t*>(words2->data_ptr()), *w1 = static_cast<const uint32_t*>(words1->data_ptr());
     const void *lp = lut->data_ptr(), *sp = scale->data_ptr();
     const uint8_t* const qp = static_cast<const uint8_t*>(xq->data_ptr());
@@ -238,16 +290,18 @@ PyObject* linear_w2a4(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!count(n, 11)) return nullptr;
     const at::Tensor* x = dev(a[0], at::kHalf, "x");
     if (!x) return nullptr;
-    const at::Tensor* words = dev(a[3], at::kInt, "words");
+    const at::Tensor* words = dev(a[3], at::kInt, "words", x);
     if (!words) return nullptr;
-    const at::Tensor* lut = dev(a[4], at::kHalf, "lut");
-    if (!lut || !integer(a[1], &B) || !real(a[2], &clip) || !integer(a[5], &group) || !ptr(a[6], "y", &y) || !ptr(a[7], "xq", &xq) ||
-        !ptr(a[8], "scale", &scale) || !ptr(a[9], "workspace", &ws) || !ptr(a[10], "S_dbg", &S))
-      return nullptr;
+    const at::Tensor* lut = dev(a[4], at::kHalf, "lut", x);
+    if (!lut || !integer(a[1], &B) || !real(a[2], &clip) || !integer(a[5], &group)) return nullptr;
     const bool two = words->dim() == 2 && x->dim() == 2;
     const int64_t N = two ? words->size(0) : 0, K = two ? x->size(1) : 0, M = two ? x->size(0) : 0;
     const bool grid = group == 0 ? has_shape(*lut, {N, 4}) : has_shape(*lut, {N, K / std::max(group, 1), 4});
     if (!two || words->size(1) * 16 != K || !grid) { bad_shapes("x, words, lut and group"); return nullptr; }
+    if (!buffer(a[6], "y", at::kHalf, *x, M * N, &y) || !buffer(a[7], "xq", at::kByte, *x, M * (K / 2), &xq) ||
+        !buffer(a[8], "scale", at::kHalf, *x, M, &scale) || !buffer(a[9], "workspace", kAny, *x, workspace_bytes(M, N, K), &ws) ||
+        !buffer(a[10], "S_dbg", at::kInt, *x, M * N * (group ? K / std::max(group, 1) : 1) * 4, &S))
+      return nullptr;
     const uint32_t* const wp = static_cast<const uint32_t*>(words->data_ptr());
     const void *lp = lut->data_ptr(), *xp = x->data_ptr();
     return on_device(*words, [&](void* st) {
@@ -262,27 +316,37 @@ PyObject* linear_w2a4_host(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded([&]() -> PyObject* {
     int B;
     float clip;
-    void *lut, *xd, *xq, *scale, *yd, *ws;
+    void *xd, *xq, *scale, *yd, *ws;
     if (!count(n, 11)) return nullptr;
-    if (!THPVariable_Check(a[0]) || !THPVariable_Check(a[5]) || !THPVariable_Check(a[3])) {
-      PyErr_SetString(PyExc_TypeError, "x_host, words and y_host must be tensors");
+    if (!THPVariable_Check(a[0]) || !THPVariable_Check(a[5])) {
+      PyErr_SetString(PyExc_TypeError, "x_host and y_host must be tensors");
       return nullptr;
     }
-    const at::Tensor &x = THPVariable_Unpack(a[0]), &y = THPVariable_Unpack(a[5]), &words = THPVariable_Unpack(a[3]);
-    if (x.is_cuda() || y.is_cuda() || x.scalar_type() != at::kHalf || y.scalar_type() != at::kHalf) {
-      PyErr_SetString(PyExc_TypeError, "x_host / y_host must be fp16 host tensors");
+    const at::Tensor &x = THPVariable_Unpack(a[0]), &y = THPVariable_Unpack(a[5]);
+    if (!x.is_cpu() || !y.is_cpu() || x.scalar_type() != at::kHalf || y.scalar_type() != at::kHalf || !x.is_contiguous() ||
+        !y.is_contiguous()) {
+      PyErr_SetString(PyExc_TypeError, "x_host / y_host must be contiguous fp16 host tensors");
       return nullptr;
     }
-    if (!integer(a[1], &B) || !real(a[2], &clip) || !ptr(a[4], "lut", &lut) || !ptr(a[6], "x_dev", &xd) || !ptr(a[7], "xq_dev", &xq) ||
-        !ptr(a[8], "scale_dev", &scale) || !ptr(a[9], "y_dev", &yd) || !ptr(a[10], "workspace", &ws))
+    const at::Tensor* words = dev(a[3], at::kInt, "words");
+    if (!words) return nullptr;
+    const at::Tensor* lut = dev(a[4], at::kHalf, "lut", words);
+    if (!lut || !integer(a[1], &B) || !real(a[2], &clip)) return nullptr;
+    const bool two = words->dim() == 2 && x.dim() == 2;
+    const int64_t N = two ? words->size(0) : 0, K = two ? x.size(1) : 0, M = two ? x.size(0) : 0;
+    if (!two || words->size(1) * 16 != K || lut->numel() != 4 * N || y.numel() < M * N) {
+      bad_shapes("x_host, words, lut and y_host");
       return nullptr;
-    if (x.dim() != 2 || !words.is_cuda()) { bad_shapes("x_host and [M][K]"); return nullptr; }
-    const int M = (int)x.size(0), K = (int)x.size(1), N = (int)words.size(0);
-    const void* const xp = x.data_ptr();
+    }
+    if (!buffer(a[6], "x_dev", at::kHalf, *words, M * K, &xd) || !buffer(a[7], "xq_dev", at::kByte, *words, M * (K / 2), &xq) ||
+        !buffer(a[8], "scale_dev", at::kHalf, *words, M, &scale) || !buffer(a[9], "y_dev", at::kHalf, *words, M * N, &yd) ||
+        !buffer(a[10], "workspace", kAny, *words, workspace_bytes(M, N, K), &ws))
+      return nullptr;
+    const void *const xp = x.data_ptr(), *const lp = lut->data_ptr();
     void* const yp = y.data_ptr();
-    const uint32_t* const wp = static_cast<const uint32_t*>(words.data_ptr());
-    return on_device(words, [&](void* st) {
-      return g_fn.linear_host(xp, M, K, B, clip, wp, lut, N, yp, xd, static_cast<uint8_t*>(xq), scale, yd, ws, st);
+    const uint32_t* const wp = static_cast<const uint32_t*>(words->data_ptr());
+    return on_device(*words, [&](void* st) {
+      return g_fn.linear_host(xp, (int)M, (int)K, B, clip, wp, lp, (int)N, yp, xd, static_cast<uint8_t*>(xq), scale, yd, ws, st);
     });
   });
 }
