@@ -121,7 +121,6 @@ struct GemvParams {
   int off_bar, off_T0c, off_scale, off_red, off_bs;   // shared-memory byte offsets from the aligned base
   int bs_bytes, red_bytes, part_bytes;                // sizes of the areas at off_bs, off_red, off_part (guarded build)
   int stage_stride;     // bytes from one ring stage to the next: kStageBytes, plus the stage's activation area (SB)
-  int late_start;       // tensor-core kernels: the next kernel may start when this one ends, not at once (see the end)
 };
 
 // ----------------------------------------------------------------------------- PTX wrappers
@@ -267,8 +266,10 @@ __global__ void wait_timeout_kernel(int32_t* status, uint32_t polls) {
 //       consumers like the producer does. The token count and K then no longer meet in shared memory: no K in
 //       parts, up to sixteen tokens for any K, and the expansion (2 us at eight tokens of 8192) leaves the
 //       critical path. The host keeps (warps sharing a group) x tokens at 32 or less per stage.
+// LATE  tensor-core kernels: the next kernel may start when this one ends, not at once (see the end). A form of its own: as a
+//       run-time flag it cost 0.3 % at sixteen tokens and 1 % of the weight-only calls.
 template <int MODE, int MTOK, bool GRP, int FQ = 0, bool A16 = false, bool SPLIT = false, bool SDBG = false,
-          bool SB = false>
+          bool SB = false, bool LATE = false>
 __global__ void __launch_bounds__(SB ? kGThreads + 32 * kExpWarps : kGThreads, 1)
 gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -320,8 +321,8 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
 
   const int b = blockIdx.x;
   // Launched with programmatic stream serialization; when the next kernel may start is explained at the end.
-  const bool late_start = MODE == kModeMma && p.late_start;
-  if (!late_start) asm volatile("griddepcontrol.launch_dependents;");
+  static_assert(!LATE || MODE == kModeMma, "late start: tensor-core kernels");
+  if constexpr (!LATE) asm volatile("griddepcontrol.launch_dependents;");
   int* const s_T0tot = reinterpret_cast<int*>(s_scale + 32);   // [16]: sum of q per token, behind scales and maxima
   // The producer warp sets up the ring's barriers and only announces that (bar.arrive): its first
   // requests go out without waiting for anybody. The consumer warps wait for the announcement.
@@ -1371,11 +1372,11 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   // inside), cannot fit beside this CTA, and takes over SM by SM (2048x2048 in a chain 2.76 us, 2.97 with the trigger here).
   // So do the kernels for more tokens when they are called on activations quantized before, one set of which serves
   // several GEMVs (4096x4096 at three tokens 4.2 us a call, 4.6 with the trigger here; 10240x8192 at nine 17.9 and 19.2).
-  // Inside a call that has a quantizer of its own (late_start) the next kernel is the next call's quantizer, and behind
+  // Inside a call that has a quantizer of its own (LATE) the next kernel is the next call's quantizer, and behind
   // that comes a GEMV whose CTAs take every SM that the quantizer leaves and fill the memory system with weights while
   // its few CTAs still fetch their tokens: started from here, a chain of such calls takes 6.0 us instead of 7.1 at 4096x4096 and
   // eight tokens, 8.6 instead of 9.9 at sixteen, 13.5 instead of 14.0 at 10240x8192 and eight.
-  if (late_start) asm volatile("griddepcontrol.launch_dependents;");
+  if constexpr (LATE) asm volatile("griddepcontrol.launch_dependents;");
 }
 
 }  // namespace rcp

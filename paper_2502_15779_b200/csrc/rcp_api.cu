@@ -266,12 +266,12 @@ cudaError_t set_max_smem(Kern kern, int bytes, std::mutex& mu, bool (&done)[kMax
   return cudaSuccess;
 }
 
-template <int MODE, int MTOK, bool GRP, int FQ, bool A16, bool SPLIT, bool SDBG, bool SB = false>
-int launch_stream_s(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
+template <int MODE, int MTOK, bool GRP, int FQ, bool A16, bool SPLIT, bool SDBG, bool SB, bool LATE>
+int launch_stream_k(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
   // cudaFuncAttributeMaxDynamicSharedMemorySize belongs to the (kernel, device) pair: set once per device
   static std::mutex mu;
   static bool attr_set[kMaxDevices] = {};
-  auto kern = rcp::gemv_stream_kernel<MODE, MTOK, GRP, FQ, A16, SPLIT, SDBG, SB>;
+  auto kern = rcp::gemv_stream_kernel<MODE, MTOK, GRP, FQ, A16, SPLIT, SDBG, SB, LATE>;
   int dev = 0;
   RCP_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxDevices) return RCP_ERR_LIMIT;
@@ -286,18 +286,32 @@ int launch_stream_s(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const 
   return RCP_OK;
 }
 
+// late: which of its two forms a tensor-core kernel is taken in. (The checked instantiations have the
+// early form alone; digit columns of more than one token always have the kernel that splits them in front: late.)
+template <int MODE, int MTOK, bool GRP, int FQ, bool A16, bool SPLIT, bool SDBG, bool SB = false>
+int launch_stream_s(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, bool late, cudaStream_t st) {
+  constexpr bool kBoth = MODE == rcp::kModeMma && !SDBG, kAlways = kBoth && A16 && (SPLIT || MTOK == 16);
+  if constexpr (kAlways) {
+    return launch_stream_k<MODE, MTOK, GRP, FQ, A16, SPLIT, SDBG, SB, true>(maps, gp, pl, st);
+  } else {
+    if constexpr (kBoth)
+      if (late) return launch_stream_k<MODE, MTOK, GRP, FQ, A16, SPLIT, SDBG, SB, true>(maps, gp, pl, st);
+    return launch_stream_k<MODE, MTOK, GRP, FQ, A16, SPLIT, SDBG, SB, false>(maps, gp, pl, st);
+  }
+}
+
 // streamed activations (tensor-core kernels of the per-row grid; MTOK 0: up to eight tokens, 16: nine to sixteen)
 template <int MTOK>
-int launch_stream_sb(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
-  if (gp.S_out) return launch_stream_s<rcp::kModeMma, MTOK, false, 0, false, false, true, true>(maps, gp, pl, st);
-  return launch_stream_s<rcp::kModeMma, MTOK, false, 0, false, false, false, true>(maps, gp, pl, st);
+int launch_stream_sb(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, bool late, cudaStream_t st) {
+  if (gp.S_out) return launch_stream_s<rcp::kModeMma, MTOK, false, 0, false, false, true, true>(maps, gp, pl, late, st);
+  return launch_stream_s<rcp::kModeMma, MTOK, false, 0, false, false, false, true>(maps, gp, pl, late, st);
 }
 
 // gp.S_out set: the checked instantiation of the same kernel, which also stores its integer sums.
 template <int MODE, int MTOK, bool GRP = false, int FQ = 0, bool A16 = false, bool SPLIT = false>
-int launch_stream_t(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
-  if (gp.S_out) return launch_stream_s<MODE, MTOK, GRP, FQ, A16, SPLIT, true>(maps, gp, pl, st);
-  return launch_stream_s<MODE, MTOK, GRP, FQ, A16, SPLIT, false>(maps, gp, pl, st);
+int launch_stream_t(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, bool late, cudaStream_t st) {
+  if (gp.S_out) return launch_stream_s<MODE, MTOK, GRP, FQ, A16, SPLIT, true>(maps, gp, pl, late, st);
+  return launch_stream_s<MODE, MTOK, GRP, FQ, A16, SPLIT, false>(maps, gp, pl, late, st);
 }
 
 // One launch: M tokens (their expanded activations fit in shared memory). grouped: lut_f16 is
@@ -327,20 +341,20 @@ bool full_block(int K, int B) { return B == K && (K == 2048 || K == 4096 || K ==
 bool fused_ok(int M, int K, int B) { return M == 1 && (full_block(K, B) || (B <= 512 && K <= 16384)); }
 
 template <bool GRP>
-int launch_fused(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, cudaStream_t st) {
+int launch_fused(const rcp::GemvMaps& maps, const rcp::GemvParams& gp, const StreamPlan& pl, bool late, cudaStream_t st) {
   if (full_block(gp.K, gp.had_block)) {
-    if (gp.K == 2048) return launch_stream_t<rcp::kModeDp4a, 1, GRP, 4>(maps, gp, pl, st);
-    if (gp.K == 4096) return launch_stream_t<rcp::kModeDp4a, 1, GRP, 8>(maps, gp, pl, st);
-    return launch_stream_t<rcp::kModeDp4a, 1, GRP, 16>(maps, gp, pl, st);
+    if (gp.K == 2048) return launch_stream_t<rcp::kModeDp4a, 1, GRP, 4>(maps, gp, pl, late, st);
+    if (gp.K == 4096) return launch_stream_t<rcp::kModeDp4a, 1, GRP, 8>(maps, gp, pl, late, st);
+    return launch_stream_t<rcp::kModeDp4a, 1, GRP, 16>(maps, gp, pl, late, st);
   }
-  if (gp.K <= 8192) return launch_stream_t<rcp::kModeDp4a, 1, GRP, -1>(maps, gp, pl, st);
-  return launch_stream_t<rcp::kModeDp4a, 1, GRP, -2>(maps, gp, pl, st);
+  if (gp.K <= 8192) return launch_stream_t<rcp::kModeDp4a, 1, GRP, -1>(maps, gp, pl, late, st);
+  return launch_stream_t<rcp::kModeDp4a, 1, GRP, -2>(maps, gp, pl, late, st);
 }
 
 int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16,
                   int M, int N, int K, void* y_f16, void* workspace, cudaStream_t st, bool grouped = false,
                   const FusedAct* fa = nullptr, const float* unit = nullptr, int nsplit = 1,
-                  const SplitAct* sa = nullptr, int32_t* S_out = nullptr, bool stream_act = false, bool late_start = false) {
+                  const SplitAct* sa = nullptr, int32_t* S_out = nullptr, bool stream_act = false, bool late = false) {
   if (stream_act && (mode != rcp::kModeMma || fa || unit || sa || nsplit > 1 || M > (grouped ? 8 : rcp::kMaxTokens))) return RCP_ERR_VARIANT;
   if (nsplit > 1 && (mode != rcp::kModeMma || grouped || fa || M > 8)) return RCP_ERR_VARIANT;
   if (sa && (mode != rcp::kModeMma || grouped || fa || unit || nsplit > 1 || M != 4 || K > 16384)) return RCP_ERR_VARIANT;
@@ -424,7 +438,6 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
   gp.off_part = pl.off_part;
   gp.act_parts = std::max(1, rcp::kCWarps / M);
   gp.inv_act_parts = (256 + gp.act_parts - 1) / gp.act_parts;
-  gp.late_start = late_start;
   gp.nphase = pl.nphase;
   for (int i = 0; i < rcp::kMaxPhases; i++) gp.phase[i] = i < pl.nphase ? pl.phase[i] : make_phase(1, 0, 0, 1, 0, pl.nchunk);
   gp.stages = pl.stages;
@@ -444,43 +457,43 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
     gp.inv_sqrt_b = (float)(1.0 / std::sqrt((double)fa->B));
     gp.clip_ratio = std::min(fa->clip_ratio, rcp::kClipRatioCap);
     gp.had_block = fa->B;
-    return grouped ? launch_fused<true>(maps, gp, pl, st) : launch_fused<false>(maps, gp, pl, st);
+    return grouped ? launch_fused<true>(maps, gp, pl, late, st) : launch_fused<false>(maps, gp, pl, late, st);
   }
   if (sa) {
     gp.x = static_cast<const __half*>(sa->x_f16);
     gp.xq_out = reinterpret_cast<uint8_t*>(sa->digits_out);
     gp.unit_out = sa->unit_out;
-    return launch_stream_t<rcp::kModeMma, 0, false, 0, true>(maps, gp, pl, st);
+    return launch_stream_t<rcp::kModeMma, 0, false, 0, true>(maps, gp, pl, late, st);
   }
   if (unit) {
-    if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, 0, true, true>(maps, gp, pl, st);
-    return M > 8 ? launch_stream_t<rcp::kModeMma, 16, false, 0, true>(maps, gp, pl, st)
-                 : launch_stream_t<rcp::kModeMma, 0, false, 0, true>(maps, gp, pl, st);
+    if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, 0, true, true>(maps, gp, pl, late, st);
+    return M > 8 ? launch_stream_t<rcp::kModeMma, 16, false, 0, true>(maps, gp, pl, late, st)
+                 : launch_stream_t<rcp::kModeMma, 0, false, 0, true>(maps, gp, pl, late, st);
   }
   if (grouped) {
     if (mode == rcp::kModeDp4a)
-      return M == 1 ? launch_stream_t<rcp::kModeDp4a, 1, true>(maps, gp, pl, st)
-                    : launch_stream_t<rcp::kModeDp4a, 2, true>(maps, gp, pl, st);
+      return M == 1 ? launch_stream_t<rcp::kModeDp4a, 1, true>(maps, gp, pl, late, st)
+                    : launch_stream_t<rcp::kModeDp4a, 2, true>(maps, gp, pl, late, st);
     if (stream_act)
-      return gp.S_out ? launch_stream_s<rcp::kModeMma, 0, true, 0, false, false, true, true>(maps, gp, pl, st)
-                      : launch_stream_s<rcp::kModeMma, 0, true, 0, false, false, false, true>(maps, gp, pl, st);
-    if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, true, 0, false, false, false>(maps, gp, pl, st);
-    return launch_stream_t<rcp::kModeMma, 0, true>(maps, gp, pl, st);
+      return gp.S_out ? launch_stream_s<rcp::kModeMma, 0, true, 0, false, false, true, true>(maps, gp, pl, late, st)
+                      : launch_stream_s<rcp::kModeMma, 0, true, 0, false, false, false, true>(maps, gp, pl, late, st);
+    if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, true, 0, false, false, false>(maps, gp, pl, late, st);
+    return launch_stream_t<rcp::kModeMma, 0, true>(maps, gp, pl, late, st);
   }
   if (mode == rcp::kModeHybrid)
-    return M == 1 ? launch_stream_t<rcp::kModeHybrid, 1>(maps, gp, pl, st)
-                  : launch_stream_t<rcp::kModeHybrid, 2>(maps, gp, pl, st);
+    return M == 1 ? launch_stream_t<rcp::kModeHybrid, 1>(maps, gp, pl, late, st)
+                  : launch_stream_t<rcp::kModeHybrid, 2>(maps, gp, pl, late, st);
   if (mode == rcp::kModeDp4a)
-    return M == 1 ? launch_stream_t<rcp::kModeDp4a, 1>(maps, gp, pl, st)
-                  : launch_stream_t<rcp::kModeDp4a, 2>(maps, gp, pl, st);
+    return M == 1 ? launch_stream_t<rcp::kModeDp4a, 1>(maps, gp, pl, late, st)
+                  : launch_stream_t<rcp::kModeDp4a, 2>(maps, gp, pl, late, st);
   if (stream_act) {
-    if (M == 8 && !gp.S_out) return launch_stream_sb<8>(maps, gp, pl, st);
-    return M > 8 ? launch_stream_sb<16>(maps, gp, pl, st) : launch_stream_sb<0>(maps, gp, pl, st);
+    if (M == 8 && !gp.S_out) return launch_stream_sb<8>(maps, gp, pl, late, st);
+    return M > 8 ? launch_stream_sb<16>(maps, gp, pl, late, st) : launch_stream_sb<0>(maps, gp, pl, late, st);
   }
-  if (pl.nsplit > 1 && M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, false, 0, false, true, false>(maps, gp, pl, st);
-  if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, 0, false, true>(maps, gp, pl, st);
-  if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, false, 0, false, false, false>(maps, gp, pl, st);   // token count known at compile time
-  return M > 8 ? launch_stream_t<rcp::kModeMma, 16>(maps, gp, pl, st) : launch_stream_t<rcp::kModeMma, 0>(maps, gp, pl, st);
+  if (pl.nsplit > 1 && M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, false, 0, false, true, false>(maps, gp, pl, late, st);
+  if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, 0, false, true>(maps, gp, pl, late, st);
+  if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, false, 0, false, false, false>(maps, gp, pl, late, st);   // token count known at compile time
+  return M > 8 ? launch_stream_t<rcp::kModeMma, 16>(maps, gp, pl, late, st) : launch_stream_t<rcp::kModeMma, 0>(maps, gp, pl, late, st);
 }
 
 // All M tokens: as many launches as it takes for the expanded activations to fit (`cap` tokens at most each).
