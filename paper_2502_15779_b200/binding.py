@@ -202,8 +202,7 @@ def rcp_nf3_export(w, sig_beta, sig_gamma, sig_s1, table, zero_index, group):
 def rcp_quantize_act(x: torch.Tensor, had_block: int, clip_ratio: float = 1.0, xq=None, scale=None):
     """x fp16 [M][K] -> (xq uint8 [M][K/2], scale fp16 [M])."""
     if xq is None or scale is None:
-        _dev(x, torch.float16, "x")
-        M, K = x.shape
+        M, K = _matrix(x, torch.float16, "x")
         if xq is None:
             xq = torch.empty((M, K // 2), dtype=torch.uint8, device=x.device)
         if scale is None:
@@ -231,18 +230,24 @@ def _variant(variant):
 def rcp_gemv_w2a4(words, lut, xq, scale, y=None, workspace=None, S_dbg=None, variant="auto"):
     """words int32 [N][K/16], lut fp16 [N][4], xq uint8 [M][K/2], scale fp16 [M] -> y fp16 [M][N]."""
     if y is None or workspace is None:
-        y, workspace = _results(words, xq, y, workspace)
+        y, workspace = _results(words, xq, torch.uint8, "xq", y, workspace)
     st = (_m or _native()).gemv_w2a4(_variant(variant), words, lut, 0, xq, scale, y, workspace, S_dbg)
     if st:
         _check("rcp_gemv_w2a4", st)
     return y
 
 
-def _results(words, x, y, workspace):
-    """The buffers a caller did not pass: y fp16 [M][N] and the workspace."""
-    _dev(words, torch.int32, "words")
-    N, K = words.shape[0], words.shape[1] * 16
-    M = x.shape[0]
+def _matrix(t, dtype, name):
+    """Rows and columns of a matrix whose sizes buffers are allocated from."""
+    if _dev(t, dtype, name).dim() != 2:
+        raise ValueError(f"{name}: expected a matrix, got shape {tuple(t.shape)}")
+    return t.shape
+
+
+def _results(words, x, dtype, name, y, workspace):
+    """The buffers a caller did not pass: y fp16 [M][N] and the workspace. x: xq or x, one row per token."""
+    N, K = _matrix(words, torch.int32, "words")
+    M, K = _matrix(x, dtype, name)[0], K * 16
     if y is None:
         y = torch.empty((M, N), dtype=torch.float16, device=words.device)
     if workspace is None and rcp_gemv_workspace_bytes(M, N, K) > 0:
@@ -256,7 +261,7 @@ def rcp_gemv_w2a4_grouped(words, lut, xq, scale, group=128, y=None, workspace=No
     if int(group) < 1:
         raise ValueError("shape mismatch between words, lut, group, xq and scale")
     if y is None or workspace is None:
-        y, workspace = _results(words, xq, y, workspace)
+        y, workspace = _results(words, xq, torch.uint8, "xq", y, workspace)
     st = (_m or _native()).gemv_w2a4(_variant(variant), words, lut, int(group), xq, scale, y, workspace, S_dbg)
     if st:
         _check("rcp_gemv_w2a4_grouped", st)
@@ -268,11 +273,13 @@ def rcp_gemv_w2a16(words, lut, x, y=None, digits=None, unit=None, workspace=None
     digits int8 [M][4][K] and unit fp32 [M][4] receive the fixed-point form of x the kernels used.
     S_dbg int32 [4 M][N][4]: the per-code sums of every digit plane (checked instantiation of the kernel)."""
     if y is None or workspace is None:
-        y, workspace = _results(words, x, y, workspace)
-    if digits is None:
-        digits = torch.empty((x.shape[0], 4, x.shape[1]), dtype=torch.int8, device=words.device)
-    if unit is None:
-        unit = torch.empty((x.shape[0], 4), dtype=torch.float32, device=words.device)
+        y, workspace = _results(words, x, torch.float16, "x", y, workspace)
+    if digits is None or unit is None:
+        M, K = _matrix(x, torch.float16, "x")
+        if digits is None:
+            digits = torch.empty((M, 4, K), dtype=torch.int8, device=x.device)
+        if unit is None:
+            unit = torch.empty((M, 4), dtype=torch.float32, device=x.device)
     st = (_m or _native()).gemv_w2a16(words, lut, x, y, digits, unit, workspace, S_dbg)
     if st:
         _check("rcp_gemv_w2a16", st)
@@ -295,8 +302,8 @@ def rcp_gemv_w3a4(words2, words1, lut, xq, scale, group=0, y=None, S_dbg=None):
     """W3A4 GEMV: words2 int32 [N][K/16], words1 int32 [N][K/32], lut fp16 [N][8] (group=0) or [N][K/128][8]
     (group=128), xq uint8 [M][K/2], scale fp16 [M] -> y fp16 [M][N]."""
     if y is None:
-        _dev(words2, torch.int32, "words2")
-        y = torch.empty((xq.shape[0], words2.shape[0]), dtype=torch.float16, device=words2.device)
+        N, M = _matrix(words2, torch.int32, "words2")[0], _matrix(xq, torch.uint8, "xq")[0]
+        y = torch.empty((M, N), dtype=torch.float16, device=words2.device)
     st = (_m or _native()).gemv_w3a4(words2, words1, lut, int(group), xq, scale, y, S_dbg)
     if st:
         _check("rcp_gemv_w3a4", st)
@@ -338,7 +345,7 @@ def rcp_linear_w2a4(x, had_block, clip_ratio, words, lut, group=0, y=None, xq=No
     them to be safe). S_dbg int32 [M][N][4] ([M][N][K/group][4]): the integer sums, from the checked instantiation
     of the kernel that runs anyway."""
     if y is None or workspace is None:
-        y, workspace = _results(words, x, y, workspace)
+        y, workspace = _results(words, x, torch.float16, "x", y, workspace)
     st = (_m or _native()).linear_w2a4(x, had_block, clip_ratio, words, lut, group, y, xq, scale, workspace, S_dbg)
     if st:
         _check("rcp_linear_w2a4", st)

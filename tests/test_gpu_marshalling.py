@@ -149,3 +149,39 @@ def test_host_form_checks_what_it_reads_and_writes():
         with pytest.raises(error):
             rcp.rcp_linear_w2a4_host(**dict(good, **change))
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("bad,error", [(None, TypeError), (3, TypeError), ("1d", ValueError), ("0d", ValueError), ("host", TypeError)])
+def test_operands_that_are_no_matrix(bad, error, given):
+    """The same exceptions whether the result buffers are passed or allocated."""
+    x = synth.make_activations(M, K, 2, device=DEV)
+    words, lut = _layer()
+    wordsg, lutg = _layer(128)
+    words2, words1 = rcp.rcp_pack_weights3(torch.randint(0, 8, (N, K), dtype=torch.uint8, device=DEV))
+    lut3 = torch.randn(N, 8, device=DEV).half()
+    xq, scale = rcp.rcp_quantize_act(x, 64, 1.0)
+    y = dict(y=torch.empty(M, N, dtype=torch.float16, device=DEV)) if given else {}
+    ws = dict(workspace=rcp.make_workspace(M, N, K, DEV)) if given else {}
+    dg = dict(digits=torch.empty(M, 4, K, dtype=torch.int8, device=DEV), unit=torch.empty(M, 4, device=DEV)) if given else {}
+
+    def spoil(t):
+        return {"1d": t.reshape(-1), "0d": t.reshape(-1)[0], "host": t.cpu()}.get(bad, bad) if isinstance(bad, str) else bad
+
+    calls = [
+        lambda: rcp.rcp_gemv_w2a4(spoil(words), lut, xq, scale, **y, **ws),
+        lambda: rcp.rcp_gemv_w2a4(words, lut, spoil(xq), scale, **y, **ws),
+        lambda: rcp.rcp_gemv_w2a4_grouped(spoil(wordsg), lutg, xq, scale, **y, **ws),
+        lambda: rcp.rcp_gemv_w2a4_grouped(wordsg, lutg, spoil(xq), scale, **y, **ws),
+        lambda: rcp.rcp_gemv_w2a16(spoil(words), lut, x, **y, **ws, **dg),
+        lambda: rcp.rcp_gemv_w2a16(words, lut, spoil(x), **y, **ws, **dg),
+        lambda: rcp.rcp_gemv_w3a4(spoil(words2), words1, lut3, xq, scale, **y),
+        lambda: rcp.rcp_gemv_w3a4(words2, words1, lut3, spoil(xq), scale, **y),
+        lambda: rcp.rcp_linear_w2a4(spoil(x), 64, 1.0, words, lut, **y, **ws, **(_buffers() if given else {})),
+        lambda: rcp.rcp_linear_w2a4(x, 64, 1.0, spoil(words), lut, **y, **ws, **(_buffers() if given else {})),
+        lambda: rcp.rcp_quantize_act(spoil(x), 64, 1.0, **(_buffers() if given else {})),
+    ]
+    for call in calls:
+        with pytest.raises(error):
+            call()
+    torch.cuda.synchronize()
