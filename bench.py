@@ -47,7 +47,7 @@ def source_sha():
     import hashlib
     h = hashlib.sha1()
     d = os.path.join(ROOT, "paper_2502_15779_b200", "csrc")
-    for name in sorted(os.listdir(d)):
+    for name in sorted(n for n in os.listdir(d) if not n.endswith(".cpp")):   # (the marshalling is no kernel)
         h.update(name.encode())
         h.update(open(os.path.join(d, name), "rb").read())
     return h.hexdigest()[:16]

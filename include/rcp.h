@@ -47,6 +47,10 @@ const char* rcp_status_str(int status);
 /* cudaError_t (as int) of the last failed CUDA call made by this library on this thread. */
 int rcp_last_cuda_error(void);
 
+/* A number for the declarations of this header that the library was built from (set by its build; 0 otherwise). A caller
+ * that was compiled apart from the library can compare it with its own. */
+unsigned long long rcp_header_id(void);
+
 /*
  * Weight packing (Section 4.4: W_q is pre-computed offline and stored sub-byte packed along the
  * input channel). codes: uint8 [N][K], each in {0,1,2,3}. words: uint32 [N][K/16].

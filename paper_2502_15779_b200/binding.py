@@ -12,6 +12,8 @@ import os
 
 import torch
 
+from .build import marshal_path
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # RCP_W2A4_LIB names another build of the same library (the tests use it for the guarded build)
 LIB_PATH = os.environ.get("RCP_W2A4_LIB") or os.path.join(_HERE, "librcp_w2a4.so")
@@ -22,9 +24,10 @@ VARIANTS = {"auto": GEMV_AUTO, "simple": GEMV_SIMPLE, "dp4a": GEMV_DP4A, "mma": 
 
 _lib = None
 _m = None   # the native marshalling module, bound to _lib
-_MARSHAL_PATH = os.path.join(_HERE, "_marshal.so")
+_MARSHAL_PATH = marshal_path()
 _MARSHALLED = ("rcp_quantize_act", "rcp_gemv_w2a4_variant", "rcp_gemv_w2a4_grouped_variant", "rcp_gemv_w2a16_checked",
-               "rcp_gemv_w3a4", "rcp_linear_w2a4_checked", "rcp_linear_w2a4_host", "rcp_gemv_workspace_bytes")
+               "rcp_gemv_w3a4", "rcp_linear_w2a4_checked", "rcp_linear_w2a4_host", "rcp_gemv_workspace_bytes",
+               "rcp_header_id")
 
 
 class RcpError(RuntimeError):
@@ -91,15 +94,20 @@ def lib():
 
 
 def _native():
-    """The marshalling module, loaded and bound to the library on first use."""
+    """The marshalling module, loaded and bound to the library on first use. It calls the library through prototypes compiled
+    into it, so binding fails where the two were not built from the same declarations."""
     global _m
     if _m is None:
         L = lib()
         if not os.path.exists(_MARSHAL_PATH):
-            raise RuntimeError(f"{_MARSHAL_PATH} not found: build it with `python -m paper_2502_15779_b200.build`")
+            raise RuntimeError(f"{_MARSHAL_PATH} not found (it is built for one Python and one torch): build it with "
+                               "`python -m paper_2502_15779_b200.build`")
         spec = importlib.util.spec_from_file_location(__package__ + "._marshal", _MARSHAL_PATH)
         m = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(m)
+        missing = [name for name in _MARSHALLED if not hasattr(L, name)]
+        if missing:
+            raise RuntimeError(f"{LIB_PATH} has no {', '.join(missing)}: build it anew with `python -m paper_2502_15779_b200.build`")
         m.bind({name: C.cast(getattr(L, name), C.c_void_p).value for name in _MARSHALLED})
         _m = m
     return _m

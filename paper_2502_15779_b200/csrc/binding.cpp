@@ -12,6 +12,10 @@
 
 #include "../../include/rcp.h"
 
+#ifndef RCP_HEADER_ID
+#define RCP_HEADER_ID 0ull
+#endif
+
 namespace {
 
 struct Entry {
@@ -164,6 +168,14 @@ PyObject* bind(PyObject*, PyObject* table) {
       !take("rcp_gemv_w3a4", g_fn.gemv_w3a4) || !take("rcp_linear_w2a4_checked", g_fn.linear) ||
       !take("rcp_linear_w2a4_host", g_fn.linear_host) || !take("rcp_gemv_workspace_bytes", g_fn.workspace_bytes))
     return nullptr;
+  decltype(&rcp_header_id) header_id = nullptr;
+  if (!take("rcp_header_id", header_id)) return nullptr;
+  if (header_id() != RCP_HEADER_ID) {
+    g_fn = {};
+    PyErr_SetString(PyExc_RuntimeError, "the library and its marshalling module were not built from the same include/rcp.h: build both anew "
+                                        "with `python -m paper_2502_15779_b200.build`");
+    return nullptr;
+  }
   Py_RETURN_NONE;
 }
 

@@ -716,6 +716,11 @@ const char* rcp_status_str(int status) {
 
 int rcp_last_cuda_error(void) { return g_last_cuda_error; }
 
+#ifndef RCP_HEADER_ID
+#define RCP_HEADER_ID 0ull
+#endif
+unsigned long long rcp_header_id(void) { return RCP_HEADER_ID; }
+
 int rcp_pack_weights(const uint8_t* codes, int N, int K, uint32_t* words, void* stream) {
   if (!codes || !words) return RCP_ERR_NULL;
   if (N < 1 || !k_ok(K)) return RCP_ERR_SHAPE;

@@ -52,3 +52,41 @@ def test_binding_fails_loudly_without_library(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "LIB_PATH", str(tmp_path / "missing.so"))
     with pytest.raises(RuntimeError, match="no CPU or PyTorch fallback"):
         binding.lib()
+
+
+def test_library_and_marshalling_module_are_of_one_header(libpath):
+    from paper_2502_15779_b200 import build
+    L = ctypes.CDLL(libpath)
+    L.rcp_header_id.restype = ctypes.c_ulonglong
+    assert L.rcp_header_id() == build.header_id() != 0
+    assert os.path.exists(build.marshal_path())   # build() makes it as well
+
+
+def test_binding_refuses_a_library_of_another_header(libpath, monkeypatch, tmp_path):
+    """The marshalling module calls by address, with the prototypes it was compiled with."""
+    from paper_2502_15779_b200 import binding
+    monkeypatch.setattr(binding, "_m", None)
+    monkeypatch.setattr(binding, "_lib", None)
+    m = binding._native()
+    other = ctypes.CFUNCTYPE(ctypes.c_ulonglong)(lambda: 12345)
+    table = {name: ctypes.cast(getattr(binding.lib(), name), ctypes.c_void_p).value for name in binding._MARSHALLED}
+    m.bind(table)
+    with pytest.raises(RuntimeError, match="same include/rcp.h"):
+        m.bind(dict(table, rcp_header_id=ctypes.cast(other, ctypes.c_void_p).value))
+    m.bind(table)
+    monkeypatch.setattr(binding, "_m", None)
+    monkeypatch.setattr(binding, "_MARSHAL_PATH", str(tmp_path / "_marshal.of-another-torch.so"))
+    with pytest.raises(RuntimeError, match="one Python and one torch"):
+        binding._native()
+
+
+def test_header_id_follows_declarations_alone(monkeypatch, tmp_path):
+    from paper_2502_15779_b200 import build
+    text = open(build.HEADER).read()
+    was = build.header_id()
+    for change, same in ((lambda t: t.replace("/*", "/* more", 1), True), (lambda t: t.replace("int M, int N", "int N, int M", 1), False)):
+        p = tmp_path / "rcp.h"
+        p.write_text(change(text))
+        assert p.read_text() != text
+        monkeypatch.setattr(build, "HEADER", str(p))
+        assert (build.header_id() == was) == same
