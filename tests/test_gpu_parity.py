@@ -74,16 +74,79 @@ def test_quantize_act_bit_exact(M, K, B, clip):
 def test_quantize_act_one_cta_per_token(M, K, B, clip):
     """The kernels with a CTA per token, at the ends of their ranges: token counts around the CTAs of the grid, words
     that fill no warp, one and two words per thread; all-zero tokens, scales among the fp16 subnormals (where the
-    clamp of the rounding acts) and quotients on and next to ties."""
+    clamp of the rounding acts) and exact quotients."""
     x = synth.make_activations(M, K, 31 * M + K)
     x[M // 2] = 0
     if M > 2:
         x[0] = x[0] * 1e-6                                     # a subnormal scale
-        x[1] = (torch.arange(K) % 15 - 7).to(torch.float16) * 0.5   # with no rotation: halves of the scale, ties
+        x[1] = (torch.arange(K) % 15 - 7).to(torch.float16) * 0.5   # with no rotation: whole quotients
     ref = oracle.quantize_act(f16_bits(x), B, clip)
     xq, scale = rcp.rcp_quantize_act(x.to(DEV), B, clip)
     assert np.array_equal(f16_bits(scale), ref["scale"])
     assert np.array_equal(xq.cpu().numpy(), ref["xq"])
+
+
+def _tie_rows(rows, K):
+    """fp16 rows whose quotients without rotation lie on ties and one fp16 number beside them: the largest magnitude is 7 s (or its
+    nearest fp16 number), the others (n + 1/2) s, s mostly a number whose reciprocal is inexact. No clamping acts."""
+    scales = [3 * 2.0 ** -6, 5 * 2.0 ** -7, 11 * 2.0 ** -8, 2.0 ** -3, 13 * 2.0 ** -5, 1.0009765625, 0.00732421875, 937.5]
+    x = np.zeros((rows, K), dtype=np.float16)
+    n = np.arange(-6, 6) + 0.5
+    for r in range(rows):
+        amax = np.float16(7 * scales[r % len(scales)])
+        s = np.float64(np.float16(np.float32(amax) / np.float32(7)))
+        t = (n * s).astype(np.float16)
+        some = np.concatenate([t, np.nextafter(t, np.float16(np.inf)), np.nextafter(t, np.float16(-np.inf)), [amax]])
+        x[r] = np.resize(np.roll(some, r), K)
+        x[r, 0] = -amax if r & 1 else amax
+    return torch.from_numpy(x)
+
+
+def _rotated_ties(rows):
+    """Tokens of 4096 whose rotation over the whole token is exact (1 / 64) and lands on ties: impulses of 3.5, 2.25 and
+    1.25 S make every rotated magnitude 7, 4.5, 2.5 or 0 s, s = S / 64."""
+    x = torch.zeros(rows, 4096)
+    for r in range(rows):
+        S = (3 + 2 * r) * 2.0 ** -4
+        for i, v in ((5 + r, 3.5), (1030 + 3 * r, 2.25), (4000 - 7 * r, -1.25)):
+            x[r, i] = v * S
+    return x.to(torch.float16)
+
+
+@pytest.mark.parametrize("M,K", [(9, 64), (16, 576), (24, 8192), (160, 8064), (24, 14336), (300, 14336), (3, 28672), (40, 28672)])
+def test_quantize_act_on_ties(M, K):
+    x = _tie_rows(M, K)
+    ref = oracle.quantize_act(f16_bits(x), 1, 1.0)
+    q = x.numpy().astype(np.float64) / ref["scale"].view(np.float16).astype(np.float64)[:, None]
+    on = np.mean(np.abs(np.abs(q) % 1 - 0.5) < 1e-6)
+    assert on > 0.05 and np.max(np.abs(q)) < 7.5, "the inputs hold no ties"
+    xq, scale = rcp.rcp_quantize_act(x.to(DEV), 1, 1.0)
+    assert np.array_equal(f16_bits(scale), ref["scale"])
+    assert np.array_equal(xq.cpu().numpy(), ref["xq"])
+
+
+def test_quantize_act_on_ties_after_an_exact_rotation():
+    x = _rotated_ties(20)
+    ref = oracle.quantize_act(f16_bits(x), 4096, 1.0)
+    xq, scale = rcp.rcp_quantize_act(x.to(DEV), 4096, 1.0)
+    assert np.array_equal(f16_bits(scale), ref["scale"])
+    assert np.array_equal(xq.cpu().numpy(), ref["xq"])
+    assert len(np.unique(ref["xq"])) > 8
+
+
+@pytest.mark.parametrize("K", [64, 2048, 4096, 8192, 14336, 16384])
+def test_linear_on_ties(K):
+    """The quantizer inside the GEMV: one and two words per thread without rotation, and a whole token rotated exactly."""
+    N = 32
+    words = torch.randint(-2 ** 31, 2 ** 31 - 1, (N, K // 16), dtype=torch.int32, device=DEV)
+    lut = torch.ones(N, 4, dtype=torch.float16, device=DEV)
+    for x, B in [(_tie_rows(3, K)[r:r + 1], 1) for r in range(3)] + ([(_rotated_ties(2)[1:], 4096)] if K == 4096 else []):
+        assert rcp.rcp_linear_w2a4_launches(1, N, K, B) == 1
+        xq = torch.zeros(1, K // 2, dtype=torch.uint8, device=DEV)
+        scale = torch.zeros(1, dtype=torch.float16, device=DEV)
+        rcp.rcp_linear_w2a4(x.to(DEV), B, 1.0, words, lut, xq=xq, scale=scale)
+        ref = oracle.quantize_act(f16_bits(x), B, 1.0)
+        assert np.array_equal(f16_bits(scale), ref["scale"]) and np.array_equal(xq.cpu().numpy(), ref["xq"])
 
 
 @pytest.mark.parametrize("K,B", [(5120, 1024), (14336, 2048), (28672, 128), (28672, 4096)])
