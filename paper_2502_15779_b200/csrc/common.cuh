@@ -9,6 +9,14 @@ namespace rcp {
 constexpr int kMaxTokens = 16;   // skinny regime of the GEMV
 constexpr int kMaxK = 65536;
 
+// Loads of what the kernel in front may write (activations, their scales and digits, exported layers). Kernels here are
+// launched while that one still runs and wait for it with griddepcontrol.wait, so this data is not constant for their
+// lifetime. __ldg promises that it is, and the compiler moves such loads in front of the wait: a layer on the results of the
+// layer in front of it read those of an earlier pass. An ordinary load stays behind the wait; its latency (some 0.3 us from
+// L2 at worst: one token in a chain, 2048x2048 2.77 -> 2.87 us, 4096x4096 3.71 -> 4.05) is what the data costs.
+template <typename T>
+__device__ __forceinline__ T ld_input(const T* p) { return *p; }
+
 // dot products of four bytes: unsigned or signed bytes of a, signed bytes of b
 __device__ __forceinline__ void dp4a_u8s8(int& d, uint32_t a, uint32_t b) {
   asm("dp4a.u32.s32 %0, %1, %2, %0;" : "+r"(d) : "r"(a), "r"(b));

@@ -427,7 +427,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
                   const int j = (int)(((uint32_t)v * inv_box) >> 20), w = v - j * per_box;
                   const int col = w >> 4, lo = w & 3, hi = (w >> 2) & 3;
                   const int wx = (s * KS + j) * kChunkWords + (kRelabel ? 8 * hi + 2 * lo : 8 * lo + 2 * hi);   // first of the unit's two words
-                  if (wx < W) x[r] = __ldg(reinterpret_cast<const uint4*>(p.xq + (size_t)col * (p.K / 2)) + (wx >> 1));
+                  if (wx < W) x[r] = ld_input(reinterpret_cast<const uint4*>(p.xq + (size_t)col * (p.K / 2)) + (wx >> 1));
                 }
               }
             };
@@ -601,7 +601,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
       int tsum = 0;
 #pragma unroll
       for (int v4 = 0; v4 < 4; v4++) {
-        const uint4 x = gi < ngroups ? __ldg(src + v4) : make_uint4(0, 0, 0, 0);
+        const uint4 x = gi < ngroups ? ld_input(src + v4) : make_uint4(0, 0, 0, 0);
         const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
         for (int h = 0; h < 4; h++) {
@@ -621,7 +621,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
     for (int col = 0; col < M; col++) {
       int tsum = 0;
       for (int i = tid; i < nvec; i += kCWarps * 32) {
-        const uint4 x = __ldg(reinterpret_cast<const uint4*>(p.xq + (size_t)col * (p.K / 2)) + i);
+        const uint4 x = ld_input(reinterpret_cast<const uint4*>(p.xq + (size_t)col * (p.K / 2)) + i);
         const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
         for (int h = 0; h < 4; h++) {
@@ -659,7 +659,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
         for (int r = 0; r < 4; r++) {
           const int i = tid + r * (kCWarps * 32);
           xr[r] = make_uint4(0, 0, 0, 0);
-          if (i < nvec) xr[r] = __ldg(reinterpret_cast<const uint4*>(p.x) + i);
+          if (i < nvec) xr[r] = ld_input(reinterpret_cast<const uint4*>(p.x) + i);
           amax = split_amax8(xr[r], amax);
         }
         amax = __reduce_max_sync(0xffffffffu, amax);
@@ -693,7 +693,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
       }
     }
     float my_scale = 0.f;   // asked for now, stored when the activations are done
-    if (tid < M && !(A16 && p.x)) my_scale = A16 ? __ldg(p.unit + tid) : __half2float(__ldg(p.scale + tid));
+    if (tid < M && !(A16 && p.x)) my_scale = A16 ? ld_input(p.unit + tid) : __half2float(ld_input(p.scale + tid));
     const int W = p.K / 16;
     // A column is shared by act_parts warps (16 / columns, at least one); a warp takes every act_parts-th pair of chunks, a
     // lane one unit of two words in each: lo and hi say which. So nothing is worked out per unit but a bound, and
@@ -721,7 +721,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
         if (ch + i * ch_step < p.nchunk && wx + i * wx_step < W) {
           const uint4* const at = reinterpret_cast<const uint4*>(src + (size_t)i * wx_step * (A16 ? 16 : 8)) + w;
           if (A16 && p.x) x[w] = *at;   // planes made above
-          else x[w] = __ldg(at);
+          else x[w] = ld_input(at);
         }
       }
     };

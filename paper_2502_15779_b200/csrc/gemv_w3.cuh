@@ -275,8 +275,8 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
 #pragma unroll
     for (int h = 0; h < 2; h++) {
       const bool ok = row < p.N && u + h * unit_h < nunit;
-      d.a[h] = ok ? __ldg(reinterpret_cast<const uint4*>(p.words2) + e + h * unit_h) : make_uint4(0, 0, 0, 0);
-      d.z[h] = ok ? __ldg(reinterpret_cast<const uint2*>(p.words1) + e + h * unit_h) : make_uint2(0, 0);
+      d.a[h] = ok ? ld_input(reinterpret_cast<const uint4*>(p.words2) + e + h * unit_h) : make_uint4(0, 0, 0, 0);
+      d.z[h] = ok ? ld_input(reinterpret_cast<const uint2*>(p.words1) + e + h * unit_h) : make_uint2(0, 0);
     }
   };
   // Rows are dealt round-robin to all warps of the grid (one resident wave of CTAs). Launched with programmatic stream
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
   int tsum = 0;
   for (int w = tid; w < nit * 256; w += kW3Threads) {
     uint2 x = make_uint2(0, 0);
-    if (w < W) x = __ldg(reinterpret_cast<const uint2*>(p.xq) + w);   // 16 nibbles
+    if (w < W) x = ld_input(reinterpret_cast<const uint2*>(p.xq) + w);   // 16 nibbles
     // four nibbles at a time: nibble k of a register goes to byte k / 2 of e (k even) or o (k odd), is sign-extended
     // inside its byte, then the bytes are gathered by position (byte j of position pp = code 4 j + pp)
     const uint32_t e0 = w3_sext4x4(x.x & 0x0F0F0F0Fu), o0 = w3_sext4x4((x.x >> 4) & 0x0F0F0F0Fu);   // codes 0,2,4,6 / 1,3,5,7
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
       o[0] = make_int4(S[0], S[1], S[2], S[3]);
       o[1] = make_int4(S[4], S[5], S[6], S[7]);
     }
-    return w3_lut_dot(__ldg(p.lut + (size_t)row * ngrp + gi), S);
+    return w3_lut_dot(ld_input(p.lut + (size_t)row * ngrp + gi), S);
   };
   // Per-row grid: the rows first, first + warps, .. (cnt of them), one per lane, from their sums.
   auto finish_rows = [&](int first, int cnt) {
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(kW3Threads, 4) gemv_w3a4_kernel(const W3Params
       const int t[8] = {T0, lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z};
       int S[8];
       w3_percode(t, S);
-      p.y[row] = __float2half_rn(s * w3_lut_dot(__ldg(p.lut + row), S));
+      p.y[row] = __float2half_rn(s * w3_lut_dot(ld_input(p.lut + row), S));
       if constexpr (SDBG) {
         int4* o = reinterpret_cast<int4*>(p.S_out + (size_t)row * 8);
         o[0] = make_int4(S[0], S[1], S[2], S[3]);

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(1024) quantize_act_kernel(const QuantParams p)
 
   float v[8];
   if (mine) {
-    const uint4 raw = __ldg(reinterpret_cast<const uint4*>(xm + base));
+    const uint4 raw = ld_input(reinterpret_cast<const uint4*>(xm + base));
     const __half2* h2 = reinterpret_cast<const __half2*>(&raw);
 #pragma unroll
     for (int e = 0; e < 4; e++) {
@@ -408,8 +408,8 @@ __global__ void __launch_bounds__(NT, kFullRowsThreads / NT) quantize_act_full_r
   uint4 raw[2];
   auto fetch = [&](int m) {
     const uint4* const src = reinterpret_cast<const uint4*>(p.x + (size_t)m * (NT * 16)) + 2 * tid;
-    raw[0] = __ldg(src);
-    raw[1] = __ldg(src + 1);
+    raw[0] = ld_input(src);
+    raw[1] = ld_input(src + 1);
   };
   int par = 0;
   fetch(blockIdx.x);
@@ -536,12 +536,12 @@ __device__ __forceinline__ float rotate_full_token(const __half* x, float inv_sq
   {
     uint32_t raw[NP];
     if constexpr (E == 4) {
-      const uint2 r = __ldg(reinterpret_cast<const uint2*>(x) + tid);
+      const uint2 r = ld_input(reinterpret_cast<const uint2*>(x) + tid);
       raw[0] = r.x; raw[1] = r.y;
     } else {
 #pragma unroll
       for (int i = 0; i < E / 8; i++) {
-        const uint4 r = __ldg(reinterpret_cast<const uint4*>(x) + tid * (E / 8) + i);
+        const uint4 r = ld_input(reinterpret_cast<const uint4*>(x) + tid * (E / 8) + i);
         raw[4 * i] = r.x; raw[4 * i + 1] = r.y; raw[4 * i + 2] = r.z; raw[4 * i + 3] = r.w;
       }
     }
@@ -601,7 +601,7 @@ __device__ __forceinline__ float rotate_block_token(const __half* x, int W, int 
   for (int r = 0; r < NR; r++) {
     const int w = r * 512 + tid;
     raw[r][0] = raw[r][1] = make_uint4(0, 0, 0, 0);
-    if (w < W) { raw[r][0] = __ldg(reinterpret_cast<const uint4*>(x) + 2 * w); raw[r][1] = __ldg(reinterpret_cast<const uint4*>(x) + 2 * w + 1); }
+    if (w < W) { raw[r][0] = ld_input(reinterpret_cast<const uint4*>(x) + 2 * w); raw[r][1] = ld_input(reinterpret_cast<const uint4*>(x) + 2 * w + 1); }
   }
   float amax = 0.f;
 #pragma unroll

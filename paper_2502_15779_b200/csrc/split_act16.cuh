@@ -52,25 +52,23 @@ __device__ __forceinline__ void split_digits8(uint4 v, float mult, uint32_t (&ou
 // out its digits; each of them looks for the largest magnitude itself, which is a load and a few maxima per eight
 // elements, where the digits are some 200 instructions. Latency bound: with one CTA per token the whole call took 17.6 us at
 // 4096x14336 with two tokens and 34.8 at 8192x28672 with one; now 15.1 and 30.3.
-__global__ void __launch_bounds__(kSplitThreads) split_act16_kernel(const __half* __restrict__ x, int K, int parts,
-                                                                     int8_t* __restrict__ digits,
-                                                                     float* __restrict__ unit) {
+__global__ void __launch_bounds__(kSplitThreads) split_act16_kernel(const __half* x, int K, int parts,
+                                                                     int8_t* digits, float* unit) {
   __shared__ unsigned s_max[kSplitThreads / 32];
   const int m = blockIdx.x / parts, part = blockIdx.x - m * parts, tid = threadIdx.x;
   const uint4* const xv = reinterpret_cast<const uint4*>(x + (size_t)m * K);
   const int nvec = K / 8;
-  asm volatile("griddepcontrol.launch_dependents;");
   asm volatile("griddepcontrol.launch_dependents;");
   // the token on its way to L2 (nothing stale: that is where the kernel in front would write it)
   if (part == 0 && tid * 64 < K) asm volatile("prefetch.global.L2 [%0];" ::"l"(x + (size_t)m * K + tid * 64));
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // this part's vectors, and the first of them asked for at once
   const int v0 = (int)((long long)nvec * part / parts), v1 = (int)((long long)nvec * (part + 1) / parts);
-  const uint4 first = v0 + tid < v1 ? __ldg(xv + v0 + tid) : make_uint4(0, 0, 0, 0);
+  const uint4 first = v0 + tid < v1 ? ld_input(xv + v0 + tid) : make_uint4(0, 0, 0, 0);
   // largest magnitude: the bit patterns of finite fp16 magnitudes order like the values
   unsigned amax = 0;
 #pragma unroll 4
-  for (int i = tid; i < nvec; i += kSplitThreads) amax = split_amax8(__ldg(xv + i), amax);
+  for (int i = tid; i < nvec; i += kSplitThreads) amax = split_amax8(ld_input(xv + i), amax);
   amax = __reduce_max_sync(0xffffffffu, amax);
   if ((tid & 31) == 0) s_max[tid >> 5] = amax;
   __syncthreads();
@@ -81,7 +79,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_act16_kernel(const __half
   int8_t* const dg = digits + (size_t)m * 4 * K;
   for (int i = v0 + tid; i < v1; i += kSplitThreads) {
     uint32_t out[4][2];
-    split_digits8(i == v0 + tid ? first : __ldg(xv + i), mult, out);
+    split_digits8(i == v0 + tid ? first : ld_input(xv + i), mult, out);
 #pragma unroll
     for (int d = 0; d < 4; d++)
       *reinterpret_cast<uint2*>(dg + (size_t)d * K + (size_t)i * 8) = make_uint2(out[d][0], out[d][1]);

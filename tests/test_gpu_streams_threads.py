@@ -150,3 +150,56 @@ def test_back_to_back_calls_that_share_their_buffers(M, group):
         assert torch.equal(o.view(torch.int16), w.view(torch.int16))
     for _, _, ws in layers:
         assert int(ws.abs().max()) == 0
+
+
+@pytest.mark.parametrize("form", ["linear", "grouped", "separate", "w2a16", "w3a4"])
+@pytest.mark.parametrize("K,B,M", [(2048, 2048, 1), (4096, 4096, 1), (8192, 8192, 1), (4096, 128, 1), (11008, 128, 1), (1024, 1024, 1),
+                                   (28672, 128, 1), (2048, 2048, 2), (4096, 4096, 8), (4096, 4096, 16), (8192, 8192, 4), (5184, 64, 3),
+                                   (14336, 128, 2), (1024, 1024, 8)])
+def test_a_layer_on_the_results_of_the_layer_in_front(K, B, M, form):
+    """Two layers, the second one's activations being the first one's results, with nothing in between: the second call's
+    first kernel is started early and has to wait for them. The results change from pass to pass, so that a value read
+    too early is the one of another pass."""
+    if form == "grouped" and K % 128:
+        pytest.skip("group does not divide K")
+    group = 128 if form == "grouped" else 0
+    g = torch.Generator(device=DEV).manual_seed(K + M)
+    words = [torch.randint(-2 ** 31, 2 ** 31 - 1, (n, K // 16), generator=g, dtype=torch.int32, device=DEV) for n in (K, 512)]
+    top = [torch.randint(-2 ** 31, 2 ** 31 - 1, (n, K // 32), generator=g, dtype=torch.int32, device=DEV) for n in (K, 512)]
+    levels = 8 if form == "w3a4" else 4
+    luts = [(torch.randn(*((n, K // group, levels) if group else (n, levels)), generator=g, device=DEV) * 0.02).half() for n in (K, 512)]
+    ws = [rcp.make_workspace(M, n, K, DEV) for n in (K, 512)]
+    xs = [synth.make_activations(M, K, 500 + i, device=DEV) * (1 + i % 3) for i in range(8)]
+    h = torch.zeros(M, K, dtype=torch.float16, device=DEV)
+    ys = torch.zeros(len(xs), M, 512, dtype=torch.float16, device=DEV)
+    extra = [dict(digits=torch.empty(M, 4, K, dtype=torch.int8, device=DEV), unit=torch.empty(M, 4, device=DEV)) if form == "w2a16" else
+             dict(xq=torch.empty(M, K // 2, dtype=torch.uint8, device=DEV), scale=torch.empty(M, dtype=torch.float16, device=DEV)) for _ in range(2)]
+
+    def layer(i, x, y):
+        if form == "w2a16":
+            rcp.rcp_gemv_w2a16(words[i], luts[i], x, y=y, workspace=ws[i], **extra[i])
+        elif form == "w3a4":
+            rcp.rcp_quantize_act(x, B, 1.0, **extra[i])
+            rcp.rcp_gemv_w3a4(words[i], top[i], luts[i], y=y, **extra[i])
+        elif form == "separate":
+            rcp.rcp_quantize_act(x, B, 1.0, **extra[i])
+            rcp.rcp_gemv_w2a4(words[i], luts[i], y=y, workspace=ws[i], **extra[i])
+        else:
+            rcp.rcp_linear_w2a4(x, B, 1.0, words[i], luts[i], group=group, y=y, workspace=ws[i], **extra[i])
+
+    for x, y in zip(xs, ys):
+        layer(0, x, h)
+        torch.cuda.synchronize()
+        layer(1, h, y)
+        torch.cuda.synchronize()
+    want = ys.clone()
+    assert torch.isfinite(want).all() and not torch.equal(want[0], want[1])
+    for rep in range(10):
+        ys.zero_()
+        h.fill_(rep)
+        torch.cuda.synchronize()
+        for x, y in zip(xs, ys):
+            layer(0, x, h)
+            layer(1, h, y)
+        torch.cuda.synchronize()
+        assert torch.equal(ys.view(torch.int16), want.view(torch.int16)), f"repetition {rep}"
