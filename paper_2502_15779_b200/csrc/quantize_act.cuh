@@ -341,8 +341,10 @@ __global__ void __launch_bounds__(T_MAX, 1024 / T_MAX) quantize_act_rows_kernel(
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  // words beyond the token: zeros, which no copy ever lands on (a store and a later asynchronous copy are not ordered)
 #pragma unroll
-  for (int i = 0; i < 2 * R; i++) s_next[i * T + tid] = make_uint4(0, 0, 0, 0);   // (threads beyond the token keep zeros)
+  for (int r = 0; r < R; r++)
+    if (r * T + tid >= W) s_next[2 * r * T + tid] = s_next[(2 * r + 1) * T + tid] = make_uint4(0, 0, 0, 0);
   int par = 0;
   fetch(blockIdx.x);
   for (int m = blockIdx.x; m < M; m += gridDim.x, par ^= 1) {
