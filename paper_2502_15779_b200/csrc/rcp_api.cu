@@ -686,9 +686,20 @@ int launch_w3(const rcp::W3Params& wp, size_t smem, cudaStream_t st) {
   auto kern = rcp::gemv_w3a4_kernel<GRP, SDBG, HALF>;
   RCP_CUDA(set_max_smem(kern, rcp::kMaxK + 128, mu, attr_set));
   // One wave of resident CTAs, rows dealt round-robin to their warps (measured: CTAs beyond the resident wave,
-  // and warps sharing a row along K, both cost more than the evener load returns). CTAs per SM: four by registers, or
-  // what the expanded activations (and some 9 KB beside them, 1 KB of it the system's) leave of 228 KB.
-  const int per_sm = std::max<int>(1, std::min<size_t>(4, 228 * 1024 / (smem + 9472 + 1024)));
+  // and warps sharing a row along K, both cost more than the evener load returns). How many that is depends on the kernel
+  // and on smem, a multiple of 4096 bytes up to kMaxK: asked once for each.
+  static int resident[kMaxDevices][rcp::kMaxK / 4096 + 1] = {};
+  int dev = 0, per_sm = 0;
+  RCP_CUDA(cudaGetDevice(&dev));   // (below kMaxDevices: set_max_smem has looked)
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    int& known = resident[dev][smem / 4096];
+    if (!known) {
+      RCP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&known, kern, rcp::kW3Threads, smem));
+      known = std::max(known, 1);
+    }
+    per_sm = known;
+  }
   const int warps_per_cta = rcp::kW3Threads / 32;
   const int grid = std::min(sm_count() * per_sm, (wp.N + warps_per_cta - 1) / warps_per_cta);
   RCP_CUDA(launch_overlapped(kern, dim3(grid), dim3(rcp::kW3Threads), smem, st, wp));
