@@ -9,8 +9,10 @@
 // activations. Twelve masked words (three planes x four positions) cover a word; each costs one
 // LOP3 on the 64-lane/clk logic pipe, the scarce resource. The products go to int8 mma.sync
 // (16 rows x 32 bytes per instruction, tokens in the n dimension) and/or to dp4a on the FMA pipe.
-// Even positions meet activations pre-multiplied by 4, so positions {0,1} and {2,3} share an
-// accumulator (scaled by 4 and 64, twice that for the planes masked at the b1 bit).
+// Even positions meet activations pre-multiplied by 4 << kQ, odd ones by 1 << kQ (kQ: 2, or 0 where the
+// quantizer is inside and for digit columns), so positions {0,1} and {2,3} share an accumulator (scaled
+// by 4 << kQ and 64 << kQ, twice that for the planes masked at the b1 bit). Largest value
+// of an accumulator: K = 65536, |q| = 8, half of the codes at 4096 each: 2^27.
 //
 // Data movement. The packed weights are the only large stream. One persistent CTA per SM: a
 // producer thread streams boxes of rows x 128 bytes into a shared-memory ring with TMA
@@ -239,7 +241,7 @@ __global__ void wait_timeout_kernel(int32_t* status, uint32_t polls) {
 // (chunk, i, pr) and token column there are two 16-byte halves per lane slice t; half h holds
 // positions 2h and 2h+1:
 //   { q[p=2h][word x], q[2h][word y], q[2h+1][word x], q[2h+1][word y] },  byte j of q[p][w] =
-//   activation of code 16 w + 4 j + p, times 4 when p is even.
+//   activation of code 16 w + 4 j + p, times 4 << kQ when p is even, times 1 << kQ when it is odd.
 // Byte address of (chunk, i, pr, half, col, t): ((((chunk*2 + i)*2 + pr)*2 + half)*ncol + col)*64 + t*16.
 
 // MODE  kModeMma: all three planes on the tensor cores; kModeHybrid: b0 and b1 planes on the tensor
@@ -306,7 +308,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   int* const s_red = reinterpret_cast<int*>(gen + p.off_red);           // [2][8 groups][16 rows][M][3]
   float* const s_redf = reinterpret_cast<float*>(gen + p.off_red);      // GRP: a slot per warp, [token pairs][32], see red_index
   const int red_plane = ((M + 1) >> 1) * 32;
-  // tensor-core GRP: the same area as floats [4 nchunk][Mp], 8 x the sum of q of a group, tokens padded to even
+  // tensor-core GRP: the same area as floats [4 nchunk][Mp], (8 << kQ) x the sum of q of a group, tokens padded to even
   float* const s_T0f = reinterpret_cast<float*>(gen + p.off_T0c);
   const int ng4 = 4 * p.nchunk;
   const int Mp = (M + 1) & ~1;
@@ -481,7 +483,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
   }
 
   // What needs nothing of the kernel before this one: clearing the sums, and x in fp16 on its way to L2 if it is not there
-  // (the L2 is where a kernel in front would write it, so this can fetch nothing stale).
+  // (the L2 is where a kernel in front would write it, so this can fetch nothing stale); a line per CTA, 9472 elements.
   if constexpr (!GRP)
     for (int i = tid; i < 2 * 8 * 16 * M * 3; i += kCWarps * 32) s_red[i] = 0;
   if constexpr (FQ != 0 || A16)
@@ -592,7 +594,7 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
     }
   } else if constexpr (SB && GRP) {
     // Streamed activations, group-wise grid: the sum of q of every (token, group of 128) is needed up front, as
-    // 8 x the sum in fp32 (what the finish works with). A group is 64 bytes of packed activations.
+    // (8 << kQ) x the sum in fp32 (what the finish works with). A group is 64 bytes of packed activations.
     // (the last chunk may reach beyond K: its missing groups get a sum of zero, they meet a grid of zeros)
     const int ngroups = p.K / 128;
     for (int i = tid; i < M * ng4; i += kCWarps * 32) {
@@ -1052,8 +1054,9 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
             else mma_u8s8(accM[f][0], au0[f], av0[f], au1[f], av1[f], bM[pp][0], bM[pp][1]);
           }
         }
-        // The accumulators hold 4 T1, 8 T2 and 8 T3. Everything below works on 8 x the sums, in fp32 (small
-        // integers: exact); the 1/8 goes into the final scale. With the levels L0..L3 of the (row, group),
+        // The accumulators hold 4 T1, 8 T2 and 8 T3, all << kQ. Everything below works on (8 << kQ) x the sums, in fp32
+        // (integers up to 32 x 128 x 8 = 2^15, far below the 2^22 of small_int_to_float: exact); kGrpScale takes the factor out
+        // again. With the levels L0..L3 of the (row, group) and kQ = 0,
         //   8 y = L0 (8 T0) + 2 (L1 - L0) (4 T1) + (L2 - L0) (8 T2) + ((L3 - L1) - (L2 - L0)) (8 T3):
         // the coefficients are made once per row and serve all its tokens.
         const int gi = ch * 4 + j;
@@ -1073,9 +1076,9 @@ gemv_stream_kernel(const __grid_constant__ GemvMaps maps, const GemvParams p) {
         }
 #pragma unroll
         for (int r = 0; r < 4; r++) {
-          const float F1 = small_int_to_float(accM[0][0][r]);   // 4 T1
-          const float F2 = small_int_to_float(accM[1][0][r]);   // 8 T2
-          const float F3 = small_int_to_float(accM[2][0][r]);   // 8 T3
+          const float F1 = small_int_to_float(accM[0][0][r]);   // 4 T1 << kQ
+          const float F2 = small_int_to_float(accM[1][0][r]);   // 8 T2 << kQ
+          const float F3 = small_int_to_float(accM[2][0][r]);   // 8 T3 << kQ
           const float (&c)[4] = cf[r >> 1];
           yacc[r] = fmaf(c[0], (r & 1) ? t0.y : t0.x, fmaf(c[1], F1, fmaf(c[2], F2, fmaf(c[3], F3, yacc[r]))));
           if constexpr (SDBG) {

@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(1024) quantize_act_kernel(const QuantParams p)
 // adds, products and the rounding work on pairs (the two-wide fp32 instructions round each half like the scalar ones)
 // and the clamp of the rounding is left out where it cannot act. Same operations on the same operands in the same
 // order as above: bit-identical results. 2048 tokens, us before (cluster, or one CTA of 512 threads with four barriers)
-// and now, memory floor: K = 4096 27.1, 10.6, 3.3; K = 8192 33.8, 21.5, 6.5; K = 14336 in blocks of 128 78.4, 25.5, 11.4.
+// and now, memory floor: K = 4096 27.1, 10.8, 3.3; K = 8192 33.8, 21.4, 6.5; K = 14336 in blocks of 128 78.4, 25.8, 11.4.
 // Fewer barriers also make it the faster form for one token (K = 4096: 2.8 -> 1.8 us).
 
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }

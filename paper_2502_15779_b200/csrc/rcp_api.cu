@@ -577,11 +577,11 @@ int static_scratch_address(void** out) {
 }
 
 // Whether one CTA takes a whole token (quantize_act_rows_kernel, quantize_act_full_rows_kernel) or a cluster shares it.
-// Measured on B200, cluster -> one CTA, us a call. One block over the token: one CTA at any count (K = 4096: 2.8 -> 1.8
-// for one token, 27 -> 12 for 2048). Blocks inside a warp: one CTA up to K = 8192 (2560: 1.95 -> 1.61 and 9.3 -> 6.7;
-// 8064: 2.8 -> 2.1 and 38 -> 19), above that once the tokens fill the GPU better than eight CTAs each would: 11008 and
-// 14336 even at 24 tokens (14336: 3.4 -> 3.6 at 16, 4.25 -> 3.5 at 32, 78 -> 28 at 2048), 28672 at 40 (5.2 -> 5.7
-// at 32, 8.0 -> 5.8 at 64, 178 -> 60 at 2048).
+// Measured on B200, cluster -> one CTA, us a call in a chain of them. One block over the token: one CTA at any count
+// (K = 4096: 2.7 -> 1.7 for one token, 26 -> 10.8 for 2048). Blocks inside a warp: one CTA up to K = 8192 (8064: 2.7 -> 2.0
+// and 34 -> 14.6), above that once the tokens fill the GPU better than eight CTAs each would: 11008 and 14336 even at
+// 24 tokens (14336: 2.8 -> 3.6 at 16, 4.2 -> 3.2 at 32, 74 -> 25.8 at 2048), 28672 at 40 (4.7 -> 5.7 at 32, 8.0 -> 5.2
+// at 64, 177 -> 50.5 at 2048).
 bool rows_form(int M, int K, int B) {
   if (B > 512) return B == K && (K == 2048 || K == 4096 || K == 8192);
   return K <= 8192 || (K <= 16384 && M >= 24) || (K <= 32768 && M >= 40);
@@ -620,7 +620,7 @@ int launch_quantize_rows(const rcp::QuantParams& qp, int M, cudaStream_t st) {
   if (qp.B == 128) {
     if (W <= 512) return launch_block_rows<1, 512, 128>(qp, M, st);
     // up to one token per SM a thread per word (14336, 96 tokens: 3.6 us against 4.9 with two words per thread), beyond
-    // that two smaller CTAs per SM (2048 tokens: 28.5 against 30.0)
+    // that two smaller CTAs per SM (2048 tokens, with an earlier form of the kernel: 28.5 against 30.0)
     if (W <= 1024 && M <= sm_count()) return launch_block_rows<1, 1024, 128>(qp, M, st);
     if (W <= 896) return launch_block_rows<2, 448, 128>(qp, M, st);
     return launch_block_rows<2, 1024, 128>(qp, M, st);
@@ -781,8 +781,8 @@ int rcp_gemv_w3a4(const uint32_t* words2, const uint32_t* words1, const void* lu
       (reinterpret_cast<uintptr_t>(y_f16) & 1u) || (reinterpret_cast<uintptr_t>(scale_f16) & 1u))
     return RCP_ERR_ALIGN;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // The last lane step of a row (64 units of 64 codes) is at most half full, and the row so short that leaving the empty half
-  // out returns more than the form's spills cost (half of one step in nit against 8 %: K = 14336, four steps, 15.1 -> 13.9 us)
+  // The last lane step of a row (64 units of 64 codes) is at most half full, and the row has so few steps that leaving half of
+  // one out returns more than the 8 % that the form costs by its spills (4096x14336, an eighth of four steps: 15.1 -> 13.9 us)
   const bool half = (K / 64 - 1) % 64 < 32 && K <= 5 * 4096;
   const int ngrp = group ? K / 128 : 1;
   const size_t smem = (size_t)((K / 64 + 63) / 64) * 4096;   // expanded activations, K padded to whole lane steps of 4096 codes

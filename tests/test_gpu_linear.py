@@ -1,5 +1,5 @@
-"""GPU parity of rcp_linear_w2a4 (activation quantization and LUT GEMV in one call; one kernel for one
-or two tokens) against the CPU oracle: xq and scale bit for bit, y within the GEMV's tolerance."""
+"""GPU parity of rcp_linear_w2a4 (activation quantization and LUT GEMV in one call; one kernel for most one-token
+shapes) against the CPU oracle: xq and scale bit for bit, y within the GEMV's tolerance."""
 import numpy as np
 import pytest
 import torch
@@ -50,8 +50,8 @@ def _check(N, K, B, M, group, clip, seed, kind="uniform", rows=None, staging=Tru
 
 
 CASES = [
-    # N, K, B, M. One token of 4096 or 8192 under one block takes the single kernel (several row counts:
-    # rounds, leftover phases, ragged tail); everything else the two kernels
+    # N, K, B, M. One token under one block of 2048, 4096 or 8192, or in blocks of at most 512 with K <= 16384, takes the
+    # single kernel (several row counts: rounds, leftover phases, ragged tail); everything else the two kernels
     (40, 64, 1, 1), (40, 64, 64, 2), (100, 256, 16, 1), (33, 512, 128, 2), (64, 512, 512, 1), (129, 1024, 1024, 1),
     (300, 2048, 2048, 1), (300, 2048, 2048, 2), (256, 4096, 4096, 1), (77, 8192, 8192, 2), (500, 8192, 128, 1),
     (77, 8192, 8192, 1), (2500, 8192, 8192, 1), (4097, 4096, 4096, 1), (1, 4096, 4096, 1), (5000, 8192, 8192, 1),
