@@ -204,9 +204,9 @@ __global__ void __launch_bounds__(1024) quantize_act_kernel(const QuantParams p)
 // One CTA per token. The cluster kernel above shares a token out to get at its latency; with many tokens (the
 // activations of a prompt) most of its threads wait at barriers or for the cluster while little else is resident. Here
 // a persistent CTA takes token after token, one thread per word (16 consecutive elements) or two, the next token's
-// activations already on their way, several CTAs per SM, so that one computes while another waits. That is bound by
-// instruction issue (17 to 19 warp instructions per 32 elements against 2.5 bytes per element of traffic), so
-// adds, products and the rounding work on pairs (the two-wide fp32 instructions round each half like the scalar ones)
+// activations already on their way, several CTAs per SM, so that one computes while another waits. Nothing is full then:
+// issue slots and shared-memory pipe are half busy (16 to 23 warp instructions per 32 elements) with the 1024 threads per SM
+// that the registers leave, the rest is latency between exchanges and barriers. Fewer instructions shorten it: adds, products and the rounding work on pairs (the two-wide fp32 instructions round each half like the scalar ones)
 // and the clamp of the rounding is left out where it cannot act. Same operations on the same operands in the same
 // order as above: bit-identical results. 2048 tokens, us before (cluster, or one CTA of 512 threads with four barriers)
 // and now, memory floor: K = 4096 27.1, 10.8, 3.3; K = 8192 33.8, 21.4, 6.5; K = 14336 in blocks of 128 78.4, 25.8, 11.4.

@@ -334,7 +334,7 @@ struct SplitAct {
 
 // Shapes the in-kernel quantizer takes: one token under one rotation block of 2048, 4096 or 8192 elements, or in blocks
 // of at most 512 with K up to 16384. Measured on B200, us a call in a chain of calls, cold weights, two kernels -> one:
-// 2048x2048 3.95 -> 2.74, 4096x4096 5.4 -> 3.9, 57344x8192 33.4 -> 31.6, 333x5184 4.6 -> 3.6, 4096x14336 9.6 -> 8.4.
+// 2048x2048 3.8 -> 2.9, 4096x4096 5.0 -> 4.05, 57344x8192 32.6 -> 30.7, 333x5184 4.5 -> 3.5, 4096x14336 8.95 -> 8.0.
 // At K = 28672 (four words per thread) the stand-alone quantizer's cluster of eight CTAs is faster than all CTAs doing
 // the whole token (8192x28672 21.6 -> 22.3), and two tokens are twice the serial work.
 bool full_block(int K, int B) { return B == K && (K == 2048 || K == 4096 || K == 8192); }
@@ -505,8 +505,8 @@ int launch_stream_passes(int mode, int cap, const uint32_t* words, const void* l
   // Where the launch would have to go through K in more than four parts (several tokens, a very long K), the form that
   // streams the activations beside the weights is faster: it expands them once per phase, but chunk by chunk among the mask
   // arithmetic, where parts pay a barrier, a fill of the ring's first stage and a set of parked sums each. Measured at eight
-  // tokens, parts against streamed: 8192x28672 (three) 30.3 and 32.2 us, 8192x40960 (four) 39.8 and 43.6, 8192x65536 (six)
-  // 67.2 and 58.3.
+  // tokens, parts against streamed: 8192x28672 (three) 28.7 and 31.6 us, 8192x40960 (four) 37.8 and 42.9, 8192x65536 (six)
+  // 67.2 and 57.3.
   if (mode == rcp::kModeMma && !grouped && nsplit > 4 && mp == std::min(M, 8)) {
     const StreamPlan sp = make_plan(mp, N, K, sm_count(), false, 0, 1, true);
     if (sp.stages >= 3 && sp.smem <= kSmemMax) {
