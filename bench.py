@@ -724,7 +724,7 @@ def main():
            "vs_baseline": None, "dtype": "int32", "data": "synthetic",
            "config": {"workload": workload_name(cfg, M),
                       "step": "per linear: rcp_linear_w2a4 (activation quantization + LUT GEMV: one kernel for one "
-                              "token where that is faster (qkv, o and gate_up here), else rcp_quantize_act then "
+                              "token where that is faster, else rcp_quantize_act then "
                               "rcp_gemv_w2a4), replayed from a CUDA graph",
                       "cold_l2": f"{copies} distinct weight copies in rotation ({copies * wbytes / 1e6:.0f} MB > 2x L2 "
                                  f"of {L2 / 1e6:.0f} MB)",
