@@ -80,7 +80,8 @@ int rcp_quantize_act(const void* x_f16, int M, int K, int had_block, float clip_
 
 /*
  * Kernel variants of the LUT GEMV (all compute the same result).
- *   RCP_GEMV_AUTO    library picks (as measured on B200): DP4A for one token, MMA_ONLY otherwise.
+ *   RCP_GEMV_AUTO    library picks (as measured on B200): UMMA for large layers (how large depends on M), otherwise DP4A
+ *                    for one token and MMA_ONLY for more.
  *   RCP_GEMV_SIMPLE  one warp per output row, scalar decode; also the variant behind S_dbg.
  *   RCP_GEMV_DP4A    streaming kernel, CUDA cores only: masked code planes times int8 activations
  *                    with dp4a, two tokens per launch.
@@ -97,11 +98,14 @@ int rcp_quantize_act(const void* x_f16, int M, int K, int had_block, float clip_
  *                    ring stage carries the int8 activations of the chunks of K its boxes cover, written by a
  *                    warp of its own ahead of the consumers. Nothing is expanded up front, K never has to be
  *                    gone through in parts, and one launch takes up to sixteen tokens whatever K is.
+ *   RCP_GEMV_UMMA    the weights' bits, moved to the top of a byte, as the A operand of tcgen05.mma in tensor memory, read as
+ *                    unsigned, signed and e4m3 numbers; up to sixteen tokens per launch, K in parts where their activations
+ *                    do not fit in shared memory and the rows are one tile per CTA (fewer tokens per launch otherwise).
  * The streaming kernel: persistent CTAs, weights through a TMA/mbarrier shared-memory ring, 16-row
  * groups owned by warps, no exchange between CTAs.
  */
 enum { RCP_GEMV_AUTO = 0, RCP_GEMV_SIMPLE = 1, RCP_GEMV_DP4A = 2, RCP_GEMV_MMA = 3, RCP_GEMV_MMA_ONLY = 4,
-       RCP_GEMV_MMA_STREAM = 5 };
+       RCP_GEMV_MMA_STREAM = 5, RCP_GEMV_UMMA = 6 };
 
 /*
  * Weight-only form of the LUT GEMV (Section 5, the W2-only setting of Table "W2_inference": the codes

@@ -11,6 +11,7 @@
 #include "common.cuh"
 #include "gemv_simple.cuh"
 #include "gemv_stream.cuh"
+#include "gemv_umma.cuh"
 #include "gemv_w3.cuh"
 #include "ldp_export.cuh"
 #include "split_act16.cuh"
@@ -238,6 +239,173 @@ EncodeTiledFn encode_tiled_fn() {
 
 constexpr int kMaxDevices = 64;
 
+// Tensor maps of boxes of 16 gpcs[i] rows x 128 bytes (those with a count of 0 repeat the first). Encoding one costs the
+// host about a microsecond, so the maps of the last few (weights, shape, boxes) combinations are remembered per thread.
+int phase_maps(const uint32_t* words, int N, int K, int nphase, const int* gpcs, const rcp::GemvMaps** out) {   // gpcs [kMaxPhases]
+  struct MapKey { const void* words; int N, K, nphase, gpc[rcp::kMaxPhases]; };
+  struct MapSlot { MapKey key; rcp::GemvMaps maps; bool used; };
+  constexpr int kMapSlots = 16;
+  thread_local MapSlot map_cache[kMapSlots] = {};
+  thread_local int map_next = 0;
+  MapKey key = {};
+  key.words = words; key.N = N; key.K = K; key.nphase = nphase;
+  for (int i = 0; i < rcp::kMaxPhases; i++) key.gpc[i] = gpcs[i];
+  for (int i = 0; i < kMapSlots; i++)
+    if (map_cache[i].used && std::memcmp(&map_cache[i].key, &key, sizeof(MapKey)) == 0) { *out = &map_cache[i].maps; return RCP_OK; }
+  EncodeTiledFn enc = encode_tiled_fn();
+  if (!enc) return cuda_fail(cudaErrorNotSupported);
+  MapSlot& slot = map_cache[map_next];
+  map_next = (map_next + 1) % kMapSlots;
+  slot.used = false;
+  const cuuint64_t gdim[2] = {(cuuint64_t)(K / 16), (cuuint64_t)N};
+  const cuuint64_t gstride[1] = {(cuuint64_t)(K / 4)};
+  const cuuint32_t estr[2] = {1, 1};
+  for (int i = 0; i < rcp::kMaxPhases; i++) {
+    if (gpcs[i] < 1 && i > 0) { slot.maps.m[i] = slot.maps.m[0]; continue; }
+    const int gpc = std::max(1, gpcs[i]);
+    const cuuint32_t box[2] = {(cuuint32_t)rcp::kChunkWords, (cuuint32_t)(16 * gpc)};
+    const CUresult r = enc(&slot.maps.m[i], CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t*>(words), gdim,
+                           gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return cuda_fail(cudaErrorInvalidValue);
+  }
+  slot.key = key;
+  slot.used = true;
+  *out = &slot.maps;
+  return RCP_OK;
+}
+
+// ---------------------------------------------------------------------------------------------
+// GEMV on tcgen05: launch plan.
+struct UmmaPlan {
+  int nchunk, nphase, grid, kpl, lg_kpl, bgroup, bstep, bhalf, lg_m2, slots, dcols, nbuf, stages, helpers;
+  rcp::UmmaPhase phase[rcp::kMaxPhases];
+  int part_chunks;   // nchunk (rounded up to kpl): all of K at once
+  long long clocks;  // estimate of its items
+  int off_bar, off_misc, off_red, off_bs, off_qbuf, red_bytes, bs_bytes;
+  size_t smem;
+};
+
+// columns of the instruction for kp chunks side by side: a column per token and one of ones for each
+int umma_columns(int M, int kp) {
+  const int n = kp * (M + 1);
+  return n <= 8 ? 8 : (n + 15) / 16 * 16;
+}
+int floor_pow2(int v) { int p = 1; while (2 * p <= v) p *= 2; return p; }
+
+// stages 0: does not fit. qbuf: bytes of scratch for the quantizer inside.
+//   An item takes the longest of: 16 KB of weights for every SM from HBM, 720 clocks (a part of that where fewer lanes are in
+// use); its 48 instructions, 600 clocks up to 16 columns, 24 a column from there on; a slot's turn, 860 clocks where the
+// accumulators (three times 48 columns) leave room for two slots only. Columns buy lanes (kp chunks side by side), which is
+// what short or few rows need; up to 32 or up to 48 of them, whichever comes out cheaper.
+UmmaPlan umma_plan_for(int M, int N, int K, int sms, size_t qbuf, int max_cols, bool parts, long long* total) {
+  UmmaPlan pl = {};
+  pl.grid = sms;
+  pl.nchunk = (K / 16 + rcp::kChunkWords - 1) / rcp::kChunkWords;
+  int kp_cap = 8;
+  while (kp_cap > 1 && (umma_columns(M, kp_cap) > max_cols || kp_cap >= 2 * pl.nchunk)) kp_cap /= 2;
+  auto kp_of = [&](int g) { return std::min(kp_cap, floor_pow2(8 / g)); };
+  auto items_of = [&](int g) { return (pl.nchunk + kp_of(g) - 1) / kp_of(g); };
+  auto cost_of = [&](int g) {
+    const int ncol = umma_columns(M, kp_of(g));
+    return (long long)items_of(g) * std::max(std::max(720 * g * kp_of(g) / 8, max_cols > 32 ? 860 : 600), 24 * ncol) + 400;
+  };
+  const int groups = (N + 15) / 16, per_round = 8 * sms, rounds = groups / per_round, left0 = groups - rounds * per_round;
+  *total = 0;
+  if (parts && groups > per_round) return pl;   // K in parts: one tile per CTA
+  // the groups left over from the rounds of eight per CTA: phases of 4, 2, 1 groups per CTA, and one last for what remains
+  int best_mask = 0;
+  long long best = -1;
+  for (int mask = 0; mask < (parts ? 1 : 8); mask++) {
+    int left = left0;
+    long long cost = 0;
+    bool ok = true;
+    for (int i = 0; i < 3; i++) {
+      if (!(mask >> i & 1)) continue;
+      const int g = 4 >> i;
+      if (left < g * sms) { ok = false; break; }
+      left -= g * sms;
+      cost += cost_of(g);
+    }
+    if (!ok) continue;
+    if (left > 0) cost += cost_of((left + sms - 1) / sms);
+    if (best < 0 || cost < best) { best = cost; best_mask = mask; }
+  }
+  *total = pl.clocks = best + (rounds > 0 ? rounds * cost_of(8) : 0);
+  int first = 0;
+  auto add = [&](int g, int n, int ncta, int reps) {
+    rcp::UmmaPhase& ph = pl.phase[pl.nphase++];
+    ph.gpc = g; ph.first = first; ph.total = n; ph.ncta = ncta; ph.reps = reps;
+    ph.q = n / ncta; ph.r = n % ncta;
+    ph.kp = kp_of(g); ph.items = items_of(g); ph.ncol = umma_columns(M, ph.kp);
+    ph.inv_rows = (65536 + 16 * g - 1) / (16 * g);
+    first += n * reps;
+  };
+  int left = left0;
+  for (int i = 0; i < 3; i++) {
+    if (!(best_mask >> i & 1)) continue;
+    const int g = 4 >> i;
+    add(g, g * sms, sms, 1);
+    left -= g * sms;
+  }
+  if (left > 0) {
+    const int ncta = std::min(left, sms);
+    add((left + ncta - 1) / ncta, left, ncta, 1);
+  }
+  if (rounds > 0) add(8, per_round, sms, rounds);
+  pl.kpl = 1;
+  int ncol = 8;
+  for (int i = 0; i < pl.nphase; i++) { pl.kpl = std::max(pl.kpl, pl.phase[i].kp); ncol = std::max(ncol, pl.phase[i].ncol); }
+  while ((1 << pl.lg_kpl) < pl.kpl) pl.lg_kpl++;
+  while ((1 << pl.lg_m2) < M) pl.lg_m2++;
+  pl.dcols = ncol;
+  pl.slots = 3 * ncol <= 128 ? 3 : 2;
+  pl.nbuf = std::min(rcp::kUMaxBuf, (512 - 128 * pl.slots) / (3 * ncol));
+  // activations: odd strides (in 16 bytes) between the halves and two pieces more between the steps keep the quantizer's
+  // narrow stores out of one another's banks
+  pl.bhalf = (pl.kpl * (M + 1)) | 1;
+  pl.bstep = 8 * pl.bhalf + 2;
+  pl.bgroup = 4 * pl.bstep;
+  bool shared = false;
+  for (int i = 0; i < pl.nphase; i++) shared |= pl.phase[i].kp > 1;
+  pl.red_bytes = shared ? M * 3 * rcp::kULanes * 4 : 0;
+  const size_t bar_bytes = 8 * (2 * rcp::kUMaxStages + 2 * rcp::kUMaxSlots + 2 * rcp::kUMaxBuf + 3), misc_bytes = 256;
+  const size_t fixed = 1024 + bar_bytes + misc_bytes + pl.red_bytes + qbuf + 64 + 16 * ncol;
+  // as few parts of K as leave room for three stages (one part: for two)
+  for (int n = parts ? 2 : 1; n <= (parts ? 8 : 1); n++) {
+    pl.part_chunks = ((pl.nchunk + n - 1) / n + pl.kpl - 1) / pl.kpl * pl.kpl;
+    const long long bytes = (long long)(pl.part_chunks / pl.kpl) * pl.bgroup * 16;
+    const long long room = (long long)kSmemMax - (long long)fixed - bytes;
+    pl.stages = room < 0 ? 0 : (int)std::min<long long>(rcp::kUMaxStages, room / rcp::kUItemBytes);
+    pl.bs_bytes = (int)std::min<long long>(bytes + 16 * ncol, 1 << 20);
+    if (pl.stages >= (parts ? 3 : 2)) break;
+    pl.stages = 0;
+  }
+  if (!pl.stages) return pl;
+  // Up to eight tokens are finished by half of the workers; the others help to convert. Two teams want a ring of five stages:
+  // a team that waits for a stage's next fill must know that the one before has come, and it does know that of the items five
+  // back (their slots were free before it wrote its last).
+  pl.helpers = M <= 2 * rcp::kUTok && pl.stages >= 5 && !parts;   // (K in parts: the workers are busy with the next part)
+  size_t off = (size_t)pl.stages * rcp::kUItemBytes;
+  pl.off_bar = (int)off; off += (bar_bytes + 15) / 16 * 16;
+  pl.off_misc = (int)off; off += misc_bytes;
+  pl.off_red = (int)off; off += pl.red_bytes;
+  pl.off_bs = (int)off; off += pl.bs_bytes;
+  pl.off_qbuf = (int)off; off += qbuf;
+  pl.smem = off + 1024;
+  return pl;
+}
+UmmaPlan make_umma_plan(int M, int N, int K, int sms, size_t qbuf) {
+  long long cost[2];
+  UmmaPlan a = umma_plan_for(M, N, K, sms, qbuf, 32, false, &cost[0]), b = umma_plan_for(M, N, K, sms, qbuf, 48, false, &cost[1]);
+  if (a.stages && b.stages) return cost[1] < cost[0] ? b : a;
+  if (a.stages || b.stages || qbuf || M == 1) return a.stages ? a : b;
+  // the activations do not fit: K in parts
+  a = umma_plan_for(M, N, K, sms, qbuf, 32, true, &cost[0]);
+  b = umma_plan_for(M, N, K, sms, qbuf, 48, true, &cost[1]);
+  return !b.stages || (a.stages && cost[0] <= cost[1]) ? a : b;
+}
+
 // SMs of the current device (remembered per device; 148 if the query fails)
 int sm_count() {
   static std::mutex mu;
@@ -364,8 +532,6 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
   if (M > 8 && (grouped || fa || M > rcp::kMaxTokens)) return RCP_ERR_VARIANT;
   if (grouped && (mode == rcp::kModeHybrid || K % 128)) return RCP_ERR_VARIANT;
   if (fa && (mode != rcp::kModeDp4a || !fused_ok(M, K, fa->B))) return RCP_ERR_VARIANT;
-  EncodeTiledFn enc = encode_tiled_fn();
-  if (!enc) return cuda_fail(cudaErrorNotSupported);
   // The plan depends on sizes and form alone; working it out costs the host a quarter of a microsecond, so the last few
   // are remembered per thread.
   struct PlanKey { size_t qbuf; int M, N, K, sms, nsplit, grouped, stream_act, unused; };   // (no padding: compared as bytes)
@@ -388,39 +554,11 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
   }
   const StreamPlan& pl = *found;
   if (pl.stages < 2 || pl.smem > kSmemMax) return RCP_ERR_SHAPE;
-  // Tensor maps of the phases in use (the others repeat the first). Encoding one costs the host about a
-  // microsecond, so the maps of the last few (weights, shape, boxes) combinations are remembered per thread.
-  struct MapKey { const void* words; int N, K, nphase, gpc[rcp::kMaxPhases]; };
-  struct MapSlot { MapKey key; rcp::GemvMaps maps; bool used; };
-  constexpr int kMapSlots = 16;
-  thread_local MapSlot map_cache[kMapSlots] = {};
-  thread_local int map_next = 0;
-  MapKey key = {};
-  key.words = words; key.N = N; key.K = K; key.nphase = pl.nphase;
-  for (int i = 0; i < pl.nphase; i++) key.gpc[i] = pl.phase[i].gpc;
+  int gpc[rcp::kMaxPhases] = {};
+  for (int i = 0; i < pl.nphase; i++) gpc[i] = pl.phase[i].gpc;
   const rcp::GemvMaps* cached = nullptr;
-  for (int i = 0; i < kMapSlots; i++)
-    if (map_cache[i].used && std::memcmp(&map_cache[i].key, &key, sizeof(MapKey)) == 0) { cached = &map_cache[i].maps; break; }
-  if (!cached) {
-    MapSlot& slot = map_cache[map_next];
-    map_next = (map_next + 1) % kMapSlots;
-    slot.used = false;
-    const cuuint64_t gdim[2] = {(cuuint64_t)(K / 16), (cuuint64_t)N};
-    const cuuint64_t gstride[1] = {(cuuint64_t)(K / 4)};
-    const cuuint32_t estr[2] = {1, 1};
-    for (int i = 0; i < rcp::kMaxPhases; i++) {
-      if (i >= pl.nphase && i > 0) { slot.maps.m[i] = slot.maps.m[0]; continue; }
-      const int gpc = i < pl.nphase ? pl.phase[i].gpc : 1;
-      const cuuint32_t box[2] = {(cuuint32_t)rcp::kChunkWords, (cuuint32_t)(16 * gpc)};
-      const CUresult r = enc(&slot.maps.m[i], CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t*>(words), gdim,
-                             gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-      if (r != CUDA_SUCCESS) return cuda_fail(cudaErrorInvalidValue);
-    }
-    slot.key = key;
-    slot.used = true;
-    cached = &slot.maps;
-  }
+  const int rc_maps = phase_maps(words, N, K, pl.nphase, gpc, &cached);
+  if (rc_maps != RCP_OK) return rc_maps;
   const rcp::GemvMaps& maps = *cached;
   rcp::GemvParams gp;
   gp.lut = static_cast<const uint2*>(lut_f16);
@@ -494,6 +632,133 @@ int launch_stream(int mode, const uint32_t* words, const void* lut_f16, const ui
   if (pl.nsplit > 1) return launch_stream_t<rcp::kModeMma, 0, false, 0, false, true>(maps, gp, pl, late, st);
   if (M == 8 && !gp.S_out) return launch_stream_s<rcp::kModeMma, 8, false, 0, false, false, false>(maps, gp, pl, late, st);   // token count known at compile time
   return M > 8 ? launch_stream_t<rcp::kModeMma, 16>(maps, gp, pl, late, st) : launch_stream_t<rcp::kModeMma, 0>(maps, gp, pl, late, st);
+}
+
+template <int FQ, bool SDBG, bool LATE, bool PARTS = false>
+int launch_umma_k(const rcp::GemvMaps& maps, const rcp::UmmaParams& up, const UmmaPlan& pl, cudaStream_t st) {
+  static std::mutex mu;
+  static bool attr_set[kMaxDevices] = {};
+  auto kern = rcp::gemv_umma_kernel<FQ, SDBG, LATE, PARTS>;
+  RCP_CUDA(set_max_smem(kern, (int)kSmemMax, mu, attr_set));
+  RCP_CUDA(launch_overlapped(kern, dim3(pl.grid), dim3(rcp::kUThreads), pl.smem, st, maps, up));
+  return RCP_OK;
+}
+template <int FQ>
+int launch_umma_f(const rcp::GemvMaps& maps, const rcp::UmmaParams& up, const UmmaPlan& pl, cudaStream_t st) {
+  return up.S_out ? launch_umma_k<FQ, true, false>(maps, up, pl, st) : launch_umma_k<FQ, false, false>(maps, up, pl, st);
+}
+
+// Whether the tcgen05 kernel is the faster one, its host-side plan against the streaming kernel's. In clocks of an SM: the
+// streaming kernels take 77 a KB of weights for one token, 80 for up to eight, 171 for sixteen in one launch; the tcgen05
+// kernel what its plan adds up to. Against that it starts and ends slower by what a call with little to stream shows (the
+// conversion, three instruction streams and the sums' way back through tensor memory lie on its path, and there is more
+// code to fetch; one token, whose calls are otherwise launches of one and the same kernel, most: a layer of 54144x4096, 4447x896
+// and 1920x14336 took 55.9 -> 56.6 with the first of them here). us a linear call in a chain, streaming -> tcgen05: one token 4096x4096 3.9 -> 5.2, 10240x8192 9.9 -> 9.5,
+// 57344x8192 33.2 -> 27.0; three 10007x4096 8.3 -> 8.8, 10240x8192 13.7 -> 11.8, 57344x8192 42.2 -> 29.1; eight 22016x4096
+// 12.3 -> 13.4, 8192x28672 32.2 -> 29.5, 57344x8192 41.1 -> 33.2; sixteen 6144x4096 9.7 -> 11.3, 12288x4096 13.5 -> 12.2,
+// 28672x4096 23.9 -> 16.9, 57344x8192 78.5 -> 42.
+bool umma_faster(int M, int N, int K, int sms, int tokens, const UmmaPlan& pl) {
+  int nsplit = 1;
+  const int ms = M == 1 ? 1 : tokens_and_parts(M, N, K, 16, sms, &nsplit);
+  const long long kb = (long long)(((N + 15) / 16 + sms - 1) / sms) * K / 256;   // of the CTA with the most rows
+  const long long per_launch = 2500, streaming = (M + ms - 1) / ms * (kb * (M == 1 ? 77 : ms <= 8 ? 80 : 171) + per_launch);
+  const long long slower = M == 1 ? 11000 : M <= 3 ? 3000 : M <= 8 ? 6000 : 7200;
+  return (M + tokens - 1) / tokens * (pl.clocks + per_launch) + slower < streaming;
+}
+
+// What the host works out for a call of M tokens: the plan for `tokens` of them at a time (as many as fit beside a ring of two
+// stages; 0: not even one does), and whether that is faster than the streaming kernels. Remembered per thread like their plans.
+struct UmmaChoice { UmmaPlan plan; int tokens; bool faster; };
+const UmmaChoice& umma_choice(int M, int N, int K, size_t qbuf) {
+  struct Key { size_t qbuf; int M, N, K, sms; };
+  struct Slot { Key key; UmmaChoice choice; };
+  constexpr int kSlots = 32;
+  thread_local Slot cache[kSlots] = {};   // (M is 0 in an unused slot)
+  thread_local int next = 0, last = 0;
+  Key k = {};
+  k.qbuf = qbuf; k.M = M; k.N = N; k.K = K; k.sms = sm_count();
+  if (std::memcmp(&cache[last].key, &k, sizeof(Key)) == 0) return cache[last].choice;
+  for (int i = 0; i < kSlots; i++)
+    if (std::memcmp(&cache[i].key, &k, sizeof(Key)) == 0) { last = i; return cache[i].choice; }
+  last = next;
+  Slot& slot = cache[next];
+  next = (next + 1) % kSlots;
+  slot.key = k;
+  UmmaChoice& c = slot.choice;
+  c.tokens = 0;
+  c.faster = false;
+  for (int parts = 1; parts <= M && !c.tokens; parts++) {
+    const int m = (M + parts - 1) / parts;
+    c.plan = make_umma_plan(m, N, K, k.sms, qbuf);
+    if (c.plan.stages) c.tokens = m;
+  }
+  if (c.tokens) c.faster = umma_faster(M, N, K, k.sms, c.tokens, c.plan);
+  return c;
+}
+
+// One launch of the tcgen05 kernel by the plan pl. fa: one token still to be rotated and quantized (xq and scale unused).
+int launch_umma(const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16, int M, int N, int K,
+                void* y_f16, void* workspace, cudaStream_t st, const UmmaPlan& pl, const FusedAct* fa, int32_t* S_out, bool late) {
+  int gpc[rcp::kMaxPhases] = {};
+  for (int i = 0; i < pl.nphase; i++) {   // (five phases at most)
+    gpc[i] = pl.phase[i].gpc;
+    if (pl.phase[i].r > 0) gpc[rcp::kMaxPhases - 1] = pl.phase[i].gpc - 1;
+  }
+  const rcp::GemvMaps* maps = nullptr;
+  const int rc = phase_maps(words, N, K, pl.nphase, gpc, &maps);
+  if (rc != RCP_OK) return rc;
+  rcp::UmmaParams up;
+  up.lut = static_cast<const uint2*>(lut_f16);
+  up.xq = xq;
+  up.scale = static_cast<const __half*>(scale_f16);
+  up.y = static_cast<__half*>(y_f16);
+  up.status = static_cast<int32_t*>(workspace);
+  up.S_out = S_out;
+  up.M = M; up.N = N; up.K = K; up.nchunk = pl.nchunk; up.nphase = pl.nphase;
+  for (int i = 0; i < rcp::kMaxPhases; i++) up.phase[i] = pl.phase[i];
+  up.kpl = pl.kpl; up.lg_kpl = pl.lg_kpl; up.bgroup = pl.bgroup; up.bstep = pl.bstep; up.bhalf = pl.bhalf; up.lg_m2 = pl.lg_m2; up.helpers = pl.helpers; up.part_chunks = pl.part_chunks;
+  up.slots = pl.slots; up.dcols = pl.dcols; up.nbuf = pl.nbuf; up.stages = pl.stages;
+  // one item per CTA at about 6 TB/s for the whole grid, in SM clocks (about 2 GHz)
+  up.ramp_clk = (int)((double)rcp::kUItemBytes * pl.grid / 6.0e12 * 1.9e9);
+  up.off_bar = pl.off_bar; up.off_misc = pl.off_misc; up.off_red = pl.off_red; up.off_bs = pl.off_bs; up.off_qbuf = pl.off_qbuf;
+  up.red_bytes = pl.red_bytes; up.bs_bytes = pl.bs_bytes;
+  up.x = nullptr; up.xq_out = nullptr; up.scale_out = nullptr;
+  up.inv_sqrt_b = 1.f; up.clip_ratio = 1.f; up.had_block = 1;
+  if (fa) {
+    up.x = static_cast<const __half*>(fa->x_f16);
+    up.xq_out = fa->xq_out;
+    up.scale_out = static_cast<__half*>(fa->scale_out);
+    up.inv_sqrt_b = (float)(1.0 / std::sqrt((double)fa->B));
+    up.clip_ratio = std::min(fa->clip_ratio, rcp::kClipRatioCap);
+    up.had_block = fa->B;
+    if (full_block(K, fa->B)) {
+      if (K == 2048) return launch_umma_f<4>(*maps, up, pl, st);
+      if (K == 4096) return launch_umma_f<8>(*maps, up, pl, st);
+      return launch_umma_f<16>(*maps, up, pl, st);
+    }
+    return K <= 8192 ? launch_umma_f<-1>(*maps, up, pl, st) : launch_umma_f<-2>(*maps, up, pl, st);
+  }
+  if (pl.part_chunks < pl.nchunk) {
+    if (S_out) return launch_umma_k<0, true, false, true>(*maps, up, pl, st);
+    return late ? launch_umma_k<0, false, true, true>(*maps, up, pl, st) : launch_umma_k<0, false, false, true>(*maps, up, pl, st);
+  }
+  if (S_out) return launch_umma_k<0, true, false>(*maps, up, pl, st);
+  return late ? launch_umma_k<0, false, true>(*maps, up, pl, st) : launch_umma_k<0, false, false>(*maps, up, pl, st);
+}
+
+int launch_umma_passes(const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16, int M, int N, int K,
+                       void* y_f16, void* workspace, cudaStream_t st, int32_t* S_out, bool late) {
+  const int mp = umma_choice(M, N, K, 0).tokens;
+  if (!mp) return RCP_ERR_VARIANT;
+  for (int m0 = 0; m0 < M; m0 += mp) {
+    const int mm = std::min(mp, M - m0);
+    const UmmaPlan& pl = m0 == 0 ? umma_choice(M, N, K, 0).plan : umma_choice(mm, N, K, 0).plan;   // (fewer tokens fit, too)
+    const int rc = launch_umma(words, lut_f16, xq + (size_t)m0 * (K / 2), static_cast<const __half*>(scale_f16) + m0, mm, N, K,
+                               static_cast<__half*>(y_f16) + (size_t)m0 * N, workspace, st, pl, nullptr,
+                               S_out ? S_out + (size_t)m0 * N * 4 : nullptr, late);
+    if (rc != RCP_OK) return rc;
+  }
+  return RCP_OK;
 }
 
 // All M tokens: as many launches as it takes for the expanded activations to fit (`cap` tokens at most each).
@@ -940,6 +1205,8 @@ size_t rcp_gemv_workspace_bytes(int M, int N, int K) {
   return 16;   // a status word for the kernels' bounded waits; no sums pass through global memory
 }
 
+static int auto_variant(int M, int N, int K) { return umma_choice(M, N, K, 0).faster ? RCP_GEMV_UMMA : M == 1 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY; }
+
 // late_start: the call quantizes its activations itself (see the end of gemv_stream_kernel)
 static int gemv_w2a4(int variant, const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16, int M,
                      int N, int K, void* y_f16, void* workspace, int32_t* S_dbg, void* stream, bool late_start) {
@@ -955,7 +1222,7 @@ static int gemv_w2a4(int variant, const uint32_t* words, const void* lut_f16, co
   // that streaming kernel, which stores the sums it finishes its rows from.
   if (S_dbg && variant == RCP_GEMV_AUTO) variant = RCP_GEMV_SIMPLE;
   // measured on B200: one token runs fastest on the CUDA cores alone, more tokens on the tensor cores
-  if (variant == RCP_GEMV_AUTO) variant = (M == 1) ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY;
+  if (variant == RCP_GEMV_AUTO) variant = auto_variant(M, N, K);
   // the streaming kernels wait on barriers with a bound and report a wait that gave up through the workspace
   if (variant != RCP_GEMV_SIMPLE && !workspace) return RCP_ERR_WORKSPACE;
   switch (variant) {
@@ -978,6 +1245,8 @@ static int gemv_w2a4(int variant, const uint32_t* words, const void* lut_f16, co
       // CUDA-core path: two tokens per launch
       return launch_stream_passes(rcp::kModeDp4a, 2, words, lut_f16, xq, scale_f16, M, N, K, y_f16, workspace, st, false,
                                   S_dbg);
+    case RCP_GEMV_UMMA:
+      return launch_umma_passes(words, lut_f16, xq, scale_f16, M, N, K, y_f16, workspace, st, S_dbg, late_start);
     case RCP_GEMV_MMA_STREAM: {
       // tensor-core path with the activations streamed beside the weights: all tokens in one launch, any K
       const StreamPlan pl = make_plan(M, N, K, sm_count(), false, 0, 1, true);
@@ -1151,7 +1420,8 @@ int rcp_linear_w2a4_launches(int M, int N, int K, int had_block, int group) {
   if (group != 0 && group != 128) return 2;
   const int cap = group == 0 ? (M == 1 ? 2 : 16) : (M <= 2 ? 2 : 8);   // tokens per launch of the variant AUTO picks
   int nsplit = 1;
-  const int mp = (group != 0 || cap < 8) ? tokens_per_pass(M, K, cap) : tokens_and_parts(M, N, K, cap, sm_count(), &nsplit);
+  const int mp = group == 0 && umma_choice(M, N, K, 0).faster ? umma_choice(M, N, K, 0).tokens
+                 : (group != 0 || cap < 8) ? tokens_per_pass(M, K, cap) : tokens_and_parts(M, N, K, cap, sm_count(), &nsplit);
   return 1 + (M + mp - 1) / mp;
 }
 
@@ -1174,6 +1444,10 @@ int rcp_linear_w2a4_checked(const void* x_f16, int M, int K, int had_block, floa
   if (!(M == 1 && B == K && (K == 4096 || K == 8192)) && (!xq || !scale_f16)) return RCP_ERR_NULL;
   if (fused_ok(M, K, B) && (group == 0 || group == 128)) {
     const FusedAct fa{x_f16, B, clip_ratio, xq, scale_f16};
+    if (group == 0) {
+      const UmmaChoice& c = umma_choice(M, N, K, full_block(K, B) ? rcp::full_rotate_bytes(K) : 0);
+      if (c.faster) return launch_umma(words, lut_f16, nullptr, nullptr, M, N, K, y_f16, workspace, st, c.plan, &fa, S_dbg, false);
+    }
     return launch_stream(rcp::kModeDp4a, words, lut_f16, nullptr, nullptr, M, N, K, y_f16, workspace, st, group == 128,
                          &fa, nullptr, 1, nullptr, S_dbg);
   }
@@ -1183,7 +1457,7 @@ int rcp_linear_w2a4_checked(const void* x_f16, int M, int K, int had_block, floa
   if (rc != RCP_OK) return rc;
   // with S_dbg: the streaming kernel AUTO would pick, in its checked instantiation
   if (group == 0)
-    return gemv_w2a4(S_dbg ? (M == 1 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY) : RCP_GEMV_AUTO, words, lut_f16, xq, scale_f16, M,
+    return gemv_w2a4(S_dbg ? auto_variant(M, N, K) : RCP_GEMV_AUTO, words, lut_f16, xq, scale_f16, M,
                      N, K, y_f16, workspace, S_dbg, stream, true);
   return gemv_w2a4_grouped(S_dbg && group == 128 ? (M <= 2 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY) : RCP_GEMV_AUTO, words,
                            lut_f16, group, xq, scale_f16, M, N, K, y_f16, workspace, S_dbg, stream, true);

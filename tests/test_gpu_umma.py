@@ -1,0 +1,76 @@
+"""The GEMV on the fifth-generation tensor cores (variant "umma"): exact sums against the oracle at the edges of its tiles, of its
+columns and of what fits in shared memory, in the production and in the guarded build; the linear call whose quantizer is inside
+that kernel; and the host's choice between the kernels."""
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2502_15779_b200 as rcp
+from gen import synth
+from helpers import f16_bits
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+# N, K, M: groups of 16 rows around the SMs and their rounds of eight, chunks of 512 around the lane blocks, tokens around the
+# columns (8, 16, 32, 48) and the workers' fours; the last ones go through K in parts
+CASES = [(1, 64, 1), (17, 192, 3), (16, 512, 1), (129, 576, 7), (300, 2048, 4), (2369, 1024, 2), (2368, 4096, 5), (4737, 1088, 9),
+         (700, 8192, 8), (18945, 512, 1), (21300, 1024, 16), (333, 5184, 12), (64, 65536, 1), (300, 11008, 15), (300, 28672, 8),
+         (2400, 14336, 16), (40, 65536, 7)]
+
+
+def run_case(i):
+    N, K, M = CASES[i]
+    codes, lut = synth.make_layer(N, K, 64, "uniform", 900 + i, device=DEV)
+    words = rcp.rcp_pack_weights(codes)
+    xq, scale = rcp.rcp_quantize_act(synth.make_activations(M, K, 900 + i, device=DEV), 64, 1.0)
+    ws = rcp.make_workspace(M, N, K, DEV)
+    S = torch.full((M, N, 4), 77, dtype=torch.int32, device=DEV)
+    checked = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="umma", S_dbg=S)
+    y = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="umma")
+    torch.cuda.synchronize()
+    assert int(ws.abs().max()) == 0
+    assert np.array_equal(f16_bits(y), f16_bits(checked))
+    ref = oracle.gemv_w2a4(words.cpu().numpy().view(np.uint32), f16_bits(lut), xq.cpu().numpy(), f16_bits(scale))
+    assert np.array_equal(S.cpu().numpy(), ref["S"])
+    assert np.all(np.abs(y.float().cpu().numpy().astype(np.float64) - ref["y"]) <= ref["tol"])
+
+
+@pytest.mark.parametrize("i", range(len(CASES)), ids=["x".join(map(str, c)) for c in CASES])
+def test_sums_are_the_oracles(i):
+    run_case(i)
+
+
+def test_guarded_build_reports_nothing():
+    from paper_2502_15779_b200 import build
+    env = dict(os.environ, RCP_W2A4_LIB=build.build_checked(), PYTHONPATH=os.pathsep.join([ROOT, os.path.join(ROOT, "tests")]))
+    subprocess.run([sys.executable, "-c", "import test_gpu_umma as t\nfor i in range(len(t.CASES)): t.run_case(i)"], check=True,
+                   env=env, cwd=ROOT, timeout=900)
+
+
+# shapes whose linear call runs as one kernel of this kind (large ones), every form of the quantizer inside
+@pytest.mark.parametrize("N,K,B", [(60000, 8192, 8192), (90000, 4096, 4096), (180000, 2048, 2048), (90000, 5184, 64),
+                                   (40000, 11008, 128)])
+def test_linear_with_the_quantizer_inside(N, K, B):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N)
+    words = torch.randint(-2 ** 31, 2 ** 31 - 1, (N, K // 16), dtype=torch.int32, device=DEV, generator=g)
+    lut = torch.sort(torch.randn(N, 4, device=DEV, generator=g) * 0.02, dim=1)[0].half()
+    x = synth.make_activations(1, K, 5, device=DEV)
+    ws = rcp.make_workspace(1, N, K, DEV)
+    xq, scale = rcp.rcp_quantize_act(x, B, 1.0)
+    want = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="dp4a")
+    xq2, scale2 = torch.zeros_like(xq), torch.zeros_like(scale)
+    y = rcp.rcp_linear_w2a4(x, B, 1.0, words, lut, xq=xq2, scale=scale2, workspace=ws)
+    torch.cuda.synchronize()
+    assert int(ws.abs().max()) == 0
+    assert torch.equal(xq, xq2) and torch.equal(scale, scale2)
+    assert np.array_equal(f16_bits(y), f16_bits(want))
+    zero = rcp.rcp_linear_w2a4(torch.zeros_like(x), B, 1.0, words, lut, xq=xq2, scale=scale2, workspace=ws)
+    assert not zero.any() and not xq2.any() and not scale2.any()
