@@ -74,3 +74,30 @@ def test_linear_with_the_quantizer_inside(N, K, B):
     assert np.array_equal(f16_bits(y), f16_bits(want))
     zero = rcp.rcp_linear_w2a4(torch.zeros_like(x), B, 1.0, words, lut, xq=xq2, scale=scale2, workspace=ws)
     assert not zero.any() and not xq2.any() and not scale2.any()
+
+
+# Sums of fp32 products stay exact where they grow largest: every code 1 (the e4m3 reading is +2 throughout) against the largest
+# activations over the longest K, then a few codes that change the last bits; +2 and -2 in long runs likewise.
+@pytest.mark.parametrize("K", [65536, 28672])
+def test_sums_at_the_ends_of_their_range(K):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(K)
+    N, M = 48, 2
+    codes = torch.ones(N, K, dtype=torch.uint8, device=DEV)
+    rnd = torch.randint(0, 4, (N, K), generator=g, device=DEV, dtype=torch.uint8)
+    codes[1:8, -64:] = rnd[1:8, -64:]
+    codes[8:16, ::129] = rnd[8:16, ::129]
+    codes[16:24, K // 2:] = 3
+    codes[24:32, 0::2] = 3
+    codes[32:40] = 3 * (rnd[32:40] > 0).to(torch.uint8)
+    codes[40:48] = 2 + rnd[40:48] // 3
+    words = rcp.rcp_pack_weights(codes)
+    lut = torch.sort(torch.randn(N, 4, device=DEV, generator=g) * 0.02, dim=1)[0].half()
+    xq = torch.full((M, K // 2), 0x77, dtype=torch.uint8, device=DEV)
+    xq[1, 1::3] = torch.randint(0, 256, xq[1, 1::3].shape, generator=g, device=DEV, dtype=torch.uint8)
+    scale = torch.tensor([0.01, 0.02], dtype=torch.float16, device=DEV)
+    S = torch.empty(M, N, 4, dtype=torch.int32, device=DEV)
+    rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=rcp.make_workspace(M, N, K, DEV), variant="umma", S_dbg=S)
+    torch.cuda.synchronize()
+    ref = oracle.gemv_w2a4(words.cpu().numpy().view(np.uint32), f16_bits(lut), xq.cpu().numpy(), f16_bits(scale))
+    assert np.array_equal(S.cpu().numpy(), ref["S"])
