@@ -20,10 +20,11 @@
 // Work. Groups of 16 rows are shared out over the CTAs in phases like in gemv_stream.cuh; an item is 128 lanes x 128
 // bytes of packed weights (16 KB): 16 gpc rows x kp chunks of K side by side in the lanes, each chunk with columns of its own
 // (lane block j uses column block j, the other products are dropped). Warps: a producer streams the items' boxes into a ring
-// (TMA, 128-byte swizzle); twelve converters in three sets of four (a warp reads and writes the 32 lanes its number gives it),
-// set s filling slot s of tensor memory with item after item; three issuers, one per reading; four finishers, who turn the sums
-// of a tile into y while the next is worked on. Slots of 128 columns (a whole item): with 64 the handshakes cost 55
-// clocks per KB of weights, so 40, less than the 44 to 49 that HBM needs.
+// (TMA, 128-byte swizzle); eight converters, two to a quarter of the lanes (a warp reads and writes the 32 lanes its number
+// gives it), each half of an item's bytes, fill the slots of tensor memory with item after item; three issuers, one per
+// reading; sixteen workers prepare the activations, then turn the sums of a tile into y while the next is worked on (four tokens
+// to a warp; up to eight tokens the last eight of them convert too). Slots of 128 columns (a whole item): with 64 the handshakes
+// cost 55 clocks per KB of weights, so 40, less than the 44 to 49 that HBM needs.
 // What it measured (B200, us a call of the whole linear in a chain, cold weights; before: dp4a for one token, mma.sync for more):
 // 57344x8192 at 1, 3, 8, 12, 16 tokens 33.2, 42.2, 41.1, 79.3, 78.5 -> 27.3, 29.1, 33.8, 35.9, 43.0; 28672x4096 at 16 23.9 -> 16.9;
 // 8192x28672 at 8 32.2 -> 29.5. Bound: HBM in the loop (an item per SM in 720 clocks is 6.4 TB/s) up to eight tokens; at

@@ -652,11 +652,11 @@ int launch_umma_f(const rcp::GemvMaps& maps, const rcp::UmmaParams& up, const Um
 // streaming kernels take 77 a KB of weights for one token, 80 for up to eight, 171 for sixteen in one launch; the tcgen05
 // kernel what its plan adds up to. Against that it starts and ends slower by what a call with little to stream shows (the
 // conversion, three instruction streams and the sums' way back through tensor memory lie on its path, and there is more
-// code to fetch; one token, whose calls are otherwise launches of one and the same kernel, most: a layer of 54144x4096, 4447x896
-// and 1920x14336 took 55.9 -> 56.6 with the first of them here). us a linear call in a chain, streaming -> tcgen05: one token 4096x4096 3.9 -> 5.2, 10240x8192 9.9 -> 9.5,
-// 57344x8192 33.2 -> 27.0; three 10007x4096 8.3 -> 8.8, 10240x8192 13.7 -> 11.8, 57344x8192 42.2 -> 29.1; eight 22016x4096
-// 12.3 -> 13.4, 8192x28672 32.2 -> 29.5, 57344x8192 41.1 -> 33.2; sixteen 6144x4096 9.7 -> 11.3, 12288x4096 13.5 -> 12.2,
-// 28672x4096 23.9 -> 16.9, 57344x8192 78.5 -> 42.
+// code to fetch; one token, whose calls are otherwise launches of one and the same kernel, most: layers of 54144x4096, 4447x896
+// and 1920x14336 took 55.9 -> 56.6 with the first of them here). us a linear call in a chain, streaming -> tcgen05: one token
+// 4096x4096 3.9 -> 5.2, 10240x8192 9.9 -> 9.5, 57344x8192 33.2 -> 27.0; three 10007x4096 8.3 -> 8.8, 10240x8192 13.7 -> 11.8,
+// 57344x8192 42.2 -> 29.1; eight 22016x4096 12.3 -> 13.4, 8192x28672 32.2 -> 29.5, 57344x8192 41.1 -> 33.2; sixteen 6144x4096
+// 9.7 -> 11.3, 12288x4096 13.5 -> 12.2, 28672x4096 23.9 -> 16.9, 57344x8192 78.5 -> 42.
 bool umma_faster(int M, int N, int K, int sms, int tokens, const UmmaPlan& pl) {
   int nsplit = 1;
   const int ms = M == 1 ? 1 : tokens_and_parts(M, N, K, 16, sms, &nsplit);
