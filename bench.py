@@ -605,8 +605,8 @@ def main():
     g_us = gms * 1e3 / g_launches
     achieved = g_bytes_per_launch / g_us / 1e3
     peaks, peak_kind = measured_peaks()
-    roofline = {"bound": "hbm", "kernel": "gemv_stream_kernel (with the activation quantizer inside where the step "
-                                          "uses the single kernel)", "achieved": round(achieved, 1),
+    roofline = {"bound": "hbm", "kernel": "gemv_stream_kernel, gemv_umma_kernel for large layers (with the activation "
+                                          "quantizer inside where the step uses the single kernel)", "achieved": round(achieved, 1),
                 "peak": peaks["hbm_gbs"], "peak_kind": peak_kind, "unit": "GB/s",
                 "frac": round(achieved / peaks["hbm_gbs"], 4), "frac_of_nominal_8TBs": round(achieved / NOMINAL_HBM_GBS, 4),
                 "avg_launch_us": round(g_us, 3), "bytes_per_launch": int(g_bytes_per_launch), "traffic": None}
@@ -618,8 +618,8 @@ def main():
     pgraphs = [capture(lambda c=c: plain_gemv(c), stream) for c in range(copies)]
     time_graph_replays(pgraphs, order[:8], stream)
     pms = min(time_graph_replays(pgraphs, order, stream) for _ in range(3))
-    # had_block 1 never takes the single kernel: the count is the quantizer plus the GEMV launches
-    p_launches = args.steps * sum(rcp.rcp_linear_w2a4_launches(M, L.N, L.K, 1) - 1 if args.variant == "auto"
+    # one token is one launch; more never take the single kernel: the count is the quantizer plus the GEMV launches
+    p_launches = args.steps * sum((rcp.rcp_linear_w2a4_launches(M, L.N, L.K, 1) - 1 if M > 1 else 1) if args.variant == "auto"
                                   else -(-M // (8 if args.variant in ("mma", "mma_only") else 2))
                                   for L in layer.layers)
     p_us = pms * 1e3 / p_launches

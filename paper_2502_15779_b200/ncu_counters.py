@@ -1,7 +1,7 @@
 """Turns an ncu launch log into the per-launch counters the benchmark reports beside its roofline.
 
     ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,smsp__inst_executed.sum,gpu__time_duration.sum \
-        --clock-control none -k regex:gemv_stream -s <warm-up launches> -c <launches of one step> \
+        --clock-control none -k "regex:gemv_(stream|umma)" -s <warm-up launches> -c <launches of one step> \
         --csv --log-file counters.csv python bench.py --profile --steps 2 --warmup 3
     python -m paper_2502_15779_b200.ncu_counters counters.csv llama2_70b_M1_auto
 
