@@ -232,9 +232,6 @@ __global__ void __launch_bounds__(kUThreads, 1) gemv_umma_kernel(const __grid_co
             ok = mbar_wait_warp(aempty0 + 8 * slot, apar);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          } else {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(empty0 + 8 * stage);   // this warp has read its part of the stage
           }
           tmem_st32(a_at + 128u * (uint32_t)slot + 32u * s, f);
         }
@@ -242,7 +239,13 @@ __global__ void __launch_bounds__(kUThreads, 1) gemv_umma_kernel(const __grid_co
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(afull0 + 8 * slot);
+        // The stage is given back when what was read from it is in tensor memory, not right behind the reads: an arrival there
+        // got ahead of the last of them, and where the producer was waiting for the stage (rings of two or three) that read
+        // met the next item's bytes.
+        if (lane == 0) {
+          mbar_arrive(afull0 + 8 * slot);
+          mbar_arrive(empty0 + 8 * stage);
+        }
       }
       if (++slot == slots) { slot = 0; apar ^= 1u; }
       if (++stage == stages) { stage = 0; rpar ^= 1u; }

@@ -54,6 +54,30 @@ def test_guarded_build_reports_nothing():
                    env=env, cwd=ROOT, timeout=900)
 
 
+# Rings of two and three stages, whose stages are filled again as soon as they have been read: the sums of many calls in a row
+# are those of the plain kernel.
+@pytest.mark.parametrize("N,K,M", [(28672, 20992, 8), (28672, 20480, 7), (5217, 23040, 6), (20000, 11008, 12)])
+def test_a_short_ring_keeps_what_is_being_read(N, K, M):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N + K)
+    words = torch.randint(-2 ** 31, 2 ** 31 - 1, (N, K // 16), dtype=torch.int32, device=DEV, generator=g)
+    lut = torch.sort(torch.randn(N, 4, device=DEV, generator=g) * 0.02, dim=1)[0].half()
+    xq = torch.randint(0, 256, (M, K // 2), dtype=torch.uint8, device=DEV, generator=g)
+    scale = (torch.rand(M, device=DEV, generator=g) * 0.1 + 0.01).half()
+    ws = rcp.make_workspace(M, N, K, DEV)
+    S, want = torch.empty(M, N, 4, dtype=torch.int32, device=DEV), torch.empty(M, N, 4, dtype=torch.int32, device=DEV)
+    y = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="simple", S_dbg=want)
+    ys = torch.empty(12, M, N, dtype=torch.float16, device=DEV)
+    for rep in range(10):
+        for out in ys:
+            rcp.rcp_gemv_w2a4(words, lut, xq, scale, y=out, workspace=ws, variant="umma")
+        rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="umma", S_dbg=S)
+        torch.cuda.synchronize()
+        assert int(ws.abs().max()) == 0
+        assert torch.equal(S, want), f"repetition {rep}"
+        assert all(torch.equal(out.view(torch.int16), y.view(torch.int16)) for out in ys), f"repetition {rep}"
+
+
 # shapes whose linear call runs as one kernel of this kind (large ones), every form of the quantizer inside
 @pytest.mark.parametrize("N,K,B", [(60000, 8192, 8192), (90000, 4096, 4096), (180000, 2048, 2048), (90000, 5184, 64),
                                    (40000, 11008, 128)])
