@@ -222,6 +222,19 @@ size_t rcp_gemv_workspace_bytes(int M, int N, int K);
 int rcp_gemv_plan(int M, int N, int K, int sms, int* out, int cap);
 
 /*
+ * The same for the tcgen05 kernel (RCP_GEMV_UMMA). had_block 0: the form on given activations; otherwise the one that
+ * rcp_linear_w2a4 runs with the quantizer inside (RCP_ERR_VARIANT where it has none). out[0] whether rcp_gemv_w2a4 (or
+ * rcp_linear_w2a4) takes this kernel, out[1] launches (0: nothing fits); then per launch: its tokens, the tokens its plan is
+ * made for, ring stages, shared-memory bytes, chunks of K, chunks whose activations are in shared memory at a time, chunks side
+ * by side at most, the strides bhalf, bstep, bgroup of the activations in units of 16 bytes, log2 of the tokens rounded up,
+ * tensor-memory slots of 128 columns, columns of an accumulator, sets of three accumulators, whether the second half of the
+ * workers helps to convert, the offsets and sizes of the shared-memory areas (barriers, scales, reduction and its bytes,
+ * activations and their bytes, quantizer), the number of phases; and per phase: groups per CTA at most, first group, groups,
+ * CTAs, repetitions, chunks side by side, items per repetition, columns of the instruction.
+ */
+int rcp_gemv_umma_plan(int M, int N, int K, int sms, int had_block, int* out, int cap);
+
+/*
  * LUT GEMV / skinny GEMM (Section 4.4, Eq. "deqgrid"):
  *   S_c[m][n] = sum over k with code[n][k] == c of q[m][k]       (exact integers)
  *   y[m][n]   = fp16( scale[m] * sum_c lut[n][c] * S_c[m][n] )   (fp32 arithmetic)

@@ -278,6 +278,7 @@ int phase_maps(const uint32_t* words, int N, int K, int nphase, const int* gpcs,
 // ---------------------------------------------------------------------------------------------
 // GEMV on tcgen05: launch plan.
 struct UmmaPlan {
+  int tokens;        // that it is made for
   int nchunk, nphase, grid, kpl, lg_kpl, bgroup, bstep, bhalf, lg_m2, slots, dcols, nbuf, stages, helpers;
   rcp::UmmaPhase phase[rcp::kMaxPhases];
   int part_chunks;   // nchunk (rounded up to kpl): all of K at once
@@ -298,11 +299,12 @@ int floor_pow2(int v) { int p = 1; while (2 * p <= v) p *= 2; return p; }
 // use); its 48 instructions, 600 clocks up to 16 columns, 24 a column from there on; a slot's turn, 860 clocks where the
 // accumulators (three times 48 columns) leave room for two slots only. Columns buy lanes (kp chunks side by side), which is
 // what short or few rows need; up to 32 or up to 48 of them, whichever comes out cheaper.
-UmmaPlan umma_plan_for(int M, int N, int K, int sms, size_t qbuf, int max_cols, bool parts, long long* total) {
+UmmaPlan umma_plan_for(int M, int N, int K, int sms, size_t qbuf, int kp_max, int max_cols, bool parts, long long* total) {
   UmmaPlan pl = {};
+  pl.tokens = M;
   pl.grid = sms;
   pl.nchunk = (K / 16 + rcp::kChunkWords - 1) / rcp::kChunkWords;
-  int kp_cap = 8;
+  int kp_cap = kp_max;
   while (kp_cap > 1 && (umma_columns(M, kp_cap) > max_cols || kp_cap >= 2 * pl.nchunk)) kp_cap /= 2;
   auto kp_of = [&](int g) { return std::min(kp_cap, floor_pow2(8 / g)); };
   auto items_of = [&](int g) { return (pl.nchunk + kp_of(g) - 1) / kp_of(g); };
@@ -395,14 +397,15 @@ UmmaPlan umma_plan_for(int M, int N, int K, int sms, size_t qbuf, int max_cols, 
   pl.smem = off + 1024;
   return pl;
 }
-UmmaPlan make_umma_plan(int M, int N, int K, int sms, size_t qbuf) {
+// kp_max: most chunks side by side
+UmmaPlan make_umma_plan(int M, int N, int K, int sms, size_t qbuf, int kp_max = 8) {
   long long cost[2];
-  UmmaPlan a = umma_plan_for(M, N, K, sms, qbuf, 32, false, &cost[0]), b = umma_plan_for(M, N, K, sms, qbuf, 48, false, &cost[1]);
+  UmmaPlan a = umma_plan_for(M, N, K, sms, qbuf, kp_max, 32, false, &cost[0]), b = umma_plan_for(M, N, K, sms, qbuf, kp_max, 48, false, &cost[1]);
   if (a.stages && b.stages) return cost[1] < cost[0] ? b : a;
   if (a.stages || b.stages || qbuf || M == 1) return a.stages ? a : b;
   // the activations do not fit: K in parts
-  a = umma_plan_for(M, N, K, sms, qbuf, 32, true, &cost[0]);
-  b = umma_plan_for(M, N, K, sms, qbuf, 48, true, &cost[1]);
+  a = umma_plan_for(M, N, K, sms, qbuf, kp_max, 32, true, &cost[0]);
+  b = umma_plan_for(M, N, K, sms, qbuf, kp_max, 48, true, &cost[1]);
   return !b.stages || (a.stages && cost[0] <= cost[1]) ? a : b;
 }
 
@@ -648,6 +651,9 @@ int launch_umma_f(const rcp::GemvMaps& maps, const rcp::UmmaParams& up, const Um
   return up.S_out ? launch_umma_k<FQ, true, false>(maps, up, pl, st) : launch_umma_k<FQ, false, false>(maps, up, pl, st);
 }
 
+// What the host works out for a call of M tokens, see umma_choose.
+struct UmmaChoice { UmmaPlan plan, last; int tokens, launches; bool faster; };
+
 // Whether the tcgen05 kernel is the faster one, its host-side plan against the streaming kernel's. In clocks of an SM: the
 // streaming kernels take 77 a KB of weights for one token, 80 for up to eight, 171 for sixteen in one launch; the tcgen05
 // kernel what its plan adds up to. Against that it starts and ends slower by what a call with little to stream shows (the
@@ -657,18 +663,36 @@ int launch_umma_f(const rcp::GemvMaps& maps, const rcp::UmmaParams& up, const Um
 // 4096x4096 3.9 -> 5.2, 10240x8192 9.9 -> 9.5, 57344x8192 33.2 -> 27.0; three 10007x4096 8.3 -> 8.8, 10240x8192 13.7 -> 11.8,
 // 57344x8192 42.2 -> 29.1; eight 22016x4096 12.3 -> 13.4, 8192x28672 32.2 -> 29.5, 57344x8192 41.1 -> 33.2; sixteen 6144x4096
 // 9.7 -> 11.3, 12288x4096 13.5 -> 12.2, 28672x4096 23.9 -> 16.9, 57344x8192 78.5 -> 42.
-bool umma_faster(int M, int N, int K, int sms, int tokens, const UmmaPlan& pl) {
+bool umma_faster(int M, int N, int K, int sms, const UmmaChoice& c) {
   int nsplit = 1;
   const int ms = M == 1 ? 1 : tokens_and_parts(M, N, K, 16, sms, &nsplit);
   const long long kb = (long long)(((N + 15) / 16 + sms - 1) / sms) * K / 256;   // of the CTA with the most rows
   const long long per_launch = 2500, streaming = (M + ms - 1) / ms * (kb * (M == 1 ? 77 : ms <= 8 ? 80 : 171) + per_launch);
   const long long slower = M == 1 ? 11000 : M <= 3 ? 3000 : M <= 8 ? 6000 : 7200;
-  return (M + tokens - 1) / tokens * (pl.clocks + per_launch) + slower < streaming;
+  return c.launches * (c.plan.clocks + per_launch) + slower < streaming;
 }
 
-// What the host works out for a call of M tokens: the plan for `tokens` of them at a time (as many as fit beside a ring of two
-// stages; 0: not even one does), and whether that is faster than the streaming kernels. Remembered per thread like their plans.
-struct UmmaChoice { UmmaPlan plan; int tokens; bool faster; };
+// A call of M tokens: launches of `tokens` of them each (as many as fit beside a ring of two
+// stages) by `plan`, the last one with what remains by `last` (0 launches: not even one token fits), and whether that is
+// faster than the streaming kernels.
+void umma_choose(int M, int N, int K, int sms, size_t qbuf, UmmaChoice& c) {
+  c.tokens = c.launches = 0;
+  c.faster = false;
+  for (int parts = 1; parts <= M && !c.launches; parts++) {
+    const int m = (M + parts - 1) / parts, n = (M + m - 1) / m, rest = M - (n - 1) * m;
+    c.plan = make_umma_plan(m, N, K, sms, qbuf);
+    if (!c.plan.stages) continue;
+    // What remains may fit only with no more chunks side by side than the others have: fewer tokens would take more, and K is
+    // padded to a multiple of them.
+    c.last = rest == m ? c.plan : make_umma_plan(rest, N, K, sms, qbuf);
+    for (int kp = c.plan.kpl; kp >= 1 && !c.last.stages; kp /= 2) c.last = make_umma_plan(rest, N, K, sms, qbuf, kp);
+    if (!c.last.stages) continue;
+    c.tokens = m;
+    c.launches = n;
+  }
+  if (c.launches) c.faster = umma_faster(M, N, K, sms, c);
+}
+// The same, remembered per thread like the streaming kernels' plans.
 const UmmaChoice& umma_choice(int M, int N, int K, size_t qbuf) {
   struct Key { size_t qbuf; int M, N, K, sms; };
   struct Slot { Key key; UmmaChoice choice; };
@@ -684,21 +708,14 @@ const UmmaChoice& umma_choice(int M, int N, int K, size_t qbuf) {
   Slot& slot = cache[next];
   next = (next + 1) % kSlots;
   slot.key = k;
-  UmmaChoice& c = slot.choice;
-  c.tokens = 0;
-  c.faster = false;
-  for (int parts = 1; parts <= M && !c.tokens; parts++) {
-    const int m = (M + parts - 1) / parts;
-    c.plan = make_umma_plan(m, N, K, k.sms, qbuf);
-    if (c.plan.stages) c.tokens = m;
-  }
-  if (c.tokens) c.faster = umma_faster(M, N, K, k.sms, c.tokens, c.plan);
-  return c;
+  umma_choose(M, N, K, k.sms, qbuf, slot.choice);
+  return slot.choice;
 }
 
 // One launch of the tcgen05 kernel by the plan pl. fa: one token still to be rotated and quantized (xq and scale unused).
 int launch_umma(const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16, int M, int N, int K,
                 void* y_f16, void* workspace, cudaStream_t st, const UmmaPlan& pl, const FusedAct* fa, int32_t* S_out, bool late) {
+  if (pl.tokens != M || pl.stages < 2 || pl.smem > kSmemMax) return RCP_ERR_SHAPE;   // (never: the layout is made for so many tokens)
   int gpc[rcp::kMaxPhases] = {};
   for (int i = 0; i < pl.nphase; i++) {   // (five phases at most)
     gpc[i] = pl.phase[i].gpc;
@@ -748,13 +765,12 @@ int launch_umma(const uint32_t* words, const void* lut_f16, const uint8_t* xq, c
 
 int launch_umma_passes(const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16, int M, int N, int K,
                        void* y_f16, void* workspace, cudaStream_t st, int32_t* S_out, bool late) {
-  const int mp = umma_choice(M, N, K, 0).tokens;
-  if (!mp) return RCP_ERR_VARIANT;
-  for (int m0 = 0; m0 < M; m0 += mp) {
-    const int mm = std::min(mp, M - m0);
-    const UmmaPlan& pl = m0 == 0 ? umma_choice(M, N, K, 0).plan : umma_choice(mm, N, K, 0).plan;   // (fewer tokens fit, too)
-    const int rc = launch_umma(words, lut_f16, xq + (size_t)m0 * (K / 2), static_cast<const __half*>(scale_f16) + m0, mm, N, K,
-                               static_cast<__half*>(y_f16) + (size_t)m0 * N, workspace, st, pl, nullptr,
+  const UmmaChoice& c = umma_choice(M, N, K, 0);
+  if (!c.launches) return RCP_ERR_VARIANT;
+  for (int i = 0, m0 = 0; i < c.launches; i++, m0 += c.tokens) {
+    const int rc = launch_umma(words, lut_f16, xq + (size_t)m0 * (K / 2), static_cast<const __half*>(scale_f16) + m0,
+                               std::min(c.tokens, M - m0), N, K, static_cast<__half*>(y_f16) + (size_t)m0 * N, workspace, st,
+                               i + 1 < c.launches ? c.plan : c.last, nullptr,
                                S_out ? S_out + (size_t)m0 * N * 4 : nullptr, late);
     if (rc != RCP_OK) return rc;
   }
@@ -1200,6 +1216,33 @@ int rcp_gemv_plan(int M, int N, int K, int sms, int* out, int cap) {
   return n;
 }
 
+int rcp_gemv_umma_plan(int M, int N, int K, int sms, int had_block, int* out, int cap) {
+  if (!out && cap > 0) return RCP_ERR_NULL;
+  if (M < 1 || M > rcp::kMaxTokens || N < 1 || !k_ok(K)) return RCP_ERR_SHAPE;
+  if (sms <= 0) sms = 148;
+  if (had_block != 0 && !fused_ok(M, K, had_block)) return RCP_ERR_VARIANT;
+  UmmaChoice c;
+  umma_choose(M, N, K, sms, had_block != 0 && full_block(K, had_block) ? rcp::full_rotate_bytes(K) : 0, c);
+  int n = 0;
+  auto put = [&](long long v) { if (n < cap) out[n] = (int)v; n++; };
+  put(c.faster);
+  put(c.launches);
+  for (int i = 0; i < c.launches; i++) {
+    const UmmaPlan& pl = i + 1 < c.launches ? c.plan : c.last;
+    for (const long long v : {(long long)std::min(c.tokens, M - i * c.tokens), (long long)pl.tokens, (long long)pl.stages, (long long)pl.smem,
+                              (long long)pl.nchunk, (long long)pl.part_chunks, (long long)pl.kpl, (long long)pl.bhalf, (long long)pl.bstep,
+                              (long long)pl.bgroup, (long long)pl.lg_m2, (long long)pl.slots, (long long)pl.dcols, (long long)pl.nbuf,
+                              (long long)pl.helpers, (long long)pl.off_bar, (long long)pl.off_misc, (long long)pl.off_red, (long long)pl.red_bytes,
+                              (long long)pl.off_bs, (long long)pl.bs_bytes, (long long)pl.off_qbuf, (long long)pl.nphase})
+      put(v);
+    for (int j = 0; j < pl.nphase; j++) {
+      const rcp::UmmaPhase& ph = pl.phase[j];
+      for (const int v : {ph.gpc, ph.first, ph.total, ph.ncta, ph.reps, ph.kp, ph.items, ph.ncol}) put(v);
+    }
+  }
+  return n;
+}
+
 size_t rcp_gemv_workspace_bytes(int M, int N, int K) {
   if (M < 1 || M > rcp::kMaxTokens || N < 1 || !k_ok(K)) return 0;
   return 16;   // a status word for the kernels' bounded waits; no sums pass through global memory
@@ -1420,8 +1463,8 @@ int rcp_linear_w2a4_launches(int M, int N, int K, int had_block, int group) {
   if (group != 0 && group != 128) return 2;
   const int cap = group == 0 ? (M == 1 ? 2 : 16) : (M <= 2 ? 2 : 8);   // tokens per launch of the variant AUTO picks
   int nsplit = 1;
-  const int mp = group == 0 && umma_choice(M, N, K, 0).faster ? umma_choice(M, N, K, 0).tokens
-                 : (group != 0 || cap < 8) ? tokens_per_pass(M, K, cap) : tokens_and_parts(M, N, K, cap, sm_count(), &nsplit);
+  if (group == 0 && umma_choice(M, N, K, 0).faster) return 1 + umma_choice(M, N, K, 0).launches;
+  const int mp = (group != 0 || cap < 8) ? tokens_per_pass(M, K, cap) : tokens_and_parts(M, N, K, cap, sm_count(), &nsplit);
   return 1 + (M + mp - 1) / mp;
 }
 

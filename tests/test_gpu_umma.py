@@ -25,6 +25,37 @@ CASES = [(1, 64, 1), (17, 192, 3), (16, 512, 1), (129, 576, 7), (300, 2048, 4), 
          (2400, 14336, 16), (40, 65536, 7)]
 
 
+# several launches with an uneven last one (N, K, M): as many rows as make K in parts impossible
+UNEVEN = [(28672, 20800, 15), (28672, 20992, 15), (20000, 14336, 13)]
+
+
+def run_uneven(i):
+    N, K, M = UNEVEN[i]
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N + K)
+    words = torch.randint(-2 ** 31, 2 ** 31 - 1, (N, K // 16), dtype=torch.int32, device=DEV, generator=g)
+    lut = torch.sort(torch.randn(N, 4, device=DEV, generator=g) * 0.02, dim=1)[0].half()
+    xq = torch.randint(0, 256, (M, K // 2), dtype=torch.uint8, device=DEV, generator=g)
+    scale = (torch.rand(M, device=DEV, generator=g) * 0.1 + 0.01).half()
+    ws = rcp.make_workspace(M, N, K, DEV)
+    S = torch.full((M, N, 4), 77, dtype=torch.int32, device=DEV)
+    checked = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="umma", S_dbg=S)
+    y = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="umma")
+    torch.cuda.synchronize()
+    assert int(ws.abs().max()) == 0
+    assert torch.equal(y.view(torch.int16), checked.view(torch.int16))
+    want = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="simple")
+    assert torch.equal(y.view(torch.int16), want.view(torch.int16))
+    rows = torch.cat([torch.arange(0, N, 997, device=DEV), torch.tensor([N - 1], device=DEV)])
+    ref = oracle.gemv_w2a4(words[rows].cpu().numpy().view(np.uint32), f16_bits(lut[rows]), xq.cpu().numpy(), f16_bits(scale))
+    assert np.array_equal(S[:, rows].cpu().numpy(), ref["S"])
+
+
+@pytest.mark.parametrize("i", range(len(UNEVEN)), ids=["x".join(map(str, c)) for c in UNEVEN])
+def test_uneven_launches(i):
+    run_uneven(i)
+
+
 def run_case(i):
     N, K, M = CASES[i]
     codes, lut = synth.make_layer(N, K, 64, "uniform", 900 + i, device=DEV)
@@ -50,7 +81,8 @@ def test_sums_are_the_oracles(i):
 def test_guarded_build_reports_nothing():
     from paper_2502_15779_b200 import build
     env = dict(os.environ, RCP_W2A4_LIB=build.build_checked(), PYTHONPATH=os.pathsep.join([ROOT, os.path.join(ROOT, "tests")]))
-    subprocess.run([sys.executable, "-c", "import test_gpu_umma as t\nfor i in range(len(t.CASES)): t.run_case(i)"], check=True,
+    subprocess.run([sys.executable, "-c", "import test_gpu_umma as t\nfor i in range(len(t.CASES)): t.run_case(i)\n"
+                    "for i in range(len(t.UNEVEN)): t.run_uneven(i)"], check=True,
                    env=env, cwd=ROOT, timeout=900)
 
 
