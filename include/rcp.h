@@ -227,10 +227,10 @@ int rcp_gemv_plan(int M, int N, int K, int sms, int* out, int cap);
  * rcp_linear_w2a4) takes this kernel, out[1] launches (0: nothing fits); then per launch: its tokens, the tokens its plan is
  * made for, ring stages, shared-memory bytes, chunks of K, chunks whose activations are in shared memory at a time, chunks side
  * by side at most, the strides bhalf, bstep, bgroup of the activations in units of 16 bytes, log2 of the tokens rounded up,
- * tensor-memory slots of 128 columns, columns of an accumulator, sets of three accumulators, whether the second half of the
+ * tensor-memory slots of 128 columns, columns of an integer accumulator and of a set of three, sets, whether the second half of the
  * workers helps to convert, the offsets and sizes of the shared-memory areas (barriers, scales, reduction and its bytes,
  * activations and their bytes, quantizer), the number of phases; and per phase: groups per CTA at most, first group, groups,
- * CTAs, repetitions, chunks side by side, items per repetition, columns of the instruction.
+ * CTAs, repetitions, chunks side by side, items per repetition, columns of the integer and of the e4m3 instruction.
  */
 int rcp_gemv_umma_plan(int M, int N, int K, int sms, int had_block, int* out, int cap);
 

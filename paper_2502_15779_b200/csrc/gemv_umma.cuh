@@ -49,7 +49,8 @@ struct UmmaPhase {
   int gpc, first, total, ncta, reps, q, r;   // as in GemvPhase
   int kp;      // chunks of K side by side in the lanes (a power of two; 16 gpc kp <= 128)
   int items;   // per repetition: ceil(nchunk / kp)
-  int ncol;    // columns of the instruction: kp (M + 1), rounded up to 8 or a multiple of 16
+  int ncol;    // columns of the kind::i8 instructions: kp (M + 1), rounded up to 8 or a multiple of 16
+  int ncol_f8; // of the e4m3 one: 16 at least
   int inv_rows;   // ceil(2^16 / (16 gpc)): v / (16 gpc) == (v * inv_rows) >> 16 for v < 512
 };
 struct UmmaParams {
@@ -73,7 +74,9 @@ struct UmmaParams {
   int part_chunks;      // chunks of K whose activations are in shared memory at a time (nchunk: all; else one tile per CTA at most)
   int helpers;          // the last eight workers have no tokens to finish: they become converters
   int lg_m2;            // log2 of M rounded up to a power of two
-  int slots, dcols, nbuf;   // tensor memory: slots of 128 columns at the top, accumulators (3 dcols columns) nbuf times at the bottom
+  // tensor memory: slots of 128 columns at the top, at the bottom nbuf sets of accumulators (acc_cols: dcols columns for each integer
+  // reading, dcols or 16 for the e4m3 one behind them)
+  int slots, dcols, acc_cols, nbuf;
   int stages, ramp_clk;
   int off_bar, off_misc, off_red, off_bs, off_qbuf;
   int red_bytes, bs_bytes;
@@ -319,14 +322,14 @@ __global__ void __launch_bounds__(kUThreads, 1) gemv_umma_kernel(const __grid_co
     const uint32_t elected = elect_one() ? 1u : 0u;
     const uint32_t b_hi = (128u >> 4) | (1u << 14);   // eight columns further on: 128 bytes
     const uint32_t b0 = (bs >> 4) | ((uint32_t)p.bhalf << 16);
-    const uint32_t step = (uint32_t)p.bstep, half2 = 2u * (uint32_t)p.bhalf, dcols = (uint32_t)p.dcols;
+    const uint32_t step = (uint32_t)p.bstep, half2 = 2u * (uint32_t)p.bhalf, dcols = (uint32_t)p.dcols, acc_cols = (uint32_t)p.acc_cols;
     bool ok = true, ready = false;
     int slot = 0, buf = 0;
     uint32_t apar = 0, dpar = 0;
     for (int pi = 0; pi < p.nphase && ok; pi++) {
       const UmmaPhase ph = p.phase[pi];
       if (b >= ph.ncta) continue;
-      const uint32_t shape = ((uint32_t)(ph.ncol >> 3) << 17) | (8u << 24);   // 128 rows
+      const uint32_t shape = ((uint32_t)((which == 2 ? ph.ncol_f8 : ph.ncol) >> 3) << 17) | (8u << 24);   // 128 rows
       const uint32_t idesc = which == 2 ? (1u << 4) | shape                   // fp32 += e4m3 x e4m3
                                         : (2u << 4) | ((uint32_t)which << 7) | (1u << 10) | shape;   // int32 += u8 or s8 x s8
       if (!ready) { ok = mbar_wait_warp(bfull, 0); ready = true; }   // the activations, when everything else is at hand
@@ -335,7 +338,7 @@ __global__ void __launch_bounds__(kUThreads, 1) gemv_umma_kernel(const __grid_co
       uint32_t bpar = 0;
       for (int rp = 0; rp < ph.reps && ok; rp++) {
         ok = mbar_wait_warp(dempty0 + 8 * buf, dpar ^ 1u);
-        const uint32_t d = (uint32_t)(buf * 3 + which) * dcols;
+        const uint32_t d = (uint32_t)buf * acc_cols + (uint32_t)which * dcols;
         uint32_t b_lo = b0;
         int kp0 = 0;
         for (int it = 0; it < ph.items && ok; it++) {
@@ -573,7 +576,7 @@ __global__ void __launch_bounds__(kUThreads, 1) gemv_umma_kernel(const __grid_co
           ok = mbar_wait_warp(dfull0 + 8 * buf, dpar);
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t dA = t_lane + (uint32_t)(buf * 3 * p.dcols + kpA * R1), dB = dA + (uint32_t)((kpB - kpA) * R1);
+          const uint32_t dA = t_lane + (uint32_t)(buf * p.acc_cols + kpA * R1), dB = dA + (uint32_t)((kpB - kpA) * R1);
           USums t[kUTok];
           if (some) {
             uint32_t o[3], o2[3], v[3][4], v2[3][4];

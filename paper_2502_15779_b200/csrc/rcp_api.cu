@@ -279,7 +279,7 @@ int phase_maps(const uint32_t* words, int N, int K, int nphase, const int* gpcs,
 // GEMV on tcgen05: launch plan.
 struct UmmaPlan {
   int tokens;        // that it is made for
-  int nchunk, nphase, grid, kpl, lg_kpl, bgroup, bstep, bhalf, lg_m2, slots, dcols, nbuf, stages, helpers;
+  int nchunk, nphase, grid, kpl, lg_kpl, bgroup, bstep, bhalf, lg_m2, slots, dcols, acc_cols, nbuf, stages, helpers;
   rcp::UmmaPhase phase[rcp::kMaxPhases];
   int part_chunks;   // nchunk (rounded up to kpl): all of K at once
   long long clocks;  // estimate of its items
@@ -287,11 +287,14 @@ struct UmmaPlan {
   size_t smem;
 };
 
-// columns of the instruction for kp chunks side by side: a column per token and one of ones for each
+// Columns of the kind::i8 instructions for kp chunks side by side: a column per token and one of ones for each.
 int umma_columns(int M, int kp) {
   const int n = kp * (M + 1);
   return n <= 8 ? 8 : (n + 15) / 16 * 16;
 }
+// kind::f8f6f4 with 128 rows is specified for multiples of 16 columns alone. (Sixteen for all three: 57344x8192 at three tokens
+// 25.6 -> 26.2 us a call, half as many sets of accumulators fitting; for that one alone, no difference.)
+int umma_columns_f8(int ncol) { return std::max(16, ncol); }
 int floor_pow2(int v) { int p = 1; while (2 * p <= v) p *= 2; return p; }
 
 // stages 0: does not fit. qbuf: bytes of scratch for the quantizer inside.
@@ -340,6 +343,7 @@ UmmaPlan umma_plan_for(int M, int N, int K, int sms, size_t qbuf, int kp_max, in
     ph.gpc = g; ph.first = first; ph.total = n; ph.ncta = ncta; ph.reps = reps;
     ph.q = n / ncta; ph.r = n % ncta;
     ph.kp = kp_of(g); ph.items = items_of(g); ph.ncol = umma_columns(M, ph.kp);
+    ph.ncol_f8 = umma_columns_f8(ph.ncol);
     ph.inv_rows = (65536 + 16 * g - 1) / (16 * g);
     first += n * reps;
   };
@@ -361,8 +365,9 @@ UmmaPlan umma_plan_for(int M, int N, int K, int sms, size_t qbuf, int kp_max, in
   while ((1 << pl.lg_kpl) < pl.kpl) pl.lg_kpl++;
   while ((1 << pl.lg_m2) < M) pl.lg_m2++;
   pl.dcols = ncol;
-  pl.slots = 3 * ncol <= 128 ? 3 : 2;
-  pl.nbuf = std::min(rcp::kUMaxBuf, (512 - 128 * pl.slots) / (3 * ncol));
+  pl.acc_cols = 2 * ncol + umma_columns_f8(ncol);
+  pl.slots = pl.acc_cols <= 128 ? 3 : 2;
+  pl.nbuf = std::min(rcp::kUMaxBuf, (512 - 128 * pl.slots) / pl.acc_cols);
   // activations: odd strides (in 16 bytes) between the halves and two pieces more between the steps keep the quantizer's
   // narrow stores out of one another's banks
   pl.bhalf = (pl.kpl * (M + 1)) | 1;
@@ -372,14 +377,14 @@ UmmaPlan umma_plan_for(int M, int N, int K, int sms, size_t qbuf, int kp_max, in
   for (int i = 0; i < pl.nphase; i++) shared |= pl.phase[i].kp > 1;
   pl.red_bytes = shared ? M * 3 * rcp::kULanes * 4 : 0;
   const size_t bar_bytes = 8 * (2 * rcp::kUMaxStages + 2 * rcp::kUMaxSlots + 2 * rcp::kUMaxBuf + 3), misc_bytes = 256;
-  const size_t fixed = 1024 + bar_bytes + misc_bytes + pl.red_bytes + qbuf + 64 + 16 * ncol;
+  const size_t fixed = 1024 + bar_bytes + misc_bytes + pl.red_bytes + qbuf + 64 + 16 * umma_columns_f8(ncol);
   // as few parts of K as leave room for three stages (one part: for two)
   for (int n = parts ? 2 : 1; n <= (parts ? 8 : 1); n++) {
     pl.part_chunks = ((pl.nchunk + n - 1) / n + pl.kpl - 1) / pl.kpl * pl.kpl;
     const long long bytes = (long long)(pl.part_chunks / pl.kpl) * pl.bgroup * 16;
     const long long room = (long long)kSmemMax - (long long)fixed - bytes;
     pl.stages = room < 0 ? 0 : (int)std::min<long long>(rcp::kUMaxStages, room / rcp::kUItemBytes);
-    pl.bs_bytes = (int)std::min<long long>(bytes + 16 * ncol, 1 << 20);
+    pl.bs_bytes = (int)std::min<long long>(bytes + 16 * umma_columns_f8(ncol), 1 << 20);
     if (pl.stages >= (parts ? 3 : 2)) break;
     pl.stages = 0;
   }
@@ -734,7 +739,7 @@ int launch_umma(const uint32_t* words, const void* lut_f16, const uint8_t* xq, c
   up.M = M; up.N = N; up.K = K; up.nchunk = pl.nchunk; up.nphase = pl.nphase;
   for (int i = 0; i < rcp::kMaxPhases; i++) up.phase[i] = pl.phase[i];
   up.kpl = pl.kpl; up.lg_kpl = pl.lg_kpl; up.bgroup = pl.bgroup; up.bstep = pl.bstep; up.bhalf = pl.bhalf; up.lg_m2 = pl.lg_m2; up.helpers = pl.helpers; up.part_chunks = pl.part_chunks;
-  up.slots = pl.slots; up.dcols = pl.dcols; up.nbuf = pl.nbuf; up.stages = pl.stages;
+  up.slots = pl.slots; up.dcols = pl.dcols; up.acc_cols = pl.acc_cols; up.nbuf = pl.nbuf; up.stages = pl.stages;
   // one item per CTA at about 6 TB/s for the whole grid, in SM clocks (about 2 GHz)
   up.ramp_clk = (int)((double)rcp::kUItemBytes * pl.grid / 6.0e12 * 1.9e9);
   up.off_bar = pl.off_bar; up.off_misc = pl.off_misc; up.off_red = pl.off_red; up.off_bs = pl.off_bs; up.off_qbuf = pl.off_qbuf;
@@ -1231,13 +1236,13 @@ int rcp_gemv_umma_plan(int M, int N, int K, int sms, int had_block, int* out, in
     const UmmaPlan& pl = i + 1 < c.launches ? c.plan : c.last;
     for (const long long v : {(long long)std::min(c.tokens, M - i * c.tokens), (long long)pl.tokens, (long long)pl.stages, (long long)pl.smem,
                               (long long)pl.nchunk, (long long)pl.part_chunks, (long long)pl.kpl, (long long)pl.bhalf, (long long)pl.bstep,
-                              (long long)pl.bgroup, (long long)pl.lg_m2, (long long)pl.slots, (long long)pl.dcols, (long long)pl.nbuf,
+                              (long long)pl.bgroup, (long long)pl.lg_m2, (long long)pl.slots, (long long)pl.dcols, (long long)pl.acc_cols, (long long)pl.nbuf,
                               (long long)pl.helpers, (long long)pl.off_bar, (long long)pl.off_misc, (long long)pl.off_red, (long long)pl.red_bytes,
                               (long long)pl.off_bs, (long long)pl.bs_bytes, (long long)pl.off_qbuf, (long long)pl.nphase})
       put(v);
     for (int j = 0; j < pl.nphase; j++) {
       const rcp::UmmaPhase& ph = pl.phase[j];
-      for (const int v : {ph.gpc, ph.first, ph.total, ph.ncta, ph.reps, ph.kp, ph.items, ph.ncol}) put(v);
+      for (const int v : {ph.gpc, ph.first, ph.total, ph.ncta, ph.reps, ph.kp, ph.items, ph.ncol, ph.ncol_f8}) put(v);
     }
   }
   return n;

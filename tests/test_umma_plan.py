@@ -7,7 +7,7 @@ import pytest
 from paper_2502_15779_b200 import build
 from gen.configs import CONFIGS
 
-FIELDS = ("launched tokens stages smem nchunk part_chunks kpl bhalf bstep bgroup lg_m2 slots dcols nbuf helpers off_bar off_misc "
+FIELDS = ("launched tokens stages smem nchunk part_chunks kpl bhalf bstep bgroup lg_m2 slots dcols acc_cols nbuf helpers off_bar off_misc "
           "off_red red_bytes off_bs bs_bytes off_qbuf nphase").split()
 ITEM = 128 * 128        # an item of the ring: 128 lanes of 128 bytes
 
@@ -27,8 +27,8 @@ def plan(L, M, N, K, sms=148, block=0):
     for _ in range(buf[1]):
         p = dict(zip(FIELDS, buf[at:at + len(FIELDS)]))
         at += len(FIELDS)
-        p["phases"] = [tuple(buf[at + 8 * i: at + 8 * i + 8]) for i in range(p["nphase"])]
-        at += 8 * p["nphase"]
+        p["phases"] = [tuple(buf[at + 9 * i: at + 9 * i + 9]) for i in range(p["nphase"])]
+        at += 9 * p["nphase"]
         launches.append(p)
     assert at == n
     return bool(buf[0]), launches
@@ -44,20 +44,22 @@ def check(L, M, N, K, sms=148, block=0, qbytes=0):
         assert 1 << p["lg_m2"] >= m > (1 << p["lg_m2"]) // 2
         nxt, chunks = 0, -(-K // 512)
         assert p["nchunk"] == chunks and 1 <= p["nphase"] <= 5
-        for gpc, first, total, ncta, reps, kp, items, ncol in p["phases"]:   # every group of 16 rows once, in order
+        for gpc, first, total, ncta, reps, kp, items, ncol, ncol_f8 in p["phases"]:   # every group of 16 rows once, in order
             assert first == nxt and 1 <= ncta <= sms and -(-total // ncta) <= gpc <= 8
             assert gpc * kp <= 8 and kp & (kp - 1) == 0 and kp <= p["kpl"] and kp * items >= chunks > kp * (items - 1)
-            assert ncol >= kp * (m + 1) and ncol <= p["dcols"] <= 256
+            # with 128 rows: kind::i8 takes 8 or a multiple of 16 columns, kind::f8f6f4 a multiple of 16
+            assert ncol >= kp * (m + 1) and ncol <= p["dcols"] <= 256 and (ncol == 8 or ncol % 16 == 0)
+            assert ncol_f8 >= ncol and ncol_f8 % 16 == 0 and ncol_f8 >= 16 and 2 * p["dcols"] + ncol_f8 <= p["acc_cols"]
             nxt += total * reps
         assert nxt == -(-N // 16)
         # tensor memory: slots of 128 columns at the top, sets of three accumulators below
-        assert 2 <= p["slots"] <= 3 and 1 <= p["nbuf"] <= 4 and 128 * p["slots"] + 3 * p["dcols"] * p["nbuf"] <= 512
+        assert 2 <= p["slots"] <= 3 and 1 <= p["nbuf"] <= 4 and 128 * p["slots"] + p["acc_cols"] * p["nbuf"] <= 512
         # activations: rows of a half, halves of a step and steps of a group of chunks do not overlap; the last group is whole
         assert p["bhalf"] >= p["kpl"] * (m + 1) and p["bstep"] >= 8 * p["bhalf"] and p["bgroup"] >= 4 * p["bstep"]
         parts = -(-chunks // p["part_chunks"])
         assert p["part_chunks"] % p["kpl"] == 0 or parts == 1
         groups = -(-min(chunks, p["part_chunks"]) // p["kpl"])
-        assert p["bs_bytes"] >= (groups * p["bgroup"] + p["dcols"]) * 16
+        assert p["bs_bytes"] >= (groups * p["bgroup"] + max(ph[8] for ph in p["phases"])) * 16
         if parts > 1:
             assert p["nphase"] == 1 and p["phases"][0][4] == 1 and not block and p["part_chunks"] % p["phases"][0][5] == 0
         # shared memory
