@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(kUThreads, 1) gemv_umma_kernel(const __grid_co
       const uint32_t t_lane = (uint32_t)(quad * 32) << 16;
       int* const red = reinterpret_cast<int*>(gen + p.off_red) + m0 * 3 * kULanes;   // [token][3][128]
       bool ok = !bad;
-      int buf = 0;
+      int buf = 0, met = 0;   // met: tiles at whose barriers this warp has met the other three of its tokens
       uint32_t dpar = 0;
       auto finish = [&](int m, int row, uint2 lut4, const USums& t) {
         const int S3 = t.t3, S1 = t.t1 - t.t3, S2 = t.t2 - t.t3, S0 = s_T0tot[m] - S1 - S2 - S3;
@@ -574,6 +574,10 @@ __global__ void __launch_bounds__(kUThreads, 1) gemv_umma_kernel(const __grid_co
           const int mine = ph.kp == 1 ? L : L - kp * rows;  // the row whose grid this lane fetches ahead
           const uint2 lut4 = mine < nrow ? __ldg(p.lut + row0 + mine) : make_uint2(0, 0);
           ok = mbar_wait_warp(dfull0 + 8 * buf, dpar);
+#ifdef RCP_CHECKED
+          // (a test's way to let this warp's wait give up)
+          if (p.status && __shfl_sync(0xffffffffu, *(volatile int32_t*)p.status, 0) == -1 - warp) ok = false;
+#endif
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t dA = t_lane + (uint32_t)(buf * p.acc_cols + kpA * R1), dB = dA + (uint32_t)((kpB - kpA) * R1);
@@ -634,11 +638,21 @@ __global__ void __launch_bounds__(kUThreads, 1) gemv_umma_kernel(const __grid_co
               }
             }
             asm volatile("bar.sync %0, 128;" ::"r"(4 + (warp >> 2)) : "memory");
+            met++;
           }
           if (++buf == nbuf) { buf = 0; dpar ^= 1u; }
         }
       }
-      if (!ok && lane == 0 && p.status) atomicExch(p.status, 3);
+      if (!ok) {
+        if (lane == 0 && p.status) atomicExch(p.status, 3);
+        // the other three may have made it: they are not left alone at the barriers of the tiles still to come
+        int left = -2 * met;   // (two a tile)
+#pragma unroll 1
+        for (int pi = 0; pi < p.nphase; pi++)
+          if (b < p.phase[pi].ncta && p.phase[pi].kp > 1) left += 2 * p.phase[pi].reps;
+#pragma unroll 1
+        for (; left > 0; left--) asm volatile("bar.sync %0, 128;" ::"r"(4 + (warp >> 2)) : "memory");
+      }
     }
   }
   // When the next kernel may start: as in gemv_stream_kernel.

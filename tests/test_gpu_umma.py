@@ -78,12 +78,38 @@ def test_sums_are_the_oracles(i):
     run_case(i)
 
 
-def test_guarded_build_reports_nothing():
+def in_guarded_build(what):
     from paper_2502_15779_b200 import build
     env = dict(os.environ, RCP_W2A4_LIB=build.build_checked(), PYTHONPATH=os.pathsep.join([ROOT, os.path.join(ROOT, "tests")]))
-    subprocess.run([sys.executable, "-c", "import test_gpu_umma as t\nfor i in range(len(t.CASES)): t.run_case(i)\n"
-                    "for i in range(len(t.UNEVEN)): t.run_uneven(i)"], check=True,
-                   env=env, cwd=ROOT, timeout=900)
+    subprocess.run([sys.executable, "-c", "import test_gpu_umma as t\n" + what], check=True, env=env, cwd=ROOT, timeout=900)
+
+
+def test_guarded_build_reports_nothing():
+    in_guarded_build("for i in range(len(t.CASES)): t.run_case(i)\nfor i in range(len(t.UNEVEN)): t.run_uneven(i)")
+
+
+# A worker whose wait gives up (in the guarded build the status word can ask one for it) leaves with the code, and the other three
+# warps of its tokens are not left at the barriers where the lane blocks of a row add up. One tile per CTA: nothing else waits.
+def run_one_warp_gives_up():
+    for N, K, M, warps in [(300, 4096, 1, (0, 3)), (2368, 8192, 3, (2,)), (500, 4096, 16, (5, 15))]:
+        codes, lut = synth.make_layer(N, K, 64, "uniform", 5, device=DEV)
+        words = rcp.rcp_pack_weights(codes)
+        xq, scale = rcp.rcp_quantize_act(synth.make_activations(M, K, 5, device=DEV), 64, 1.0)
+        ws = rcp.make_workspace(M, N, K, DEV)
+        want = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="umma")
+        for warp in warps:
+            ws[0] = -1 - warp
+            rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="umma")
+            torch.cuda.synchronize()
+            assert int(ws[0]) == 3
+            ws.zero_()
+        y = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="umma")
+        torch.cuda.synchronize()
+        assert int(ws.abs().max()) == 0 and torch.equal(y.view(torch.int16), want.view(torch.int16))
+
+
+def test_one_warp_gives_up():
+    in_guarded_build("t.run_one_warp_gives_up()")
 
 
 # Rings of two and three stages, whose stages are filled again as soon as they have been read: the sums of many calls in a row
