@@ -223,8 +223,8 @@ int rcp_gemv_plan(int M, int N, int K, int sms, int* out, int cap);
 
 /*
  * The same for the tcgen05 kernel (RCP_GEMV_UMMA). had_block 0: the form on given activations; otherwise the one that
- * rcp_linear_w2a4 runs with the quantizer inside (RCP_ERR_VARIANT where it has none). out[0] whether rcp_gemv_w2a4 (or
- * rcp_linear_w2a4) takes this kernel, out[1] launches (0: nothing fits); then per launch: its tokens, the tokens its plan is
+ * rcp_linear_w2a4 runs with the quantizer inside (RCP_ERR_VARIANT where it has none). out[0] whether the library
+ * takes this kernel: 1 (rcp_gemv_w2a4) + 2 (rcp_linear_w2a4; with had_block 0: behind a quantizer in front of it), out[1] launches (0: nothing fits); then per launch: its tokens, the tokens its plan is
  * made for, ring stages, shared-memory bytes, chunks of K, chunks whose activations are in shared memory at a time, chunks side
  * by side at most, the strides bhalf, bstep, bgroup of the activations in units of 16 bytes, log2 of the tokens rounded up,
  * tensor-memory slots of 128 columns, columns of an integer accumulator and of a set of three, sets, whether the second half of the

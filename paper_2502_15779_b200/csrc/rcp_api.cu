@@ -311,10 +311,10 @@ UmmaPlan umma_plan_for(int M, int N, int K, int sms, size_t qbuf, int kp_max, in
   while (kp_cap > 1 && (umma_columns(M, kp_cap) > max_cols || kp_cap >= 2 * pl.nchunk)) kp_cap /= 2;
   auto kp_of = [&](int g) { return std::min(kp_cap, floor_pow2(8 / g)); };
   auto items_of = [&](int g) { return (pl.nchunk + kp_of(g) - 1) / kp_of(g); };
-  auto cost_of = [&](int g) {
-    const int ncol = umma_columns(M, kp_of(g));
-    return (long long)items_of(g) * std::max(std::max(720 * g * kp_of(g) / 8, max_cols > 32 ? 860 : 600), 24 * ncol) + 400;
+  auto item_of = [&](int g, int hbm) {
+    return (long long)std::max(std::max(hbm * g * kp_of(g) / 8, max_cols > 32 ? 860 : 600), 24 * umma_columns(M, kp_of(g)));
   };
+  auto cost_of = [&](int g) { return items_of(g) * item_of(g, 720) + 400; };
   const int groups = (N + 15) / 16, per_round = 8 * sms, rounds = groups / per_round, left0 = groups - rounds * per_round;
   *total = 0;
   if (parts && groups > per_round) return pl;   // K in parts: one tile per CTA
@@ -389,6 +389,11 @@ UmmaPlan umma_plan_for(int M, int N, int K, int sms, size_t qbuf, int kp_max, in
     pl.stages = 0;
   }
   if (!pl.stages) return pl;
+  // Two stages do not keep enough requests in flight for 720 clocks an item (12288x20800, us a call: 22.0 at six tokens with three
+  // stages, 30.3 at eight with two).
+  if (pl.stages == 2)
+    for (int i = 0; i < pl.nphase; i++)
+      pl.clocks += pl.phase[i].reps * pl.phase[i].items * (item_of(pl.phase[i].gpc, 1100) - item_of(pl.phase[i].gpc, 720));
   // Up to eight tokens are finished by half of the workers; the others help to convert. Two teams want a ring of five stages:
   // a team that waits for a stage's next fill must know that the one before has come, and it does know that of the items five
   // back (their slots were free before it wrote its last).
@@ -657,7 +662,7 @@ int launch_umma_f(const rcp::GemvMaps& maps, const rcp::UmmaParams& up, const Um
 }
 
 // What the host works out for a call of M tokens, see umma_choose.
-struct UmmaChoice { UmmaPlan plan, last; int tokens, launches; bool faster; };
+struct UmmaChoice { UmmaPlan plan, last; int tokens, launches; bool faster, faster_late; };   // late: behind a quantizer of its own
 
 // Whether the tcgen05 kernel is the faster one, its host-side plan against the streaming kernel's. In clocks of an SM: the
 // streaming kernels take 77 a KB of weights for one token, 80 for up to eight, 171 for sixteen in one launch; the tcgen05
@@ -668,13 +673,26 @@ struct UmmaChoice { UmmaPlan plan, last; int tokens, launches; bool faster; };
 // 4096x4096 3.9 -> 5.2, 10240x8192 9.9 -> 9.5, 57344x8192 33.2 -> 27.0; three 10007x4096 8.3 -> 8.8, 10240x8192 13.7 -> 11.8,
 // 57344x8192 42.2 -> 29.1; eight 22016x4096 12.3 -> 13.4, 8192x28672 32.2 -> 29.5, 57344x8192 41.1 -> 33.2; sixteen 6144x4096
 // 9.7 -> 11.3, 12288x4096 13.5 -> 12.2, 28672x4096 23.9 -> 16.9, 57344x8192 78.5 -> 42.
-bool umma_faster(int M, int N, int K, int sms, const UmmaChoice& c) {
+// Up to eight tokens it also prepares their activations more slowly than the streaming kernels: all of K before the first
+// instruction, and behind a quantizer (`late`) nothing hides that, least of all behind the clusters that quantize long tokens
+// (a linear call takes up to 5.4 us longer than the plain one there, 2.7 on the streaming kernels; four tokens and more, or tokens a
+// power of two apart). Hence a second comparison with a charge that grows with tokens x channels, where going through K in parts
+// costs the streaming kernels 4500 clocks each. Set from 800 shapes of 1 to 90000 rows (a linear call, streaming -> tcgen05: 2368x28672 at
+// three tokens 11.4 -> 13.1, 5000x24576 at six 22.0 -> 25.4, 5000x40960 at eight 34.5 -> 38.4, 10240x12288 at five 16.5 -> 18.4, which stay on the
+// streaming kernels; 9001x28672 at three 25.4 -> 20.9, at eight 31.2 -> 28.8, 12288x14336 at four 20.7 -> 19.0, which do not). Without it the
+// worst of them took 1.15 times as long; with it none takes more than 1.03.
+bool umma_faster(int M, int N, int K, int sms, const UmmaChoice& c, bool late) {
   int nsplit = 1;
   const int ms = M == 1 ? 1 : tokens_and_parts(M, N, K, 16, sms, &nsplit);
   const long long kb = (long long)(((N + 15) / 16 + sms - 1) / sms) * K / 256;   // of the CTA with the most rows
   const long long per_launch = 2500, streaming = (M + ms - 1) / ms * (kb * (M == 1 ? 77 : ms <= 8 ? 80 : 171) + per_launch);
   const long long slower = M == 1 ? 11000 : M <= 3 ? 3000 : M <= 8 ? 6000 : 7200;
-  return c.launches * (c.plan.clocks + per_launch) + slower < streaming;
+  const long long own = c.launches * (c.plan.clocks + per_launch), mk = (long long)M * K;
+  if (own + slower >= streaming) return false;
+  if (M == 1 || M > 8) return true;
+  if (!late) return own + 3000 + mk * 2 / 100 < streaming;
+  const int cluster = K > 8192 && (M > 3 || (K & (K - 1)) == 0) ? 2000 : 0;
+  return own + 2000 + mk * 7 / 100 + cluster < streaming + (nsplit <= 4 ? (nsplit - 1) * 4500 : 0);
 }
 
 // A call of M tokens: launches of `tokens` of them each (as many as fit beside a ring of two
@@ -682,7 +700,7 @@ bool umma_faster(int M, int N, int K, int sms, const UmmaChoice& c) {
 // faster than the streaming kernels.
 void umma_choose(int M, int N, int K, int sms, size_t qbuf, UmmaChoice& c) {
   c.tokens = c.launches = 0;
-  c.faster = false;
+  c.faster = c.faster_late = false;
   for (int parts = 1; parts <= M && !c.launches; parts++) {
     const int m = (M + parts - 1) / parts, n = (M + m - 1) / m, rest = M - (n - 1) * m;
     c.plan = make_umma_plan(m, N, K, sms, qbuf);
@@ -695,7 +713,10 @@ void umma_choose(int M, int N, int K, int sms, size_t qbuf, UmmaChoice& c) {
     c.tokens = m;
     c.launches = n;
   }
-  if (c.launches) c.faster = umma_faster(M, N, K, sms, c);
+  if (c.launches) {
+    c.faster = umma_faster(M, N, K, sms, c, false);
+    c.faster_late = umma_faster(M, N, K, sms, c, true);
+  }
 }
 // The same, remembered per thread like the streaming kernels' plans.
 const UmmaChoice& umma_choice(int M, int N, int K, size_t qbuf) {
@@ -1230,7 +1251,7 @@ int rcp_gemv_umma_plan(int M, int N, int K, int sms, int had_block, int* out, in
   umma_choose(M, N, K, sms, had_block != 0 && full_block(K, had_block) ? rcp::full_rotate_bytes(K) : 0, c);
   int n = 0;
   auto put = [&](long long v) { if (n < cap) out[n] = (int)v; n++; };
-  put(c.faster);
+  put(c.faster + 2 * c.faster_late);
   put(c.launches);
   for (int i = 0; i < c.launches; i++) {
     const UmmaPlan& pl = i + 1 < c.launches ? c.plan : c.last;
@@ -1253,7 +1274,11 @@ size_t rcp_gemv_workspace_bytes(int M, int N, int K) {
   return 16;   // a status word for the kernels' bounded waits; no sums pass through global memory
 }
 
-static int auto_variant(int M, int N, int K) { return umma_choice(M, N, K, 0).faster ? RCP_GEMV_UMMA : M == 1 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY; }
+// The kernel for a call, as measured on B200: umma_faster; otherwise one token runs fastest on the CUDA cores, more tokens on mma.sync.
+static int auto_variant(int M, int N, int K, bool late_start) {
+  const UmmaChoice& c = umma_choice(M, N, K, 0);
+  return (late_start ? c.faster_late : c.faster) ? RCP_GEMV_UMMA : M == 1 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY;
+}
 
 // late_start: the call quantizes its activations itself (see the end of gemv_stream_kernel)
 static int gemv_w2a4(int variant, const uint32_t* words, const void* lut_f16, const uint8_t* xq, const void* scale_f16, int M,
@@ -1269,8 +1294,7 @@ static int gemv_w2a4(int variant, const uint32_t* words, const void* lut_f16, co
   // S_dbg without a variant of the caller's choice: the plain kernel. With one: the checked instantiation of
   // that streaming kernel, which stores the sums it finishes its rows from.
   if (S_dbg && variant == RCP_GEMV_AUTO) variant = RCP_GEMV_SIMPLE;
-  // measured on B200: one token runs fastest on the CUDA cores alone, more tokens on the tensor cores
-  if (variant == RCP_GEMV_AUTO) variant = auto_variant(M, N, K);
+  if (variant == RCP_GEMV_AUTO) variant = auto_variant(M, N, K, late_start);
   // the streaming kernels wait on barriers with a bound and report a wait that gave up through the workspace
   if (variant != RCP_GEMV_SIMPLE && !workspace) return RCP_ERR_WORKSPACE;
   switch (variant) {
@@ -1468,7 +1492,7 @@ int rcp_linear_w2a4_launches(int M, int N, int K, int had_block, int group) {
   if (group != 0 && group != 128) return 2;
   const int cap = group == 0 ? (M == 1 ? 2 : 16) : (M <= 2 ? 2 : 8);   // tokens per launch of the variant AUTO picks
   int nsplit = 1;
-  if (group == 0 && umma_choice(M, N, K, 0).faster) return 1 + umma_choice(M, N, K, 0).launches;
+  if (group == 0 && umma_choice(M, N, K, 0).faster_late) return 1 + umma_choice(M, N, K, 0).launches;
   const int mp = (group != 0 || cap < 8) ? tokens_per_pass(M, K, cap) : tokens_and_parts(M, N, K, cap, sm_count(), &nsplit);
   return 1 + (M + mp - 1) / mp;
 }
@@ -1505,7 +1529,7 @@ int rcp_linear_w2a4_checked(const void* x_f16, int M, int K, int had_block, floa
   if (rc != RCP_OK) return rc;
   // with S_dbg: the streaming kernel AUTO would pick, in its checked instantiation
   if (group == 0)
-    return gemv_w2a4(S_dbg ? auto_variant(M, N, K) : RCP_GEMV_AUTO, words, lut_f16, xq, scale_f16, M,
+    return gemv_w2a4(S_dbg ? auto_variant(M, N, K, true) : RCP_GEMV_AUTO, words, lut_f16, xq, scale_f16, M,
                      N, K, y_f16, workspace, S_dbg, stream, true);
   return gemv_w2a4_grouped(S_dbg && group == 128 ? (M <= 2 ? RCP_GEMV_DP4A : RCP_GEMV_MMA_ONLY) : RCP_GEMV_AUTO, words,
                            lut_f16, group, xq, scale_f16, M, N, K, y_f16, workspace, S_dbg, stream, true);

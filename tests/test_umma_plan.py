@@ -31,7 +31,7 @@ def plan(L, M, N, K, sms=148, block=0):
         at += 9 * p["nphase"]
         launches.append(p)
     assert at == n
-    return bool(buf[0]), launches
+    return buf[0], launches
 
 
 def check(L, M, N, K, sms=148, block=0, qbytes=0):
@@ -72,7 +72,7 @@ def check(L, M, N, K, sms=148, block=0, qbytes=0):
         assert p["off_bs"] % 16 == 0 and p["off_qbuf"] + qbytes + 1024 <= p["smem"] <= 232448
     if not block and sms == 148:
         n = L.rcp_linear_w2a4_launches(M, N, K, 1, 0)
-        if taken and M > 1:
+        if taken & 2 and M > 1:
             assert n == 1 + len(launches)
     return taken, launches
 
@@ -105,10 +105,29 @@ def test_plans_with_the_quantizer_inside(L):
             check(L, 1, N, K, block=B, qbytes=q)
 
 
+# Measured on B200: the first were slower on this kernel than on the streaming kernels (by 4 to 15 %; (rows, channels, tokens), as a
+# linear call with a quantizer kernel and as a call on given activations), the others are faster by 10 % and more.
+SLOWER_LINEAR = [(300, 28672, 3), (2368, 28672, 2), (2368, 28672, 3), (5000, 11008, 3), (5000, 20800, 6), (5000, 24576, 6), (5000, 40960, 8),
+                 (5000, 65536, 8), (9001, 14336, 8), (9001, 24576, 8), (12288, 14336, 8), (12288, 20800, 8), (7000, 16384, 2), (10240, 12288, 5),
+                 (10240, 16384, 5), (14000, 9216, 5)]
+SLOWER_PLAIN = [(2368, 28672, 3), (5000, 11008, 2), (5000, 24576, 6), (5000, 40960, 8), (5000, 65536, 8), (12288, 20800, 8)]
+FASTER_BOTH = [(57344, 8192, 2), (57344, 8192, 3), (57344, 8192, 8), (57344, 8192, 16), (8192, 28672, 3), (28672, 4096, 16), (9001, 28672, 3),
+               (12288, 20800, 4), (8192, 28672, 8), (9001, 28672, 8), (5000, 28672, 2), (20000, 5184, 3), (9001, 11008, 9), (12288, 4096, 12)]
+
+
+def test_the_choice_is_the_faster_kernel(L):
+    for N, K, M in SLOWER_LINEAR:
+        assert not plan(L, M, N, K)[0] & 2, (N, K, M)
+    for N, K, M in SLOWER_PLAIN:
+        assert not plan(L, M, N, K)[0] & 1, (N, K, M)
+    for N, K, M in FASTER_BOTH:
+        assert plan(L, M, N, K)[0] == 3, (N, K, M)
+
+
 def test_uneven_launches(L):
     # fewer tokens take more chunks side by side, which pads K: by themselves seven tokens would not fit where eight do
-    taken, launches = check(L, 15, 28672, 20992)
-    assert taken and [p["launched"] for p in launches] == [8, 7]
+    _, launches = check(L, 15, 28672, 20992)
+    assert [p["launched"] for p in launches] == [8, 7]
     assert launches[1]["bhalf"] >= 8 * launches[1]["kpl"]
 
 
