@@ -185,12 +185,13 @@ __global__ void __launch_bounds__(kUThreads, 1) gemv_umma_kernel(const __grid_co
 #ifdef RCP_CHECKED
   auto ck_fail = [&](int site) { if (p.status) atomicMax(p.status, 16 + site); };
 #endif
-  if constexpr (!LATE) asm volatile("griddepcontrol.launch_dependents;");
   // The producer sets up the barriers and only announces that; the first issuer takes all of the tensor memory (which
-  // therefore starts at column 0).
+  // therefore starts at column 0). The next kernel may start when every CTA has it, not before: one that fits beside these CTAs and
+  // takes tensor memory of its own in front of its wait for this kernel would keep a CTA waiting that it waits for.
   if (warp == kUFirstIssue) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (!LATE) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
   // Barriers and tensor memory: the producer only announces, converters and issuers wait, the workers learn of it from the
   // first issuer when they have prepared the activations.

@@ -1,6 +1,7 @@
 """The GEMV on the fifth-generation tensor cores (variant "umma"): exact sums against the oracle at the edges of its tiles, of its
 columns and of what fits in shared memory, in the production and in the guarded build; the linear call whose quantizer is inside
-that kernel; and the host's choice between the kernels."""
+that kernel; and its neighbours on the stream. (The host's plans and its choice between the kernels: test_umma_plan.py.)"""
+import ctypes as C
 import os
 import subprocess
 import sys
@@ -134,6 +135,66 @@ def test_a_short_ring_keeps_what_is_being_read(N, K, M):
         assert int(ws.abs().max()) == 0
         assert torch.equal(S, want), f"repetition {rep}"
         assert all(torch.equal(out.view(torch.int16), y.view(torch.int16)) for out in ys), f"repetition {rep}"
+
+
+# Somebody else's small kernel behind a call, let in early, that takes all of the tensor memory of an SM before it waits for that
+# call: it gets it when the call's CTA has given it back.
+BEHIND = r"""
+#include <cuda_runtime.h>
+__global__ void behind(const short* y, short* copy, int n) {
+  __shared__ unsigned at;
+  const unsigned a = (unsigned)__cvta_generic_to_shared(&at);
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(a) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  for (int i = blockIdx.x * 32 + threadIdx.x; i < n; i += gridDim.x * 32) copy[i] = ((volatile const short*)y)[i];
+  __syncwarp();
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(*(volatile unsigned*)&at) : "memory");
+}
+extern "C" int run_behind(const void* y, void* copy, int n, void* stream) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(148);
+  c.blockDim = dim3(32);
+  c.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return (int)cudaLaunchKernelEx(&c, behind, (const short*)y, (short*)copy, n);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def run_behind(tmp_path_factory):
+    d = tmp_path_factory.mktemp("behind")
+    (d / "b.cu").write_text(BEHIND)
+    subprocess.run([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-O2", "--shared",
+                    "-Xcompiler", "-fPIC", "-o", str(d / "b.so"), str(d / "b.cu")], check=True)
+    lib = C.CDLL(str(d / "b.so"))
+    lib.run_behind.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p]
+    return lib.run_behind
+
+
+@pytest.mark.parametrize("N,K,M", [(40, 128, 1), (2368, 2048, 3), (57344, 8192, 1), (300, 28672, 8)])
+def test_a_kernel_behind_that_takes_tensor_memory(run_behind, N, K, M):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N)
+    words = torch.randint(-2 ** 31, 2 ** 31 - 1, (N, K // 16), dtype=torch.int32, device=DEV, generator=g)
+    lut = torch.sort(torch.randn(N, 4, device=DEV, generator=g) * 0.02, dim=1)[0].half()
+    xq = torch.randint(0, 256, (M, K // 2), dtype=torch.uint8, device=DEV, generator=g)
+    scale = torch.full((M,), 0.1, dtype=torch.float16, device=DEV)
+    ws = rcp.make_workspace(M, N, K, DEV)
+    want = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="simple")
+    y, copy = torch.zeros_like(want), torch.zeros_like(want)
+    for rep in range(5):
+        y.zero_()
+        rcp.rcp_gemv_w2a4(words, lut, xq, scale, y=y, workspace=ws, variant="umma")
+        assert run_behind(y.data_ptr(), copy.data_ptr(), y.numel(), torch.cuda.current_stream().cuda_stream) == 0
+        torch.cuda.synchronize()
+        assert int(ws.abs().max()) == 0
+        assert torch.equal(copy.view(torch.int16), want.view(torch.int16)), rep
 
 
 # shapes whose linear call runs as one kernel of this kind (large ones), every form of the quantizer inside
