@@ -1,10 +1,11 @@
 """The GEMV on the fifth-generation tensor cores (variant "umma"): exact sums against the oracle at the edges of its tiles, of its
-columns and of what fits in shared memory, in the production and in the guarded build; the linear call whose quantizer is inside
-that kernel; and its neighbours on the stream. (The host's plans and its choice between the kernels: test_umma_plan.py.)"""
+columns and of what fits in shared memory, in the production and in the guarded build; linear calls that run it,
+with the quantizer inside and in front; and its neighbours on the stream. (The host's plans and its choice between the kernels: test_umma_plan.py.)"""
 import ctypes as C
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -12,6 +13,7 @@ import torch
 
 import oracle
 import paper_2502_15779_b200 as rcp
+import test_gpu_streams_threads as streams
 from gen import synth
 from helpers import f16_bits
 
@@ -24,6 +26,12 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CASES = [(1, 64, 1), (17, 192, 3), (16, 512, 1), (129, 576, 7), (300, 2048, 4), (2369, 1024, 2), (2368, 4096, 5), (4737, 1088, 9),
          (700, 8192, 8), (18945, 512, 1), (21300, 1024, 16), (333, 5184, 12), (64, 65536, 1), (300, 11008, 15), (300, 28672, 8),
          (2400, 14336, 16), (40, 65536, 7)]
+
+
+def taken(M, N, K, B):   # whether a linear call runs this kernel; B: with the quantizer for such blocks inside, 0: behind it
+    out = (C.c_int * 2)()
+    assert rcp.lib().rcp_gemv_umma_plan(M, N, K, 0, B, out, 2) > 2
+    return bool(out[0] & 2)
 
 
 # several launches with an uneven last one (N, K, M): as many rows as make K in parts impossible
@@ -207,6 +215,7 @@ def test_linear_with_the_quantizer_inside(N, K, B):
     lut = torch.sort(torch.randn(N, 4, device=DEV, generator=g) * 0.02, dim=1)[0].half()
     x = synth.make_activations(1, K, 5, device=DEV)
     ws = rcp.make_workspace(1, N, K, DEV)
+    assert taken(1, N, K, B)
     xq, scale = rcp.rcp_quantize_act(x, B, 1.0)
     want = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="dp4a")
     xq2, scale2 = torch.zeros_like(xq), torch.zeros_like(scale)
@@ -217,6 +226,100 @@ def test_linear_with_the_quantizer_inside(N, K, B):
     assert np.array_equal(f16_bits(y), f16_bits(want))
     zero = rcp.rcp_linear_w2a4(torch.zeros_like(x), B, 1.0, words, lut, xq=xq2, scale=scale2, workspace=ws)
     assert not zero.any() and not xq2.any() and not scale2.any()
+
+
+# Linear calls that run this kernel (N, K, B, M): its quantizer-inside forms, and the forms behind a quantizer, K at once and in parts,
+# one and several launches. Results and sums, also those of the checked instantiations, are the plain kernel's.
+LINEARS = [(60000, 8192, 8192, 1), (90000, 4096, 4096, 1), (180000, 2048, 2048, 1), (90000, 5184, 64, 1), (40000, 11008, 128, 1),
+           (8192, 28672, 128, 1), (57344, 8192, 8192, 8), (8192, 28672, 128, 8), (28672, 4096, 4096, 16), (28672, 20992, 128, 15),
+           (5000, 28672, 128, 12), (5000, 65536, 128, 2)]
+
+
+def run_linear(i):
+    N, K, B, M = LINEARS[i]
+    inside = rcp.rcp_linear_w2a4_launches(M, N, K, B) == 1
+    assert taken(M, N, K, B if inside else 0)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N + M)
+    words = torch.randint(-2 ** 31, 2 ** 31 - 1, (N, K // 16), dtype=torch.int32, device=DEV, generator=g)
+    lut = torch.sort(torch.randn(N, 4, device=DEV, generator=g) * 0.02, dim=1)[0].half()
+    x = synth.make_activations(M, K, 6, device=DEV)
+    ws = rcp.make_workspace(M, N, K, DEV)
+    xq, scale = rcp.rcp_quantize_act(x, B, 1.0)
+    want_S, S = (torch.full((M, N, 4), v, dtype=torch.int32, device=DEV) for v in (1, 2))
+    want = rcp.rcp_gemv_w2a4(words, lut, xq, scale, workspace=ws, variant="simple", S_dbg=want_S)
+    for S_dbg in (None, S):
+        xq2, scale2 = torch.zeros_like(xq), torch.zeros_like(scale)
+        y = rcp.rcp_linear_w2a4(x, B, 1.0, words, lut, xq=xq2, scale=scale2, workspace=ws, S_dbg=S_dbg)
+        torch.cuda.synchronize()
+        assert int(ws.abs().max()) == 0
+        assert torch.equal(xq, xq2) and torch.equal(scale, scale2)
+        assert torch.equal(y.view(torch.int16), want.view(torch.int16))
+    assert torch.equal(S, want_S)
+
+
+@pytest.mark.parametrize("i", range(len(LINEARS)), ids=["x".join(map(str, c)) for c in LINEARS])
+def test_linear_calls(i):
+    run_linear(i)
+
+
+def test_linear_calls_in_the_guarded_build():
+    in_guarded_build("for i in range(len(t.LINEARS)): t.run_linear(i)")
+
+
+# Calls of this kernel beside one another and beside a streaming one: several streams, several host threads, a captured step
+BESIDE = [(57344, 8192, 8192, 1), (57344, 8192, 8192, 8), (8192, 28672, 128, 3), (4096, 4096, 4096, 1), (28672, 4096, 4096, 16)]
+
+
+def test_streams_threads_and_replays():
+    probs = [streams._problem(N, K, B, M, 700 + i) for i, (N, K, B, M) in enumerate(BESIDE)]
+    want = []
+    for p in probs:
+        streams._run(p)
+        torch.cuda.synchronize()
+        want.append(p["y"].clone())
+
+    def check(what):
+        torch.cuda.synchronize()
+        for p, w in zip(probs, want):
+            assert torch.equal(p["y"].view(torch.int16), w.view(torch.int16)), what
+            assert int(p["ws"].abs().max()) == 0
+            p["y"].zero_()
+        torch.cuda.synchronize()
+
+    lanes = [torch.cuda.Stream() for _ in probs]
+    for rep in range(20):
+        for p, st in zip(probs, lanes):
+            with torch.cuda.stream(st):
+                streams._run(p)
+    check("streams")
+    errors = []
+
+    def worker(p, st):
+        try:
+            torch.cuda.set_device(0)
+            with torch.cuda.stream(st):
+                for rep in range(30):
+                    streams._run(p)
+                st.synchronize()
+        except Exception as e:   # noqa: BLE001
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=worker, args=a) for a in zip(probs, lanes)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    check("threads")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for p in probs:
+            streams._run(p)
+    for rep in range(3):
+        graph.replay()
+        graph.replay()
+        check(f"replay {rep}")
 
 
 # Sums of fp32 products stay exact where they grow largest: every code 1 (the e4m3 reading is +2 throughout) against the largest
