@@ -80,8 +80,8 @@ int rcp_quantize_act(const void* x_f16, int M, int K, int had_block, float clip_
 
 /*
  * Kernel variants of the LUT GEMV (all compute the same result).
- *   RCP_GEMV_AUTO    library picks (as measured on B200): UMMA for large layers (how large depends on M), otherwise DP4A
- *                    for one token and MMA_ONLY for more.
+ *   RCP_GEMV_AUTO    library picks (as measured on B200): UMMA for large layers (how large depends on M and K; also few rows
+ *                    over a very long K), otherwise DP4A for one token and MMA_ONLY for more.
  *   RCP_GEMV_SIMPLE  one warp per output row, scalar decode; also the variant behind S_dbg.
  *   RCP_GEMV_DP4A    streaming kernel, CUDA cores only: masked code planes times int8 activations
  *                    with dp4a, two tokens per launch.
@@ -241,7 +241,8 @@ int rcp_gemv_umma_plan(int M, int N, int K, int sms, int had_block, int* out, in
  * Constraints: 1 <= M <= 16, N >= 1, K % 64 == 0, 64 <= K <= 65536.
  *   workspace  rcp_gemv_workspace_bytes(M,N,K) bytes, see above. Required (RCP_ERR_WORKSPACE without it): every
  *              wait inside the streaming kernels is bounded, and a wait that gives up writes a non-zero code
- *              into its first word (2: the weight producer, 3: a consumer warp) and ends the kernel; the
+ *              into its first word (2: the weight producer, 3: a consumer warp; RCP_GEMV_UMMA: 3 a converter or a warp that
+ *              finishes rows, 4 one that prepares activations, 5 one that issues instructions) and ends the kernel; the
  *              results of that call are then invalid. Only RCP_GEMV_SIMPLE (no waits) takes NULL.
  *   words, lut_f16 are the constants of the layer: the kernel may start fetching them while earlier
  *              work on the stream is still running (programmatic dependent launch), so that work

@@ -15,7 +15,8 @@
 // shifts per 16 codes, where the CUDA-core kernel needs 23 operations and the mma.sync kernels 18 and 6 MMA slots.
 // The activations are bytes 0..15, u = q + 8: as e4m3 such a byte is u / 512 (subnormals and the first binade are evenly
 // spaced), so one copy serves all three instructions. A column of ones beside the tokens measures what the + 8 adds.
-// Everything is exact: int32 sums, and fp32 sums of multiples of 2^-8 below 2^13.
+// The sums are exact: int32, and fp32 sums of multiples of 2^-8 below 2^13, 20 bits of 24. (That kind::f8f6f4 drops no bits below
+// its largest product while it adds is measured, at the ends of the range too, not documented.)
 //
 // Work. Groups of 16 rows are shared out over the CTAs in phases like in gemv_stream.cuh; an item is 128 lanes x 128
 // bytes of packed weights (16 KB): 16 gpc rows x kp chunks of K side by side in the lanes, each chunk with columns of its own
@@ -26,9 +27,10 @@
 // to a warp; up to eight tokens the last eight of them convert too). Slots of 128 columns (a whole item): with 64 the handshakes
 // cost 55 clocks per KB of weights, so 40, less than the 44 to 49 that HBM needs.
 // What it measured (B200, us a call of the whole linear in a chain, cold weights; before: dp4a for one token, mma.sync for more):
-// 57344x8192 at 1, 3, 8, 12, 16 tokens 33.2, 42.2, 41.1, 79.3, 78.5 -> 27.3, 29.1, 33.8, 35.9, 43.0; 28672x4096 at 16 23.9 -> 16.9;
-// 8192x28672 at 8 32.2 -> 29.5. Bound: HBM in the loop (an item per SM in 720 clocks is 6.4 TB/s) up to eight tokens; at
-// sixteen the 32 columns take 768 clocks an item; beside it some 5 us from launch to the first sums and from the last to y.
+// 57344x8192 at 1, 3, 8, 12, 16 tokens 30.5, 39.7, 38.8, 76.7, 75.7 -> 24.8, 28.1, 31.2, 33.5, 40.1; 28672x4096 at 16 23.7 -> 16.8;
+// 8192x28672 at 8 31.3 -> 28.5. Bound: HBM in the loop up to eight tokens (an item per SM in 720 clocks is 6.4 TB/s; four times the
+// weights, 28672x4096 at two tokens and 57344x8192 at one, take 14.2 us longer, 6.2 TB/s); at sixteen the 32 columns take 768 clocks
+// an item; beside it some 5 us from launch to the first sums and from the last to y.
 #pragma once
 #include "gemv_stream.cuh"
 

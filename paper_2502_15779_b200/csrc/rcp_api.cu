@@ -670,9 +670,9 @@ struct UmmaChoice { UmmaPlan plan, last; int tokens, launches; bool faster, fast
 // conversion, three instruction streams and the sums' way back through tensor memory lie on its path, and there is more
 // code to fetch; one token, whose calls are otherwise launches of one and the same kernel, most: layers of 54144x4096, 4447x896
 // and 1920x14336 took 55.9 -> 56.6 with the first of them here). us a linear call in a chain, streaming -> tcgen05: one token
-// 4096x4096 3.9 -> 5.2, 10240x8192 9.9 -> 9.5, 57344x8192 33.2 -> 27.0; three 10007x4096 8.3 -> 8.8, 10240x8192 13.7 -> 11.8,
-// 57344x8192 42.2 -> 29.1; eight 22016x4096 12.3 -> 13.4, 8192x28672 32.2 -> 29.5, 57344x8192 41.1 -> 33.2; sixteen 6144x4096
-// 9.7 -> 11.3, 12288x4096 13.5 -> 12.2, 28672x4096 23.9 -> 16.9, 57344x8192 78.5 -> 42.
+// 4096x4096 3.9 -> 5.2, 10240x8192 9.9 -> 9.5, 57344x8192 30.5 -> 24.8; three 10007x4096 8.3 -> 8.8, 10240x8192 13.3 -> 11.8,
+// 57344x8192 39.7 -> 28.1; eight 22016x4096 12.3 -> 13.4, 8192x28672 31.3 -> 28.5, 57344x8192 38.8 -> 31.2; sixteen 6144x4096
+// 9.7 -> 11.3, 12288x4096 14.7 -> 12.1, 28672x4096 23.7 -> 16.8, 57344x8192 75.7 -> 40.1.
 // Up to eight tokens it also prepares their activations more slowly than the streaming kernels: all of K before the first
 // instruction, and behind a quantizer (`late`) nothing hides that, least of all behind the clusters that quantize long tokens
 // (a linear call takes up to 5.4 us longer than the plain one there, 2.7 on the streaming kernels; four tokens and more, or tokens a
